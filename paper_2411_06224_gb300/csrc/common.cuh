@@ -158,7 +158,12 @@ int level0_bf16_launch(gs_ctx ctx, gs_mas mas, bool f32_node_major, int nrhs, co
 bool level0_f64tc_usable(gs_ctx ctx, gs_mas mas, int nrhs);
 // FP32 level-0 product from a bulk-copied inverse (mas_apply.cu)
 bool level0_f32_bulk_usable(gs_mas mas, int nrhs);
+// digit storage for every level, filled by invert_domains_launch; then what
+// other storage the context's GS_TUNE_F64_TC asks for, from the inverses
+int level0_f64tc_alloc(gs_ctx ctx, gs_mas mas);
 int level0_f64tc_prepare(gs_ctx ctx, gs_mas mas);
+// Inverts the level matrices in place and cuts their digit matrices (mas_invert.cu)
+int invert_domains_launch(gs_ctx ctx, gs_mas mas, double* fac0);
 // skip (device, may be null): the kernels return at once while *skip is set
 int level0_f64tc_launch(gs_ctx ctx, gs_mas mas, int nrhs, const double* r, int64_t stride, const double* zl,
                         int64_t lstride, double* z, const int* skip = nullptr);

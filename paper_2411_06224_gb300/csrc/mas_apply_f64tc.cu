@@ -69,44 +69,6 @@ __device__ __forceinline__ double scaled_to_double(long long hi, long long lo, i
   return combine_to_double(hi, lo, 32, e);
 }
 
-// Balanced base-256 digits of x (|x| < 2^55): x = sum_p d[p] 256^(6-p), d[0] the
-// most significant; d[1..6] in [-128, 127], |d[0]| <= 128.
-__device__ __forceinline__ void digits(long long x, int (&d)[kDigits]) {
-#pragma unroll
-  for (int p = kDigits - 1; p >= 1; --p) {
-    int t = (int)(x & 255);
-    if (t >= 128) t -= 256;
-    d[p] = t;
-    x = (x - t) >> 8;
-  }
-  d[0] = (int)x;
-}
-
-// Build time: digit matrices of the level-0 inverses.  One CTA per domain,
-// thread i = row i.  Output per domain: kDigits matrices of ld*ld BF16 in the
-// K-major operand layout [k/8][i/8][i%8][k%8], then the row exponents.
-__global__ void k_split_inverse(const double* __restrict__ inv, int ld, __nv_bfloat16* __restrict__ out,
-                                int32_t* __restrict__ row_exp) {
-  const int64_t d = blockIdx.x;
-  const int i = threadIdx.x;
-  if (i >= ld) return;
-  const double* Mi = inv + d * ld * ld + (int64_t)i * ld;
-  int emax = 0;
-  for (int k = 0; k < ld; ++k) emax = max(emax, biased_exp(Mi[k]));
-  const int a = emax - 1021;  // |M_ik| < 2^(emax - 1022) = 2^(a - 1)
-  row_exp[d * ld + i] = emax ? a : -100000;
-  __nv_bfloat16* base = out + d * kDigits * ld * ld;
-  const int groups = ld / 8;
-  for (int k = 0; k < ld; ++k) {
-    int dg[kDigits];
-    digits(emax ? scaled_rint(Mi[k], a) : 0, dg);
-    const int64_t pos = (int64_t)(k >> 3) * (groups * 64) + (i >> 3) * 64 + (i & 7) * 8 + (k & 7);
-#pragma unroll
-    for (int p = 0; p < kDigits; ++p) base[(int64_t)p * ld * ld + pos] = __int2bfloat16_rn(dg[p]);
-  }
-}
-
-
 // kCoarse = false: level 0, CTA = level-0 domain, r gathered through remap0,
 //   z = level-0 product + prolongated coarse results, written per node;
 // kCoarse = true: one coarse-level domain per CTA (job tables), r and z are the
@@ -630,32 +592,29 @@ bool level0_f64tc_usable(gs_ctx ctx, gs_mas mas, int nrhs) {
   return (t == 1 || t == 2 || t == 4) && !mas->dig64.empty();
 }
 
-int level0_f64tc_prepare(gs_ctx ctx, gs_mas mas) {
+int level0_f64tc_alloc(gs_ctx ctx, gs_mas mas) {
   const int ld = 3 * mas->N;
   const int t = ctx->tune[GS_TUNE_F64_TC];
-  if (mas->precision != GS_PREC_FP64 || t == 0) return GS_OK;
-  if (t == 3) return f64sym_shape_ok(mas->N) ? f64sym_prepare(ctx, mas) : GS_OK;  // 1, 2, 4: BF16 digits
-  if (ld % 16 != 0 || ld > f64tc::kM || !mas->dig64.empty()) return GS_OK;
+  if (t == 0 || t == 3 || ld % 16 != 0 || ld > f64tc::kM || !mas->dig64.empty()) return GS_OK;
   for (int l = 0; l < mas->L; ++l) {  // every level: level 0 and the coarse levels
-    const int64_t n_dom = mas->n_domains[l];
+    const size_t n_dom = (size_t)std::max(mas->n_domains[l], 1);
     void* dg = nullptr;
     int32_t* ex = nullptr;
-    GS_TRY(ctx->alloc(&dg, (size_t)std::max<int64_t>(n_dom, 1) * f64tc::kDigits * ld * ld * 2));
+    GS_TRY(ctx->alloc(&dg, n_dom * f64tc::kDigits * ld * ld * 2));
     mas->dig64.push_back(dg);
-    GS_TRY(ctx->alloc((void**)&ex, (size_t)std::max<int64_t>(n_dom, 1) * ld * 4));
+    GS_TRY(ctx->alloc((void**)&ex, n_dom * ld * 4));
     mas->dig64_exp.push_back(ex);
-    if (n_dom) {
-      GS_PROF(ctx, GS_K_MAS_INVERT);
-      f64tc::k_split_inverse<<<n_dom, ((ld + 31) / 32) * 32, 0, ctx->stream>>>(mas->inv64[l], ld,
-                                                                               (__nv_bfloat16*)dg, ex);
-    }
   }
   GS_TRY(ctx->alloc((void**)&mas->d_dig_tab, 16 * sizeof(void*)));
   std::vector<void*> hp(16, nullptr);
   for (int l = 0; l < mas->L; ++l) hp[l] = mas->dig64[l], hp[8 + l] = mas->dig64_exp[l];
   GS_CUDA(cudaMemcpyAsync(mas->d_dig_tab, hp.data(), 16 * sizeof(void*), cudaMemcpyHostToDevice, ctx->stream));
-  GS_CUDA(cudaGetLastError());
   return GS_OK;
+}
+
+int level0_f64tc_prepare(gs_ctx ctx, gs_mas mas) {  // 3: symmetric digit bytes; 1, 2, 4 were cut with the inverses
+  if (mas->precision != GS_PREC_FP64 || ctx->tune[GS_TUNE_F64_TC] != 3) return GS_OK;
+  return f64sym_shape_ok(mas->N) ? f64sym_prepare(ctx, mas) : GS_OK;
 }
 
 static f64tc::Levels f64tc_levels(gs_mas mas) {

@@ -19,9 +19,7 @@
 // level-0 domain are first summed per (item, item) pair of that domain --
 // one warp per domain, the paper's warp reduction -- and added atomically;
 // blocks between level-0 domains are added atomically one by one.
-// Inverses (Alg. 1 "invert unpadded parts"): one CTA per domain factorises
-// the real items' part in shared memory (Cholesky, FP64), inverts the
-// factor and forms L^-T L^-1, overwriting the matrix with its inverse.
+// Inverses (Alg. 1 "invert unpadded parts"): mas_invert.cu.
 #include <cub/device/device_scan.cuh>
 #include <cuda_bf16.h>
 
@@ -262,137 +260,6 @@ __global__ void k_domain_reduce(const int32_t* __restrict__ remap, int32_t n_dom
   }
 }
 
-// ------------------------------------------------------------------ inversion
-struct InvJob {
-  double* mat;              // 3N x 3N row-major, overwritten by the inverse
-  const int32_t* remap;     // level 0: slot -> node (-1 padding); nullptr for l >= 1
-  int32_t items_in_domain;  // l >= 1: real items of this domain
-};
-
-// One CTA per domain.  Shared memory holds the lower triangle of the
-// compacted real part, packed by rows (entry (i, j), j <= i, at
-// i (i + 1) / 2 + j: 37 KB at 3k = 96, so five CTAs share an SM), plus a
-// contiguous copy of the current Cholesky column.  The arithmetic is that of
-// the full-storage form, operation for operation.
-__device__ __forceinline__ int tri(int i, int j) { return i * (i + 1) / 2 + j; }
-
-__global__ void __launch_bounds__(256) k_invert_domains(double* const* mats,
-                                                         const int32_t* __restrict__ remap0, int32_t n_dom0,
-                                                         const int32_t* __restrict__ dom_level,
-                                                         const int32_t* __restrict__ dom_index,
-                                                         const int32_t* __restrict__ n_items, int N, int* flags,
-                                                         double* __restrict__ fac0) {
-  extern __shared__ double sA[];
-  __shared__ double colp[96];  // column p of the factor, rows p+1 ..
-  __shared__ int s_lane[32];
-  __shared__ int s_k;
-  __shared__ int s_bad;
-  __shared__ double s_rdiag;  // 1 / L_pp of the current Cholesky step
-  const int job = blockIdx.x;
-  const int l = dom_level[job];
-  const int d = dom_index[job];
-  const int ld = 3 * N;
-  double* M = mats[l] + (int64_t)d * ld * ld;
-  const int tid = threadIdx.x, T = blockDim.x;
-  const int lane = tid & 31, wid = tid >> 5, nw = T >> 5;
-  if (tid < 32) {
-    bool real;
-    if (l == 0)
-      real = tid < N && remap0[(int64_t)d * N + tid] >= 0;
-    else
-      real = tid < N && (int64_t)d * N + tid < n_items[l];
-    uint32_t rm = __ballot_sync(kFull, real);
-    if (real) s_lane[__popc(rm & ((1u << tid) - 1u))] = tid;
-    if (tid == 0) {
-      s_k = __popc(rm);
-      s_bad = 0;
-    }
-  }
-  __syncthreads();
-  const int k = s_k;
-  const int n3 = 3 * k;
-  if (k == 0) return;
-  // load the lower triangle of the compacted real part (a warp per row)
-  for (int i = wid; i < n3; i += nw) {
-    const int gi = 3 * s_lane[i / 3] + i % 3;
-    for (int j = lane; j <= i; j += 32) sA[tri(i, j)] = M[(int64_t)gi * ld + 3 * s_lane[j / 3] + j % 3];
-  }
-  __syncthreads();
-  // right-looking Cholesky, lower triangle.  FP64 is the scarce unit: one
-  // reciprocal per step (not one per thread), and the trailing update walks
-  // only the lower triangle (a warp per row, lanes along it, the column read
-  // from its contiguous copy).
-  for (int p = 0; p < n3; ++p) {
-    if (tid == 0) {
-      double dpp = sA[tri(p, p)];
-      if (!(dpp > 0.0)) {
-        s_bad = 1;
-        dpp = 1.0;
-      }
-      const double lpp = sqrt(dpp);
-      sA[tri(p, p)] = lpp;
-      s_rdiag = 1.0 / lpp;
-    }
-    __syncthreads();
-    if (s_bad) break;
-    const double inv = s_rdiag;
-    for (int i = p + 1 + tid; i < n3; i += T) {
-      const double v = sA[tri(i, p)] * inv;
-      sA[tri(i, p)] = v;
-      colp[i] = v;
-    }
-    __syncthreads();
-    for (int i = p + 1 + wid; i < n3; i += nw) {
-      const double lip = colp[i];
-      const int ri = tri(i, 0);
-      for (int j = p + 1 + lane; j <= i; j += 32) sA[ri + j] -= lip * colp[j];
-    }
-    __syncthreads();
-  }
-  if (s_bad) {
-    if (tid == 0) atomicOr(flags, kErrNotSPD);
-    return;
-  }
-  // W = L^{-1} in place.  The diagonal first becomes 1 / L_jj (= W_jj), then
-  // W_ij = -(sum_{q=j+1..i} W_iq L_qj) W_jj, column by column from the last.
-  for (int j = tid; j < n3; j += T) sA[tri(j, j)] = 1.0 / sA[tri(j, j)];
-  __syncthreads();
-  for (int j = n3 - 1; j >= 0; --j) {
-    const double wjj = sA[tri(j, j)];
-    double w = 0.0;
-    const int i = j + 1 + tid;
-    if (i < n3) {
-      double acc = 0.0;
-      const int ri = tri(i, 0);
-      for (int q = j + 1; q <= i; ++q) acc += sA[ri + q] * sA[tri(q, j)];
-      w = -acc * wjj;
-    }
-    __syncthreads();
-    if (i < n3) sA[tri(i, j)] = w;
-    __syncthreads();
-  }
-  // level 0, low-precision form: keep the factor W = L^{-1} (M^{-1} = W^T W)
-  if (fac0 && l == 0) {
-    double* F = fac0 + (int64_t)d * ld * ld;
-    for (int i = wid; i < n3; i += nw) {
-      const int gi = 3 * s_lane[i / 3] + i % 3;
-      for (int j = lane; j <= i; j += 32) F[(int64_t)gi * ld + 3 * s_lane[j / 3] + j % 3] = sA[tri(i, j)];
-    }
-  }
-  // inverse = W^T W, written over the real part of the global matrix; entry
-  // (i, j) and (j, i) are the same sum in the same order, so the lower
-  // triangle is computed and mirrored
-  for (int e = tid; e < n3 * n3; e += T) {
-    int i = e / n3, j = e % n3;
-    if (j > i) continue;
-    double acc = 0.0;
-    for (int q = i; q < n3; ++q) acc += sA[tri(q, i)] * sA[tri(q, j)];
-    int gi = 3 * s_lane[i / 3] + i % 3, gj = 3 * s_lane[j / 3] + j % 3;
-    M[(int64_t)gi * ld + gj] = acc;
-    M[(int64_t)gj * ld + gi] = acc;
-  }
-}
-
 __global__ void k_to_float(const double* __restrict__ a, float* __restrict__ b, int64_t n) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) b[i] = (float)a[i];
@@ -452,26 +319,6 @@ static int mas_numeric(gs_ctx ctx, gs_mas mas, gs_mat mat) {
   if (mat->nnzb > 0)
     { GS_PROF(ctx, GS_K_MAS_MATRICES); k_scatter_blocks<<<ceil_div(mat->nnzb, 256), 256, 0, st>>>(mat->rid, mat->cid, mat->au, mat->nnzb, lp); }
   if (L > 1) { GS_PROF(ctx, GS_K_MAS_MATRICES); k_domain_reduce<<<ceil_div((int64_t)n_dom0 * 32, 256), 256, 0, st>>>(mas->remap0, n_dom0, lp); }
-  // inversion jobs: every domain of every level
-  std::vector<int32_t> h_level, h_index;
-  for (int l = 0; l < L; ++l)
-    for (int32_t d = 0; d < mas->n_domains[l]; ++d) h_level.push_back(l), h_index.push_back(d);
-  const int jobs = (int)h_level.size();
-  int32_t* djobs = nullptr;
-  if ((s = ctx->scratch_buf(kSlotMasBuild3, (size_t)jobs * 8 + (L + 1) * 8 + 8 * sizeof(double*) + 64,
-                            (void**)&djobs)))
-    return s;
-  int32_t* d_items = djobs + 2 * jobs;
-  double** d_mats = (double**)(((uintptr_t)(d_items + L + 1) + 15) & ~(uintptr_t)15);
-  std::vector<double*> hm(mas->inv64.begin(), mas->inv64.end());
-  if (cudaMemcpyAsync(djobs, h_level.data(), jobs * 4, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-      cudaMemcpyAsync(djobs + jobs, h_index.data(), jobs * 4, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-      cudaMemcpyAsync(d_items, mas->n_items.data(), L * 4, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-      cudaMemcpyAsync(d_mats, hm.data(), L * sizeof(double*), cudaMemcpyHostToDevice, st) != cudaSuccess)
-    return GS_ERR_CUDA;
-  const size_t smem = (size_t)(3 * N) * (3 * N + 1) / 2 * sizeof(double);  // packed lower triangle
-  if (cudaFuncSetAttribute(k_invert_domains, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return GS_ERR_CUDA;
   // BF16 form: level 0 keeps its inverse Cholesky factors (rounding W keeps
   // W^T W positive semi-definite; rounding M^{-1} itself does not once a
   // domain's condition number passes ~1e3), coarse levels FP32 inverses
@@ -481,8 +328,9 @@ static int mas_numeric(gs_ctx ctx, gs_mas mas, gs_mat mat) {
     if ((s = ctx->alloc((void**)&fac0, (size_t)std::max<int64_t>(cnt0, 1) * 8))) return s;
     if (cudaMemsetAsync(fac0, 0, (size_t)cnt0 * 8, st) != cudaSuccess) return GS_ERR_CUDA;
   }
-  { GS_PROF(ctx, GS_K_MAS_INVERT); k_invert_domains<<<jobs, 256, smem, st>>>(d_mats, mas->remap0, n_dom0, djobs, djobs + jobs, d_items, N,
-                                            ctx->d_flags, fac0); }
+  // the FP64 form's digit matrices are cut by the same kernel
+  if (precision == GS_PREC_FP64 && (s = level0_f64tc_alloc(ctx, mas))) return s;
+  if ((s = invert_domains_launch(ctx, mas, fac0))) return s;
   if (precision == GS_PREC_BF16) {
     void* f = nullptr;
     s = ctx->alloc(&f, (size_t)std::max<int64_t>(cnt0, 1) * 2);
