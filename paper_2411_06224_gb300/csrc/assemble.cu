@@ -6,16 +6,24 @@
 // index, and reduce runs with FastSegmentReduction (a warp head-segmented
 // reduction; segments crossing a warp boundary finish with atomics).
 //
-// GB300 choices: keys are packed as (row << b) | col with b the bit width
-// of n, which keeps the (row, col) order of the paper's (row << 32) | col
-// encoding while shortening the radix sort to 2b bits; values are gathered
-// through the sorted index instead of being sorted along (72-byte payloads
-// are read once, in the reduction).
+// GB300 choices: the sort is a counting sort by row (one atomic per input
+// counts the rows and ranks the input within its row, one scatter of 8-byte
+// (column, index) keys) followed by a sort of every row's keys in a warp's
+// registers or a block's shared memory; the runs of a sorted row are then
+// summed by one warp, nine lanes to a block (reduce_rows).  A row of more
+// than 4,096 inputs sends the matrix to the general path: keys packed as
+// (row << b) | col with b the bit width of n, which keeps the (row, col) order
+// of the paper's (row << 32) | col encoding while shortening the radix sort
+// to 2b bits, values gathered through the sorted index, run flags, scan and
+// FastSegmentReduction (reduce_sorted_keys).
 #include <cub/device/device_reduce.cuh>
+
+#include <algorithm>
 
 #include "common.cuh"
 #include "sort_scan.cuh"
 #include "primitives.cuh"
+#include "run_reduce.cuh"
 
 namespace gs {
 
@@ -105,84 +113,347 @@ __global__ void k_row_ptr(const int32_t* __restrict__ rid, int64_t U, int32_t n,
   for (int32_t r = r_prev + 1; r <= r_here; ++r) row_ptr[r] = (int32_t)u;
 }
 
-// Reduce (rows, cols, blocks) to a new matrix.  Shared by gs_assemble and
-// the second level of gs_assemble_abd.
-int reduce_blocks(gs_ctx ctx, int32_t n, const int32_t* rows, const int32_t* cols, const double* blocks,
-                  int64_t nb, gs_mat* out) {
+// ---------------------------------------------------------------- rows sorted one by one
+// What bounds it: 80 bytes per input and stored block, and the additions
+// (run_reduce.cuh).  A radix sort of 13.4M inputs (64^3 body) moved 24 bytes
+// per key and pass, and its reduction read each 72-byte block by one thread,
+// nine loads spread over 32 blocks.  Here a key is written once and read
+// twice.  Measured, gs_assemble and gs_mat_export: 2.48 -> 1.29 ms (64^3, 13.4M
+// inputs), 0.21 -> 0.13 ms (16^3, 0.18M), two-level 1.34 -> 0.80 ms (40^3 and
+// 1,000 bodies).
+constexpr int kRowWarp = 256;   // longest row sorted by one warp
+constexpr int kRowBlock = kRowSerial;  // longest row sorted by one block (32 KB of keys)
+
+// Words the host reads back: [0] rows longer than kRowWarp, [1] set if a row
+// is longer than kRowBlock.
+struct RowWords {
+  int32_t n_long, too_long;
+};
+
+__global__ void k_row_count(const int32_t* __restrict__ rows, const int32_t* __restrict__ cols, int64_t nb, int32_t n,
+                            int32_t* __restrict__ cnt, int32_t* __restrict__ rank, int32_t* __restrict__ key_of_input,
+                            int* __restrict__ flags) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nb) return;
+  const int32_t r = rows[i], c = cols[i];
+  int32_t k = -1;
+  if (r < 0 || r >= n || c < 0 || c >= n)
+    atomicOr(flags, kErrIndex);
+  else if (r <= c)
+    k = atomicAdd(&cnt[r], 1);
+  rank[i] = k;
+  if (k < 0) key_of_input[i] = -1;
+}
+
+// The ranks of a row's inputs are in no fixed order; the sort by (column,
+// input index) that follows makes it one.
+__global__ void k_row_scatter(const int32_t* __restrict__ rows, const int32_t* __restrict__ cols,
+                              const int32_t* __restrict__ rank, const int32_t* __restrict__ start, int64_t nb,
+                              uint64_t* __restrict__ list) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nb) return;
+  const int32_t k = rank[i];
+  if (k >= 0) list[(int64_t)start[rows[i]] + k] = ((uint64_t)(uint32_t)cols[i] << 32) | (uint32_t)i;
+}
+
+// Bitonic sort of 32 kR keys, element q * 32 + lane in a[q]; then the sorted
+// keys go back and the distinct columns are counted.
+template <int kR>
+__device__ __forceinline__ int32_t sort_row(uint64_t* __restrict__ row, int32_t len, int lane) {
+  uint64_t a[kR];
+#pragma unroll
+  for (int q = 0; q < kR; ++q) a[q] = q * 32 + lane < len ? row[q * 32 + lane] : ~0ull;
+#pragma unroll
+  for (int k = 2; k <= 32 * kR; k <<= 1) {
+#pragma unroll
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      if (j >= 32) {
+#pragma unroll
+        for (int q = 0; q < kR; ++q) {
+          const int o = q ^ (j / 32);
+          if (o > q) {
+            const bool up = ((q * 32) & k) == 0;
+            const uint64_t lo = a[q] < a[o] ? a[q] : a[o], hi = a[q] < a[o] ? a[o] : a[q];
+            a[q] = up ? lo : hi, a[o] = up ? hi : lo;
+          }
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < kR; ++q) {
+          const uint64_t b = __shfl_xor_sync(kFull, a[q], j);
+          const bool up = (k < 32 ? (lane & k) : ((q * 32) & k)) == 0;
+          const bool keep_min = up == ((lane & j) == 0);
+          a[q] = (a[q] < b) == keep_min ? a[q] : b;
+        }
+      }
+    }
+  }
+  int32_t unique = 0;
+#pragma unroll
+  for (int q = 0; q < kR; ++q) {
+    const uint32_t c = (uint32_t)(a[q] >> 32);
+    uint32_t p = __shfl_up_sync(kFull, c, 1);
+    if (q > 0) {
+      const uint32_t last = __shfl_sync(kFull, (uint32_t)(a[q - 1] >> 32), 31);
+      if (lane == 0) p = last;
+    }
+    const bool in = q * 32 + lane < len;
+    if (in) row[q * 32 + lane] = a[q];
+    unique += __popc(__ballot_sync(kFull, in && (c != p || (q == 0 && lane == 0))));
+  }
+  return unique;
+}
+
+__global__ void __launch_bounds__(256) k_row_sort(const int32_t* __restrict__ start, int32_t n,
+                                                  uint64_t* __restrict__ list, int32_t* __restrict__ unique,
+                                                  RowWords* __restrict__ words, int32_t* __restrict__ long_rows) {
+  const int32_t r = (int32_t)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  const int lane = threadIdx.x & 31;
+  if (r >= n) return;  // whole warp
+  const int32_t s0 = start[r], len = start[r + 1] - s0;
+  uint64_t* row = list + s0;
+  int32_t u = 0;
+  if (len > kRowWarp) {
+    if (lane == 0) {
+      if (len > kRowBlock)
+        words->too_long = 1;
+      else
+        long_rows[atomicAdd(&words->n_long, 1)] = r;
+    }
+    return;  // k_row_sort_block writes this row's count
+  }
+  if (len > 128)
+    u = sort_row<8>(row, len, lane);
+  else if (len > 64)
+    u = sort_row<4>(row, len, lane);
+  else if (len > 32)
+    u = sort_row<2>(row, len, lane);
+  else if (len > 0)
+    u = sort_row<1>(row, len, lane);
+  if (lane == 0) unique[r] = u;
+}
+
+// The long rows, a block each.
+__global__ void __launch_bounds__(256) k_row_sort_block(const int32_t* __restrict__ start, uint64_t* __restrict__ list,
+                                                        int32_t* __restrict__ unique,
+                                                        const RowWords* __restrict__ words,
+                                                        const int32_t* __restrict__ long_rows) {
+  __shared__ uint64_t a[kRowBlock];
+  __shared__ int32_t s_unique;
+  const int32_t n_long = words->n_long;
+  for (int32_t w = blockIdx.x; w < n_long; w += gridDim.x) {
+    const int32_t r = long_rows[w], s0 = start[r], len = start[r + 1] - s0;
+    int size = 2 * kRowWarp;
+    while (size < len) size *= 2;
+    for (int e = threadIdx.x; e < size; e += blockDim.x) a[e] = e < len ? list[s0 + e] : ~0ull;
+    if (threadIdx.x == 0) s_unique = 0;
+    __syncthreads();
+    for (int k = 2; k <= size; k <<= 1)
+      for (int j = k >> 1; j > 0; j >>= 1) {
+        for (int e = threadIdx.x; e < size; e += blockDim.x) {
+          const int o = e ^ j;
+          if (o > e) {
+            const uint64_t x = a[e], y = a[o];
+            if ((x > y) == ((e & k) == 0)) a[e] = y, a[o] = x;
+          }
+        }
+        __syncthreads();
+      }
+    int32_t u = 0;
+    for (int e = threadIdx.x; e < len; e += blockDim.x) {
+      list[s0 + e] = a[e];
+      u += e == 0 || (a[e] >> 32) != (a[e - 1] >> 32);
+    }
+    atomicAdd(&s_unique, u);
+    __syncthreads();
+    if (threadIdx.x == 0) unique[r] = s_unique;
+    __syncthreads();
+  }
+}
+
+// The runs of every sorted row, a warp per row: in pieces of 256 entries it
+// finds the runs, writes their keys and each input's stored block, and sums
+// them (run_reduce.cuh).
+__global__ void __launch_bounds__(256) k_row_reduce(const int32_t* __restrict__ start,
+                                                    const int32_t* __restrict__ row_ptr,
+                                                    const uint64_t* __restrict__ list,
+                                                    const double* __restrict__ blocks, int32_t n,
+                                                    double* __restrict__ R, int32_t* __restrict__ rid,
+                                                    int32_t* __restrict__ cid, int32_t* __restrict__ key_of_input) {
+  __shared__ uint32_t s_idx[8][kPiece];
+  __shared__ int32_t s_dst[8][kPiece];
+  const int32_t r = (int32_t)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (r >= n) return;  // whole warp
+  const int32_t s0 = start[r], len = start[r + 1] - s0;
+  if (len == 0) return;
+  int32_t next = row_ptr[r];  // the next run's stored block
+  uint32_t before = 0;        // column of the last entry of the previous 32
+  double cv = 0.0;
+  int32_t cd = -1;
+  for (int32_t p0 = 0; p0 < len; p0 += kPiece) {
+    const int m = min(kPiece, len - p0);
+    for (int j = 0; j < m; j += 32) {
+      const int32_t p = p0 + j + lane;
+      const bool in = j + lane < m;
+      const uint64_t key = in ? list[s0 + p] : ~0ull;
+      const uint32_t c = (uint32_t)(key >> 32);
+      uint32_t prev = __shfl_up_sync(kFull, c, 1);
+      if (lane == 0) prev = before;
+      before = __shfl_sync(kFull, c, 31);
+      const bool head = in && (p == 0 || c != prev);
+      const uint32_t hm = __ballot_sync(kFull, head);
+      const int32_t u = next + __popc(hm & (0xffffffffu >> (31 - lane))) - 1;
+      if (head) {
+        rid[u] = r;
+        cid[u] = (int32_t)c;
+      }
+      if (in) {
+        s_idx[w][j + lane] = (uint32_t)key;
+        s_dst[w][j + lane] = u;
+        key_of_input[(uint32_t)key] = u;
+      }
+      next += __popc(hm);
+    }
+    __syncwarp();
+    sum_piece<false>(blocks, s_idx[w], s_dst[w], m, R, cv, cd, lane);
+    __syncwarp();
+  }
+  if (lane < 9) R[(size_t)cd * 9 + lane] = cv;
+}
+
+// Rows sorted one by one.  *done stays false when a row is too long for it
+// (nothing but scratch and m->row_ptr, m->key_of_input was touched).
+static int reduce_rows(gs_ctx ctx, gs_mat m, const int32_t* rows, const int32_t* cols, const double* blocks, int64_t nb,
+                       bool* done) {
   cudaStream_t st = ctx->stream;
-  gs_mat m = new gs_mat_s();
-  m->n = n;
-  m->owner = ctx;
+  const int32_t n = m->n;
+  const int T = 256;
+  // counts / unique counts, row starts, worklist of long rows, words
+  int32_t *cnt = nullptr, *rank = nullptr;
+  uint64_t* list = nullptr;
+  void* temp = nullptr;
+  const size_t tb = scan_temp_bytes((int64_t)n + 1);
+  GS_TRY(ctx->scratch_buf(kSlotScan, (3 * (size_t)n + 8) * 4, (void**)&cnt));
+  GS_TRY(ctx->scratch_buf(kSlotSortValsIn, (size_t)nb * 4, (void**)&rank));
+  GS_TRY(ctx->scratch_buf(kSlotSortKeysIn, (size_t)nb * 8, (void**)&list));
+  GS_TRY(ctx->scratch_buf(kSlotSortTemp, tb, &temp));
+  int32_t *start = cnt + n + 1, *long_rows = start + n + 1;
+  RowWords* words = (RowWords*)(long_rows + n);
+  GS_CUDA(cudaMemsetAsync(cnt, 0, ((size_t)n + 1) * 4, st));
+  GS_CUDA(cudaMemsetAsync(words, 0, sizeof(RowWords), st));
+  { GS_PROF(ctx, GS_K_ASSEMBLE); k_row_count<<<ceil_div(nb, T), T, 0, st>>>(rows, cols, nb, n, cnt, rank, m->key_of_input, ctx->d_flags); }
+  { GS_PROF(ctx, GS_K_ASSEMBLE); GS_TRY(exclusive_scan_i32(st, cnt, start, (int64_t)n + 1, temp, tb)); }
+  { GS_PROF(ctx, GS_K_ASSEMBLE); k_row_scatter<<<ceil_div(nb, T), T, 0, st>>>(rows, cols, rank, start, nb, list); }
+  { GS_PROF(ctx, GS_K_ASSEMBLE); k_row_sort<<<ceil_div(32LL * n, T), T, 0, st>>>(start, n, list, cnt, words, long_rows); }
+  {
+    GS_PROF(ctx, GS_K_ASSEMBLE);
+    k_row_sort_block<<<std::max(1, std::min(2 * ctx->sm_count, n)), T, 0, st>>>(start, list, cnt, words, long_rows);
+  }
+  { GS_PROF(ctx, GS_K_ASSEMBLE); GS_TRY(exclusive_scan_i32(st, cnt, m->row_ptr, (int64_t)n + 1, temp, tb)); }
+  GS_CUDA(cudaMemcpyAsync(ctx->h_pinned + 4, words, sizeof(RowWords), cudaMemcpyDeviceToHost, st));
+  GS_CUDA(cudaMemcpyAsync(ctx->h_pinned + 8, m->row_ptr + n, 4, cudaMemcpyDeviceToHost, st));
+  int flags = 0;
+  GS_TRY(ctx->take_flags(&flags));
+  if (flags) return status_from_flags(flags);
+  const RowWords h = *(const RowWords*)(ctx->h_pinned + 4);
+  if (h.too_long) return GS_OK;
+  const int64_t U = ctx->h_pinned[8];
+  m->nnzb = U;
+  GS_TRY(ctx->alloc((void**)&m->au, (size_t)U * 72));
+  GS_TRY(ctx->alloc((void**)&m->rid, (size_t)U * 4));
+  GS_TRY(ctx->alloc((void**)&m->cid, (size_t)U * 4));
+  if (U > 0) {
+    { GS_PROF(ctx, GS_K_ASSEMBLE); k_row_reduce<<<ceil_div(32LL * n, T), T, 0, st>>>(start, m->row_ptr, list, blocks, n, m->au, m->rid, m->cid,
+                                                                                    m->key_of_input); }
+  }
+  *done = true;
+  return GS_OK;
+}
+
+// The general path: radix sort of (key, input) pairs, run flags, exclusive
+// scan, FastSegmentReduction.
+static int reduce_sorted_keys(gs_ctx ctx, gs_mat m, const int32_t* rows, const int32_t* cols, const double* blocks,
+                              int64_t nb) {
+  cudaStream_t st = ctx->stream;
+  const int32_t n = m->n;
   const int shift = bits_for(n);
   const uint64_t sentinel = (shift * 2 >= 64) ? ~0ull : ((1ull << (2 * shift)) - 1);
   const int end_bit = 2 * shift;
   uint64_t *k_in = nullptr, *k_out = nullptr;
   uint32_t *i_in = nullptr, *i_out = nullptr;
   int32_t *P = nullptr, *O = nullptr;
-  int64_t U = 0;
-  auto fail = [&](int s) {
-    gs_mat_destroy(m);
-    return s;
-  };
-  if (nb > 0) {
-    int s;
-    if ((s = ctx->scratch_buf(kSlotSortKeysIn, nb * 8, (void**)&k_in)) ||
-        (s = ctx->scratch_buf(kSlotSortKeysOut, nb * 8, (void**)&k_out)) ||
-        (s = ctx->scratch_buf(kSlotSortValsIn, nb * 4, (void**)&i_in)) ||
-        (s = ctx->scratch_buf(kSlotSortValsOut, nb * 4, (void**)&i_out)) ||
-        (s = ctx->scratch_buf(kSlotScan, nb * 8, (void**)&P)))
-      return fail(s);
-    O = P + nb;
-    const int T = 256;
-    { GS_PROF(ctx, GS_K_ASSEMBLE); k_encode_keys<<<ceil_div(nb, T), T, 0, st>>>(rows, cols, nb, n, shift, sentinel, k_in, i_in, ctx->d_flags); }
-    // radix sort of (key, index) and the exclusive scan of the run flags
-    // (sort_scan.cu: hand-written, stable)
-    const size_t tb = std::max(radix_sort_temp_bytes(nb), scan_temp_bytes(nb));
-    void* temp = nullptr;
-    if ((s = ctx->scratch_buf(kSlotSortTemp, tb, &temp))) return fail(s);
-    {
-      GS_PROF(ctx, GS_K_ASSEMBLE);
-      if ((s = radix_sort_pairs(st, k_in, k_out, i_in, i_out, nb, end_bit, temp, tb))) return fail(s);
-    }
-    { GS_PROF(ctx, GS_K_ASSEMBLE); k_run_flags<<<ceil_div(nb, T), T, 0, st>>>(k_out, nb, P); }
-    {
-      GS_PROF(ctx, GS_K_ASSEMBLE);
-      if ((s = exclusive_scan_i32(st, P, O, nb, temp, tb))) return fail(s);
-    }
-    // U = distinct keys, minus the sentinel group if present.
-    uint64_t* hk = (uint64_t*)ctx->h_pinned;
-    int32_t* ho = (int32_t*)(ctx->h_pinned + 4);
-    if (cudaMemcpyAsync(hk, k_out + nb - 1, 8, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(ho, O + nb - 1, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess) {
-      set_error("assembly readback failed");
-      return fail(GS_ERR_CUDA);
-    }
-    U = (int64_t)ho[0] + 1 - (hk[0] == sentinel ? 1 : 0);
-  }
+  const int T = 256;
+  GS_TRY(ctx->scratch_buf(kSlotSortKeysIn, nb * 8, (void**)&k_in));
+  GS_TRY(ctx->scratch_buf(kSlotSortKeysOut, nb * 8, (void**)&k_out));
+  GS_TRY(ctx->scratch_buf(kSlotSortValsIn, nb * 4, (void**)&i_in));
+  GS_TRY(ctx->scratch_buf(kSlotSortValsOut, nb * 4, (void**)&i_out));
+  GS_TRY(ctx->scratch_buf(kSlotScan, nb * 8, (void**)&P));
+  O = P + nb;
+  { GS_PROF(ctx, GS_K_ASSEMBLE); k_encode_keys<<<ceil_div(nb, T), T, 0, st>>>(rows, cols, nb, n, shift, sentinel, k_in, i_in, ctx->d_flags); }
+  // radix sort of (key, index) and the exclusive scan of the run flags
+  // (sort_scan.cu: hand-written, stable)
+  const size_t tb = std::max(radix_sort_temp_bytes(nb), scan_temp_bytes(nb));
+  void* temp = nullptr;
+  GS_TRY(ctx->scratch_buf(kSlotSortTemp, tb, &temp));
+  { GS_PROF(ctx, GS_K_ASSEMBLE); GS_TRY(radix_sort_pairs(st, k_in, k_out, i_in, i_out, nb, end_bit, temp, tb)); }
+  { GS_PROF(ctx, GS_K_ASSEMBLE); k_run_flags<<<ceil_div(nb, T), T, 0, st>>>(k_out, nb, P); }
+  { GS_PROF(ctx, GS_K_ASSEMBLE); GS_TRY(exclusive_scan_i32(st, P, O, nb, temp, tb)); }
+  // U = distinct keys, minus the sentinel group if present.
+  uint64_t* hk = (uint64_t*)(ctx->h_pinned + 4);
+  int32_t* ho = (int32_t*)(ctx->h_pinned + 8);
+  GS_CUDA(cudaMemcpyAsync(hk, k_out + nb - 1, 8, cudaMemcpyDeviceToHost, st));
+  GS_CUDA(cudaMemcpyAsync(ho, O + nb - 1, 4, cudaMemcpyDeviceToHost, st));
   int flags = 0;
   GS_TRY(ctx->take_flags(&flags));
-  if (flags) return fail(status_from_flags(flags));
+  if (flags) return status_from_flags(flags);
+  const int64_t U = (int64_t)ho[0] + 1 - (hk[0] == sentinel ? 1 : 0);
   m->nnzb = U;
-  int s;
-  m->n_input = nb;
-  if ((s = ctx->alloc((void**)&m->key_of_input, (size_t)std::max<int64_t>(nb, 1) * 4)) ||
-      (s = ctx->alloc((void**)&m->au, (size_t)U * 9 * sizeof(double))) ||
-      (s = ctx->alloc((void**)&m->rid, (size_t)U * 4)) || (s = ctx->alloc((void**)&m->cid, (size_t)U * 4)) ||
-      (s = ctx->alloc((void**)&m->row_ptr, (size_t)(n + 1) * 4)))
-    return fail(s);
+  GS_TRY(ctx->alloc((void**)&m->au, (size_t)U * 72));
+  GS_TRY(ctx->alloc((void**)&m->rid, (size_t)U * 4));
+  GS_TRY(ctx->alloc((void**)&m->cid, (size_t)U * 4));
   if (U > 0) {
-    if (cudaMemsetAsync(m->au, 0, (size_t)U * 9 * sizeof(double), st) != cudaSuccess) return fail(GS_ERR_CUDA);
-    const int T = 256;
-    { GS_PROF(ctx, GS_K_ASSEMBLE); k_fast_segment_reduce<<<ceil_div(nb, T), T, 0, st>>>(k_out, i_out, O, blocks, nb, sentinel, shift, m->au,
-                                                            m->rid, m->cid, m->key_of_input); }
+    GS_CUDA(cudaMemsetAsync(m->au, 0, (size_t)U * 72, st));
+    GS_PROF(ctx, GS_K_ASSEMBLE);
+    k_fast_segment_reduce<<<ceil_div(nb, T), T, 0, st>>>(k_out, i_out, O, blocks, nb, sentinel, shift, m->au, m->rid,
+                                                         m->cid, m->key_of_input);
+  } else {
+    GS_CUDA(cudaMemsetAsync(m->key_of_input, 0xff, (size_t)nb * 4, st));
   }
-  if (U == 0 && nb > 0 && cudaMemsetAsync(m->key_of_input, 0xff, (size_t)nb * 4, st) != cudaSuccess)
-    return fail(GS_ERR_CUDA);
   { GS_PROF(ctx, GS_K_ASSEMBLE); k_row_ptr<<<ceil_div(U + 1, 256), 256, 0, st>>>(m->rid, U, n, m->row_ptr); }
-  if (cudaGetLastError() != cudaSuccess) {
-    set_error("assembly kernel launch failed");
-    return fail(GS_ERR_CUDA);
+  return GS_OK;
+}
+
+// Reduce (rows, cols, blocks) to a new matrix.  Shared by gs_assemble and
+// the second level of gs_assemble_abd.
+int reduce_blocks(gs_ctx ctx, int32_t n, const int32_t* rows, const int32_t* cols, const double* blocks,
+                  int64_t nb, gs_mat* out) {
+  gs_mat m = new gs_mat_s();
+  m->n = n;
+  m->owner = ctx;
+  m->n_input = nb;
+  auto run = [&]() -> int {
+    GS_TRY(ctx->alloc((void**)&m->key_of_input, (size_t)std::max<int64_t>(nb, 1) * 4));
+    GS_TRY(ctx->alloc((void**)&m->row_ptr, (size_t)(n + 1) * 4));
+    if (nb == 0) {
+      int flags = 0;
+      GS_TRY(ctx->take_flags(&flags));
+      if (flags) return status_from_flags(flags);
+      GS_CUDA(cudaMemsetAsync(m->row_ptr, 0, (size_t)(n + 1) * 4, ctx->stream));
+      return GS_OK;
+    }
+    bool done = false;
+    // every row, empty ones too, costs the row path a warp and 12 bytes of
+    // scratch; the general path costs passes over the inputs alone
+    if (n <= 4 * nb + 65536) GS_TRY(reduce_rows(ctx, m, rows, cols, blocks, nb, &done));
+    if (!done) GS_TRY(reduce_sorted_keys(ctx, m, rows, cols, blocks, nb));
+    GS_CUDA(cudaGetLastError());
+    return GS_OK;
+  };
+  const int s = run();
+  if (s != GS_OK) {
+    gs_mat_destroy(m);
+    return s;
   }
   *out = m;
   return GS_OK;

@@ -1,0 +1,87 @@
+// Sums of runs of 3x3 blocks, a matrix row at a time by one warp (Sec. 5.2,
+// the reduction of blocks with equal keys).  Shared by the assembly from
+// triplets (assemble.cu) and the numeric assembly through a stored order
+// (elastic.cu): both give the same bits for the same inputs.
+//
+// What bounds it: 72 bytes gathered and 9 FP64 additions per input, and the
+// additions as much as the bytes: an FP64 instruction costs its 16 cycles per
+// SM however few lanes take part (13.4M inputs: 0.19 ms of additions with full
+// warps, 0.2 ms of reads).  So nine neighbouring lanes read one block (three
+// blocks per warp instruction, 9 sectors), and the three lane groups take
+// equal thirds of a row's entries whatever its runs are: every step is one
+// addition for the whole warp.  A group per run left the warp waiting for the
+// longest run (the diagonal's) at three times the additions.
+#pragma once
+
+#include "primitives.cuh"
+
+namespace gs {
+
+constexpr int kPiece = 256;      // entries of a row summed at a time
+constexpr int kRowSerial = 4096; // longest row that one warp sums piece by piece
+
+template <bool kAtomic>
+__device__ __forceinline__ void put_sum(double* dst, double v) {
+  if (kAtomic)
+    atomicAdd(dst, v);
+  else
+    *dst = v;
+}
+
+// Whole warp.  Entries 0 .. m-1 (m <= kPiece, m > 0) of a row: s_idx their
+// blocks, s_dst their destination blocks in R, ascending.  cv (component
+// lane % 9) and cd carry the unfinished run between a row's pieces (cd = -1:
+// none); the last run stays in them.  Each lane group sums its third in
+// order; a run that spans groups is added group by group.
+template <bool kAtomic>
+__device__ __forceinline__ void sum_piece(const double* __restrict__ blocks, const uint32_t* s_idx,
+                                          const int32_t* s_dst, int m, double* __restrict__ R, double& cv, int32_t& cd,
+                                          int lane) {
+  constexpr int kLoads = 6;  // blocks in flight per lane group
+  const int g = lane / 9, q = lane - 9 * g;
+  const int T = (m + 2) / 3;
+  const int b = g * T, e = g < 3 ? min(b + T, m) : b;
+  const int32_t f = b < e ? s_dst[b] : -1;  // the group's first run
+  int32_t cur = f;
+  double acc = 0.0, lead = 0.0;
+  for (int t = 0; t < T; t += kLoads) {
+    double v[kLoads];
+#pragma unroll
+    for (int k = 0; k < kLoads; ++k) {
+      const int p = b + t + k;
+      v[k] = p < e ? blocks[(size_t)s_idx[p] * 9 + q] : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < kLoads; ++k) {
+      if (t + k >= T) break;  // whole warp
+      const int p = b + t + k;
+      const int32_t d = p < e ? s_dst[p] : cur;
+      if (d != cur) {
+        if (cur == f)
+          lead = acc;
+        else
+          put_sum<kAtomic>(R + (size_t)cur * 9 + q, acc);
+        acc = 0.0;
+        cur = d;
+      }
+      acc += v[k];
+    }
+  }
+#pragma unroll
+  for (int h = 0; h < 3; ++h) {  // the groups' first and last runs, in order
+    const int from = 9 * h + lane % 9;
+    const int32_t hf = __shfl_sync(kFull, f, from), hc = __shfl_sync(kFull, cur, from);
+    const double first = __shfl_sync(kFull, cur == f ? acc : lead, from), last = __shfl_sync(kFull, acc, from);
+    if (hf < 0) continue;  // whole warp
+    if (cd >= 0 && cd != hf && lane < 9) put_sum<kAtomic>(R + (size_t)cd * 9 + lane, cv);
+    cv = (cd == hf ? cv : 0.0) + first;
+    cd = hf;
+    if (hc != hf) {
+      if (lane < 9) put_sum<kAtomic>(R + (size_t)hf * 9 + lane, cv);
+      cv = last;
+      cd = hc;
+    }
+  }
+}
+
+}  // namespace gs
