@@ -507,6 +507,7 @@ int gs_mat_destroy(gs_mat m) {
   c->release(m->au_ff);
   c->release(m->ff_k);
   c->release(m->row_order);
+  gs::release_sliced(c, m, true);
   c->release(m->key_of_input);
   delete m;
   return GS_OK;

@@ -86,6 +86,7 @@ struct gs_ctx_s {
   int sm_count = 0;
   int tune[GS_TUNE_COUNT] = {2, 2, 4, 4096, 1, 4, 1024, 1, 8};  // GS_TUNE_* launch shapes
   cudaStream_t capture_stream = nullptr;  // private stream for CUDA-graph capture
+  cudaEvent_t poll_event[2] = {nullptr, nullptr};  // convergence polls in flight (PCG)
   int* d_flags = nullptr;     // 256 device bytes: [0] error word, [kSpmvCounterWord] SpMV work counter
   int* h_pinned = nullptr;    // pinned host staging (small readbacks), 4 KiB
   double* noalloc_scratch = nullptr;  // gs_mas_apply_noalloc's fixed array in this context
@@ -165,10 +166,14 @@ int level0_f64tc_prepare(gs_ctx ctx, gs_mas mas);
 // Inverts the level matrices in place and cuts their digit matrices (mas_invert.cu)
 int invert_domains_launch(gs_ctx ctx, gs_mas mas, double* fac0);
 // skip (device, may be null): the kernels return at once while *skip is set
+// dot (GS_TUNE_F64_TC 1 or 4): also partial sums of r . z, one per domain
+struct Partials;
 int level0_f64tc_launch(gs_ctx ctx, gs_mas mas, int nrhs, const double* r, int64_t stride, const double* zl,
-                        int64_t lstride, double* z, const int* skip = nullptr);
+                        int64_t lstride, double* z, const int* skip = nullptr, const Partials* dot = nullptr);
+// from_kids: levels >= 2 sum their r from the level below themselves (at most
+// one such level)
 int coarse_f64tc_launch(gs_ctx ctx, gs_mas mas, int nrhs, const double* rl, double* zl, int64_t lstride,
-                        const int* skip = nullptr);
+                        const int* skip = nullptr, bool from_kids = false);
 // The same product from the block lower triangles of the symmetric inverses
 // as digit bytes (GS_TUNE_F64_TC = 3, N = 16 or 32); mas_apply_f64sym.cu.
 bool f64sym_shape_ok(int N);
@@ -187,6 +192,10 @@ int mas_apply_launch_skip(gs_ctx ctx, gs_mas mas, const double* r, double* z, in
 // x_k[3 node + c] * 2^(ff_k[node] - F[k]) (|.| <= 1), F device int[nrhs];
 // spmv_ff_launch splits x itself (two extra passes).
 int ensure_ff(gs_ctx ctx, gs_mat m);
+int ensure_ff_scales(gs_ctx ctx, gs_mat m);  // the row exponents ff_k alone
+// Sliced copy for PCG's product (sliced.cu)
+int ensure_sliced(gs_ctx ctx, gs_mat m, bool ff);
+void release_sliced(gs_ctx ctx, gs_mat m, bool all);
 int spmv_ff_split_launch(gs_ctx ctx, gs_mat m, const float2* xs, const int* F, double* y, int nrhs, const int* skip);
 int spmv_ff_launch(gs_ctx ctx, gs_mat m, const double* x, double* y, int nrhs, const int* skip);
 }  // namespace gs
@@ -214,6 +223,16 @@ struct gs_mat_s {
   // (hi, lo) = (rn(a), rn(a - hi)) floats.
   float2* au_ff = nullptr;    // nnzb * 9
   int32_t* ff_k = nullptr;    // n + 1: k_i - K per row; [n] holds K = max_i k_i
+  // Sliced copy of the full matrix for PCG's product (sliced.cu, built lazily):
+  // 32 rows of row_order per slice, entry e of slice s at (sl_ptr[s] + e) * 32 + row.
+  int32_t* sl_ptr = nullptr;  // slices + 1
+  int32_t* sl_len = nullptr;  // n: entries of every row of the order
+  int32_t* sl_col = nullptr;  // per entry: column
+  int32_t* sl_blk = nullptr;  // per entry: stored block, complemented where used transposed
+  float2* sl_ff = nullptr;    // values, float-float: [(sl_ptr[s] + e) * 9 + q][32]
+  double* sl_f64 = nullptr;   // the same in FP64
+  int64_t sl_entries = 0;
+  int32_t sl_window = -1;     // row_order_window it was built for
   const void* pattern_owner = nullptr;  // the elastic body whose fixed pattern this matrix uses (or null)
   uint64_t pattern_version = 0;        // and that pattern's version
   gs_ctx owner = nullptr;
@@ -229,6 +248,8 @@ struct gs_mas_s {
   std::vector<int32_t*> coarse;    // per level: device int32[n] (level 0 = map)
   std::vector<int32_t*> up;        // per level l >= 1 below the top: device int32[n_domains[l] * N],
                                    // the level-(l+1) item of each level-l item (-1: padding)
+  std::vector<int2*> kids;         // per level l >= 2: per item its children of level l - 1, (first item of their
+                                   // domain, lane mask); the same map as up[l - 1]
   int32_t* remap0 = nullptr;       // device int32[n_items[0]], slot -> node or -1
   std::vector<double*> inv64;      // per level: n_domains * (3N)^2
   std::vector<float*> inv32;       // per level (FP32 precision, or made for the mixed solve)

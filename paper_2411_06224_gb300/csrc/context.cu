@@ -249,6 +249,8 @@ int gs_destroy(gs_ctx ctx) {
   for (auto& b : ctx->scratch) ctx->release(b.ptr);
   cudaStreamSynchronize(ctx->stream);
   if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
+  for (cudaEvent_t e : ctx->poll_event)
+    if (e) cudaEventDestroy(e);
   cudaFree(ctx->d_flags);
   cudaFreeHost(ctx->h_pinned);
   delete ctx;

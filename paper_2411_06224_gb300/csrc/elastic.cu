@@ -1082,6 +1082,7 @@ int refill(gs_ctx ctx, gs_fem f, const double* x, gs_mat m) {
   m->au32 = nullptr;
   m->au_ff = nullptr;
   m->ff_k = nullptr;
+  release_sliced(ctx, m, false);
   GS_CUDA(cudaGetLastError());
   return GS_OK;
 }

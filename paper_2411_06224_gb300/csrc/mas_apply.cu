@@ -14,9 +14,11 @@
 // the inverse is symmetric, so row i is read as column i (coalesced).
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
+#include "pcg_state.cuh"
 #include "primitives.cuh"
 #include "umma.cuh"
 
@@ -24,6 +26,7 @@ namespace gs {
 
 struct ApplyLevels {
   const int32_t* coarse[8];
+  const int2* kids[8];  // levels whose r is summed from the level below in the product itself, else null
   int64_t vec_off[8];
   int L;
   int N;
@@ -194,7 +197,7 @@ __global__ void __launch_bounds__(1024) k_domain_product(
 }
 
 // FP32 level 0 + prolongation: one CTA of 3N threads per domain, thread i
-// owning row i for all (at most 8) right-hand sides.  The domain's inverse is
+// owning row i for the kR >= nrhs right-hand sides.  The domain's inverse is
 // stored as its lower triangle packed by rows (18.6 KB at N = 32, half the
 // full matrix), so ten CTAs share an SM, and comes into shared memory by one
 // bulk asynchronous copy issued first; the right-hand sides are gathered into
@@ -202,18 +205,24 @@ __global__ void __launch_bounds__(1024) k_domain_product(
 // are loaded while it lands.  Row i of the symmetric inverse is its packed
 // row for j <= i and column i below it (entry (j, i) of row j) for j > i,
 // summed in ascending j; four steps' shared-memory loads are issued before
-// their FMAs (one step at a time left the warps waiting on each load).  The
-// copy wait is bounded: on a timeout the kernel sets kErrTimeout, waits
-// (bounded) for the copy to land and writes nothing.
+// their FMAs (one step at a time left the warps waiting on each load).  kDot:
+// r . z as well (FP64).  The copy wait is bounded: on a timeout the kernel sets
+// kErrTimeout, waits (bounded) for the copy to land and writes nothing.
+// What bounds it: the gathers of r and of the coarse results.  kR per RHS count
+// rather than 8 for all: 30 -> 24 us at 40^3, 4 RHS, with r . z.
 constexpr int kF32Unroll = 4;
 
-__global__ void __launch_bounds__(96) k_level0_f32_cta(const float* __restrict__ invp, int pitch, int N, int nrhs,
-                                                        const double* __restrict__ r, double* __restrict__ z,
-                                                        int64_t stride, const int32_t* __restrict__ remap0,
-                                                        const double* __restrict__ zl, int64_t lstride,
-                                                        ApplyLevels al, const int* __restrict__ skip,
-                                                        int* __restrict__ flags) {
+template <int kR, bool kDot>
+__global__ void __launch_bounds__(96) k_level0_f32(const float* __restrict__ invp, int pitch, int N, int nrhs,
+                                                   const double* __restrict__ r, double* __restrict__ z,
+                                                   int64_t stride, const int32_t* __restrict__ remap0,
+                                                   const double* __restrict__ zl, int64_t lstride, ApplyLevels al,
+                                                   const int* __restrict__ skip, int* __restrict__ flags,
+                                                   Partials dot) {
   using namespace umma;
+  // with kDot the kernel before is this preconditioner's coarse product or the
+  // update of r: it wrote neither the inverses nor *skip
+  if (!kDot) wait_for_previous_kernel();
   if (skip && *skip) return;  // every RHS of the solve has converged
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int ld = 3 * N;
@@ -221,16 +230,18 @@ __global__ void __launch_bounds__(96) k_level0_f32_cta(const float* __restrict__
   const int tid = threadIdx.x;
   const uint32_t mbytes = (uint32_t)pitch * 4;
   float* sp = (float*)smem_raw;
-  float* sr = sp + pitch;  // [ld][8]
+  float* sr = sp + pitch;  // [ld][kR]
   uint64_t* bar = (uint64_t*)(sr + ld * 8);
+  __shared__ int s_ok;
   if (tid == 0) {
     mbar_init(bar, 1);
     fence_mbar_init();
     mbar_arrive_expect_tx(bar, mbytes);
     bulk_g2s(sp, invp + (int64_t)d * pitch, mbytes, bar);
   }
-  for (int e = tid; e < ld * 8; e += blockDim.x) {  // e = j * 8 + k
-    const int j = e >> 3, k = e & 7;
+  if (kDot) wait_for_previous_kernel();
+  for (int e = tid; e < ld * kR; e += blockDim.x) {  // e = j * kR + k
+    const int j = e / kR, k = e % kR;
     float v = 0.0f;
     if (k < nrhs) {
       const int32_t node = remap0[(int64_t)d * N + j / 3];
@@ -242,20 +253,27 @@ __global__ void __launch_bounds__(96) k_level0_f32_cta(const float* __restrict__
   const bool act = i < ld;
   const int32_t node = act ? remap0[(int64_t)d * N + i / 3] : -1;
   const int x = i % 3;
-  float acc[8];
+  float acc[kR];
+  double dacc[kR];
+  int dex[kR];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) acc[k] = 0.0f;
+  for (int k = 0; k < kR; ++k) acc[k] = 0.0f, dacc[k] = 0.0, dex[k] = kExpNone;
   if (node >= 0) {
 #pragma unroll
     for (int ll = 1; ll < 8; ++ll) {
       if (ll >= al.L) break;
       const int64_t ci = al.vec_off[ll] + al.coarse[ll][node];
 #pragma unroll
-      for (int k = 0; k < 8; ++k)
+      for (int k = 0; k < kR; ++k)
         if (k < nrhs) acc[k] += f64_to_f32_bits(zl[k * lstride + 3 * ci + x]);
     }
+    if (kDot) {
+#pragma unroll
+      for (int k = 0; k < kR; ++k)
+        if (k < nrhs) dacc[k] = r[k * stride + 3 * (int64_t)node + x];
+    }
   }
-  __shared__ int s_ok;
+  let_next_kernel_launch();
   if (tid == 0) s_ok = mbar_wait(bar, 0);
   __syncthreads();
   if (!s_ok) {
@@ -263,42 +281,126 @@ __global__ void __launch_bounds__(96) k_level0_f32_cta(const float* __restrict__
       atomicOr(flags, kErrTimeout);
       mbar_wait(bar, 0);  // let a late copy land before the CTA leaves
     }
-    return;
+    return;  // whole CTA
   }
-  if (!act) return;
-  const int rb = i * (i + 1) / 2;
-  int tri = 0;  // j (j + 1) / 2
-  int j0 = 0;
-  for (; j0 + kF32Unroll <= ld; j0 += kF32Unroll) {
-    float m[kF32Unroll];
-    float4 ra[kF32Unroll], rc[kF32Unroll];
+  if (act) {
+    const int rb = i * (i + 1) / 2;
+    int tri = 0;  // j (j + 1) / 2
+    int j0 = 0;
+    for (; j0 + kF32Unroll <= ld; j0 += kF32Unroll) {
+      float m[kF32Unroll], rj[kF32Unroll][kR];
 #pragma unroll
-    for (int u = 0; u < kF32Unroll; ++u) {
-      const int j = j0 + u;
-      m[u] = sp[j <= i ? rb + j : tri + i];
-      ra[u] = *reinterpret_cast<const float4*>(sr + j * 8);
-      rc[u] = *reinterpret_cast<const float4*>(sr + j * 8 + 4);
-      tri += j + 1;
+      for (int u = 0; u < kF32Unroll; ++u) {
+        const int j = j0 + u;
+        m[u] = sp[j <= i ? rb + j : tri + i];
+        if constexpr (kR % 4 == 0) {
+#pragma unroll
+          for (int k = 0; k < kR; k += 4) {
+            const float4 q = *reinterpret_cast<const float4*>(sr + j * kR + k);
+            rj[u][k] = q.x, rj[u][k + 1] = q.y, rj[u][k + 2] = q.z, rj[u][k + 3] = q.w;
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < kR; ++k) rj[u][k] = sr[j * kR + k];
+        }
+        tri += j + 1;
+      }
+#pragma unroll
+      for (int u = 0; u < kF32Unroll; ++u)
+#pragma unroll
+        for (int k = 0; k < kR; ++k) acc[k] = fmaf(m[u], rj[u][k], acc[k]);
     }
+    for (; j0 < ld; ++j0) {
+      const float m = sp[j0 <= i ? rb + j0 : tri + i];
 #pragma unroll
-    for (int u = 0; u < kF32Unroll; ++u) {
-      acc[0] = fmaf(m[u], ra[u].x, acc[0]), acc[1] = fmaf(m[u], ra[u].y, acc[1]);
-      acc[2] = fmaf(m[u], ra[u].z, acc[2]), acc[3] = fmaf(m[u], ra[u].w, acc[3]);
-      acc[4] = fmaf(m[u], rc[u].x, acc[4]), acc[5] = fmaf(m[u], rc[u].y, acc[5]);
-      acc[6] = fmaf(m[u], rc[u].z, acc[6]), acc[7] = fmaf(m[u], rc[u].w, acc[7]);
+      for (int k = 0; k < kR; ++k) acc[k] = fmaf(m, sr[j0 * kR + k], acc[k]);
+      tri += j0 + 1;
+    }
+    if (node >= 0) {
+#pragma unroll
+      for (int k = 0; k < kR; ++k)
+        if (k < nrhs) {
+          const double v = f32_to_f64_bits(acc[k]);
+          z[k * stride + 3 * (int64_t)node + x] = v;
+          if (kDot) {
+            dacc[k] *= v;
+            dex[k] = ex_bound(v);
+          }
+        }
     }
   }
-  for (; j0 < ld; ++j0) {
-    const float m = sp[j0 <= i ? rb + j0 : tri + i];
-    const float* rj = sr + j0 * 8;
+  if (kDot) {
+    __shared__ double red[3][kR];
+    __shared__ int redx[3][kR];
+    const int lane = tid & 31, w = tid >> 5, nw = blockDim.x >> 5;
+    const int k = sum_index<kR>(lane);
+    const double v = warp_sums<kR>(dacc, lane);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) acc[k] = fmaf(m, rj[k], acc[k]);
-    tri += j0 + 1;
+    for (int q = 0; q < kR; ++q) {
+      const int e = __reduce_max_sync(kFull, dex[q]);
+      if (lane == 0) redx[w][q] = e;
+    }
+    if (lane < kR) red[w][k] = v;
+    __syncthreads();
+    if (tid < nrhs) {
+      double sum = 0.0;
+      int e = kExpNone;
+      for (int q = 0; q < nw; ++q) sum += red[q][tid], e = max(e, redx[q][tid]);
+      dot.sum[(size_t)tid * dot.pitch + d] = sum;
+      dot.ex[(size_t)tid * dot.pitch + d] = e;
+    }
   }
-  if (node < 0) return;
+}
+
+// FP32 coarse domains, one CTA each: the inverse goes to shared memory whole
+// (all its loads in flight at once), then thread (i, k) sums row i for RHS k in
+// ascending j.  A level with kids takes its r as the sums of its items'
+// children.  40^3, 4 RHS, 79 domains: 15 -> 13 us, and a launch less.
+template <int kR>
+__global__ void __launch_bounds__(256) k_coarse_f32(const float* const* __restrict__ inv,
+                                                    const int32_t* __restrict__ job_level,
+                                                    const int32_t* __restrict__ job_dom, int N, int nrhs,
+                                                    const double* __restrict__ rl, double* __restrict__ zl,
+                                                    int64_t lstride, ApplyLevels al, const int* __restrict__ skip) {
+  if (skip && *skip) return;
+  extern __shared__ float sm[];  // [ld][ld], then [ld][kR]
+  const int ld = 3 * N, tid = threadIdx.x;
+  const int l = job_level[blockIdx.x];
+  const int64_t d = job_dom[blockIdx.x];
+  const float* M = inv[l] + d * ld * ld;
+  float* sr = sm + ld * ld;
+  for (int e = tid; e < ld * ld; e += 256 * 12) {
+    float v[12];
 #pragma unroll
-  for (int k = 0; k < 8; ++k)
-    if (k < nrhs) z[k * stride + 3 * (int64_t)node + x] = f32_to_f64_bits(acc[k]);
+    for (int u = 0; u < 12; ++u) v[u] = e + 256 * u < ld * ld ? __ldg(M + e + 256 * u) : 0.0f;
+#pragma unroll
+    for (int u = 0; u < 12; ++u)
+      if (e + 256 * u < ld * ld) sm[e + 256 * u] = v[u];
+  }
+  wait_for_previous_kernel();  // the restriction: it wrote neither the inverse nor *skip
+  for (int e = tid; e < ld * kR; e += 256) {
+    const int k = e / ld, j = e - k * ld;
+    double v = 0.0;
+    if (k < nrhs) {
+      if (al.kids[l]) {
+        const int2 kid = al.kids[l][d * N + j / 3];
+        const double* rk = rl + k * lstride + 3 * (al.vec_off[l - 1] + kid.x) + j % 3;
+        v = sum_children(rk, (uint32_t)kid.y);
+      } else {
+        v = rl[k * lstride + 3 * (al.vec_off[l] + d * N) + j];
+      }
+    }
+    sr[j * kR + k] = f64_to_f32_bits(v);
+  }
+  let_next_kernel_launch();
+  __syncthreads();
+  for (int e = tid; e < ld * nrhs; e += 256) {
+    const int k = e / ld, i = e - k * ld;
+    float acc = 0.0f;
+#pragma unroll 16
+    for (int j = 0; j < ld; ++j) acc = fmaf(sm[j * ld + i], sr[j * kR + k], acc);
+    zl[k * lstride + 3 * (al.vec_off[l] + d * N) + i] = f32_to_f64_bits(acc);
+  }
 }
 
 // Floats per domain of the packed level-0 inverses (16-byte multiple).
@@ -307,7 +409,7 @@ static int f32_pitch(int N) {
   return ((ld * (ld + 1) / 2 + 3) / 4) * 4;
 }
 
-// Shared memory of k_level0_f32_cta; 0 when it cannot be used (3N <= 96 rows).
+// Shared memory of k_level0_f32; 0 when it cannot be used (3N <= 96 rows).
 static size_t f32_cta_smem(int N) {
   const size_t ld = 3 * (size_t)N;
   if (ld > 96) return 0;
@@ -355,6 +457,95 @@ __global__ void __launch_bounds__(256) k_coarse_product(const Ts* const* __restr
   zl[k * lstride + 3 * (al.vec_off[l] + (int64_t)d * N) + i] = to_f64(acc);
 }
 
+static ApplyLevels apply_levels(gs_mas mas, bool from_kids) {
+  ApplyLevels al{};
+  al.L = mas->L;
+  al.N = mas->N;
+  for (int l = 0; l < mas->L; ++l) {
+    al.coarse[l] = mas->coarse[l];
+    al.vec_off[l] = mas->vec_off[l];
+    if (from_kids && l >= 2) al.kids[l] = mas->kids[l];
+  }
+  return al;
+}
+
+template <int kR>
+static int launch_coarse_f32(gs_ctx ctx, gs_mas mas, int nrhs, const double* rl, double* zl, int64_t lstride,
+                             const int* skip, bool from_kids) {
+  if (mas->n_coarse_jobs == 0) return GS_OK;
+  const size_t ld = 3 * (size_t)mas->N, smem = (ld * ld + ld * kR) * 4;
+  GS_CUDA(launch_chained(ctx, (int64_t)mas->n * nrhs, k_coarse_f32<kR>, dim3(mas->n_coarse_jobs), dim3(256), smem,
+                         (const float* const*)mas->d_inv_tab, mas->d_coarse_jobs,
+                         mas->d_coarse_jobs + mas->n_coarse_jobs, mas->N, nrhs, rl, zl, lstride,
+                         apply_levels(mas, from_kids), skip));
+  return GS_OK;
+}
+
+static int coarse_f32_launch(gs_ctx ctx, gs_mas mas, int nrhs, const double* rl, double* zl, int64_t lstride,
+                             const int* skip, bool from_kids) {
+  GS_PROF(ctx, GS_K_MAS_APPLY_COARSE);
+  if (nrhs == 1) return launch_coarse_f32<1>(ctx, mas, nrhs, rl, zl, lstride, skip, from_kids);
+  if (nrhs <= 4) return launch_coarse_f32<4>(ctx, mas, nrhs, rl, zl, lstride, skip, from_kids);
+  return launch_coarse_f32<8>(ctx, mas, nrhs, rl, zl, lstride, skip, from_kids);
+}
+
+template <int kR, bool kDot>
+static int launch_level0_f32(gs_ctx ctx, gs_mas mas, const double* r, double* z, int nrhs, const double* zl,
+                             int64_t lstride, const int* skip, const Partials& dot) {
+  if (mas->n_domains[0] == 0) return GS_OK;
+  const int ld = 3 * mas->N;
+  GS_CUDA(launch_chained(ctx, (int64_t)mas->n * nrhs, k_level0_f32<kR, kDot>, dim3(mas->n_domains[0]),
+                         dim3((ld + 31) / 32 * 32), f32_cta_smem(mas->N), mas->inv32p, f32_pitch(mas->N), mas->N, nrhs, r, z,
+                         3LL * mas->n, mas->remap0, zl, lstride, apply_levels(mas, false), skip, ctx->d_flags, dot));
+  return GS_OK;
+}
+
+template <bool kDot>
+static int level0_f32_launch(gs_ctx ctx, gs_mas mas, const double* r, double* z, int nrhs, const double* zl,
+                             int64_t lstride, const int* skip, const Partials& dot) {
+  GS_PROF(ctx, GS_K_MAS_APPLY_L0);
+  if (nrhs == 1) return launch_level0_f32<1, kDot>(ctx, mas, r, z, nrhs, zl, lstride, skip, dot);
+  if (nrhs <= 4) return launch_level0_f32<4, kDot>(ctx, mas, r, z, nrhs, zl, lstride, skip, dot);
+  return launch_level0_f32<8, kDot>(ctx, mas, r, z, nrhs, zl, lstride, skip, dot);
+}
+
+// Forms whose level-0 product can also reduce r . z: FP64 from BF16 digit
+// matrices (one CTA per domain), FP32 from packed inverses; at most 8 RHS.
+bool mas_dot_usable(gs_ctx ctx, gs_mas mas, int nrhs) {
+  if (nrhs > 8) return false;
+  if (mas->precision == GS_PREC_FP32) return level0_f32_bulk_usable(mas, nrhs);
+  const int t = ctx->tune[GS_TUNE_F64_TC];
+  return (t == 1 || t == 4) && level0_f64tc_usable(ctx, mas, nrhs);
+}
+
+// z = M^-1 r and partial sums of r . z (one per domain) from r and its level-1
+// sums (in rl, whose padding entries are zero), for the forms above.
+int mas_products_dot(gs_ctx ctx, gs_mas mas, const double* r, double* z, int nrhs, double* rl, double* zl,
+                     const int* skip, const Partials& dot) {
+  const int64_t stride = 3LL * mas->n, lstride = 3 * std::max<int64_t>(mas->vec_items, 1);
+  const bool f32 = mas->precision == GS_PREC_FP32;
+  if (mas->L > 1) {
+    // one level above level 1 sums its children itself: a launch less, which
+    // costs a large system more than it saves (64^3, 8 RHS: 22 against 18 us)
+    const bool from_kids = mas->L == 3 && (int64_t)mas->n * nrhs <= kSmallWork;
+    for (int l = 1; !from_kids && l + 1 < mas->L; ++l) {
+      GS_PROF(ctx, GS_K_MAS_APPLY_COARSE);
+      k_restrict_up<double, LevelIdxRhsMajor><<<ceil_div((int64_t)mas->n_domains[l] * 32, 128), 128, 0, ctx->stream>>>(
+          mas->up[l], mas->n_domains[l], mas->N, 3 * nrhs, LevelIdxRhsMajor{lstride, mas->vec_off[l]},
+          LevelIdxRhsMajor{lstride, mas->vec_off[l + 1]}, rl, skip);
+    }
+    if (f32) {
+      GS_TRY(coarse_f32_launch(ctx, mas, nrhs, rl, zl, lstride, skip, from_kids));
+    } else {
+      GS_PROF(ctx, GS_K_MAS_APPLY_COARSE);
+      GS_TRY(coarse_f64tc_launch(ctx, mas, nrhs, rl, zl, lstride, skip, from_kids));
+    }
+  }
+  if (f32) return level0_f32_launch<true>(ctx, mas, r, z, nrhs, zl, lstride, skip, dot);
+  GS_PROF(ctx, GS_K_MAS_APPLY_L0);
+  return level0_f64tc_launch(ctx, mas, nrhs, r, stride, zl, lstride, z, skip, &dot);
+}
+
 template <typename Ts, typename Tm>
 static int launch_apply(gs_ctx ctx, gs_mas mas, const Ts* const* d_inv, const int32_t* d_jobs, int n_coarse_jobs,
                         const double* r, double* z, int nrhs, double* rl, double* zl, const int* skip) {
@@ -362,13 +553,7 @@ static int launch_apply(gs_ctx ctx, gs_mas mas, const Ts* const* d_inv, const in
   const int N = mas->N, ld = 3 * N;
   const int64_t stride = 3LL * mas->n;
   const int64_t lstride = 3 * std::max<int64_t>(mas->vec_items, 1);
-  ApplyLevels al{};
-  al.L = mas->L;
-  al.N = N;
-  for (int l = 0; l < mas->L; ++l) {
-    al.coarse[l] = mas->coarse[l];
-    al.vec_off[l] = mas->vec_off[l];
-  }
+  const ApplyLevels al = apply_levels(mas, false);
   const int kRPT = ctx->tune[GS_TUNE_APPLY_RHS];
   const int groups = ceil_div(nrhs, kRPT);
   const int threads = ((ld * groups + 31) / 32) * 32;
@@ -387,14 +572,8 @@ static int launch_apply(gs_ctx ctx, gs_mas mas, const Ts* const* d_inv, const in
     if (level0_f64tc_usable(ctx, mas, nrhs)) {  // FP64 accuracy on the BF16 tensor cores
       GS_PROF(ctx, GS_K_MAS_APPLY_COARSE);
       GS_TRY(coarse_f64tc_launch(ctx, mas, nrhs, rl, zl, lstride, skip));
-    } else if (std::is_same<Ts, float>::value && nrhs <= 8 && n_coarse_jobs > 0) {
-      // FP32: one CTA per coarse domain, (row, 4 RHS) per thread, inverse
-      // entries loaded 16 ahead (a thread per output re-read the RHS row
-      // per output and waited on each inverse entry)
-      GS_PROF(ctx, GS_K_MAS_APPLY_COARSE);
-      const int thr = ((ld * ceil_div(nrhs, 4) + 31) / 32) * 32;
-      k_domain_product<Ts, Tm, 4, 0><<<n_coarse_jobs, thr, (size_t)ld * nrhs * sizeof(Tm), st>>>(
-          d_inv, d_jobs, d_jobs + n_coarse_jobs, N, nrhs, nullptr, nullptr, 0, nullptr, rl, zl, lstride, al);
+    } else if (std::is_same<Ts, float>::value && nrhs <= 8) {
+      GS_TRY(coarse_f32_launch(ctx, mas, nrhs, rl, zl, lstride, skip, false));
     } else {
       GS_PROF(ctx, GS_K_MAS_APPLY_COARSE);
       const int64_t outs = (int64_t)n_coarse_jobs * ld * nrhs;
@@ -406,9 +585,7 @@ static int launch_apply(gs_ctx ctx, gs_mas mas, const Ts* const* d_inv, const in
     GS_PROF(ctx, GS_K_MAS_APPLY_L0);
     GS_TRY(level0_bf16_launch(ctx, mas, false, nrhs, r, stride, zl, lstride, z, nullptr, ctx->d_flags));
   } else if (std::is_same<Ts, float>::value && level0_f32_bulk_usable(mas, nrhs)) {  // FP32, packed inverses
-    GS_PROF(ctx, GS_K_MAS_APPLY_L0);
-    k_level0_f32_cta<<<mas->n_domains[0], ((ld + 31) / 32) * 32, f32_cta_smem(N), st>>>(
-        mas->inv32p, f32_pitch(N), N, nrhs, r, z, stride, mas->remap0, zl, lstride, al, skip, ctx->d_flags);
+    GS_TRY(level0_f32_launch<false>(ctx, mas, r, z, nrhs, zl, lstride, skip, Partials{}));
   } else if (level0_f64tc_usable(ctx, mas, nrhs)) {  // FP64 accuracy on the BF16 tensor cores
     GS_PROF(ctx, GS_K_MAS_APPLY_L0);
     GS_TRY(level0_f64tc_launch(ctx, mas, nrhs, (const double*)r, stride, (const double*)zl, lstride, (double*)z,
@@ -432,8 +609,8 @@ int mas_apply_launch(gs_ctx ctx, gs_mas mas, const double* r, double* z, int nrh
   return mas_apply_launch_skip(ctx, mas, r, z, nrhs, rl, zl, nullptr);
 }
 
-// The same, but the restriction and the digit-split products return at once
-// while *skip (device) is set (PCG's all-converged word).
+// The same; the restriction and the digit-split products return at once while
+// *skip (device, may be null) is set (PCG's all-converged word).
 int mas_apply_launch_skip(gs_ctx ctx, gs_mas mas, const double* r, double* z, int nrhs, double* rl, double* zl,
                           const int* skip) {
   // the BF16 form's coarse levels are FP32 inverses

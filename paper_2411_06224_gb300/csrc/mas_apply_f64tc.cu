@@ -24,7 +24,7 @@
 // Dropped terms (p + q > 9) and the roundings of X, Y are below 2^-55 of the
 // row and column maxima, the level of FP64's own rounding.
 //
-// One CTA per domain, 128 threads; the 7 digit matrices (18 KB each) stream
+// One CTA of 256 threads per domain; the 7 digit matrices (18 KB each) stream
 // through a shared-memory ring filled by bulk asynchronous copies: 2 slots at
 // level 0 (50 KB per CTA, four CTAs share an SM and hide each other's
 // latency), 4 for the few coarse-level domains.  All waits are bounded
@@ -35,6 +35,7 @@
 
 #include "common.cuh"
 #include "fp64split.cuh"
+#include "pcg_state.cuh"
 #include "umma.cuh"
 
 namespace gs {
@@ -43,13 +44,14 @@ namespace f64tc {
 constexpr int kDigits = 7;
 constexpr int kSlots = 2;        // ring slots of the level-0 kernel (4 CTAs per SM; 3 slots and
                                  // 3 CTAs per SM measured 15 % slower)
-constexpr int kSlotsCoarse = 4;  // coarse levels: few CTAs, so a deeper ring per CTA
+constexpr int kSlotsFew = 4;     // two CTAs per SM
 constexpr int kThreads = 128;
 constexpr int kM = 128;
 constexpr int kTmemCols = 128;  // groups s = 2..10, 8 columns each (72 used)
 
 struct Levels {
   const int32_t* coarse[8];
+  const int2* kids[8];  // level l's items as sums of level l - 1's (gs_mas_s::kids), or null
   int64_t vec_off[8];
   int L;
 };
@@ -69,21 +71,29 @@ __device__ __forceinline__ double scaled_to_double(long long hi, long long lo, i
   return combine_to_double(hi, lo, 32, e);
 }
 
-// kCoarse = false: level 0, CTA = level-0 domain, r gathered through remap0,
-//   z = level-0 product + prolongated coarse results, written per node;
-// kCoarse = true: one coarse-level domain per CTA (job tables), r and z are the
-//   level's contiguous multilevel vectors rl, zl.
-template <bool kCoarse, int kS, int LD, int kT>
-__global__ void __launch_bounds__(kT) k_level0_f64tc(const __nv_bfloat16* const* __restrict__ dig_tab,
-                                                           const int32_t* const* __restrict__ exp_tab,
-                                                           const int32_t* __restrict__ job_level,
-                                                           const int32_t* __restrict__ job_dom,
-                                                           const int32_t* __restrict__ remap0, int N, int nrhs,
-                                                           Levels al, const double* __restrict__ r, int64_t stride,
-                                                           const double* __restrict__ zl, int64_t lstride,
-                                                           double* __restrict__ z, int* __restrict__ flags,
-                                                           const int* __restrict__ skip) {
+// kCoarse = false: level-0 domains, r gathered through remap0, z = level-0
+//   product + prolongated coarse results, written per node; kDot: also the
+//   domain's part of r . z per right-hand side and the exponent bound of its z;
+// kCoarse = true: coarse-level domains (job tables), r and z are the level's
+//   contiguous multilevel vectors rl, zl; a level with al.kids gathers its r
+//   as the sums of its items' children of the level below.
+// One CTA per domain (CTAs that walk several domains with everything set up
+// once and the next domain's first digits prefetched measured 0.24 ms at 64^3
+// against 0.21: the four CTAs of an SM overlap each other's prologue and
+// epilogue better than one does its own).  r . z costs a CTA ten FP64
+// instructions per warp (warp_sums), the separate pass it replaces 9 us at 45^3.
+template <bool kCoarse, bool kDot, int kS, int LD, int kT>
+__global__ void __launch_bounds__(kT, kT == 256 ? 4 : 1) k_level0_f64tc(
+    const __nv_bfloat16* const* __restrict__ dig_tab, const int32_t* const* __restrict__ exp_tab,
+    const int32_t* __restrict__ job_level, const int32_t* __restrict__ job_dom, const int32_t* __restrict__ remap0,
+    int N, int nrhs, Levels al, const double* __restrict__ r, int64_t stride,
+    const double* __restrict__ zl, int64_t lstride, double* __restrict__ z, int* __restrict__ flags,
+    const int* __restrict__ skip, Partials dot) {
   using namespace umma;
+  // The digits may be copied before the kernel ahead has ended where that is the
+  // restriction or the coarse product: it wrote neither them nor *skip.
+  constexpr bool kEarly = kCoarse || kDot;
+  if (!kEarly) wait_for_previous_kernel();
   if (skip && *skip) return;  // whole CTA, before any barrier or TMEM use
   extern __shared__ unsigned char smem_raw[];
   constexpr int ld = LD;  // 3 N
@@ -96,13 +106,12 @@ __global__ void __launch_bounds__(kT) k_level0_f64tc(const __nv_bfloat16* const*
   uint64_t* done = empty + kS;
   uint32_t* tslot = (uint32_t*)(done + 1);
   int* sfail = (int*)(tslot + 1);
-  int* sexp = sfail + 1;   // [8] biased exponent maxima of the RHS columns
-  int* snode = sexp + 8;   // [32] node of every slot of the domain (-1: padding)
+  int* sexp = sfail + 1;  // [8] biased exponent maxima of the RHS columns
+  int* snode = sexp + 8;  // [32] node of every slot of the domain (-1: padding)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int lvl = kCoarse ? job_level[blockIdx.x] : 0;
   const int32_t d = kCoarse ? job_dom[blockIdx.x] : (int32_t)blockIdx.x;
   const __nv_bfloat16* dd = dig_tab[lvl] + (int64_t)d * kDigits * ld * ld;
-  const int32_t* row_exp = exp_tab[lvl];
   const int64_t cbase = kCoarse ? 3 * (al.vec_off[lvl] + (int64_t)d * N) : 0;  // coarse: first entry of the domain
 
   if (tid == 0) {
@@ -110,6 +119,10 @@ __global__ void __launch_bounds__(kT) k_level0_f64tc(const __nv_bfloat16* const*
     mbar_init(done, 1);
     *sfail = 0;
     fence_mbar_init();
+    for (int p = 0; p < kS; ++p) {
+      mbar_arrive_expect_tx(&full[p], dig_bytes);
+      bulk_g2s(ring + p * sbytes, dd + (int64_t)p * ld * ld, dig_bytes, &full[p]);
+    }
   }
   if (tid < 8) sexp[tid] = 0;
   if (tid < 32) snode[tid] = tid < N ? (kCoarse ? 0 : remap0[(int64_t)d * N + tid]) : -1;
@@ -121,12 +134,12 @@ __global__ void __launch_bounds__(kT) k_level0_f64tc(const __nv_bfloat16* const*
   __syncthreads();
   fence_after_sync();
   const uint32_t tmem = *tslot;
-  if (tid == 0) {
-    for (int p = 0; p < kS; ++p) {
-      mbar_arrive_expect_tx(&full[p], dig_bytes);
-      bulk_g2s(ring + p * sbytes, dd + (int64_t)p * ld * ld, dig_bytes, &full[p]);
-    }
-  }
+  if (kEarly) wait_for_previous_kernel();
+  // With 256 threads, warps w and w + 4 share TMEM lane quarter w % 4 and
+  // take the right-hand sides 0..3 and 4..7 of its rows.
+  constexpr int kRpt = 8 * 128 / kT;  // right-hand sides per epilogue thread
+  const int q4 = warp & 3, k0 = (warp >> 2) * kRpt;
+  const int i_row = q4 * 32 + lane;
   // r_d once into registers (entry e = k * ld + j), column exponents by
   // shared-memory atomics, then the digits into the four pair operands
   constexpr int kPer = 8 * 128 / kT;  // entries per thread for ld <= 128
@@ -138,10 +151,17 @@ __global__ void __launch_bounds__(kT) k_level0_f64tc(const __nv_bfloat16* const*
     rv[m] = 0.0;
     if (k < nrhs && k < 8) {
       const int32_t node = snode[j / 3];
-      if (kCoarse)
-        rv[m] = r[k * lstride + cbase + j];
-      else if (node >= 0)
+      if (kCoarse) {
+        if (al.kids[lvl]) {
+          const int2 kid = al.kids[lvl][(int64_t)d * N + j / 3];
+          const double* rk = r + k * lstride + 3 * (al.vec_off[lvl - 1] + kid.x) + j % 3;
+          rv[m] = sum_children(rk, (uint32_t)kid.y);
+        } else {
+          rv[m] = r[k * lstride + cbase + j];
+        }
+      } else if (node >= 0) {
         rv[m] = r[k * stride + 3 * (int64_t)node + j % 3];
+      }
       const int eb = biased_exp(rv[m]);  // integer test: no FP64 compare
       if (eb) atomicMax(&sexp[k], eb);
     }
@@ -162,21 +182,14 @@ __global__ void __launch_bounds__(kT) k_level0_f64tc(const __nv_bfloat16* const*
   // Epilogue operands that do not depend on the MMAs, loaded now so that their
   // latency overlaps the tensor-core work: row exponent and the prolongated
   // coarse-level sum per RHS.
-  // With 256 threads, warps w and w + 4 share TMEM lane quarter w % 4 and
-  // take the right-hand sides 0..3 and 4..7 of its rows.
-  constexpr int kRpt = 8 * 128 / kT;  // right-hand sides per epilogue thread
-  const int q4 = warp & 3, k0 = (warp >> 2) * kRpt;
-  const int i_row = q4 * 32 + lane;
   const int32_t node_row = (q4 * 32 < ld && i_row < ld) ? snode[i_row / 3] : -1;
+  const int c_row = i_row % 3;
   int a_row = -100000;
   double coarse_sum[kRpt];
 #pragma unroll
   for (int k = 0; k < kRpt; ++k) coarse_sum[k] = 0.0;
-  if (node_row >= 0) {
-    a_row = row_exp[(int64_t)d * ld + i_row];
-  }
+  if (node_row >= 0) a_row = exp_tab[lvl][(int64_t)d * ld + i_row];
   if (!kCoarse && node_row >= 0) {
-    const int c = i_row % 3;
 #pragma unroll
     for (int l = 1; l < 8; ++l) {
       if (l >= al.L) break;
@@ -184,7 +197,7 @@ __global__ void __launch_bounds__(kT) k_level0_f64tc(const __nv_bfloat16* const*
 #pragma unroll
       for (int k = 0; k < kRpt; ++k)
         if (k0 + k < nrhs) {  // the first coarse level assigns: one FP64 add fewer per output
-          const double v = zl[(k0 + k) * lstride + 3 * item + c];
+          const double v = zl[(k0 + k) * lstride + 3 * item + c_row];
           coarse_sum[k] = l == 1 ? v : coarse_sum[k] + v;
         }
     }
@@ -237,6 +250,14 @@ __global__ void __launch_bounds__(kT) k_level0_f64tc(const __nv_bfloat16* const*
       mbar_arrive(done);
     }
   }
+  let_next_kernel_launch();
+  // r of this thread's row, for r . z (in cache since the gather)
+  double rrow[kRpt];
+  if (kDot) {
+#pragma unroll
+    for (int k = 0; k < kRpt; ++k)
+      rrow[k] = node_row >= 0 && k0 + k < nrhs ? r[(k0 + k) * stride + 3 * (int64_t)node_row + c_row] : 0.0;
+  }
   // warp 0 waits for the MMAs; the other warps wait at the barrier, where they
   // take no issue slots
   if (warp == 0) {
@@ -249,6 +270,10 @@ __global__ void __launch_bounds__(kT) k_level0_f64tc(const __nv_bfloat16* const*
   __syncthreads();
   const bool ok = !*sfail;
   fence_after_sync();
+  double dacc[kRpt];
+  int dex[kRpt];
+#pragma unroll
+  for (int k = 0; k < kRpt; ++k) dacc[k] = 0.0, dex[k] = kExpNone;
   if (ok && q4 * 32 < ld) {
     const uint32_t ta = tmem + ((uint32_t)(q4 * 32) << 16);
     float g[8 * kRpt];  // groups s = 2..9 of this thread's RHS: g[kRpt (s - 2) + k]
@@ -261,31 +286,46 @@ __global__ void __launch_bounds__(kT) k_level0_f64tc(const __nv_bfloat16* const*
 #pragma unroll
       for (int s = 0; s < 8; ++s) tmem_ld_32x32b_x4(ta + 8 * s + k0, g + 4 * s);
     }
-    const int32_t node = node_row;
-    if (node >= 0) {
-      const int a = a_row;
-      const int c = i_row % 3;
+    if (node_row >= 0) {
 #pragma unroll
       for (int k = 0; k < kRpt; ++k) {
         const int kk = k0 + k;
         if (kk >= nrhs) break;
         double v = 0.0;
-        if (sexp[kk] && a > -100000) {
+        if (sexp[kk] && a_row > -100000) {
           // T = hi 2^32 + lo, hi = sum_{s=2..5} G_s 256^(5-s), lo = sum_{s=6..9} G_s 256^(9-s)
           long long hi = 0, lo = 0;
 #pragma unroll
           for (int s = 0; s < 4; ++s) hi = (hi << 8) + (long long)__float2int_rn(g[kRpt * s + k]);
 #pragma unroll
           for (int s = 4; s < 8; ++s) lo = (lo << 8) + (long long)__float2int_rn(g[kRpt * s + k]);
-          const int e = a + (sexp[kk] - 1021) - 72;  // z = T 2^e, T = hi 2^32 + lo
+          const int e = a_row + (sexp[kk] - 1021) - 72;  // z = T 2^e, T = hi 2^32 + lo
           if (e < 900) v = scaled_to_double(hi, lo, e);
         }
-        if (kCoarse)
+        if (kCoarse) {
           z[kk * lstride + cbase + i_row] = v;
-        else
-          z[kk * stride + 3 * (int64_t)node + c] = v + coarse_sum[k];
+        } else {
+          v += coarse_sum[k];
+          z[kk * stride + 3 * (int64_t)node_row + c_row] = v;
+          if (kDot) {
+            dacc[k] = rrow[k] * v;
+            dex[k] = ex_bound(v);
+          }
+        }
       }
     }
+  }
+  __shared__ double red[kT / 32][kRpt];
+  __shared__ int redx[kT / 32][kRpt];
+  if (kDot) {
+    const int k = sum_index<kRpt>(lane);
+    const double v = warp_sums<kRpt>(dacc, lane);
+#pragma unroll
+    for (int q = 0; q < kRpt; ++q) {
+      const int e = __reduce_max_sync(kFull, dex[q]);
+      if (lane == 0) redx[warp][q] = e;
+    }
+    if (lane < kRpt) red[warp][k] = v;
   }
   fence_before_sync();
   __syncthreads();
@@ -293,8 +333,18 @@ __global__ void __launch_bounds__(kT) k_level0_f64tc(const __nv_bfloat16* const*
     fence_after_sync();
     tmem_dealloc(tmem, kTmemCols);
   }
+  if (kDot && tid < nrhs) {
+    double v = 0.0;
+    int e = kExpNone;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      v += red[tid / kRpt * 4 + q][tid % kRpt];
+      e = max(e, redx[tid / kRpt * 4 + q][tid % kRpt]);
+    }
+    dot.sum[(size_t)tid * dot.pitch + d] = v;
+    dot.ex[(size_t)tid * dot.pitch + d] = e;
+  }
 }
-
 
 // ---------------------------------------------------------------- persistent form
 // One CTA per SM walks domains d = blockIdx.x, + gridDim.x, ...  Warp roles:
@@ -624,8 +674,44 @@ static f64tc::Levels f64tc_levels(gs_mas mas) {
   return al;
 }
 
+template <bool kCoarse, bool kDot, int kS, int LD, int kT>
+static int launch_digits(gs_ctx ctx, gs_mas mas, int nrhs, const f64tc::Levels& al, const double* r, int64_t stride,
+                         const double* zl, int64_t lstride, double* z, const int* skip, const Partials& dot) {
+  const auto kernel = f64tc::k_level0_f64tc<kCoarse, kDot, kS, LD, kT>;
+  const size_t smem = f64tc::smem_bytes<kS>(LD);
+  GS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int jobs = kCoarse ? mas->n_coarse_jobs : mas->n_domains[0];
+  const int32_t* jt = kCoarse ? mas->d_coarse_jobs : nullptr;
+  GS_CUDA(launch_chained(ctx, (int64_t)mas->n * nrhs, kernel, dim3(jobs), dim3(kT), smem, (const __nv_bfloat16* const*)mas->d_dig_tab,
+                         (const int32_t* const*)(mas->d_dig_tab + 8), jt, jt ? jt + jobs : nullptr, mas->remap0, mas->N,
+                         nrhs, al, r, stride, zl, lstride, z, ctx->d_flags, skip, dot));
+  return GS_OK;
+}
+
+// Ring slots by the number of domains: where every SM holds one domain at
+// most, all 7 digits are copied at once (133 KB); where it holds two, 4 slots;
+// else 2, so that four CTAs share an SM (3 slots and 3 CTAs: 15 % slower).
+template <bool kCoarse, bool kDot>
+static int launch_digits_shape(gs_ctx ctx, gs_mas mas, int nrhs, const f64tc::Levels& al, const double* r,
+                               int64_t stride, const double* zl, int64_t lstride, double* z, const int* skip,
+                               const Partials& dot) {
+  const bool wide = ctx->tune[GS_TUNE_F64_TC] == 4;  // 256 threads per domain
+  const int jobs = kCoarse ? mas->n_coarse_jobs : mas->n_domains[0];
+  const int sms = std::max(ctx->sm_count, 1);
+#define GS_DIGITS(S, LD, T) launch_digits<kCoarse, kDot, S, LD, T>(ctx, mas, nrhs, al, r, stride, zl, lstride, z, skip, dot)
+  if (mas->N == 32) {  // 3 N = 96 or 48 (the digit storage is made only for N = 32 and 16)
+    if (!wide) return GS_DIGITS(f64tc::kSlots, 96, 128);
+    if (jobs <= sms) return GS_DIGITS(f64tc::kDigits, 96, 256);
+    if (jobs <= 2 * sms) return GS_DIGITS(f64tc::kSlotsFew, 96, 256);
+    return GS_DIGITS(f64tc::kSlots, 96, 256);
+  }
+  if (!wide) return GS_DIGITS(f64tc::kSlots, 48, 128);
+  return jobs <= 2 * sms ? GS_DIGITS(f64tc::kDigits, 48, 256) : GS_DIGITS(f64tc::kSlots, 48, 256);
+#undef GS_DIGITS
+}
+
 int level0_f64tc_launch(gs_ctx ctx, gs_mas mas, int nrhs, const double* r, int64_t stride, const double* zl,
-                        int64_t lstride, double* z, const int* skip) {
+                        int64_t lstride, double* z, const int* skip, const Partials* dot) {
   GS_CHECK(level0_f64tc_usable(ctx, mas, nrhs), GS_ERR_UNSUPPORTED, "FP64 tensor-core apply: not available");
   if (ctx->tune[GS_TUNE_F64_TC] == 3) return f64sym_level0_launch(ctx, mas, nrhs, r, stride, zl, lstride, z, skip);
   if (mas->n_domains[0] == 0) return GS_OK;
@@ -640,68 +726,20 @@ int level0_f64tc_launch(gs_ctx ctx, gs_mas mas, int nrhs, const double* r, int64
     GS_CUDA(cudaGetLastError());
     return GS_OK;
   }
-  const auto tabs = (const __nv_bfloat16* const*)mas->d_dig_tab;
-  const auto etabs = (const int32_t* const*)(mas->d_dig_tab + 8);
-  const size_t smem = f64tc::smem_bytes<f64tc::kSlots>(3 * mas->N);
-  // 3 N = 96 or 48 (the digit storage is made only for N = 32 and 16)
-#define GS_F64TC_L0(LD, T)                                                                                     \
-  GS_CUDA(cudaFuncSetAttribute(f64tc::k_level0_f64tc<false, f64tc::kSlots, LD, T>,                             \
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));                       \
-  f64tc::k_level0_f64tc<false, f64tc::kSlots, LD, T><<<mas->n_domains[0], T, smem, ctx->stream>>>(              \
-      tabs, etabs, nullptr, nullptr, mas->remap0, mas->N, nrhs, f64tc_levels(mas), r, stride, zl, lstride, z,   \
-      ctx->d_flags, skip)
-  const bool wide = ctx->tune[GS_TUNE_F64_TC] == 4;  // 256 threads per domain
-  if (mas->N == 32) {
-    if (wide) {
-      GS_F64TC_L0(96, 256);
-    } else {
-      GS_F64TC_L0(96, 128);
-    }
-  } else {
-    if (wide) {
-      GS_F64TC_L0(48, 256);
-    } else {
-      GS_F64TC_L0(48, 128);
-    }
-  }
-#undef GS_F64TC_L0
-  GS_CUDA(cudaGetLastError());
-  return GS_OK;
+  return dot ? launch_digits_shape<false, true>(ctx, mas, nrhs, f64tc_levels(mas), r, stride, zl, lstride, z, skip, *dot)
+             : launch_digits_shape<false, false>(ctx, mas, nrhs, f64tc_levels(mas), r, stride, zl, lstride, z, skip,
+                                                 Partials{});
 }
 
 int coarse_f64tc_launch(gs_ctx ctx, gs_mas mas, int nrhs, const double* rl, double* zl, int64_t lstride,
-                        const int* skip) {
+                        const int* skip, bool from_kids) {
   GS_CHECK(level0_f64tc_usable(ctx, mas, nrhs), GS_ERR_UNSUPPORTED, "FP64 tensor-core apply: not available");
   if (ctx->tune[GS_TUNE_F64_TC] == 3) return f64sym_coarse_launch(ctx, mas, nrhs, rl, zl, lstride, skip);
   if (mas->n_coarse_jobs == 0) return GS_OK;
-  // a few hundred coarse domains at most: a deeper ring per CTA shortens the
-  // chain of copy latencies that bounds this small launch
-  const size_t smem = f64tc::smem_bytes<f64tc::kSlotsCoarse>(3 * mas->N);
-  const auto tabs = (const __nv_bfloat16* const*)mas->d_dig_tab;
-  const auto etabs = (const int32_t* const*)(mas->d_dig_tab + 8);
-#define GS_F64TC_CO(LD, T)                                                                                       \
-  GS_CUDA(cudaFuncSetAttribute(f64tc::k_level0_f64tc<true, f64tc::kSlotsCoarse, LD, T>,                          \
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));                         \
-  f64tc::k_level0_f64tc<true, f64tc::kSlotsCoarse, LD, T><<<mas->n_coarse_jobs, T, smem, ctx->stream>>>(         \
-      tabs, etabs, mas->d_coarse_jobs, mas->d_coarse_jobs + mas->n_coarse_jobs, nullptr, mas->N, nrhs,             \
-      f64tc_levels(mas), rl, 0, nullptr, lstride, zl, ctx->d_flags, skip)
-  const bool wide = ctx->tune[GS_TUNE_F64_TC] == 4;  // 256 threads per domain
-  if (mas->N == 32) {
-    if (wide) {
-      GS_F64TC_CO(96, 256);
-    } else {
-      GS_F64TC_CO(96, 128);
-    }
-  } else {
-    if (wide) {
-      GS_F64TC_CO(48, 256);
-    } else {
-      GS_F64TC_CO(48, 128);
-    }
-  }
-#undef GS_F64TC_CO
-  GS_CUDA(cudaGetLastError());
-  return GS_OK;
+  f64tc::Levels al = f64tc_levels(mas);
+  if (from_kids)
+    for (int l = 2; l < mas->L; ++l) al.kids[l] = mas->kids[l];
+  return launch_digits_shape<true, false>(ctx, mas, nrhs, al, rl, 0, nullptr, lstride, zl, skip, Partials{});
 }
 
 }  // namespace gs

@@ -141,6 +141,15 @@ __global__ void k_up_of_item(int32_t n_items_pad, int N, const int32_t* __restri
   up[a] = id >= 0 ? dom_off[a / N] + id : -1;
 }
 
+// The same map from above: the children of every level-(l+1) item, all in one
+// level-l domain, as the domain's first item and a lane mask.
+__global__ void k_kids_of_item(int32_t n_items_pad, int N, const int32_t* __restrict__ up, int2* __restrict__ kids) {
+  int32_t a = blockIdx.x * blockDim.x + threadIdx.x;
+  if (a >= n_items_pad || up[a] < 0) return;
+  kids[up[a]].x = a / N * N;
+  atomicOr((unsigned*)&kids[up[a]].y, 1u << (a % N));
+}
+
 // ------------------------------------------------------------------ level matrices
 struct LevelPtrs {
   const int32_t* coarse[8];
@@ -440,6 +449,7 @@ int gs_mas_destroy(gs_mas mas) {
   gs_ctx c = mas->owner;
   for (auto p : mas->coarse) c->release(p);
   for (auto p : mas->up) c->release(p);
+  for (auto p : mas->kids) c->release(p);
   for (auto p : mas->inv64) c->release(p);
   for (auto p : mas->inv32) c->release(p);
   c->release(mas->inv32p);
@@ -562,6 +572,13 @@ int gs_build_mas(gs_ctx ctx, gs_mat mat, const int32_t* map, int32_t n_dom0, con
       if ((s = ctx->alloc((void**)&u, (size_t)ndom * N * 4))) return fail(s);
       mas->up[l] = u;
       { GS_PROF(ctx, GS_K_MAS_LEVELS); k_up_of_item<<<ceil_div((int64_t)ndom * N, 256), 256, 0, st>>>(ndom * N, N, local_id, dom_off, u); }
+      int2* kids = nullptr;
+      const size_t kb = (size_t)ceil_div(n_next, N) * N * sizeof(int2);
+      if ((s = ctx->alloc((void**)&kids, kb))) return fail(s);
+      mas->kids.resize(l + 1, nullptr);
+      mas->kids.push_back(kids);
+      if (cudaMemsetAsync(kids, 0, kb, st) != cudaSuccess) return fail(GS_ERR_CUDA);
+      { GS_PROF(ctx, GS_K_MAS_LEVELS); k_kids_of_item<<<ceil_div((int64_t)ndom * N, 256), 256, 0, st>>>(ndom * N, N, u, kids); }
     }
     mas->n_items.push_back(n_next);
     mas->n_domains.push_back(ceil_div(n_next, N));
@@ -569,6 +586,7 @@ int gs_build_mas(gs_ctx ctx, gs_mat mat, const int32_t* map, int32_t n_dom0, con
   }
   mas->L = (int)mas->coarse.size();
   mas->up.resize(mas->L, nullptr);
+  mas->kids.resize(mas->L, nullptr);
   if ((s = mas_numeric(ctx, mas, mat))) return fail(s);
   *out = mas;
   return GS_OK;

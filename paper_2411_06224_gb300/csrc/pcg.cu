@@ -1,24 +1,30 @@
 // Preconditioned conjugate gradients for several right-hand sides (Sec. 3.2).
 //
 // Per iteration (one SpMV per RHS):
-//   Ap = A p                         spmv.cu
-//   alpha = rz / (p . Ap)            k_dot (finalised on the device)
-//   x += alpha p, r -= alpha Ap      k_update_xr, fused with ||r||^2 and the
-//                                    per-RHS convergence test
-//   z = M^{-1} r                     mas_apply.cu
-//   beta = (r . z) / rz, rz = r . z  k_dot
-//   p = z + beta p                   k_update_p
-// Every reduction is deterministic: a fixed grid writes per-block partials
-// and the last block to finish sums them in block order and updates the
-// per-RHS scalars, so no scalar ever travels to the host inside the loop.
-// A RHS stops moving once converged (alpha = 0), which keeps each RHS on
-// exactly its own single-RHS recurrence.  Kernels return at once after
-// every RHS converged; the host only polls that flag every few iterations.
+//   Ap = A p, alpha = rz / (p . Ap)
+//   x += alpha p, r -= alpha Ap, ||r||^2 and the per-RHS convergence test
+//   z = M^{-1} r, beta = (r . z) / rz, rz = r . z
+//   p = z + beta p
+// For up to 8 right-hand sides each line but the third is one kernel
+// (pcg_fused.cu), and where the preconditioner's form allows it (mas_dot_usable)
+// the second also restricts r and the third also takes r . z: five kernels,
+// launched so that each is resident when the one before it ends.  Other counts
+// and forms run the product, the dot product or the apply as separate passes
+// (k_dot, k_update_xr here).
+// Every reduction is deterministic: a fixed grid writes partial sums, and the
+// kernels that need the scalar add them in a fixed order (pcg_state.cuh), so
+// no scalar ever travels to the host inside the loop.  The convergence test of
+// an iteration is taken with its direction update.  A RHS stops moving once
+// converged (alpha = 0), which keeps each RHS on exactly its own single-RHS
+// recurrence.  Kernels return at once after every RHS converged; the host polls
+// that flag every four iterations, one poll behind, so that the GPU always has
+// the next iterations queued.
 #include <algorithm>
 #include <cmath>
 
 #include "common.cuh"
 #include "ff.cuh"
+#include "pcg_state.cuh"
 #include "primitives.cuh"
 
 namespace gs {
@@ -28,30 +34,19 @@ int mas_apply_launch(gs_ctx ctx, gs_mas mas, const double* r, double* z, int nrh
 int mas_level_vectors(gs_ctx ctx, gs_mas mas, int nrhs, double** rl, double** zl);
 int ensure_row_order(gs_ctx ctx, gs_mat m);
 
-constexpr int kMaxRhs = 32;
+int pcg_spmv_dot(gs_ctx ctx, gs_mat m, const float2* ps, const double* p, double* Ap, int nrhs, const PcgScalars* s,
+                 Partials& pap);
+int pcg_update_xr(gs_ctx ctx, gs_mas mas, double* x, double* r, const double* p, const double* Ap, int nrhs, double* rl,
+                  int64_t lstride, PcgScalars* s, const Partials& pap, Partials& rrp, int parity);
+int pcg_update_p(gs_ctx ctx, gs_mat m, double* p, const double* z, float2* ps, int nrhs, PcgScalars* s,
+                 const Partials& rrp, const Partials& rzp, Partials fold, double tol2, int parity);
+bool mas_dot_usable(gs_ctx ctx, gs_mas mas, int nrhs);
+int mas_products_dot(gs_ctx ctx, gs_mas mas, const double* r, double* z, int nrhs, double* rl, double* zl,
+                     const int* skip, const Partials& dot);
+
 constexpr int kRedThreads = 256;
-constexpr int kMaxRedBlocks = 256;  // reduction blocks per right-hand side
-constexpr int kUnroll = 4;          // strided elements per thread and pass of k_dot and k_update_p
-
-struct PcgScalars {
-  double bnorm2[kMaxRhs];
-  double rz[kMaxRhs];
-  double alpha[kMaxRhs];
-  double beta[kMaxRhs];
-  double rr[kMaxRhs];
-  int conv[kMaxRhs];
-  int iters[kMaxRhs];
-  // float-float SpMV operand (GS_SPMV_ROW_FF): |z| < 2^fz, |p| < 2^fp, and
-  // the split copy of p holds p 2^(k_node - K - fsplit)
-  int fz[kMaxRhs];
-  int fp[kMaxRhs];
-  int fsplit[kMaxRhs];
-  int all_conv;
-  unsigned counter;
-  int flags;
-};
-
-enum DotOp : int { kOpBnorm = 0, kOpRzInit, kOpPAp, kOpRR, kOpRz };
+constexpr int kMaxChunks = 256;     // reduction blocks per right-hand side of the kernels here
+constexpr int kUnroll = 4;          // strided elements per thread and pass of k_dot
 
 // Grid of the vector kernels: (G, nrhs); block (g, k) covers a contiguous
 // chunk of right-hand side k.  G depends only on the vector length, the RHS
@@ -67,7 +62,7 @@ inline int red_blocks(int64_t len, int nrhs, int sms) {
   const int64_t want = (2LL * std::max(sms, 1) + nrhs - 1) / nrhs;
   const int64_t cap8 = (len + kRedThreads * 8 - 1) / (kRedThreads * 8);
   g = std::max(g, std::min(want, cap8));
-  return (int)std::max<int64_t>(1, std::min<int64_t>(g, kMaxRedBlocks));
+  return (int)std::max<int64_t>(1, std::min<int64_t>(g, kMaxChunks));
 }
 
 __device__ __forceinline__ double block_sum(double v) {
@@ -108,101 +103,14 @@ __device__ __forceinline__ void chunk_of(int64_t len, int64_t& b, int64_t& e) {
   e = b + per < len ? b + per : len;
 }
 
-__device__ void apply_op(PcgScalars* s, int k, double sum, int op, double tol2) {
-  if (!isfinite(sum)) {
-    atomicOr(&s->flags, kErrNonFinite);
-    s->conv[k] = 1;
-    s->alpha[k] = 0.0;
-    return;
-  }
-  switch (op) {
-    case kOpBnorm:
-      s->bnorm2[k] = sum;
-      s->conv[k] = sum == 0.0;
-      s->iters[k] = 0;
-      s->rr[k] = sum;
-      break;
-    case kOpRzInit:
-      s->rz[k] = sum;
-      break;
-    case kOpPAp:
-      if (s->conv[k]) {
-        s->alpha[k] = 0.0;
-      } else if (!(sum > 0.0)) {
-        atomicOr(&s->flags, kErrNotSPD);
-        s->conv[k] = 1;
-        s->alpha[k] = 0.0;
-      } else {
-        s->alpha[k] = s->rz[k] / sum;
-      }
-      break;
-    case kOpRR:
-      if (!s->conv[k]) {
-        s->rr[k] = sum;
-        s->iters[k] += 1;
-        if (sum <= tol2 * s->bnorm2[k]) s->conv[k] = 1;
-      }
-      break;
-    case kOpRz:
-      s->beta[k] = s->conv[k] ? 0.0 : sum / s->rz[k];
-      s->rz[k] = sum;
-      break;
-  }
-}
-
-// Write this block's partial; the last block to arrive reduces all partials
-// of every right-hand side in a fixed order and updates the scalars.  With
-// ipart, each block also posts the largest exponent bound of the vector it
-// read (my_ex, valid in thread 0), and the last block keeps the maximum per
-// RHS as fz (and fp for op kOpRzInit, where p = z).
-__device__ void finalize(PcgScalars* s, double* __restrict__ partials, double my_partial, int nrhs, int op,
-                         double tol2, int* __restrict__ ipart = nullptr, int my_ex = kExpNone) {
-  __shared__ bool last;
-  if (threadIdx.x == 0) {
-    partials[blockIdx.y * kMaxRedBlocks + blockIdx.x] = my_partial;
-    if (ipart) ipart[blockIdx.y * kMaxRedBlocks + blockIdx.x] = my_ex;
-    __threadfence();
-    const unsigned total = gridDim.x * gridDim.y;
-    last = atomicInc(&s->counter, total - 1) == total - 1;
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  // one warp per right-hand side (fixed order: lane, then stride 32, then
-  // the shuffle tree), so the tail costs one warp reduction, not nrhs block ones
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int k = w; k < nrhs; k += kRedThreads / 32) {
-    double v = 0.0;
-    for (int g = lane; g < (int)gridDim.x; g += 32) v += __ldcg(&partials[k * kMaxRedBlocks + g]);
-    v = warp_sum(v);
-    if (lane == 0) apply_op(s, k, v, op, tol2);
-    if (ipart) {
-      int e = kExpNone;
-      for (int g = lane; g < (int)gridDim.x; g += 32) e = max(e, __ldcg(&ipart[k * kMaxRedBlocks + g]));
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(kFull, e, o));
-      if (lane == 0) {
-        s->fz[k] = e;
-        if (op == kOpRzInit) s->fp[k] = e;
-      }
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int all = 1;
-    for (int k = 0; k < nrhs; ++k) all &= s->conv[k] != 0;
-    s->all_conv = all;
-  }
-}
-
-// a_k . b_k per right-hand side; kCopy also writes dst = b (p = z); kEx also
-// takes the largest exponent bound of b (z) for the float-float SpMV operand.
-template <bool kCopy, bool kEx = false>
+// Partial sums of a_k . b_k, block (g, k) its chunk of right-hand side k; kCopy
+// also writes dst = b (p = z); kEx also the exponent bound of the chunk of b
+// (z) for the float-float SpMV operand.
+template <bool kCopy, bool kEx>
 __global__ void __launch_bounds__(kRedThreads) k_dot(const double* __restrict__ a, const double* __restrict__ b,
-                                                     double* __restrict__ dst, int64_t len, int nrhs,
-                                                     PcgScalars* s, double* __restrict__ partials, int op,
-                                                     int* __restrict__ ipart = nullptr) {
-  if (s->all_conv && op != kOpBnorm && op != kOpRzInit) return;
+                                                     double* __restrict__ dst, int64_t len, const int* __restrict__ skip,
+                                                     Partials out) {
+  if (skip && *skip) return;
   const int64_t o = (int64_t)blockIdx.y * len;
   int64_t i0, i1;
   chunk_of(len, i0, i1);
@@ -229,13 +137,17 @@ __global__ void __launch_bounds__(kRedThreads) k_dot(const double* __restrict__ 
       }
     }
   }
+  v = block_sum(v);
   if (kEx) ex = block_max(ex);
-  finalize(s, partials, block_sum(v), nrhs, op, 0.0, kEx ? ipart : nullptr, ex);
+  if (threadIdx.x == 0) {
+    out.sum[blockIdx.y * out.pitch + blockIdx.x] = v;
+    if (kEx) out.ex[blockIdx.y * out.pitch + blockIdx.x] = ex;
+  }
 }
 
+// x = 0, r = b, partial sums of ||b||^2.
 __global__ void __launch_bounds__(kRedThreads) k_init(const double* __restrict__ bvec, double* __restrict__ x,
-                                                      double* __restrict__ r, int64_t len, int nrhs, PcgScalars* s,
-                                                      double* __restrict__ partials) {
+                                                      double* __restrict__ r, int64_t len, Partials out) {
   const int64_t o = (int64_t)blockIdx.y * len;
   int64_t i0, i1;
   chunk_of(len, i0, i1);
@@ -246,16 +158,55 @@ __global__ void __launch_bounds__(kRedThreads) k_init(const double* __restrict__
     r[o + i] = bb;
     v += bb * bb;
   }
-  finalize(s, partials, block_sum(v), nrhs, kOpBnorm, 0.0);
+  v = block_sum(v);
+  if (threadIdx.x == 0) out.sum[blockIdx.y * out.pitch + blockIdx.x] = v;
 }
 
+// The first scalars, block k right-hand side k (s is zeroed): ||b||^2, rz = r . z
+// of the first z, and the exponent bounds of p = z.
+__global__ void __launch_bounds__(kRedThreads) k_first_scalars(PcgScalars* s, Partials bb, Partials rz) {
+  const int k = blockIdx.x;
+  const double b2 = warp_sum_partials(bb, k), z0 = warp_sum_partials(rz, k);
+  int ex = kExpNone;
+  if (rz.ex)
+    for (int g = threadIdx.x; g < rz.n; g += kRedThreads) ex = max(ex, rz.ex[k * rz.pitch + g]);
+  ex = block_max(ex);
+  if (threadIdx.x != 0) return;
+  const bool finite = isfinite(b2) && isfinite(z0);
+  if (!finite) atomicOr(&s->flags, kErrNonFinite);
+  s->bnorm2[k] = s->rr[k] = b2;
+  s->rz[0][k] = z0;
+  s->fz[k] = s->fp[0][k] = ex;
+  s->fp[1][k] = kExpNone;
+  s->conv[k] = !finite || b2 == 0.0;
+  if (!s->conv[k]) atomicAdd(&s->running, 1);
+}
+__global__ void k_first_running(PcgScalars* s) { s->all_conv = s->running == 0; }
+
+// The last iteration's convergence tests, where no direction update follows.
+__global__ void __launch_bounds__(32) k_last_scalars(PcgScalars* s, Partials rrp, double tol2) {
+  if (s->all_conv) return;
+  const double rr = warp_sum_partials(rrp, blockIdx.x);
+  if (threadIdx.x == 0) test_convergence(s, blockIdx.x, rr, tol2, true);
+}
+
+// x += alpha p, r -= alpha Ap with alpha from the partial sums of p . Ap, and
+// partial sums of ||r||^2; block (g, k) its chunk of right-hand side k.
 __global__ void __launch_bounds__(kRedThreads) k_update_xr(double* __restrict__ x, double* __restrict__ r,
                                                            const double* __restrict__ p, const double* __restrict__ Ap,
-                                                           int64_t len, int nrhs, PcgScalars* s,
-                                                           double* __restrict__ partials, double tol2) {
+                                                           int64_t len, PcgScalars* s, Partials pap, Partials rrp,
+                                                           int parity) {
   if (s->all_conv) return;
   const int k = blockIdx.y;
-  const double al = s->alpha[k];
+  const bool record = blockIdx.x == 0 && threadIdx.x == 0;
+  __shared__ double s_alpha;
+  if (threadIdx.x < 32) {
+    const double sum = warp_sum_partials(pap, k);
+    if (threadIdx.x == 0) s_alpha = take_alpha(s, k, sum, parity, record);
+  }
+  if (record) s->fp[parity ^ 1][k] = kExpNone;  // k_pcg_p gathers there
+  __syncthreads();
+  const double al = s_alpha;
   const int64_t o = (int64_t)k * len;
   int64_t i0, i1;
   chunk_of(len, i0, i1);
@@ -269,106 +220,16 @@ __global__ void __launch_bounds__(kRedThreads) k_update_xr(double* __restrict__ 
     }
     v += rk * rk;
   }
-  finalize(s, partials, block_sum(v), nrhs, kOpRR, tol2);
+  v = block_sum(v);
+  if (threadIdx.x == 0) rrp.sum[k * rrp.pitch + blockIdx.x] = v;
 }
 
-__global__ void __launch_bounds__(kRedThreads) k_update_p(double* __restrict__ p, const double* __restrict__ z,
-                                                          int64_t len, const PcgScalars* s) {
-  const int k = blockIdx.y;
-  if (s->all_conv || s->conv[k]) return;
-  const double be = s->beta[k];
-  const int64_t o = (int64_t)k * len;
-  int64_t i0, i1;
-  chunk_of(len, i0, i1);
-  const int64_t T = blockDim.x;
-  for (int64_t i = i0 + threadIdx.x; i < i1; i += kUnroll * T) {
-    double zv[kUnroll], pv[kUnroll];
-#pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      const int64_t j = i + u * T;
-      zv[u] = j < i1 ? z[o + j] : 0.0;
-      pv[u] = j < i1 ? p[o + j] : 0.0;
-    }
-#pragma unroll
-    for (int u = 0; u < kUnroll; ++u)
-      if (i + u * T < i1) p[o + i + u * T] = zv[u] + be * pv[u];
-  }
-}
-
-// p = z + beta p (as k_update_p), and the float-float operand of the next
-// SpMV: ps = split(p 2^(k_node - K - F)) with 2^F above |p|, taken from the
-// bounds |z| < 2^fz, |p_old| < 2^fp, |beta| < 2^eb as max(fz, fp + eb) + 1.
-// ps is node-major across right-hand sides, ps[(node * nrhs + k) * 3 + c],
-// so the SpMV gathers all RHS of a column in one contiguous stretch.
-// The blocks also post the exponent bound of the new p, which the last block
-// keeps as fp.  A converged RHS keeps p, ps, fp and fsplit unchanged.
-__global__ void __launch_bounds__(kRedThreads) k_update_p_ff(double* __restrict__ p, const double* __restrict__ z,
-                                                             float2* __restrict__ ps,
-                                                             const int32_t* __restrict__ kk, int64_t len, int nrhs,
-                                                             PcgScalars* s, int* __restrict__ ipart) {
-  if (s->all_conv) return;  // every block leaves: no arrival is expected
-  const int k = blockIdx.y;
-  int ex = kExpNone;
-  if (!s->conv[k]) {
-    const double be = s->beta[k];
-    const int eb = ex_bound(be);
-    const int fp = s->fp[k], fz = s->fz[k];
-    const int fb = (fp == kExpNone || eb == kExpNone) ? kExpNone : fp + eb;
-    const int fmax = max(fz, fb);
-    const int F = fmax == kExpNone ? 0 : fmax + 1;
-    if (blockIdx.x == 0 && threadIdx.x == 0) s->fsplit[k] = F;
-    const int64_t o = (int64_t)k * len;
-    int64_t i0, i1;
-    chunk_of(len, i0, i1);
-    const int64_t T = blockDim.x;
-    for (int64_t i = i0 + threadIdx.x; i < i1; i += kUnroll * T) {
-      double zv[kUnroll], pv[kUnroll];
-#pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        const int64_t j = i + u * T;
-        zv[u] = j < i1 ? z[o + j] : 0.0;
-        pv[u] = j < i1 ? p[o + j] : 0.0;
-      }
-#pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        const int64_t j = i + u * T;
-        if (j < i1) {
-          const double v = zv[u] + be * pv[u];
-          p[o + j] = v;
-          ex = max(ex, ex_bound(v));
-          const uint32_t node = (uint32_t)j / 3u;
-          ps[((int64_t)node * nrhs + k) * 3 + ((uint32_t)j - 3u * node)] = ff_split_bits(v, kk[node] - F);
-        }
-      }
-    }
-  }
-  ex = block_max(ex);
-  __shared__ bool last;
-  if (threadIdx.x == 0) {
-    ipart[blockIdx.y * kMaxRedBlocks + blockIdx.x] = ex;
-    __threadfence();
-    const unsigned total = gridDim.x * gridDim.y;
-    last = atomicInc(&s->counter, total - 1) == total - 1;
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int q = w; q < nrhs; q += kRedThreads / 32) {
-    int e = kExpNone;
-    for (int g = lane; g < (int)gridDim.x; g += 32) e = max(e, __ldcg(&ipart[q * kMaxRedBlocks + g]));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(kFull, e, o));
-    if (lane == 0 && !s->conv[q]) s->fp[q] = e;
-  }
-}
-
-// The first split of p (p = z, |p| < 2^fp): fsplit = fp.
+// The first split of p (p = z, |p| < 2^fz): fsplit = fz.
 __global__ void __launch_bounds__(kRedThreads) k_split_p(const double* __restrict__ p, float2* __restrict__ ps,
                                                          const int32_t* __restrict__ kk, int64_t len, int nrhs,
                                                          PcgScalars* s) {
   const int k = blockIdx.y;
-  const int F = s->fp[k] == kExpNone ? 0 : s->fp[k];
+  const int F = s->fz[k] == kExpNone ? 0 : s->fz[k];
   if (blockIdx.x == 0 && threadIdx.x == 0) s->fsplit[k] = F;
   const int64_t o = (int64_t)k * len;
   int64_t i0, i1;
@@ -401,66 +262,116 @@ extern "C" int gs_pcg_solve(gs_ctx ctx, gs_mat mat, gs_mas mas, const double* b,
   GS_TRY(ctx->scratch_buf(kSlotPcgVectors, (ff ? 5 : 4) * vbytes, (void**)&vec));
   double *r = vec, *z = r + nrhs * len, *p = z + nrhs * len, *Ap = p + nrhs * len;
   float2* ps = (float2*)(Ap + nrhs * len);  // float-float operand (same size as a vector)
+  const bool fused_spmv = nrhs <= 8 && variant != GS_SPMV_SRBK;
+  // beyond kSmallWork the separate passes are faster: x, r streamed (55 us at
+  // 64^3, 8 RHS), restricted (22), r . z streamed (22)
+  const bool fused_mas = mas_dot_usable(ctx, mas, nrhs) && (int64_t)mat->n * nrhs <= kSmallWork;
+  // scalars; partial sums of p . Ap, ||r||^2, r . z (per domain where the MAS
+  // product takes it) and r . z folded
+  const int rz_pitch = std::max(kMaxRedBlocks, fused_mas ? mas->n_domains[0] : 0);
+  const size_t rows = (size_t)nrhs * (3 * kMaxRedBlocks + rz_pitch), erows = (size_t)nrhs * (kMaxRedBlocks + rz_pitch);
   char* sbuf = nullptr;
-  const size_t part_bytes = kMaxRedBlocks * kMaxRhs * sizeof(double);
-  GS_TRY(ctx->scratch_buf(kSlotPcgScalars, sizeof(PcgScalars) + part_bytes + kMaxRedBlocks * kMaxRhs * sizeof(int) + 256,
-                          (void**)&sbuf));
+  GS_TRY(ctx->scratch_buf(kSlotPcgScalars, sizeof(PcgScalars) + 256 + rows * 8 + erows * 4, (void**)&sbuf));
   PcgScalars* s = (PcgScalars*)sbuf;
-  double* partials = (double*)(sbuf + ((sizeof(PcgScalars) + 255) / 256) * 256);
-  int* ipart = (int*)((char*)partials + part_bytes);
+  double* sums = (double*)(sbuf + ((sizeof(PcgScalars) + 255) / 256) * 256);
+  int* exps = (int*)(sums + rows);
+  Partials pap, rrp, fold, rzp;
+  pap.sum = sums, pap.pitch = kMaxRedBlocks;
+  rrp.sum = sums + (size_t)nrhs * kMaxRedBlocks, rrp.pitch = kMaxRedBlocks;
+  fold.sum = sums + 2 * (size_t)nrhs * kMaxRedBlocks, fold.ex = exps, fold.pitch = kMaxRedBlocks;
+  rzp.sum = sums + 3 * (size_t)nrhs * kMaxRedBlocks, rzp.ex = exps + (size_t)nrhs * kMaxRedBlocks, rzp.pitch = rz_pitch;
   double *rl, *zl;
   GS_TRY(mas_level_vectors(ctx, mas, nrhs, &rl, &zl));
   GS_CUDA(cudaMemsetAsync(s, 0, sizeof(PcgScalars), st));
-  if (variant != GS_SPMV_SRBK) GS_TRY(ensure_row_order(ctx, mat));  // built once per matrix
-  if (ff) GS_TRY(ensure_ff(ctx, mat));
+  if (fused_spmv) {  // built once per matrix
+    GS_TRY(ensure_sliced(ctx, mat, ff));
+  } else {
+    if (variant != GS_SPMV_SRBK) GS_TRY(ensure_row_order(ctx, mat));
+    if (ff) GS_TRY(ensure_ff(ctx, mat));
+  }
 
   const double tol2 = tol * tol;
   const dim3 vg(red_blocks(len, nrhs, ctx->sm_count), nrhs);
-  { GS_PROF(ctx, GS_K_PCG_VECTOR); k_init<<<vg, kRedThreads, 0, st>>>(b, x, r, len, nrhs, s, partials); }
+  rrp.n = rzp.n = vg.x;
+  { GS_PROF(ctx, GS_K_PCG_VECTOR); k_init<<<vg, kRedThreads, 0, st>>>(b, x, r, len, rrp); }
   GS_TRY(mas_apply_launch(ctx, mas, r, z, nrhs, rl, zl));
-  if (ff) {
-    { GS_PROF(ctx, GS_K_PCG_VECTOR); k_dot<true, true><<<vg, kRedThreads, 0, st>>>(r, z, p, len, nrhs, s, partials, kOpRzInit, ipart); }
-    { GS_PROF(ctx, GS_K_PCG_VECTOR); k_split_p<<<vg, kRedThreads, 0, st>>>(p, ps, mat->ff_k, len, nrhs, s); }
-  } else {
+  {
     GS_PROF(ctx, GS_K_PCG_VECTOR);
-    k_dot<true><<<vg, kRedThreads, 0, st>>>(r, z, p, len, nrhs, s, partials, kOpRzInit);
+    if (ff)
+      k_dot<true, true><<<vg, kRedThreads, 0, st>>>(r, z, p, len, nullptr, rzp);
+    else
+      k_dot<true, false><<<vg, kRedThreads, 0, st>>>(r, z, p, len, nullptr, rzp);
   }
+  Partials rz0 = rzp;
+  if (!ff) rz0.ex = nullptr, ps = nullptr;
+  { GS_PROF(ctx, GS_K_PCG_VECTOR); k_first_scalars<<<nrhs, kRedThreads, 0, st>>>(s, rrp, rz0); }
+  { GS_PROF(ctx, GS_K_PCG_VECTOR); k_first_running<<<1, 1, 0, st>>>(s); }
+  if (ff) { GS_PROF(ctx, GS_K_PCG_VECTOR); k_split_p<<<vg, kRedThreads, 0, st>>>(p, ps, mat->ff_k, len, nrhs, s); }
+  const int64_t lstride = 3 * std::max<int64_t>(mas->vec_items, 1);
   const int poll = 4;
   int* h_conv = ctx->h_pinned + 64;
-  for (int it = 0; it < max_iter; ++it) {
-    if (ff)
-      GS_TRY(spmv_ff_split_launch(ctx, mat, ps, s->fsplit, Ap, nrhs, &s->all_conv));
-    else
-      GS_TRY(spmv_launch_skip(ctx, mat, p, Ap, nrhs, variant, &s->all_conv));
-    { GS_PROF(ctx, GS_K_PCG_VECTOR); k_dot<false><<<vg, kRedThreads, 0, st>>>(p, Ap, nullptr, len, nrhs, s, partials, kOpPAp); }
-    { GS_PROF(ctx, GS_K_PCG_VECTOR); k_update_xr<<<vg, kRedThreads, 0, st>>>(x, r, p, Ap, len, nrhs, s, partials, tol2); }
-    if (it + 1 == max_iter) break;
-    GS_TRY(mas_apply_launch_skip(ctx, mas, r, z, nrhs, rl, zl, &s->all_conv));
-    if (ff) {
-      { GS_PROF(ctx, GS_K_PCG_VECTOR); k_dot<false, true><<<vg, kRedThreads, 0, st>>>(r, z, nullptr, len, nrhs, s, partials, kOpRz, ipart); }
-      { GS_PROF(ctx, GS_K_PCG_VECTOR); k_update_p_ff<<<vg, kRedThreads, 0, st>>>(p, z, ps, mat->ff_k, len, nrhs, s, ipart); }
+  for (int q = 0; q < 2; ++q)
+    if (!ctx->poll_event[q]) GS_CUDA(cudaEventCreateWithFlags(&ctx->poll_event[q], cudaEventDisableTiming));
+  for (int it = 0, polls = 0; it < max_iter; ++it) {
+    const int parity = it & 1;
+    if (fused_spmv) {
+      GS_TRY(pcg_spmv_dot(ctx, mat, ps, p, Ap, nrhs, s, pap));
     } else {
-      { GS_PROF(ctx, GS_K_PCG_VECTOR); k_dot<false><<<vg, kRedThreads, 0, st>>>(r, z, nullptr, len, nrhs, s, partials, kOpRz); }
-      { GS_PROF(ctx, GS_K_PCG_VECTOR); k_update_p<<<vg, kRedThreads, 0, st>>>(p, z, len, s); }
+      if (ff)
+        GS_TRY(spmv_ff_split_launch(ctx, mat, ps, s->fsplit, Ap, nrhs, &s->all_conv));
+      else
+        GS_TRY(spmv_launch_skip(ctx, mat, p, Ap, nrhs, variant, &s->all_conv));
+      GS_PROF(ctx, GS_K_PCG_VECTOR);
+      pap.n = vg.x;
+      k_dot<false, false><<<vg, kRedThreads, 0, st>>>(p, Ap, nullptr, len, &s->all_conv, pap);
     }
+    if (fused_mas) {
+      GS_TRY(pcg_update_xr(ctx, mas, x, r, p, Ap, nrhs, rl, lstride, s, pap, rrp, parity));
+    } else {
+      GS_PROF(ctx, GS_K_PCG_VECTOR);
+      k_update_xr<<<vg, kRedThreads, 0, st>>>(x, r, p, Ap, len, s, pap, rrp, parity);
+    }
+    if (it + 1 == max_iter) {
+      GS_PROF(ctx, GS_K_PCG_VECTOR);
+      k_last_scalars<<<nrhs, 32, 0, st>>>(s, rrp, tol2);
+      break;
+    }
+    if (fused_mas) {
+      rzp.n = mas->n_domains[0];
+      GS_TRY(mas_products_dot(ctx, mas, r, z, nrhs, rl, zl, &s->all_conv, rzp));
+    } else {
+      GS_TRY(mas_apply_launch_skip(ctx, mas, r, z, nrhs, rl, zl, &s->all_conv));
+      GS_PROF(ctx, GS_K_PCG_VECTOR);
+      if (ff)
+        k_dot<false, true><<<vg, kRedThreads, 0, st>>>(r, z, nullptr, len, &s->all_conv, rzp);
+      else
+        k_dot<false, false><<<vg, kRedThreads, 0, st>>>(r, z, nullptr, len, &s->all_conv, rzp);
+    }
+    GS_TRY(pcg_update_p(ctx, mat, p, z, ps, nrhs, s, rrp, rzp, fold, tol2, parity));
     if ((it + 1) % poll == 0) {
-      GS_CUDA(cudaMemcpyAsync(h_conv, &s->all_conv, 4, cudaMemcpyDeviceToHost, st));
-      GS_CUDA(cudaStreamSynchronize(st));
-      if (*h_conv) break;
+      const int q = polls++ & 1;
+      GS_CUDA(cudaMemcpyAsync(h_conv + q, &s->all_conv, 4, cudaMemcpyDeviceToHost, st));
+      GS_CUDA(cudaEventRecord(ctx->poll_event[q], st));
+      if (polls > 1) {
+        GS_CUDA(cudaEventSynchronize(ctx->poll_event[q ^ 1]));
+        if (h_conv[q ^ 1]) break;
+      }
     }
   }
   GS_CUDA(cudaGetLastError());
-  PcgScalars hs;
-  GS_CUDA(cudaMemcpyAsync(&hs, s, sizeof(PcgScalars), cudaMemcpyDeviceToHost, st));
-  GS_CUDA(cudaStreamSynchronize(st));
+  // (h_pinned holds 4 KiB; its first words are the polls' and take_flags')
+  PcgScalars* hp = (PcgScalars*)(ctx->h_pinned + 256);
+  static_assert(1024 + sizeof(PcgScalars) <= 4096, "pinned staging");
+  GS_CUDA(cudaMemcpyAsync(hp, s, sizeof(PcgScalars), cudaMemcpyDeviceToHost, st));
+  int flags = 0;
+  GS_TRY(ctx->take_flags(&flags));  // synchronises
+  const PcgScalars& hs = *hp;
   bool all = true;
   for (int k = 0; k < nrhs; ++k) {
     if (iters) iters[k] = hs.iters[k];
     if (rel_res) rel_res[k] = hs.bnorm2[k] > 0 ? std::sqrt(hs.rr[k] / hs.bnorm2[k]) : 0.0;
     all = all && hs.conv[k];
   }
-  int flags = 0;
-  GS_TRY(ctx->take_flags(&flags));
   if (hs.flags) return status_from_flags(hs.flags);
   if (flags) return status_from_flags(flags);
   if (!all) {

@@ -1,0 +1,482 @@
+// The kernels of one PCG iteration (pcg.cu):
+//   k_pcg_spmv   Ap = A p (row or float-float product over the sliced matrix),
+//                partial sums of p . Ap
+//   k_pcg_xr     alpha from those; x += alpha p, r -= alpha Ap, partial sums of
+//                ||r||^2, and the level-1 sums of r, a warp per level-0 domain
+//   (the MAS products, the level-0 one with partial sums of r . z)
+//   k_pcg_p      the convergence test and beta from the partial sums; p = z +
+//                beta p (and the float-float operand of the next product)
+//
+// What bounds them: on small systems the chain of launches and reductions (ten
+// launches of 6 to 8 us each per iteration before, five now), on large ones
+// the vectors' bytes and the FP64 pipe.  A reduction has no tail: a kernel
+// writes its partial sums (block b's covers a fixed share of the rows or
+// domains), and every block of the kernel that needs the scalar adds them in
+// the same fixed order, so all see the same bits.  What a kernel reads that is
+// older than the kernel just before it is loaded before that one has ended.
+// Per iteration, before and now: 16^3, 4 RHS 110 / 42 us; 40^3, 4 RHS, FP32
+// preconditioner 205 / 122; 45^3, 1 RHS 197 / 152; 64^3, 8 RHS 655 / 603.
+#include <algorithm>
+
+#include "common.cuh"
+#include "ff_product.cuh"
+#include "pcg_state.cuh"
+
+namespace gs {
+
+constexpr int kT = 256;
+constexpr int kWarps = kT / 32;
+
+// ---------------------------------------------------------------- Ap = A p, p . Ap
+struct Sliced {  // the sliced matrix (sliced.cu)
+  const int32_t *row_order, *ptr, *len, *col;
+  const float2* ff;
+  const double* f64;
+  int32_t n;
+};
+
+// One row by kBL * kRL lanes: kRL groups take kR right-hand sides each, the kBL
+// lanes of a group share the row's entries and merge in a fixed order.  kFF:
+// float-float (spmv_ff.cu), xs the split operand; else FP64, x the operand.  An
+// entry's column is loaded one entry ahead, so that its operand's gather leaves
+// with the entry's own values.
+template <bool kFF, int kBL, int kRL, int kR, int kMin>
+__global__ void __launch_bounds__(kT, kMin) k_pcg_spmv(Sliced A, const int32_t* __restrict__ kk,
+                                                       const float2* __restrict__ xs, const double* __restrict__ p,
+                                                       double* __restrict__ Ap, int64_t stride, int nrhs,
+                                                       const PcgScalars* __restrict__ s, Partials pap) {
+  wait_for_previous_kernel();
+  if (s->all_conv) return;
+  constexpr int G = kBL * kRL;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = lane % G;
+  const int bl = sub % kBL, r0 = sub / kBL * kR;
+  const int nh = min(kR, nrhs - r0);  // may be <= 0
+  const bool vec = kR % 2 == 0 && (nrhs & 1) == 0;
+  double dot[kR];
+#pragma unroll
+  for (int q = 0; q < kR; ++q) dot[q] = 0.0;
+  const int64_t chunks = ((int64_t)A.n * G + kT - 1) / kT;
+  // blocks take one chunk of every gridDim.x, another place of it each time
+  // (rows are ordered by length within windows: the same place would always
+  // meet the same lengths)
+  const int64_t rounds = (chunks + gridDim.x - 1) / gridDim.x;
+  for (int64_t i = 0; i < rounds; ++i) {
+    const int64_t c = i * gridDim.x + (blockIdx.x + i * 37) % gridDim.x;
+    if (c >= chunks) continue;  // whole block
+    const int64_t slot = c * (kT / G) + threadIdx.x / G;
+    const bool in = slot < A.n && nh > 0;
+    const int32_t len = in ? A.len[slot] : 0;
+    const int64_t base = in ? (int64_t)A.ptr[slot >> 5] * 32 + (slot & 31) : 0;  // entry 0 of the row
+    const int32_t row = in ? A.row_order[slot] : 0;
+    int32_t next = bl < len ? A.col[base + 32 * bl] : 0;
+    double y[kR * 3];
+    if (kFF) {
+      FFSum<kR * 3> acc;
+      acc.clear();
+      const float2* v = A.ff + (base - (slot & 31)) * 9 + (slot & 31);
+      for (int32_t e = bl; e < len; e += kBL) {
+        const int32_t col = next;
+        if (e + kBL < len) next = A.col[base + 32 * (int64_t)(e + kBL)];
+        float2 H[9];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) H[q] = v[(int64_t)e * 288 + 32 * q];
+        ff_block_product<kR>(H, xs + ((int64_t)col * nrhs + r0) * 3, nh, vec, acc);
+      }
+      acc.template merge<kBL>();
+      if (in && bl == 0) {
+        const int kr = kk[row] + 2 * kk[A.n];  // k_row + K
+#pragma unroll
+        for (int q = 0; q < kR; ++q) {
+          const int f = q < nh ? s->fsplit[r0 + q] : kExpNone;
+#pragma unroll
+          for (int j = 0; j < 3; ++j) y[3 * q + j] = f == kExpNone ? 0.0 : acc.value(3 * q + j, kr + f);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < kR * 3; ++q) y[q] = 0.0;
+      const double* v = A.f64 + (base - (slot & 31)) * 9 + (slot & 31);
+      for (int32_t e = bl; e < len; e += kBL) {
+        const int32_t col = next;
+        if (e + kBL < len) next = A.col[base + 32 * (int64_t)(e + kBL)];
+        double H[9];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) H[q] = v[(int64_t)e * 288 + 32 * q];
+#pragma unroll
+        for (int q = 0; q < kR; ++q)
+          if (q < nh) {
+            const double* xr = p + (r0 + q) * stride + 3 * (int64_t)col;
+            const double x0 = xr[0], x1 = xr[1], x2 = xr[2];
+#pragma unroll
+            for (int j = 0; j < 3; ++j)
+              y[3 * q + j] = fma(H[3 * j + 2], x2, fma(H[3 * j + 1], x1, fma(H[3 * j], x0, y[3 * q + j])));
+          }
+      }
+#pragma unroll
+      for (int o = kBL / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < kR * 3; ++q) y[q] += __shfl_xor_sync(kFull, y[q], o, kBL);
+    }
+    if (in && bl == 0) {
+#pragma unroll
+      for (int q = 0; q < kR; ++q)
+        if (q < nh) {
+          const int64_t o = (r0 + q) * stride + 3 * (int64_t)row;
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            Ap[o + j] = y[3 * q + j];
+            dot[q] = fma(p[o + j], y[3 * q + j], dot[q]);
+          }
+        }
+    }
+  }
+  let_next_kernel_launch();
+  __shared__ double red[kWarps][8];
+#pragma unroll
+  for (int q = 0; q < kR; ++q) {
+#pragma unroll
+    for (int o = G; o < 32; o <<= 1) dot[q] += __shfl_xor_sync(kFull, dot[q], o);
+    if (lane < G && bl == 0) red[w][r0 + q] = dot[q];
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < nrhs) {
+    double v = 0.0;
+#pragma unroll
+    for (int i = 0; i < kWarps; ++i) v += red[i][threadIdx.x];
+    pap.sum[threadIdx.x * pap.pitch + blockIdx.x] = v;
+  }
+}
+
+// Lanes per row by size.  The large-system shapes give each lane two
+// right-hand sides and the whole row (64^3, 8 RHS: 0.19 ms; 2 lanes sharing the
+// blocks of 8 RHS: 0.23 ms); systems whose rows do not fill the GPU share a
+// row's blocks among up to 8 lanes.
+template <bool kFF, int kRL, int kR>
+static int launch_spmv(gs_ctx ctx, gs_mat m, const float2* xs, const double* p, double* Ap, int nrhs,
+                       const PcgScalars* s, Partials& pap) {
+  const Sliced A{m->row_order, m->sl_ptr, m->sl_len, m->sl_col, m->sl_ff, m->sl_f64, m->n};
+  const int64_t fill = (int64_t)std::max(ctx->sm_count, 1) * 1024;
+  int bl = 1;
+  while (bl < 8 && bl * kRL < 32 && (int64_t)m->n * kRL * bl * 2 <= fill) bl *= 2;
+  constexpr int kMin = kFF ? 4 : 3;
+  const int64_t chunks = ((int64_t)m->n * kRL * bl + kT - 1) / kT;
+  pap.n = (int)std::max<int64_t>(1, std::min<int64_t>({chunks, (int64_t)kMin * std::max(ctx->sm_count, 1),
+                                                       (int64_t)kMaxRedBlocks}));
+  auto go = [&](auto kernel) {
+    return launch_chained(ctx, (int64_t)m->n * nrhs, kernel, dim3(pap.n), dim3(kT), 0, A, m->ff_k, xs, p, Ap,
+                          3LL * m->n, nrhs, s, pap);
+  };
+  cudaError_t e = cudaSuccess;
+  switch (bl) {
+    case 1: e = go(k_pcg_spmv<kFF, 1, kRL, kR, kMin>); break;
+    case 2: e = go(k_pcg_spmv<kFF, 2, kRL, kR, kMin>); break;
+    case 4: e = go(k_pcg_spmv<kFF, 4, kRL, kR, kMin>); break;
+    default: e = go(k_pcg_spmv<kFF, 8, kRL, kR, kMin>); break;
+  }
+  GS_CUDA(e);
+  return GS_OK;
+}
+
+template <bool kFF>
+static int launch_spmv_rhs(gs_ctx ctx, gs_mat m, const float2* xs, const double* p, double* Ap, int nrhs,
+                           const PcgScalars* s, Partials& pap) {
+  if (nrhs == 1) return launch_spmv<kFF, 1, 1>(ctx, m, xs, p, Ap, nrhs, s, pap);
+  if (nrhs == 2) return launch_spmv<kFF, 2, 1>(ctx, m, xs, p, Ap, nrhs, s, pap);
+  if (nrhs <= 4) return launch_spmv<kFF, 2, 2>(ctx, m, xs, p, Ap, nrhs, s, pap);
+  return launch_spmv<kFF, 4, 2>(ctx, m, xs, p, Ap, nrhs, s, pap);
+}
+
+// Ap = A p and the partial sums of p . Ap (pap.n is set), at most 8 right-hand
+// sides, over the sliced matrix (ensure_sliced); ps: the split operand
+// (float-float product) or null (FP64 product).
+int pcg_spmv_dot(gs_ctx ctx, gs_mat m, const float2* ps, const double* p, double* Ap, int nrhs, const PcgScalars* s,
+                 Partials& pap) {
+  GS_PROF(ctx, GS_K_SPMV);
+  return ps ? launch_spmv_rhs<true>(ctx, m, ps, p, Ap, nrhs, s, pap)
+            : launch_spmv_rhs<false>(ctx, m, nullptr, p, Ap, nrhs, s, pap);
+}
+
+// ---------------------------------------------------------------- x, r, ||r||^2, level-1 sums
+// A warp takes a level-0 domain and kR right-hand sides: its 3N values of each
+// in three passes (lanes along the domain's nodes in slot order, so
+// neighbouring lanes read neighbouring entries), r kept in shared memory for
+// the sums over the domain's level-1 items.  kR = 2: two right-hand sides'
+// loads are in flight together, and more per warp leave too few warps (40^3,
+// 4 RHS: 129 us per iteration with four, 122 with two).  What does not come from the kernel just
+// before (x, r, p and the domain tables) is loaded before that one has ended.
+constexpr int kPitch = 99;  // doubles per right-hand side: 3 N <= 96, spread over the banks
+
+template <int kR>
+__global__ void __launch_bounds__(kT, 3) k_pcg_xr(double* __restrict__ x, double* __restrict__ r,
+                                                  const double* __restrict__ p, const double* __restrict__ Ap,
+                                                  int64_t stride, int nrhs, const int32_t* __restrict__ remap0,
+                                                  int32_t n_dom, int N, const int32_t* __restrict__ item1,
+                                                  int64_t off1, double* __restrict__ rl, int64_t lstride,
+                                                  PcgScalars* s, Partials pap, Partials rrp, int parity) {
+  __shared__ double sm_all[kWarps * kR * kPitch];
+  __shared__ double s_alpha[kR];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int kb = blockIdx.y * kR;
+  double* sm = sm_all + w * (kR * kPitch);
+  double rr[kR], rv[kR][3], pv[kR][3], xv[kR][3];
+  int64_t o[3];  // this lane's three entries (-1: padding)
+  int32_t node = -1, c1 = -1;
+  auto load = [&](int32_t d) {
+    node = lane < N ? remap0[(int64_t)d * N + lane] : -1;
+    c1 = node >= 0 && item1 ? item1[node] : -1;
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+      const int v = t * 32 + lane;
+      const int32_t nd = __shfl_sync(kFull, node, v / 3);
+      o[t] = v < 3 * N && nd >= 0 ? 3 * (int64_t)nd + v % 3 : -1;
+    }
+#pragma unroll
+    for (int k = 0; k < kR; ++k)
+#pragma unroll
+      for (int t = 0; t < 3; ++t) {
+        const int64_t at = (kb + k) * stride + o[t];
+        rv[k][t] = pv[k][t] = xv[k][t] = 0.0;
+        if (kb + k < nrhs && o[t] >= 0) rv[k][t] = r[at], pv[k][t] = p[at], xv[k][t] = x[at];
+      }
+  };
+  int32_t d = blockIdx.x * kWarps + w;
+  if (s->all_conv) return;  // the product did not write it
+  if (d < n_dom) load(d);
+  wait_for_previous_kernel();
+  if (w < kR && kb + w < nrhs) {
+    const int k = kb + w;
+    const double sum = warp_sum_partials(pap, k);
+    if (lane == 0) {
+      s_alpha[w] = take_alpha(s, k, sum, parity, blockIdx.x == 0);
+      if (blockIdx.x == 0) s->fp[parity ^ 1][k] = kExpNone;  // k_pcg_p gathers there
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < kR; ++k) rr[k] = 0.0;
+  while (d < n_dom) {
+    double av[kR][3], al[kR];
+#pragma unroll
+    for (int k = 0; k < kR; ++k) {
+      al[k] = kb + k < nrhs ? s_alpha[k] : 0.0;
+#pragma unroll
+      for (int t = 0; t < 3; ++t) av[k][t] = al[k] != 0.0 && o[t] >= 0 ? Ap[(kb + k) * stride + o[t]] : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < kR; ++k)
+#pragma unroll
+      for (int t = 0; t < 3; ++t) {
+        if (al[k] != 0.0 && o[t] >= 0) {
+          const int64_t at = (kb + k) * stride + o[t];
+          x[at] = fma(al[k], pv[k][t], xv[k][t]);
+          rv[k][t] = fma(-al[k], av[k][t], rv[k][t]);
+          r[at] = rv[k][t];
+        }
+        rr[k] = fma(rv[k][t], rv[k][t], rr[k]);
+        if (item1) sm[k * kPitch + t * 32 + lane] = rv[k][t];
+      }
+    if (item1) {
+      __syncwarp();
+      // value c of RHS k summed over each group's slots by kParts lanes, 32 /
+      // kParts neighbouring slots each, then the parts (an addition costs the
+      // FP64 pipe the same for 3 lanes as for 32)
+      constexpr int kV = 3 * kR, kParts = kR == 1 ? 8 : 4, kS = 32 / kParts;
+      const int part = lane / kV, kc = lane % kV, k = kc / 3, c = kc % 3;
+      const bool act = part < kParts;  // 24 lanes
+      const double* mine = sm + (act ? k : 0) * kPitch + c + 3 * kS * (act ? part : 0);
+      for (uint32_t left = __ballot_sync(kFull, node >= 0); left;) {
+        const int lead = __ffs(left) - 1;
+        const int32_t cc = __shfl_sync(kFull, c1, lead);
+        const uint32_t g = __ballot_sync(kFull, node >= 0 && c1 == cc);
+        double sum = 0.0;
+        if (g == 0xffffffffu) {  // the usual domain: full, one item
+          double q4[4];
+#pragma unroll
+          for (int q = 0; q < kS; ++q) q4[q % 4] = q < 4 ? mine[3 * q] : q4[q % 4] + mine[3 * q];
+          sum = (q4[0] + q4[1]) + (q4[2] + q4[3]);
+        } else {
+          const uint32_t gm = (g >> (act ? part * kS : 0)) & ((1u << kS) - 1u);
+          for (uint32_t m = act ? gm : 0u; m; m &= m - 1) sum += mine[3 * (__ffs(m) - 1)];
+          __syncwarp();
+        }
+#pragma unroll
+        for (int h = kParts / 2; h > 0; h /= 2) sum += __shfl_down_sync(kFull, sum, h * kV);
+        if (part == 0 && kb + k < nrhs) rl[(kb + k) * lstride + c + 3 * (off1 + cc)] = sum;
+        left &= ~g;
+      }
+      __syncwarp();
+    }
+    d += gridDim.x * kWarps;
+    if (d < n_dom) load(d);
+  }
+  let_next_kernel_launch();
+  __shared__ double red[kWarps][kR];
+  const int ks = sum_index<kR>(lane);
+  const double v = warp_sums<kR>(rr, lane);
+  if (lane < kR) red[w][ks] = v;
+  __syncthreads();
+  if ((int)threadIdx.x < kR && kb + (int)threadIdx.x < nrhs) {
+    double t = 0.0;
+#pragma unroll
+    for (int i = 0; i < kWarps; ++i) t += red[i][threadIdx.x];
+    rrp.sum[(kb + threadIdx.x) * rrp.pitch + blockIdx.x] = t;
+  }
+}
+
+// x += alpha p, r -= alpha Ap, partial sums of ||r||^2 (rrp.n is set), and rl =
+// level-1 sums of r (where the preconditioner has a level 1), at most 8
+// right-hand sides.
+int pcg_update_xr(gs_ctx ctx, gs_mas mas, double* x, double* r, const double* p, const double* Ap, int nrhs, double* rl,
+                  int64_t lstride, PcgScalars* s, const Partials& pap, Partials& rrp, int parity) {
+  GS_PROF(ctx, GS_K_PCG_VECTOR);
+  const int kr = nrhs == 1 ? 1 : 2;
+  // a domain per warp while the partial sums allow it: one wave of longer
+  // blocks left a third of the last round empty
+  rrp.n = std::max(1, std::min(ceil_div(mas->n_domains[0], kWarps), kMaxRedBlocks));
+  const bool coarse = mas->L > 1;
+  GS_CUDA(launch_chained(ctx, (int64_t)mas->n * nrhs, kr == 1 ? k_pcg_xr<1> : k_pcg_xr<2>,
+                         dim3(rrp.n, ceil_div(nrhs, kr)), dim3(kT), 0, x, r, p, Ap, 3LL * mas->n, nrhs, mas->remap0,
+                         mas->n_domains[0], mas->N, coarse ? mas->coarse[1] : nullptr, coarse ? mas->vec_off[1] : 0,
+                         rl, lstride, s, pap, rrp, parity));
+  return GS_OK;
+}
+
+// ---------------------------------------------------------------- p = z + beta p
+// Block (g, k): the convergence test of RHS k and its beta from the partial
+// sums, then its share of p.  kFF: also the float-float operand of the next
+// product, ps = split(p 2^(k_node - K - F)) with 2^F above |p| from the bounds
+// |z| < 2^fz, |p_old| < 2^fp, |beta| < 2^eb as max(fz, fp + eb) + 1, node-major
+// across right-hand sides; the new p's bound gathers in the other parity's fp.
+// A converged RHS keeps p, ps and its bounds.
+template <bool kFF>
+__global__ void __launch_bounds__(kT) k_pcg_p(double* __restrict__ p, const double* __restrict__ z,
+                                              float2* __restrict__ ps, const int32_t* __restrict__ kk, int64_t len,
+                                              int nrhs, PcgScalars* s, Partials rrp, Partials rzp, double tol2,
+                                              int parity) {
+  constexpr int kUnroll = 4;  // strided elements per thread and pass, loaded before they are used
+  __shared__ double s_beta;
+  __shared__ int s_ex[2], s_stop;
+  const int k = blockIdx.y;
+  const bool record = blockIdx.x == 0 && threadIdx.x == 0;
+  const int64_t o = (int64_t)k * len, step = (int64_t)gridDim.x * kT * kUnroll;
+  int64_t i = (int64_t)blockIdx.x * kT * kUnroll + threadIdx.x;
+  // p and ||r||^2 do not come from the kernel just before
+  double pv[kUnroll];
+#pragma unroll
+  for (int u = 0; u < kUnroll; ++u) pv[u] = i + u * kT < len ? p[o + i + u * kT] : 0.0;
+  double rr = 0.0;
+  if (threadIdx.x < 32) rr = warp_sum_partials(rrp, k);
+  wait_for_previous_kernel();
+  if (s->all_conv) return;
+  double rz = 0.0;
+  if (threadIdx.x < 32) rz = warp_sum_partials(rzp, k);
+  if (threadIdx.x == 0) {
+    s_ex[0] = s_ex[1] = kExpNone;
+    s_stop = test_convergence(s, k, rr, tol2, record);
+    s_beta = rz / s->rz[parity][k];
+  }
+  int ex = kExpNone;
+  if (kFF)
+    for (int g = threadIdx.x; g < rzp.n; g += kT) ex = max(ex, __ldcg(rzp.ex + (size_t)k * rzp.pitch + g));
+  __syncthreads();
+  if (s_stop) {
+    if (kFF && record) atomicMax(&s->fp[parity ^ 1][k], s->fp[parity][k]);
+    return;
+  }
+  const double be = s_beta;
+  if (record) {
+    s->rz[parity ^ 1][k] = rz;
+    if (!isfinite(rz)) {
+      atomicOr(&s->flags, kErrNonFinite);
+      s->bad[k] = 1;
+    }
+  }
+  int F = 0;
+  if (kFF) {
+    ex = __reduce_max_sync(kFull, ex);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_ex[0], ex);
+    __syncthreads();
+    const int eb = ex_bound(be), fp = s->fp[parity][k];
+    const int fb = (fp == kExpNone || eb == kExpNone) ? kExpNone : fp + eb;
+    const int fmax = max(s_ex[0], fb);
+    F = fmax == kExpNone ? 0 : fmax + 1;
+    if (record) s->fsplit[k] = F;
+    ex = kExpNone;
+  }
+  while (i < len) {
+    double zv[kUnroll];
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) zv[u] = i + u * kT < len ? z[o + i + u * kT] : 0.0;
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) {
+      const int64_t j = i + u * kT;
+      if (j < len) {
+        const double v = fma(be, pv[u], zv[u]);
+        p[o + j] = v;
+        if (kFF) {
+          ex = max(ex, ex_bound(v));
+          const uint32_t node = (uint32_t)j / 3u;
+          ps[((int64_t)node * nrhs + k) * 3 + ((uint32_t)j - 3u * node)] = ff_split_bits(v, kk[node] - F);
+        }
+      }
+    }
+    i += step;
+    if (i >= len) break;
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) pv[u] = i + u * kT < len ? p[o + i + u * kT] : 0.0;
+  }
+  let_next_kernel_launch();
+  if (kFF) {
+    ex = __reduce_max_sync(kFull, ex);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_ex[1], ex);
+    __syncthreads();
+    if (threadIdx.x == 0) atomicMax(&s->fp[parity ^ 1][k], s_ex[1]);
+  }
+}
+
+// Folds the partial sums of a reduction over very many domains to 64 per RHS.
+constexpr int kFold = 64;
+__global__ void __launch_bounds__(kT) k_fold(Partials a, Partials out, const int* __restrict__ skip) {
+  wait_for_previous_kernel();
+  if (*skip) return;
+  const int k = blockIdx.y, per = (a.n + kFold - 1) / kFold, g0 = blockIdx.x * per;
+  Partials mine = a;
+  mine.sum += g0;
+  mine.n = max(0, min(per, a.n - g0));
+  const double v = threadIdx.x < 32 ? warp_sum_partials(mine, k) : 0.0;
+  __shared__ int s_ex;
+  if (threadIdx.x == 0) s_ex = kExpNone;
+  __syncthreads();
+  int e = kExpNone;
+  for (int g = threadIdx.x; g < mine.n; g += kT) e = max(e, a.ex[(size_t)k * a.pitch + g0 + g]);
+  e = __reduce_max_sync(kFull, e);
+  if ((threadIdx.x & 31) == 0) atomicMax(&s_ex, e);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    out.sum[k * out.pitch + blockIdx.x] = v;
+    out.ex[k * out.pitch + blockIdx.x] = s_ex;
+  }
+}
+
+// The convergence test, beta and p = z + beta p from the partial sums of
+// ||r||^2 and r . z; fold: room for kFold partials per right-hand side.
+int pcg_update_p(gs_ctx ctx, gs_mat m, double* p, const double* z, float2* ps, int nrhs, PcgScalars* s,
+                 const Partials& rrp, const Partials& rzp, Partials fold, double tol2, int parity) {
+  GS_PROF(ctx, GS_K_PCG_VECTOR);
+  const int64_t len = 3LL * m->n, work = (int64_t)m->n * nrhs;
+  Partials rz = rzp;
+  if (rzp.n > kMaxRedBlocks) {  // every block below would read them all
+    GS_CUDA(launch_chained(ctx, work, k_fold, dim3(kFold, nrhs), dim3(kT), 0, rzp, fold, &s->all_conv));
+    rz = fold;
+    rz.n = kFold;
+  }
+  // about eight blocks per SM over all right-hand sides: each first adds the
+  // partial sums
+  const int gx = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(len, kT * 4),
+                                                             (8LL * std::max(ctx->sm_count, 1) + nrhs - 1) / nrhs));
+  GS_CUDA(launch_chained(ctx, work, ps ? k_pcg_p<true> : k_pcg_p<false>, dim3(gx, nrhs), dim3(kT), 0, p, z, ps,
+                         ps ? m->ff_k : nullptr, len, nrhs, s, rrp, rz, tol2, parity));
+  return GS_OK;
+}
+
+}  // namespace gs

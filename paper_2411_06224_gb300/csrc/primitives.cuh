@@ -86,6 +86,22 @@ struct LevelIdxNodeMajor {
   __device__ __forceinline__ int64_t operator()(int64_t item, int v) const { return (off + item) * nv + v; }
 };
 
+// Sum of rk[3 b] over the set bits b of mask, ascending, 16 loads in flight:
+// a coarse item's value from its children (the sum of k_restrict_up).
+__device__ __forceinline__ double sum_children(const double* __restrict__ rk, uint32_t mask) {
+  double sum = 0.0;
+#pragma unroll 1
+  for (int b = 0; b < 32; b += 16) {
+    double v[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) v[q] = (mask >> (b + q)) & 1u ? rk[3 * (b + q)] : 0.0;
+#pragma unroll
+    for (int q = 0; q < 16; ++q)
+      if ((mask >> (b + q)) & 1u) sum += v[q];
+  }
+  return sum;
+}
+
 // Restriction from level l >= 1 to level l + 1 (supplement Eq. 5-6, C_{l+1}
 // = C'_l C_l).  A level-(l+1) item is a connected component of one level-l
 // domain (items dN .. dN+N-1), so one warp per level-l domain sums the

@@ -43,6 +43,7 @@
 
 #include "common.cuh"
 #include "ff.cuh"
+#include "ff_product.cuh"
 #include "primitives.cuh"
 
 namespace gs {
@@ -71,12 +72,12 @@ __global__ void k_ff_half(int32_t* __restrict__ k, int32_t n) {
 }
 
 __global__ void k_ff_blocks(const int32_t* __restrict__ rid, const int32_t* __restrict__ cid,
-                            const double* __restrict__ au, int64_t nnzb, const int32_t* __restrict__ k,
+                            const double* __restrict__ au, int64_t nnzb, int32_t n, const int32_t* __restrict__ k,
                             float2* __restrict__ out) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nnzb * 9) return;
   const int64_t b = t / 9;
-  out[t] = ff_split_scaled(au[t], -(k[rid[b]] + k[cid[b]]));
+  out[t] = ff_split_scaled(au[t], -(k[rid[b]] + k[cid[b]] + 2 * k[n]));  // k[i] holds k_i - K, k[n] = K
 }
 
 __global__ void k_ff_minus_K(int32_t* __restrict__ k, int32_t n) {
@@ -84,25 +85,31 @@ __global__ void k_ff_minus_K(int32_t* __restrict__ k, int32_t n) {
   if (i < n) k[i] -= k[n];
 }
 
-int ensure_ff(gs_ctx ctx, gs_mat m) {
-  if (m->au_ff) return GS_OK;
+int ensure_ff_scales(gs_ctx ctx, gs_mat m) {
+  if (m->ff_k) return GS_OK;
   cudaStream_t st = ctx->stream;
   const int64_t nz = m->nnzb;
   GS_TRY(ctx->alloc((void**)&m->ff_k, (size_t)(m->n + 1) * 4));
-  GS_TRY(ctx->alloc((void**)&m->au_ff, (size_t)std::max<int64_t>(nz, 1) * 9 * sizeof(float2)));
-  GS_CUDA(cudaMemsetAsync(m->ff_k, 0x80, (size_t)m->n * 4, st));  // kExpNone
-  GS_CUDA(cudaMemsetAsync(m->ff_k + m->n, 0x80, 4, st));
+  GS_CUDA(cudaMemsetAsync(m->ff_k, 0x80, (size_t)(m->n + 1) * 4, st));  // kExpNone
   {
     GS_PROF(ctx, GS_K_OTHER);
     if (nz > 0) k_ff_row_exp<<<ceil_div(nz, 256), 256, 0, st>>>(m->rid, m->cid, m->au, nz, m->ff_k);
   }
   // rows that no block touched still hold kExpNone: they read as empty
   { GS_PROF(ctx, GS_K_OTHER); k_ff_half<<<ceil_div(std::max(m->n, 1), 256), 256, 0, st>>>(m->ff_k, m->n); }
-  {
-    GS_PROF(ctx, GS_K_OTHER);
-    if (nz > 0) k_ff_blocks<<<ceil_div(nz * 9, 256), 256, 0, st>>>(m->rid, m->cid, m->au, nz, m->ff_k, m->au_ff);
-  }
   { GS_PROF(ctx, GS_K_OTHER); k_ff_minus_K<<<ceil_div(std::max(m->n, 1), 256), 256, 0, st>>>(m->ff_k, m->n); }
+  GS_CUDA(cudaGetLastError());
+  return GS_OK;
+}
+
+int ensure_ff(gs_ctx ctx, gs_mat m) {
+  if (m->au_ff) return GS_OK;
+  GS_TRY(ensure_ff_scales(ctx, m));
+  const int64_t nz = m->nnzb;
+  GS_TRY(ctx->alloc((void**)&m->au_ff, (size_t)std::max<int64_t>(nz, 1) * 9 * sizeof(float2)));
+  GS_PROF(ctx, GS_K_OTHER);
+  if (nz > 0)
+    k_ff_blocks<<<ceil_div(nz * 9, 256), 256, 0, ctx->stream>>>(m->rid, m->cid, m->au, nz, m->n, m->ff_k, m->au_ff);
   GS_CUDA(cudaGetLastError());
   return GS_OK;
 }
@@ -133,42 +140,6 @@ __global__ void __launch_bounds__(256) k_ff_split(const double* __restrict__ x, 
 }
 
 // ---------------------------------------------------------------- the product
-// Accumulate the term (ah + al)(xh + xl) into the pair (S, L).  The rounded
-// intrinsics keep the compiler from contracting or reordering the
-// transformations.
-__device__ __forceinline__ void ff_term(float ah, float al, float xh, float xl, float& S, float& L) {
-  const float p = __fmul_rn(ah, xh);
-  const float e = __fmaf_rn(ah, xh, -p);
-  const float s = __fadd_rn(S, p);
-  const float bp = __fsub_rn(s, S);
-  const float err = __fadd_rn(__fsub_rn(S, __fsub_rn(s, bp)), __fsub_rn(p, bp));
-  S = s;
-  L = __fadd_rn(L, __fadd_rn(err, e));
-  L = __fmaf_rn(ah, xl, L);
-  L = __fmaf_rn(al, xh, L);
-}
-
-// (S, L) += (S2, L2): two-sum of the large parts, the rest gathered in L.
-__device__ __forceinline__ void ff_merge(float& S, float& L, float S2, float L2) {
-  const float s = __fadd_rn(S, S2);
-  const float bp = __fsub_rn(s, S);
-  const float err = __fadd_rn(__fsub_rn(S, __fsub_rn(s, bp)), __fsub_rn(S2, bp));
-  S = s;
-  L = __fadd_rn(L, __fadd_rn(L2, err));
-}
-
-// f * 2^e as a double, built from f's bit pattern (no conversion
-// instruction; on this part conversions run on the FP64 pipe).  A zero or
-// subnormal f gives 0; e keeps the result inside the double range here.
-__device__ __forceinline__ double f32_times_pow2(float f, int e) {
-  const unsigned b = __float_as_uint(f);
-  const int fe = (int)((b >> 23) & 0xffu);
-  if (fe == 0) return 0.0;
-  const int de = min(max(fe - 127 + 1023 + e, 1), 2046);
-  const unsigned hi = (b & 0x80000000u) | ((unsigned)de << 20) | ((b & 0x7fffffu) >> 3);
-  return __hiloint2double((int)hi, (int)(b << 29));
-}
-
 // One thread's share of the product for thread t of the walk over the row
 // order (kLanes threads per row).  kSplit = false: the row's lanes stride over
 // its blocks and merge their pairs at the end (any RHS count).  kSplit = true:
@@ -201,9 +172,8 @@ __device__ __forceinline__ void spmv_ff_row_group(int64_t t, const int32_t* __re
   const bool vec = kR % 2 == 0 && (nrhs & 1) == 0;
   for (int r0 = r_first; r0 < nrhs; r0 += r_step) {
     const int nh = min(kR, nrhs - r0);  // right-hand sides in this pass
-    float S[kR * 3], L[kR * 3];
-#pragma unroll
-    for (int q = 0; q < kR * 3; ++q) S[q] = 0.f, L[q] = 0.f;
+    FFSum<kR * 3> acc;
+    acc.clear();
     for (int32_t e = e_first; e < total; e += e_step) {
       const bool upper = e < nu;
       int64_t blk;
@@ -219,55 +189,15 @@ __device__ __forceinline__ void spmv_ff_row_group(int64_t t, const int32_t* __re
 #pragma unroll
       for (int q = 0; q < 9; ++q) H[q] = au[blk * 9 + q];
       if (!upper) {  // use the transpose
-        float2 t1 = H[1], t2 = H[2], t5 = H[5];
+        const float2 t1 = H[1], t2 = H[2], t5 = H[5];
         H[1] = H[3], H[2] = H[6], H[5] = H[7];
         H[3] = t1, H[6] = t2, H[7] = t5;
       }
       // the column's operand for this pass's right-hand sides is one
       // contiguous stretch (node-major); two RHS at a time in 16-byte loads
-      const float2* xb = xs + ((int64_t)col * nrhs + r0) * 3;
-#pragma unroll
-      for (int q = 0; q < kR; q += 2) {
-        float2 xv[6];
-        if (vec) {
-          if (q < nh) {
-            const float4* x4 = reinterpret_cast<const float4*>(xb + 3 * q);
-            const float4 a = x4[0], b = x4[1], c = x4[2];
-            xv[0] = make_float2(a.x, a.y), xv[1] = make_float2(a.z, a.w), xv[2] = make_float2(b.x, b.y);
-            xv[3] = make_float2(b.z, b.w), xv[4] = make_float2(c.x, c.y), xv[5] = make_float2(c.z, c.w);
-          }
-        } else {
-#pragma unroll
-          for (int i = 0; i < 6; ++i)
-            if (q + i / 3 < nh && (q + i / 3) < kR) xv[i] = xb[3 * q + i];
-        }
-#pragma unroll
-        for (int qq = 0; qq < 2; ++qq) {
-          const int qi = q + qq;
-          if (qi < kR && qi < nh) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              ff_term(H[3 * c + 0].x, H[3 * c + 0].y, xv[3 * qq].x, xv[3 * qq].y, S[3 * qi + c], L[3 * qi + c]);
-              ff_term(H[3 * c + 1].x, H[3 * c + 1].y, xv[3 * qq + 1].x, xv[3 * qq + 1].y, S[3 * qi + c],
-                      L[3 * qi + c]);
-              ff_term(H[3 * c + 2].x, H[3 * c + 2].y, xv[3 * qq + 2].x, xv[3 * qq + 2].y, S[3 * qi + c],
-                      L[3 * qi + c]);
-            }
-          }
-        }
-      }
+      ff_block_product<kR>(H, xs + ((int64_t)col * nrhs + r0) * 3, nh, vec, acc);
     }
-    if (!kSplit) {
-#pragma unroll
-      for (int q = 0; q < kR * 3; ++q) {
-#pragma unroll
-        for (int o = kLanes / 2; o > 0; o >>= 1) {
-          const float S2 = __shfl_xor_sync(kFull, S[q], o, kLanes);
-          const float L2 = __shfl_xor_sync(kFull, L[q], o, kLanes);
-          ff_merge(S[q], L[q], S2, L2);
-        }
-      }
-    }
+    if (!kSplit) acc.template merge<kLanes>();
     if (in && (kSplit || sub == 0)) {
       const int kr = kk[row] + 2 * kk[n];  // k_row + K
 #pragma unroll
@@ -277,8 +207,7 @@ __device__ __forceinline__ void spmv_ff_row_group(int64_t t, const int32_t* __re
           double* yr = y + (r0 + q) * stride + 3 * (int64_t)row;
 #pragma unroll
           for (int c = 0; c < 3; ++c)
-            yr[c] = f == kExpNone ? 0.0
-                                  : f32_times_pow2(S[3 * q + c], kr + f) + f32_times_pow2(L[3 * q + c], kr + f);
+            yr[c] = f == kExpNone ? 0.0 : acc.value(3 * q + c, kr + f);
         }
     }
   }
