@@ -425,7 +425,7 @@ def kernel_lines(B, ctx, dev, clk, spmv, prec, nrhs, N, V, nnzb, ndom, mp, live,
                 "flops_per_launch": flops, "bytes_per_launch": nbytes, "avg_launch_ms": tsec * 1e3}
 
     tune_tc = B.gs_tune_get(ctx, B.GS_TUNE_F64_TC)
-    f64tc = (prec == B.GS_PREC_FP64 and nrhs <= 8 and ld % 16 == 0 and tune_tc in (1, 3, 4))
+    f64tc = (prec == B.GS_PREC_FP64 and nrhs <= 8 and ld % 16 == 0 and tune_tc in (1, 2, 3, 4))
     if f64tc:
         if tune_tc == 3:
             # the block lower triangle of every level-0 inverse as 8 base-128
@@ -438,11 +438,11 @@ def kernel_lines(B, ctx, dev, clk, spmv, prec, nrhs, N, V, nnzb, ndom, mp, live,
                      "triangles as base-128 digit bytes, expanded to BF16 in shared memory, on tcgen05, "
                      "+ prolongation)")
         else:
-            # the 7 BF16 digit matrices of every level-0 inverse (14 B per entry)
-            dig_bytes = 7 * 2 * n_dom0 * ld * ld
+            # the 7 digit bytes per entry of every level-0 inverse
+            dig_bytes = 7 * n_dom0 * ld * ld
             kname = "k_level0_f64tc"
-            kdesc = ("k_level0_f64tc (level-0 MAS apply in FP64 accuracy by exact BF16 digit "
-                     f"splitting on tcgen05, + prolongation; {256 if tune_tc == 4 else 128} threads per domain)")
+            kdesc = ("k_level0_f64tc (level-0 MAS apply in FP64 accuracy from digit bytes by exact F16 digit "
+                     "splitting on tcgen05, + prolongation)")
         tc_bytes = dig_bytes + 2 * 8 * 3 * V * nrhs
         traffic = recorded_traffic(kname, traffic_key) if traffic_key else None
         apply_line = {"bound": "hbm", "achieved": tc_bytes / t_apply / 1e9, "peak": hbm, "unit": "GB/s",
@@ -455,12 +455,12 @@ def kernel_lines(B, ctx, dev, clk, spmv, prec, nrhs, N, V, nnzb, ndom, mp, live,
                       "kernel": kdesc}
         apply_iso_ach = tc_bytes / t_apply_iso / 1e9
     elif prec == B.GS_PREC_FP32 and nrhs <= 8:
-        # FP32 inverses streamed as packed lower triangles (k_level0_f32_cta)
+        # FP32 inverses streamed as packed lower triangles (k_level0_f32)
         apply_line = {"bound": "hbm", "achieved": apply_bytes / t_apply / 1e9, "peak": hbm, "unit": "GB/s",
                       "frac": apply_bytes / t_apply / 1e9 / hbm, "traffic": None,
                       "flops_per_launch": apply_flops, "bytes_per_launch": apply_bytes,
                       "avg_launch_ms": t_apply * 1e3,
-                      "kernel": "k_level0_f32_cta (level-0 MAS apply from packed FP32 lower triangles, + prolongation)"}
+                      "kernel": "k_level0_f32 (level-0 MAS apply from packed FP32 lower triangles, + prolongation)"}
         apply_iso_ach = apply_bytes / t_apply_iso / 1e9
     else:
         apply_line = fp64_line(apply_flops, apply_bytes, t_apply, None)

@@ -15,13 +15,12 @@ The shapes and the kernels they steer:
   * GS_TUNE_SPMV32_LANES lanes per block row of the FP32 SpMV inside the mixed solve;
   * GS_TUNE_BATCH_CHUNK  vector entries per work item of the batched PCG reductions;
   * GS_TUNE_BF16_TC      BF16 level-0 apply on the tensor cores or on the FP32 cores;
-  * GS_TUNE_F64_TC       FP64 apply on the BF16 tensor cores (exact digit
+  * GS_TUNE_F64_TC       FP64 apply on the tensor cores (exact digit
                          splitting) or on the FP64 cores.  The digit storage is
                          made when the preconditioner is built, so the sweep
                          stays within the storage built: the symmetric digit
-                         bytes (3) or the FP64 cores, or the BF16 digit
-                         matrices (one CTA per domain 1, persistent 2) or the
-                         FP64 cores;
+                         bytes (3) or the FP64 cores, or the digit bytes of
+                         every entry (1, 2 and 4 alike) or the FP64 cores;
   * GS_TUNE_SPMV_WS      one thread group per row, or a persistent grid whose
                          warps steal the next rows;
   * GS_TUNE_SPMV_FF_RHS  right-hand sides per thread of the float-float SpMV

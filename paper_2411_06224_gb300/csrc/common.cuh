@@ -257,7 +257,7 @@ struct gs_mas_s {
                                    // packed by rows (ld(ld+1)/2 floats, padded to a multiple of 4)
   std::vector<void*> inv16;        // BF16 precision: level 0 only, inverse Cholesky factor W, row-major
   void* inv16_tc = nullptr;        // BF16 precision: level-0 W in the tensor-core operand layout
-  std::vector<void*> dig64;        // FP64 precision: per level, the inverses as 7 BF16 digit matrices per domain
+  std::vector<void*> dig64;        // FP64 precision: per level, the inverses as 7 matrices of digit bytes per domain
   std::vector<int32_t*> dig64_exp; // FP64 precision: per level, their row exponents
   void** d_dig_tab = nullptr;      // device table: digit pointers [0..7], exponent pointers [8..15]
   std::vector<void*> dig8;         // FP64 precision, GS_TUNE_F64_TC = 3: per level, the inverses' block lower

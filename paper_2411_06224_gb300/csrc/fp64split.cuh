@@ -4,6 +4,7 @@
 // the integer units, so no FP64 instruction is spent on the splits.
 #pragma once
 
+#include <cuda_fp16.h>
 #include <stdint.h>
 
 namespace gs {
@@ -12,50 +13,53 @@ namespace gs {
 __device__ __forceinline__ int biased_exp(double v) { return (int)((__double_as_longlong(v) >> 52) & 0x7FF); }
 
 // rint(v * 2^(56 - b)) for |v| < 2^(b-1), in integer arithmetic (round half
-// to even), so |result| <= 2^55.
+// to even) without branches, so |result| <= 2^55; 0 for zeros and subnormals.
 __device__ __forceinline__ long long scaled_rint(double v, int b) {
   const long long bits = __double_as_longlong(v);
   const int eb = (int)((bits >> 52) & 0x7FF);
-  if (eb == 0) return 0;  // zero or subnormal: far below the column scale
-  const long long mant = (bits & 0xFFFFFFFFFFFFFLL) | 0x10000000000000LL;  // 53 bits
-  const int sh = eb - 1075 + 56 - b;  // value = mant 2^(eb - 1075); times 2^(56 - b)
-  long long q;
-  if (sh >= 0) {
-    q = mant << sh;  // sh <= 2 by the bound on |v|
-  } else {
-    const int s = -sh;
-    if (s > 54) return 0;
-    const long long half = 1LL << (s - 1);
-    q = mant >> s;
-    const long long rem = mant & ((1LL << s) - 1);
-    q += (rem > half || (rem == half && (q & 1))) ? 1 : 0;
-  }
+  // value = mant 2^(eb - 1075); times 2^(56 - b) = (4 mant) 2^-s, s >= 0 by the bound on |v|
+  const unsigned long long x4 = eb ? ((unsigned long long)bits & 0xFFFFFFFFFFFFFull | 0x10000000000000ull) << 2 : 0ull;
+  const int s = min(max(1021 - eb + b, 0), 60);  // beyond 57 everything rounds to 0
+  const unsigned long long half = (1ull << s) >> 1;
+  const unsigned long long up = half ? half - 1 + ((x4 >> s) & 1) : 0ull;
+  const long long q = (long long)((x4 + up) >> s);
   return bits < 0 ? -q : q;
 }
 
-// The digits of y (|y| < 2^55) as BF16 bit patterns, written 128 bytes apart
-// from col (digit 0, the most significant, first), for the tensor-core
-// operand of r.  Balanced digits of y are the plain digits of y + C minus the
-// offset, C holding the offset in every digit but the top one, so each digit
-// is one bit-field extract; the BF16 of a digit d is the top half of the
-// float 1.5 2^23 + d - 1.5 2^23 (exact: d has at most 8 significant bits).
+// Balanced digits of y (|y| < 2^55) are the plain digits of y + C minus the
+// offset, C holding the offset in every digit (base 256) or every digit but the
+// top one (base 128), so each digit is one bit-field extract.
+
+// The BF16 of a small integer is the top half of the float 1.5 2^23 + d - 1.5
+// 2^23 (exact: d has at most 8 significant bits).
 __device__ __forceinline__ uint16_t small_int_bf16_bits(int d) {
   return (uint16_t)(__float_as_uint(__int_as_float(0x4B400000 + d) - 12582912.0f) >> 16);
 }
 
-// base 256, digits 0..6 (d_0 in [-128, 128], the others in [-128, 127]); an
-// eighth, zero digit is written at 7 * 128
-__device__ __forceinline__ void write_digits256_bf16(long long y, unsigned char* col) {
-  const long long z = y + 0x808080808080LL;  // 128 in digits 1..6
-  const uint32_t lo = (uint32_t)z, hi = (uint32_t)((unsigned long long)z >> 32);
-  *(uint16_t*)(col + 0 * 128) = small_int_bf16_bits((int)(z >> 48));
-  *(uint16_t*)(col + 1 * 128) = small_int_bf16_bits((int)((hi >> 8) & 255u) - 128);
-  *(uint16_t*)(col + 2 * 128) = small_int_bf16_bits((int)(hi & 255u) - 128);
-  *(uint16_t*)(col + 3 * 128) = small_int_bf16_bits((int)(lo >> 24) - 128);
-  *(uint16_t*)(col + 4 * 128) = small_int_bf16_bits((int)((lo >> 16) & 255u) - 128);
-  *(uint16_t*)(col + 5 * 128) = small_int_bf16_bits((int)((lo >> 8) & 255u) - 128);
-  *(uint16_t*)(col + 6 * 128) = small_int_bf16_bits((int)(lo & 255u) - 128);
+// Base 256, digits 0..6 (the most significant first; d_0 in [-128, 128], the
+// others in [-128, 127]) as F16, written at 0 .. 6 * 128 of col; an eighth, zero digit at 7 * 128.  With 128
+// added to every digit they are the bytes of one integer, and 1024 + u, u <= 256,
+// is the F16 with the bits 0x6400 + u.
+constexpr unsigned long long kBias256 = 0x80808080808080ull;
+__device__ __forceinline__ void write_digits256_f16(long long y, unsigned char* col) {
+  const unsigned long long z = (unsigned long long)y + kBias256;
+  const uint32_t lo = (uint32_t)z, hi = (uint32_t)(z >> 32);  // hi < 2^25
+  const uint32_t u[7] = {hi >> 16, (hi >> 8) & 255u, hi & 255u, lo >> 24, (lo >> 16) & 255u, (lo >> 8) & 255u, lo & 255u};
+  const __half off = __ushort_as_half(0x6480);  // 1024 + 128
+#pragma unroll
+  for (int p = 0; p < 7; ++p)
+    *(uint16_t*)(col + p * 128) = __half_as_ushort(__hsub(__ushort_as_half((unsigned short)(0x6400u + u[p])), off));
   *(uint16_t*)(col + 7 * 128) = 0;
+}
+
+// Four digit bytes (digit + 128 each) as two F16 pairs.
+__device__ __forceinline__ void expand_digit_bytes(uint32_t w, uint32_t& d01, uint32_t& d23) {
+  const uint32_t off = 0x64806480u;
+  const uint32_t a = __byte_perm(w, 0x64646464u, 0x4140), b = __byte_perm(w, 0x64646464u, 0x4342);
+  const __half2 o = *reinterpret_cast<const __half2*>(&off);
+  const __half2 x = __hsub2(*reinterpret_cast<const __half2*>(&a), o), y = __hsub2(*reinterpret_cast<const __half2*>(&b), o);
+  d01 = *reinterpret_cast<const uint32_t*>(&x);
+  d23 = *reinterpret_cast<const uint32_t*>(&y);
 }
 
 // base 128, digits 0..7 (d_0 in [-64, 64], the others in [-64, 63]) into d[]

@@ -509,8 +509,8 @@ static int level0_f32_launch(gs_ctx ctx, gs_mas mas, const double* r, double* z,
   return launch_level0_f32<8, kDot>(ctx, mas, r, z, nrhs, zl, lstride, skip, dot);
 }
 
-// Forms whose level-0 product can also reduce r . z: FP64 from BF16 digit
-// matrices (one CTA per domain), FP32 from packed inverses; at most 8 RHS.
+// Forms whose level-0 product can also reduce r . z: FP64 from digit bytes
+// (one CTA per domain), FP32 from packed inverses; at most 8 RHS.
 bool mas_dot_usable(gs_ctx ctx, gs_mas mas, int nrhs) {
   if (nrhs > 8) return false;
   if (mas->precision == GS_PREC_FP32) return level0_f32_bulk_usable(mas, nrhs);
@@ -569,7 +569,7 @@ static int launch_apply(gs_ctx ctx, gs_mas mas, const Ts* const* d_inv, const in
           mas->up[l], mas->n_domains[l], N, 3 * nrhs, LevelIdxRhsMajor{lstride, mas->vec_off[l]},
           LevelIdxRhsMajor{lstride, mas->vec_off[l + 1]}, rl, skip);
     }
-    if (level0_f64tc_usable(ctx, mas, nrhs)) {  // FP64 accuracy on the BF16 tensor cores
+    if (level0_f64tc_usable(ctx, mas, nrhs)) {  // FP64 accuracy on the tensor cores
       GS_PROF(ctx, GS_K_MAS_APPLY_COARSE);
       GS_TRY(coarse_f64tc_launch(ctx, mas, nrhs, rl, zl, lstride, skip));
     } else if (std::is_same<Ts, float>::value && nrhs <= 8) {
@@ -586,7 +586,7 @@ static int launch_apply(gs_ctx ctx, gs_mas mas, const Ts* const* d_inv, const in
     GS_TRY(level0_bf16_launch(ctx, mas, false, nrhs, r, stride, zl, lstride, z, nullptr, ctx->d_flags));
   } else if (std::is_same<Ts, float>::value && level0_f32_bulk_usable(mas, nrhs)) {  // FP32, packed inverses
     GS_TRY(level0_f32_launch<false>(ctx, mas, r, z, nrhs, zl, lstride, skip, Partials{}));
-  } else if (level0_f64tc_usable(ctx, mas, nrhs)) {  // FP64 accuracy on the BF16 tensor cores
+  } else if (level0_f64tc_usable(ctx, mas, nrhs)) {  // FP64 accuracy on the tensor cores
     GS_PROF(ctx, GS_K_MAS_APPLY_L0);
     GS_TRY(level0_f64tc_launch(ctx, mas, nrhs, (const double*)r, stride, (const double*)zl, lstride, (double*)z,
                                skip));

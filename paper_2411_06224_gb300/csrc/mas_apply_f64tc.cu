@@ -1,4 +1,4 @@
-// Level-0 MAS product in FP64 accuracy on the BF16 tensor cores (Eq. 6 at
+// Level-0 MAS product in FP64 accuracy on the F16 tensor cores (Eq. 6 at
 // level 0), by exact integer splitting of both operands (the Ozaki scheme).
 //
 // FP64 FMA runs at 2 per clock per SM on this part, so the FP64 dense
@@ -8,29 +8,33 @@
 // combination remains per output:
 //   * build time: row i of M_d^{-1} gets an exponent a_i with |M_ik| < 2^(a_i-1);
 //     X_ik = rint(M_ik 2^(56-a_i)) (|X| < 2^55) is cut into 7 balanced base-256
-//     digits m^(1..7) in [-128, 128] (X = sum_p m^(p) 256^(7-p)), each digit
-//     matrix stored as BF16 (exact) in the K-major operand layout;
+//     digits m^(1..7) in [-128, 127] (X = sum_p m^(p) 256^(7-p)), stored as the
+//     bytes m + 128 (a row whose leading digit would be 128 takes a_i + 1);
 //   * apply: column k of r_d gets b_k with |r_jk| < 2^(b_k-1), likewise
-//     Y_jk = rint(r_jk 2^(56-b_k)) -> digits n^(1..7);
+//     Y_jk = rint(r_jk 2^(56-b_k)) -> digits n^(1..7) in [-128, 128];
 //   * G_s = sum_{p+q=s} m^(p) n^(q) for s = 2..9 (products of digits <= 2^14,
 //     96 terms, <= 7 pairs: |G_s| < 2^24, exact in FP32): the B operand holds
-//     all 7 digit columns of r (plus a zero one, N = 64), so one MMA per digit
-//     matrix and K step writes the groups p+2 .. p+9 into TMEM columns
-//     8p .. 8p+63; each G_s collects in its own 8 columns (groups above 9 are
-//     not read);
+//     all 7 digit columns of r (plus a zero one), so one MMA per digit matrix
+//     and K step writes the groups p+2 .. 9 into TMEM columns 8p .. 63 (one more
+//     group, not read, where N is rounded up to a multiple of 16); each G_s
+//     collects in its own 8 columns;
 //   * z_ik = 2^(a_i + b_k - 72) sum_{s=2..9} G_s 256^(9-s), combined in
 //     64-bit integers (two halves) and rounded once to a double in integer
 //     arithmetic, so the epilogue spends one FP64 add (the coarse levels).
-// Dropped terms (p + q > 9) and the roundings of X, Y are below 2^-55 of the
+// Dropped terms (p + q > 9) and the roundings of X, Y are below 2^-54 of the
 // row and column maxima, the level of FP64's own rounding.
 //
-// One CTA of 256 threads per domain; the 7 digit matrices (18 KB each) stream
-// through a shared-memory ring filled by bulk asynchronous copies: 2 slots at
-// level 0 (50 KB per CTA, four CTAs share an SM and hide each other's
-// latency), 4 for the few coarse-level domains.  All waits are bounded
-// (kErrTimeout); TMEM is always freed.
-#include <cuda_bf16.h>
-
+// One CTA of 256 threads per domain.  The digit bytes come into a shared-memory
+// ring by bulk asynchronous copies; two threads per row read them, expand them
+// to F16 (a byte permute and a subtraction for two entries) and store them to
+// TMEM as the MMA's A operand.  What bounds it: no longer the bytes (7 per entry;
+// BF16 digits, copied to shared memory as they lay, were 14, and 81 % of the
+// DRAM rate) but the chain of steps within a domain, about 16000 clocks with
+// four domains to an SM, half of it the seven digits.  With r . z, 45^3, 1 RHS:
+// 74 -> 51 us; 24 bodies, 1 RHS: 140 -> 99; 64^3, 8 RHS: 214 -> 172 without it.
+// Tried: digits prefetched into registers (57 us at 45^3, against 48 of the same
+// without r . z), three A operands and two CTAs per SM (70).  All waits are
+// bounded (kErrTimeout); TMEM is always freed.
 #include <algorithm>
 
 #include "common.cuh"
@@ -42,12 +46,16 @@ namespace gs {
 namespace f64tc {
 
 constexpr int kDigits = 7;
-constexpr int kSlots = 2;        // ring slots of the level-0 kernel (4 CTAs per SM; 3 slots and
-                                 // 3 CTAs per SM measured 15 % slower)
-constexpr int kSlotsFew = 4;     // two CTAs per SM
-constexpr int kThreads = 128;
+constexpr int kThreads = 256;
 constexpr int kM = 128;
-constexpr int kTmemCols = 128;  // groups s = 2..10, 8 columns each (72 used)
+
+// TMEM: groups s = 2..10, 8 columns each, then kBufs A operands of LD / 2 columns.
+constexpr int kACol = 80;
+__host__ __device__ constexpr int tmem_cols(int bufs, int ld) {
+  const int need = kACol + bufs * (ld / 2);
+  return need <= 128 ? 128 : (need <= 256 ? 256 : 512);
+}
+__host__ __device__ constexpr size_t ring_bytes(int slots, int ld) { return 128 + (size_t)slots * ld * ld; }
 
 struct Levels {
   const int32_t* coarse[8];
@@ -55,15 +63,6 @@ struct Levels {
   int64_t vec_off[8];
   int L;
 };
-
-__host__ __device__ inline uint32_t slot_bytes(int ld) {  // K-major M = 128 span of one digit matrix
-  return ((uint32_t)(ld * ld * 2 - ld * 16 + kM * 16) + 127u) & ~127u;
-}
-__host__ __device__ inline uint32_t b_bytes(int ld) { return (uint32_t)(ld / 8) * 256; }
-template <int kS>
-__host__ inline size_t smem_bytes(int ld) {
-  return 128 + (size_t)kS * slot_bytes(ld) + 4 * (size_t)b_bytes(ld) + (2 * kS + 1) * 8 + 8 + 8 * 4 + 32 * 4;
-}
 
 // T 2^e as the nearest double (ties to even), T = hi 2^32 + lo with
 // |hi|, |lo| < 2^49.
@@ -77,14 +76,16 @@ __device__ __forceinline__ double scaled_to_double(long long hi, long long lo, i
 // kCoarse = true: coarse-level domains (job tables), r and z are the level's
 //   contiguous multilevel vectors rl, zl; a level with al.kids gathers its r
 //   as the sums of its items' children of the level below.
-// One CTA per domain (CTAs that walk several domains with everything set up
-// once and the next domain's first digits prefetched measured 0.24 ms at 64^3
-// against 0.21: the four CTAs of an SM overlap each other's prologue and
-// epilogue better than one does its own).  r . z costs a CTA ten FP64
-// instructions per warp (warp_sums), the separate pass it replaces 9 us at 45^3.
-template <bool kCoarse, bool kDot, int kS, int LD, int kT>
-__global__ void __launch_bounds__(kT, kT == 256 ? 4 : 1) k_level0_f64tc(
-    const __nv_bfloat16* const* __restrict__ dig_tab, const int32_t* const* __restrict__ exp_tab,
+// kSlots: digits in the ring; kBufs: A operands in TMEM (a digit is stored while
+// the MMAs of the kBufs - 1 before it run); kCtas of them per SM.
+// Roles after the operand B is written: the warps that own rows of TMEM lanes
+// 0 .. LD - 1 expand and store the digits and later take the results, warp 3
+// issues the MMAs and the copies, warp 7 sums the prolongated coarse results.  r . z costs a
+// CTA ten FP64 instructions per warp (warp_sums), the separate pass it replaces
+// 9 us at 45^3.
+template <bool kCoarse, bool kDot, int kSlots, int kBufs, int kCtas, int LD>
+__global__ void __launch_bounds__(kThreads, kCtas) k_level0_f64tc(
+    const uint8_t* const* __restrict__ dig_tab, const int32_t* const* __restrict__ exp_tab,
     const int32_t* __restrict__ job_level, const int32_t* __restrict__ job_dom, const int32_t* __restrict__ remap0,
     int N, int nrhs, Levels al, const double* __restrict__ r, int64_t stride,
     const double* __restrict__ zl, int64_t lstride, double* __restrict__ z, int* __restrict__ flags,
@@ -94,63 +95,101 @@ __global__ void __launch_bounds__(kT, kT == 256 ? 4 : 1) k_level0_f64tc(
   // restriction or the coarse product: it wrote neither them nor *skip.
   constexpr bool kEarly = kCoarse || kDot;
   if (!kEarly) wait_for_previous_kernel();
-  if (skip && *skip) return;  // whole CTA, before any barrier or TMEM use
-  extern __shared__ unsigned char smem_raw[];
   constexpr int ld = LD;  // 3 N
-  const uint32_t sbytes = slot_bytes(ld), bb = b_bytes(ld);
-  const uint32_t dig_bytes = (uint32_t)ld * ld * 2;
+  constexpr int kPer = (8 * LD + kThreads - 1) / kThreads;  // entries of r per thread: e = tid + m kThreads = k ld + j
+  constexpr int kChunks = LD / 16, kHalf = (kChunks + 1) / 2, kRowWarps = (LD + 31) / 32;
+  __shared__ __align__(128) unsigned char sB[LD / 8 * 1024];  // 4 pair operands [n^(2j+1) | n^(2j+2)]
+  __shared__ double sr[kDot ? 8 * LD : 1];                     // r, for r . z
+  __shared__ double scoarse[kCoarse ? 1 : 8 * LD];
+  __shared__ int32_t snode[32];  // node of every slot of the domain (-1: padding)
+  __shared__ int sexp[8];        // biased exponent maxima of the RHS columns
+  __shared__ uint64_t full[kSlots], ready[kBufs], freed[kBufs], drained, summed;
+  extern __shared__ unsigned char smem_raw[];
   unsigned char* ring = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
-  unsigned char* sB = ring + kS * sbytes;  // 4 pair operands [n^(2j+1) | n^(2j+2)]
-  uint64_t* full = (uint64_t*)(sB + 4 * bb);
-  uint64_t* empty = full + kS;
-  uint64_t* done = empty + kS;
-  uint32_t* tslot = (uint32_t*)(done + 1);
-  int* sfail = (int*)(tslot + 1);
-  int* sexp = sfail + 1;  // [8] biased exponent maxima of the RHS columns
-  int* snode = sexp + 8;  // [32] node of every slot of the domain (-1: padding)
+  constexpr uint32_t dig_bytes = LD * LD, kCols = tmem_cols(kBufs, LD);
+  __shared__ uint32_t tslot;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // loads that depend on nothing leave together
   const int lvl = kCoarse ? job_level[blockIdx.x] : 0;
   const int32_t d = kCoarse ? job_dom[blockIdx.x] : (int32_t)blockIdx.x;
-  const __nv_bfloat16* dd = dig_tab[lvl] + (int64_t)d * kDigits * ld * ld;
+  const uint8_t* dd = dig_tab[lvl] + (int64_t)d * kDigits * LD * LD;
+  int32_t node_of[kPer];  // nodes of this thread's entries of r
+#pragma unroll
+  for (int m = 0; m < kPer; ++m) {
+    const int e = tid + m * kThreads;
+    node_of[m] = kCoarse ? 0 : (e / ld < nrhs && e < 8 * ld ? remap0[(int64_t)d * N + e % ld / 3] : -1);
+  }
+  const int32_t my_node = kCoarse ? 0 : remap0[(int64_t)d * N + min(lane, N - 1)];
+  if (skip && *skip) return;  // whole CTA, before any barrier or TMEM use
   const int64_t cbase = kCoarse ? 3 * (al.vec_off[lvl] + (int64_t)d * N) : 0;  // coarse: first entry of the domain
+  // Warps w and w + 4 share TMEM lane quarter w % 4: they expand half a row
+  // each and take the right-hand sides 0..3 and 4..7 of its results.
+  constexpr int kRpt = 4;  // right-hand sides per epilogue thread
+  const int q4 = warp & 3, half = warp >> 2, k0 = half * kRpt;
+  const int i_row = q4 * 32 + lane;
+  const bool rows = q4 < kRowWarps;  // whole warp
 
   if (tid == 0) {
-    for (int s = 0; s < kS; ++s) mbar_init(&full[s], 1), mbar_init(&empty[s], 1);
-    mbar_init(done, 1);
-    *sfail = 0;
+    for (int q = 0; q < kSlots; ++q) mbar_init(&full[q], 1);
+    for (int q = 0; q < kBufs; ++q) mbar_init(&freed[q], 1), mbar_init(&ready[q], 2 * kRowWarps);
+    mbar_init(&drained, 1);
+    mbar_init(&summed, 1);
     fence_mbar_init();
-    for (int p = 0; p < kS; ++p) {
-      mbar_arrive_expect_tx(&full[p], dig_bytes);
-      bulk_g2s(ring + p * sbytes, dd + (int64_t)p * ld * ld, dig_bytes, &full[p]);
+    for (int q = 0; q < kSlots; ++q) {
+      mbar_arrive_expect_tx(&full[q], dig_bytes);
+      bulk_g2s(ring + q * dig_bytes, dd + q * dig_bytes, dig_bytes, &full[q]);
     }
   }
   if (tid < 8) sexp[tid] = 0;
-  if (tid < 32) snode[tid] = tid < N ? (kCoarse ? 0 : remap0[(int64_t)d * N + tid]) : -1;
+  if (tid < 32) snode[tid] = tid < N ? my_node : -1;
   if (warp == 0) {
-    tmem_alloc(tslot, kTmemCols);
+    tmem_alloc(&tslot, kCols);
     tmem_relinquish();
   }
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
-  const uint32_t tmem = *tslot;
+  const uint32_t tmem = tslot;
   if (kEarly) wait_for_previous_kernel();
-  // With 256 threads, warps w and w + 4 share TMEM lane quarter w % 4 and
-  // take the right-hand sides 0..3 and 4..7 of its rows.
-  constexpr int kRpt = 8 * 128 / kT;  // right-hand sides per epilogue thread
-  const int q4 = warp & 3, k0 = (warp >> 2) * kRpt;
-  const int i_row = q4 * 32 + lane;
+  // Digit p of this thread's half row, chunk c (16 entries) at [c][row] of its
+  // slot, to the A operand: false where a wait gave up.
+  bool ok = true;
+  auto store_digit = [&](int p) {
+    const unsigned char* mine = ring + (p % kSlots) * dig_bytes + (half * kHalf * ld + min(i_row, ld - 1)) * 16;
+    const uint32_t ta = tmem + ((uint32_t)(q4 * 32) << 16) + kACol + half * kHalf * 8 + (p % kBufs) * (ld / 2);
+    ok = ok && mbar_wait(&full[p % kSlots], (uint32_t)(p / kSlots) & 1u);
+    uint32_t v[kHalf][8];  // expanded while the MMAs of the digit before still read the operand
+#pragma unroll
+    for (int j = 0; j < kHalf; ++j)
+      if (half * kHalf + j < kChunks) {  // whole warp
+        const uint4 b = *reinterpret_cast<const uint4*>(mine + j * ld * 16);
+        expand_digit_bytes(b.x, v[j][0], v[j][1]);
+        expand_digit_bytes(b.y, v[j][2], v[j][3]);
+        expand_digit_bytes(b.z, v[j][4], v[j][5]);
+        expand_digit_bytes(b.w, v[j][6], v[j][7]);
+      }
+    if (p >= kBufs) ok = ok && mbar_wait(&freed[p % kBufs], (uint32_t)(p / kBufs - 1) & 1u);
+    ok = __all_sync(kFull, ok);
+    if (!ok) return false;
+    fence_after_sync();
+#pragma unroll
+    for (int j = 0; j < kHalf; ++j)
+      if (half * kHalf + j < kChunks) tmem_st_32x32b_x8(ta + 8 * j, v[j]);
+    tmem_wait_st();
+    fence_before_sync();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&ready[p % kBufs]);
+    return true;
+  };
   // r_d once into registers (entry e = k * ld + j), column exponents by
   // shared-memory atomics, then the digits into the four pair operands
-  constexpr int kPer = 8 * 128 / kT;  // entries per thread for ld <= 128
   double rv[kPer];
 #pragma unroll
   for (int m = 0; m < kPer; ++m) {
-    const int e = tid + m * kT;
+    const int e = tid + m * kThreads;
     const int k = e / ld, j = e - k * ld;
     rv[m] = 0.0;
     if (k < nrhs && k < 8) {
-      const int32_t node = snode[j / 3];
       if (kCoarse) {
         if (al.kids[lvl]) {
           const int2 kid = al.kids[lvl][(int64_t)d * N + j / 3];
@@ -159,133 +198,137 @@ __global__ void __launch_bounds__(kT, kT == 256 ? 4 : 1) k_level0_f64tc(
         } else {
           rv[m] = r[k * lstride + cbase + j];
         }
-      } else if (node >= 0) {
-        rv[m] = r[k * stride + 3 * (int64_t)node + j % 3];
+      } else if (node_of[m] >= 0) {
+        rv[m] = r[k * stride + 3 * (int64_t)node_of[m] + j % 3];
       }
-      const int eb = biased_exp(rv[m]);  // integer test: no FP64 compare
-      if (eb) atomicMax(&sexp[k], eb);
+    }
+  }
+  if (rows) store_digit(0);  // while r is on its way
+#pragma unroll
+  for (int m = 0; m < kPer; ++m) {
+    const int e = tid + m * kThreads;
+    const int k = e / ld;
+    if (k >= nrhs || k >= 8) continue;
+    if (kDot) sr[e] = rv[m];
+    int eb = biased_exp(rv[m]);  // integer test: no FP64 compare
+    if (LD % 32 == 0) {          // one right-hand side per warp
+      eb = __reduce_max_sync(kFull, eb);
+      if (lane == 0) atomicMax(&sexp[k], eb);
+    } else if (eb) {
+      atomicMax(&sexp[k], eb);
     }
   }
   __syncthreads();
   // element (n, kk) of a pair operand at (kk/8)*256 + (n/8)*128 + (n%8)*16 + (kk%8)*2
 #pragma unroll
   for (int m = 0; m < kPer; ++m) {
-    const int e = tid + m * kT;
-    if (e >= 8 * ld) break;
+    const int e = tid + m * kThreads;
+    if (e >= nrhs * ld) break;  // columns of absent right-hand sides stay unset: their results are not read
     const int k = e / ld, j = e - k * ld;
     const long long y = scaled_rint(rv[m], sexp[k] - 1021);  // 0 for zero entries
     // column n = 8 q + k; q = 7: the missing 8th digit, zero
-    write_digits256_bf16(y, sB + (j >> 3) * 1024 + (j & 7) * 2 + k * 16);
+    write_digits256_f16(y, sB + (j >> 3) * 1024 + (j & 7) * 2 + k * 16);
   }
   fence_proxy_async();
   __syncthreads();
-  // Epilogue operands that do not depend on the MMAs, loaded now so that their
-  // latency overlaps the tensor-core work: row exponent and the prolongated
-  // coarse-level sum per RHS.
-  const int32_t node_row = (q4 * 32 < ld && i_row < ld) ? snode[i_row / 3] : -1;
+
+  const int32_t node_row = rows && i_row < ld ? snode[i_row / 3] : -1;
   const int c_row = i_row % 3;
   int a_row = -100000;
-  double coarse_sum[kRpt];
-#pragma unroll
-  for (int k = 0; k < kRpt; ++k) coarse_sum[k] = 0.0;
   if (node_row >= 0) a_row = exp_tab[lvl][(int64_t)d * ld + i_row];
-  if (!kCoarse && node_row >= 0) {
+  // one copy of the loops' code where each step waits for the one before anyway:
+  // a CTA runs them once, from a cold instruction cache
+  constexpr int kUnroll = kBufs == 1 ? 1 : kDigits;
+  if (rows) {
+#pragma unroll kUnroll
+    for (int p = 1; p < kDigits; ++p)
+      if (!store_digit(p)) break;
+    let_next_kernel_launch();
+    constexpr int kLast = kDigits - 1;  // the MMAs end in order
+    ok = ok && __all_sync(kFull, mbar_wait(&freed[kLast % kBufs], (uint32_t)(kLast / kBufs) & 1u));
+    if (!kCoarse) ok = ok && __all_sync(kFull, mbar_wait(&summed, 0));
+    if (!ok && lane == 0) atomicOr(flags, kErrTimeout);
+    fence_after_sync();
+  } else if (warp == 3) {
+    let_next_kernel_launch();
+    if (lane == 0) {
+      // descriptors are built once; their 14-bit address fields are advanced
+      // by adding byte offsets / 16
+      const uint64_t db0 = smem_desc(smem_u32(sB), 1024, 128);
+      int copied = kSlots;
+      bool good = true;
+#pragma unroll kUnroll
+      for (int p = 0; p < kDigits; ++p) {
+        good = good && mbar_wait(&ready[p % kBufs], (uint32_t)(p / kBufs) & 1u);
+        if (!good) break;
+        fence_after_sync();
+        const uint32_t idesc = idesc_f16_f32(kM, (64 - 8 * p + 15) / 16 * 16);
+        const uint32_t ta = tmem + kACol + (p % kBufs) * (ld / 2);
 #pragma unroll
-    for (int l = 1; l < 8; ++l) {
-      if (l >= al.L) break;
-      const int64_t item = al.vec_off[l] + al.coarse[l][node_row];
-#pragma unroll
-      for (int k = 0; k < kRpt; ++k)
-        if (k0 + k < nrhs) {  // the first coarse level assigns: one FP64 add fewer per output
-          const double v = zl[(k0 + k) * lstride + 3 * item + c_row];
-          coarse_sum[k] = l == 1 ? v : coarse_sum[k] + v;
+        for (int ks = 0; ks < kChunks; ++ks)
+          mma_f16_ts(tmem + 8u * p, ta + 8u * ks, db0 + ks * (2048u >> 4), idesc, (p > 0 || ks > 0) ? 1u : 0u);
+        mma_commit(&freed[p % kBufs]);
+        if (p + kSlots < kDigits) {  // every row warp has read this slot
+          mbar_arrive_expect_tx(&full[p % kSlots], dig_bytes);
+          bulk_g2s(ring + (p % kSlots) * dig_bytes, dd + (p + kSlots) * dig_bytes, dig_bytes, &full[p % kSlots]);
+          ++copied;
         }
-    }
-  }
-  // MMA issue and ring refills (one thread).  A slot is refilled as soon as
-  // the MMAs reading it have completed (a wait of a few hundred cycles, while
-  // the next digit's copy is still in flight), so two copies stay in flight
-  // per CTA.  Descriptors are built once; their 14-bit address fields are
-  // advanced by adding byte offsets / 16 (all addresses stay below 256 KB).
-  if (tid == 0) {
-    bool ok = true;
-    int loads[kS];  // copies issued into each slot
-    for (int s = 0; s < kS; ++s) loads[s] = 1;
-    const uint32_t lbo = (uint32_t)ld * 16;
-    const uint32_t idesc = idesc_bf16_f32(kM, 64);
-    const uint64_t da0 = smem_desc(smem_u32(ring), lbo, 128);
-    const uint64_t db0 = smem_desc(smem_u32(sB), 1024, 128);
-    const uint64_t da_ks = (2u * lbo) >> 4, db_ks = 2048u >> 4;
-    for (int p = 0; p < kDigits && ok; ++p) {
-      const int slot = p % kS;
-      if (!mbar_wait(&full[slot], (uint32_t)(p / kS) & 1u)) {
-        ok = false;
-        break;
       }
-      fence_after_sync();
-      const uint64_t da = da0 + ((uint64_t)slot * sbytes >> 4);
-      // digit p times all digit columns of r: groups s = p + 2 .. p + 9 at TMEM
-      // columns 8 p .. 8 p + 63 (group s at column 8 (s - 2))
-#pragma unroll 6
-      for (int ks = 0; ks < ld / 16; ++ks)
-        mma_bf16(tmem + 8u * p, da + ks * da_ks, db0 + ks * db_ks, idesc, (p > 0 || ks > 0) ? 1u : 0u);
-      if (p + kS < kDigits) {  // this slot takes digit p + kS once its MMAs are done
-        mma_commit(&empty[slot]);
-        if (!mbar_wait(&empty[slot], (uint32_t)(p / kS) & 1u)) {
-          ok = false;
-          break;
-        }
-        mbar_arrive_expect_tx(&full[slot], dig_bytes);
-        bulk_g2s(ring + slot * sbytes, dd + (int64_t)(p + kS) * ld * ld, dig_bytes, &full[slot]);
-        ++loads[slot];
+      if (!good) {  // whatever was issued ends before the CTA leaves
+        atomicOr(flags, kErrTimeout);
+        mma_commit(&drained);
+        mbar_wait(&drained, 0);
+        for (int q = 0; q < kSlots; ++q) mbar_wait(&full[q], (uint32_t)((copied - 1 - q) / kSlots) & 1u);
       }
     }
-    if (ok) {
-      mma_commit(done);
-    } else {
-      *sfail = 1;
-      atomicOr(flags, kErrTimeout);
-      for (int s = 0; s < kS; ++s)  // let the last copy into each slot land before the CTA leaves
-        mbar_wait(&full[s], (uint32_t)(loads[s] - 1) & 1u);
-      mbar_arrive(done);
+  } else {
+    let_next_kernel_launch();
+    if (!kCoarse && warp == 7) {
+      // the prolongated coarse results, lane s holding slot s's items; the first
+      // coarse level assigns: one FP64 add fewer per output
+      const int32_t node = lane < N ? snode[lane] : -1;
+      int32_t item[8];
+#pragma unroll
+      for (int l = 1; l < 8; ++l) item[l] = l < al.L && node >= 0 ? al.coarse[l][node] : 0;
+      constexpr int kU = 6;
+      for (int e0 = 0; e0 < nrhs * ld; e0 += 32 * kU) {
+        double v[kU];
+        int64_t at[kU];
+        int slot[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+          const int e = min(e0 + 32 * u + lane, nrhs * ld - 1);
+          const int k = e / ld, j = e - k * ld;
+          slot[u] = j / 3;
+          at[u] = k * lstride + j % 3;
+          v[u] = 0.0;
+        }
+#pragma unroll
+        for (int l = 1; l < 8; ++l) {
+          if (l >= al.L) break;
+          double t[kU];
+#pragma unroll
+          for (int u = 0; u < kU; ++u)
+            t[u] = zl[at[u] + 3 * (al.vec_off[l] + __shfl_sync(kFull, item[l], slot[u]))];
+#pragma unroll
+          for (int u = 0; u < kU; ++u) v[u] = l == 1 ? t[u] : v[u] + t[u];
+        }
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+          if (e0 + 32 * u + lane < nrhs * ld) scoarse[e0 + 32 * u + lane] = v[u];
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&summed);
     }
   }
-  let_next_kernel_launch();
-  // r of this thread's row, for r . z (in cache since the gather)
-  double rrow[kRpt];
-  if (kDot) {
-#pragma unroll
-    for (int k = 0; k < kRpt; ++k)
-      rrow[k] = node_row >= 0 && k0 + k < nrhs ? r[(k0 + k) * stride + 3 * (int64_t)node_row + c_row] : 0.0;
-  }
-  // warp 0 waits for the MMAs; the other warps wait at the barrier, where they
-  // take no issue slots
-  if (warp == 0) {
-    __syncwarp();
-    bool fin = mbar_wait(done, 0);
-    if (!fin) atomicOr(flags, kErrTimeout);
-    fin = __all_sync(0xffffffffu, fin);
-    if (lane == 0 && !fin) *sfail = 1;
-  }
-  __syncthreads();
-  const bool ok = !*sfail;
-  fence_after_sync();
   double dacc[kRpt];
   int dex[kRpt];
 #pragma unroll
   for (int k = 0; k < kRpt; ++k) dacc[k] = 0.0, dex[k] = kExpNone;
-  if (ok && q4 * 32 < ld) {
+  if (rows && ok && k0 < nrhs) {  // whole warp
     const uint32_t ta = tmem + ((uint32_t)(q4 * 32) << 16);
     float g[8 * kRpt];  // groups s = 2..9 of this thread's RHS: g[kRpt (s - 2) + k]
-    if constexpr (kRpt == 8) {
-      tmem_ld_32x32b_x16(ta + 0, g);
-      tmem_ld_32x32b_x16(ta + 16, g + 16);
-      tmem_ld_32x32b_x16(ta + 32, g + 32);
-      tmem_ld_32x32b_x16(ta + 48, g + 48);
-    } else {
-#pragma unroll
-      for (int s = 0; s < 8; ++s) tmem_ld_32x32b_x4(ta + 8 * s + k0, g + 4 * s);
-    }
+    tmem_ld_32x32b_8x4(ta + k0, 8, g);
     if (node_row >= 0) {
 #pragma unroll
       for (int k = 0; k < kRpt; ++k) {
@@ -294,35 +337,37 @@ __global__ void __launch_bounds__(kT, kT == 256 ? 4 : 1) k_level0_f64tc(
         double v = 0.0;
         if (sexp[kk] && a_row > -100000) {
           // T = hi 2^32 + lo, hi = sum_{s=2..5} G_s 256^(5-s), lo = sum_{s=6..9} G_s 256^(9-s)
-          long long hi = 0, lo = 0;
+          long long hi = __float2int_rn(g[3 * kRpt + k]), lo = __float2int_rn(g[7 * kRpt + k]);
 #pragma unroll
-          for (int s = 0; s < 4; ++s) hi = (hi << 8) + (long long)__float2int_rn(g[kRpt * s + k]);
-#pragma unroll
-          for (int s = 4; s < 8; ++s) lo = (lo << 8) + (long long)__float2int_rn(g[kRpt * s + k]);
+          for (int s = 0; s < 3; ++s) {
+            hi += (long long)__float2int_rn(g[kRpt * s + k]) * (1 << (24 - 8 * s));
+            lo += (long long)__float2int_rn(g[kRpt * (s + 4) + k]) * (1 << (24 - 8 * s));
+          }
           const int e = a_row + (sexp[kk] - 1021) - 72;  // z = T 2^e, T = hi 2^32 + lo
           if (e < 900) v = scaled_to_double(hi, lo, e);
         }
         if (kCoarse) {
           z[kk * lstride + cbase + i_row] = v;
         } else {
-          v += coarse_sum[k];
+          v += scoarse[kk * ld + i_row];
           z[kk * stride + 3 * (int64_t)node_row + c_row] = v;
           if (kDot) {
-            dacc[k] = rrow[k] * v;
+            dacc[k] = sr[kk * ld + i_row] * v;
             dex[k] = ex_bound(v);
           }
         }
       }
     }
   }
-  __shared__ double red[kT / 32][kRpt];
-  __shared__ int redx[kT / 32][kRpt];
+  __shared__ double red[kThreads / 32][kRpt];
+  __shared__ int redx[kThreads / 32][kRpt];
   if (kDot) {
+    const bool some = rows && k0 < nrhs;  // whole warp: the others add zeros at the FP64 pipe's full price
     const int k = sum_index<kRpt>(lane);
-    const double v = warp_sums<kRpt>(dacc, lane);
+    const double v = some ? warp_sums<kRpt>(dacc, lane) : 0.0;
 #pragma unroll
     for (int q = 0; q < kRpt; ++q) {
-      const int e = __reduce_max_sync(kFull, dex[q]);
+      const int e = some ? __reduce_max_sync(kFull, dex[q]) : kExpNone;
       if (lane == 0) redx[warp][q] = e;
     }
     if (lane < kRpt) red[warp][k] = v;
@@ -331,13 +376,13 @@ __global__ void __launch_bounds__(kT, kT == 256 ? 4 : 1) k_level0_f64tc(
   __syncthreads();
   if (warp == 0) {
     fence_after_sync();
-    tmem_dealloc(tmem, kTmemCols);
+    tmem_dealloc(tmem, kCols);
   }
   if (kDot && tid < nrhs) {
     double v = 0.0;
     int e = kExpNone;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < kRowWarps; ++q) {
       v += red[tid / kRpt * 4 + q][tid % kRpt];
       e = max(e, redx[tid / kRpt * 4 + q][tid % kRpt]);
     }
@@ -346,293 +391,9 @@ __global__ void __launch_bounds__(kT, kT == 256 ? 4 : 1) k_level0_f64tc(
   }
 }
 
-// ---------------------------------------------------------------- persistent form
-// One CTA per SM walks domains d = blockIdx.x, + gridDim.x, ...  Warp roles:
-//   warp 0 (one lane)  producer: streams the 7 digit matrices of domain after
-//                      domain through a kRing-slot shared-memory ring;
-//   warp 1 (one lane)  MMA issuer: group sums of domain n into TMEM buffer n%2;
-//   warps 2-3          stagers: r of domain n -> column exponents and digits
-//                      into B-operand buffer n%2;
-//   warps 4-7          epilogue: TMEM lane quarter (warp % 4), rounding to
-//                      FP64, prolongated coarse sums, z.
-// Barriers (phase parity = use count & 1): ring full/empty per slot, B-buffer
-// full/empty (empty needs the MMAs and the epilogue), TMEM full/empty.  Copies,
-// MMAs, staging and epilogue of consecutive domains overlap.  Every wait is
-// bounded; a timeout sets an abort word that every role checks, so all roles
-// leave their loops, wait (bounded) for their asynchronous work and meet at
-// the final barrier that precedes the TMEM release.
-constexpr int kRing = 10;
-constexpr int kPThreads = 256;
-
-// Layout after the 128-byte alignment slack: ring, B buffers [2][4], barriers
-// (full, empty [kRing]; bfull, bempty, tfull, tempty [2]; drain), a 64-byte
-// word area (TMEM address, abort word), exponents [2][8], node map [2][32].
-__host__ inline size_t psmem_bytes(int ld) {
-  return 128 + (size_t)kRing * slot_bytes(ld) + 2 * 4 * (size_t)b_bytes(ld) + (2 * kRing + 9) * 8 + 64 + 2 * 8 * 4 +
-         2 * 32 * 4;
-}
-
-__device__ __forceinline__ void named_sync(int id, int count) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
-
-// Named barrier that also ORs a predicate over the participating threads, so
-// that a decision to leave a loop is the same in every one of them.
-__device__ __forceinline__ bool named_sync_or(int id, int count, bool pred) {
-  uint32_t out;
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.red.or.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}"
-      : "=r"(out)
-      : "r"((uint32_t)pred), "r"(id), "r"(count)
-      : "memory");
-  return out != 0;
-}
-
-__global__ void __launch_bounds__(kPThreads, 1) k_level0_f64tc_persistent(
-    const __nv_bfloat16* __restrict__ dig, const int32_t* __restrict__ row_exp, const int32_t* __restrict__ remap0,
-    int32_t n_dom, int N, int nrhs, Levels al, const double* __restrict__ r, int64_t stride,
-    const double* __restrict__ zl, int64_t lstride, double* __restrict__ z, int* __restrict__ flags) {
-  using namespace umma;
-  extern __shared__ unsigned char smem_raw[];
-  const int ld = 3 * N;
-  const uint32_t sbytes = slot_bytes(ld), bb = b_bytes(ld);
-  const uint32_t dig_bytes = (uint32_t)ld * ld * 2;
-  unsigned char* ring = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
-  unsigned char* sBbuf = ring + kRing * sbytes;  // [2][4 pair operands]
-  uint64_t* full = (uint64_t*)(sBbuf + 2 * 4 * bb);
-  uint64_t* empty = full + kRing;
-  uint64_t* bfull = empty + kRing;  // [2]
-  uint64_t* bempty = bfull + 2;     // [2]
-  uint64_t* tfull = bempty + 2;     // [2]
-  uint64_t* tempty = tfull + 2;     // [2]
-  uint64_t* drain = tempty + 2;     // [1]
-  uint32_t* tslot = (uint32_t*)(drain + 1);
-  volatile int* abort_word = (volatile int*)(tslot + 1);
-  int* sexp = (int*)(tslot + 16);  // [2][8]
-  int* snode = sexp + 16;          // [2][32]
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n_local = n_dom > (int)blockIdx.x ? (n_dom - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-
-  if (tid == 0) {
-    for (int s = 0; s < kRing; ++s) mbar_init(&full[s], 1), mbar_init(&empty[s], 1);
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&bfull[b], 1);
-      mbar_init(&bempty[b], 2);  // the MMAs (commit) and the epilogue
-      mbar_init(&tfull[b], 1);
-      mbar_init(&tempty[b], 1);
-    }
-    mbar_init(drain, 1);
-    *abort_word = 0;
-    fence_mbar_init();
-  }
-  if (warp == 0) {
-    tmem_alloc(tslot, 256);
-    tmem_relinquish();
-  }
-  fence_before_sync();
-  __syncthreads();
-  fence_after_sync();
-  const uint32_t tmem = *tslot;
-
-  if (warp == 0) {
-    // ------------------------------------------------------------ producer
-    if (lane == 0) {
-      int seq = 0;
-      for (int n = 0; n < n_local && !*abort_word; ++n) {
-        const __nv_bfloat16* dd = dig + (int64_t)(blockIdx.x + (int64_t)n * gridDim.x) * kDigits * ld * ld;
-        for (int p = 0; p < kDigits; ++p) {
-          const int slot = seq % kRing, use = seq / kRing;
-          if (use > 0 && !mbar_wait(&empty[slot], (uint32_t)(use - 1) & 1u)) {
-            *abort_word = 1;
-            atomicOr(flags, kErrTimeout);
-          }
-          if (*abort_word) break;
-          mbar_arrive_expect_tx(&full[slot], dig_bytes);
-          bulk_g2s(ring + slot * sbytes, dd + (int64_t)p * ld * ld, dig_bytes, &full[slot]);
-          ++seq;
-        }
-      }
-      // every copy issued lands before the CTA can leave (the last use of each slot)
-      for (int s = 0; s < kRing && s < seq; ++s) mbar_wait(&full[s], (uint32_t)((seq - 1 - s) / kRing) & 1u);
-    }
-  } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      const uint32_t lbo = (uint32_t)ld * 16;
-      const uint32_t idesc = idesc_bf16_f32(kM, 64);
-      const uint64_t da0 = smem_desc(smem_u32(ring), lbo, 128);
-      const uint64_t db0 = smem_desc(smem_u32(sBbuf), 1024, 128);
-      const uint64_t da_ks = (2u * lbo) >> 4, db_ks = 2048u >> 4, db_buf = (4u * bb) >> 4;
-      int seq = 0;
-      bool issued = false;
-      for (int n = 0; n < n_local && !*abort_word; ++n) {
-        const int b = n & 1, use = n >> 1;
-        bool ok = (use == 0 || mbar_wait(&tempty[b], (uint32_t)(use - 1) & 1u)) &&
-                  mbar_wait(&bfull[b], (uint32_t)use & 1u);
-        if (ok) {
-          fence_after_sync();
-          const uint32_t tbase = tmem + 128u * b;
-          for (int p = 0; p < kDigits && ok; ++p, ++seq) {
-            const int slot = seq % kRing;
-            if (!mbar_wait(&full[slot], (uint32_t)(seq / kRing) & 1u)) {
-              ok = false;
-              break;
-            }
-            fence_after_sync();
-            const uint64_t da = da0 + ((uint64_t)slot * sbytes >> 4);
-            const uint64_t db = db0 + b * db_buf;
-#pragma unroll 6
-            for (int ks = 0; ks < ld / 16; ++ks)
-              mma_bf16(tbase + 8u * p, da + ks * da_ks, db + ks * db_ks, idesc, (p > 0 || ks > 0) ? 1u : 0u);
-            mma_commit(&empty[slot]);
-            issued = true;
-          }
-        }
-        if (!ok) {
-          *abort_word = 1;
-          atomicOr(flags, kErrTimeout);
-          break;
-        }
-        mma_commit(&tfull[b]);
-        mma_commit(&bempty[b]);
-      }
-      if (issued) {  // every MMA issued finishes before TMEM can be released
-        mma_commit(drain);
-        mbar_wait(drain, 0);
-      }
-    }
-  } else if (warp < 4) {
-    // ------------------------------------------------------------ stagers (64 threads)
-    const int st = tid - 64;
-    for (int n = 0; n < n_local; ++n) {
-      const int b = n & 1, use = n >> 1;
-      const int32_t d = blockIdx.x + n * gridDim.x;
-      bool bad = *abort_word != 0;
-      if (!bad && use > 0 && !mbar_wait(&bempty[b], (uint32_t)(use - 1) & 1u)) {
-        bad = true;
-        *abort_word = 1;
-        atomicOr(flags, kErrTimeout);
-      }
-      if (named_sync_or(1, 64, bad)) break;
-      int* se = sexp + 8 * b;
-      int* sn = snode + 32 * b;
-      if (st < 8) se[st] = 0;
-      if (st < 32) sn[st] = st < N ? remap0[(int64_t)d * N + st] : -1;
-      named_sync(1, 64);
-      constexpr int kSPer = 8 * 128 / 64;
-      double rv[kSPer];
-#pragma unroll
-      for (int m = 0; m < kSPer; ++m) {
-        const int e = st + m * 64;
-        const int k = e / ld, j = e - k * ld;
-        rv[m] = 0.0;
-        if (k < nrhs && k < 8) {
-          const int32_t node = sn[j / 3];
-          if (node >= 0) rv[m] = r[k * stride + 3 * (int64_t)node + j % 3];
-          const int eb = biased_exp(rv[m]);
-          if (eb) atomicMax(&se[k], eb);
-        }
-      }
-      named_sync(1, 64);
-      unsigned char* sB = sBbuf + b * 4 * bb;
-#pragma unroll
-      for (int m = 0; m < kSPer; ++m) {
-        const int e = st + m * 64;
-        if (e >= 8 * ld) break;
-        const int k = e / ld, j = e - k * ld;
-        const long long y = scaled_rint(rv[m], se[k] - 1021);
-        write_digits256_bf16(y, sB + (j >> 3) * 1024 + (j & 7) * 2 + k * 16);
-      }
-      fence_proxy_async();
-      named_sync(1, 64);
-      if (st == 0) mbar_arrive(&bfull[b]);
-    }
-  } else {
-    // ------------------------------------------------------------ epilogue (128 threads)
-    const int q4 = warp & 3;  // TMEM lane quarter
-    const int i_row = q4 * 32 + lane;
-    for (int n = 0; n < n_local; ++n) {
-      const int b = n & 1, use = n >> 1;
-      const int32_t d = blockIdx.x + n * gridDim.x;
-      bool bad = *abort_word != 0;
-      if (!bad && !mbar_wait(&bfull[b], (uint32_t)use & 1u)) {  // this domain's node map and exponents
-        bad = true;
-        *abort_word = 1;
-        atomicOr(flags, kErrTimeout);
-      }
-      if (named_sync_or(2, 128, bad)) break;
-      const int* se = sexp + 8 * b;
-      const int32_t node = i_row < ld ? snode[32 * b + i_row / 3] : -1;
-      int a = -100000;
-      double coarse_sum[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) coarse_sum[k] = 0.0;
-      const int c = i_row % 3;
-      if (node >= 0) {
-        a = row_exp[(int64_t)d * ld + i_row];
-#pragma unroll
-        for (int l = 1; l < 8; ++l) {
-          if (l >= al.L) break;
-          const int64_t item = al.vec_off[l] + al.coarse[l][node];
-#pragma unroll
-          for (int k = 0; k < 8; ++k)
-            if (k < nrhs) {  // the first coarse level assigns: one FP64 add fewer per output
-          const double v = zl[k * lstride + 3 * item + c];
-          coarse_sum[k] = l == 1 ? v : coarse_sum[k] + v;
-        }
-        }
-      }
-      bad = !mbar_wait(&tfull[b], (uint32_t)use & 1u);
-      if (bad) {
-        *abort_word = 1;
-        atomicOr(flags, kErrTimeout);
-      }
-      if (named_sync_or(2, 128, bad)) break;
-      fence_after_sync();
-      if (q4 * 32 < ld) {
-        const uint32_t ta = tmem + 128u * b + ((uint32_t)(q4 * 32) << 16);
-        float g[64];
-        tmem_ld_32x32b_x16(ta + 0, g);
-        tmem_ld_32x32b_x16(ta + 16, g + 16);
-        tmem_ld_32x32b_x16(ta + 32, g + 32);
-        tmem_ld_32x32b_x16(ta + 48, g + 48);
-        if (node >= 0) {
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            if (k >= nrhs) break;
-            double v = 0.0;
-            if (se[k] && a > -100000) {
-              long long hi = 0, lo = 0;
-#pragma unroll
-              for (int s = 0; s < 4; ++s) hi = (hi << 8) + (long long)__float2int_rn(g[8 * s + k]);
-#pragma unroll
-              for (int s = 4; s < 8; ++s) lo = (lo << 8) + (long long)__float2int_rn(g[8 * s + k]);
-              const int e = a + (se[k] - 1021) - 72;
-              if (e < 900) v = scaled_to_double(hi, lo, e);
-            }
-            z[k * stride + 3 * (int64_t)node + c] = v + coarse_sum[k];
-          }
-        }
-      }
-      fence_before_sync();
-      named_sync(2, 128);
-      if (tid == 128) {
-        mbar_arrive(&tempty[b]);
-        mbar_arrive(&bempty[b]);
-      }
-    }
-  }
-  fence_before_sync();
-  __syncthreads();
-  if (warp == 0) {
-    fence_after_sync();
-    tmem_dealloc(tmem, 256);
-  }
-}
-
 }  // namespace f64tc
 
-// GS_TUNE_F64_TC: 1 / 2 / 4 stream the BF16 digit matrices of this file, 3 the
+// GS_TUNE_F64_TC: 1 / 2 / 4 stream the digit bytes of this file, 3 the
 // symmetric digit bytes of mas_apply_f64sym.cu; the storage is made when the
 // preconditioner is built for the value set then.
 bool level0_f64tc_usable(gs_ctx ctx, gs_mas mas, int nrhs) {
@@ -650,7 +411,7 @@ int level0_f64tc_alloc(gs_ctx ctx, gs_mas mas) {
     const size_t n_dom = (size_t)std::max(mas->n_domains[l], 1);
     void* dg = nullptr;
     int32_t* ex = nullptr;
-    GS_TRY(ctx->alloc(&dg, n_dom * f64tc::kDigits * ld * ld * 2));
+    GS_TRY(ctx->alloc(&dg, n_dom * f64tc::kDigits * ld * ld));
     mas->dig64.push_back(dg);
     GS_TRY(ctx->alloc((void**)&ex, n_dom * ld * 4));
     mas->dig64_exp.push_back(ex);
@@ -674,39 +435,39 @@ static f64tc::Levels f64tc_levels(gs_mas mas) {
   return al;
 }
 
-template <bool kCoarse, bool kDot, int kS, int LD, int kT>
+template <bool kCoarse, bool kDot, int kSlots, int kBufs, int kCtas, int LD>
 static int launch_digits(gs_ctx ctx, gs_mas mas, int nrhs, const f64tc::Levels& al, const double* r, int64_t stride,
                          const double* zl, int64_t lstride, double* z, const int* skip, const Partials& dot) {
-  const auto kernel = f64tc::k_level0_f64tc<kCoarse, kDot, kS, LD, kT>;
-  const size_t smem = f64tc::smem_bytes<kS>(LD);
+  const auto kernel = f64tc::k_level0_f64tc<kCoarse, kDot, kSlots, kBufs, kCtas, LD>;
+  const size_t smem = f64tc::ring_bytes(kSlots, LD);
   GS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const int jobs = kCoarse ? mas->n_coarse_jobs : mas->n_domains[0];
   const int32_t* jt = kCoarse ? mas->d_coarse_jobs : nullptr;
-  GS_CUDA(launch_chained(ctx, (int64_t)mas->n * nrhs, kernel, dim3(jobs), dim3(kT), smem, (const __nv_bfloat16* const*)mas->d_dig_tab,
-                         (const int32_t* const*)(mas->d_dig_tab + 8), jt, jt ? jt + jobs : nullptr, mas->remap0, mas->N,
-                         nrhs, al, r, stride, zl, lstride, z, ctx->d_flags, skip, dot));
+  GS_CUDA(launch_chained(ctx, (int64_t)mas->n * nrhs, kernel, dim3(jobs), dim3(f64tc::kThreads), smem,
+                         (const uint8_t* const*)mas->d_dig_tab, (const int32_t* const*)(mas->d_dig_tab + 8), jt,
+                         jt ? jt + jobs : nullptr, mas->remap0, mas->N, nrhs, al, r, stride, zl, lstride, z,
+                         ctx->d_flags, skip, dot));
   return GS_OK;
 }
 
-// Ring slots by the number of domains: where every SM holds one domain at
-// most, all 7 digits are copied at once (133 KB); where it holds two, 4 slots;
-// else 2, so that four CTAs share an SM (3 slots and 3 CTAs: 15 % slower).
+// By the number of domains: where every SM holds one at most, all 7 digits are
+// copied at once and each has its own A operand in TMEM, so that no step waits
+// for an MMA; where it holds two, 3 operands; else one, and a ring of 3 digits,
+// so that four CTAs share an SM.  One operand for the 128 domains of a 16^3 body
+// as well: 6.2 against 5.5 ms for its solve.
 template <bool kCoarse, bool kDot>
 static int launch_digits_shape(gs_ctx ctx, gs_mas mas, int nrhs, const f64tc::Levels& al, const double* r,
                                int64_t stride, const double* zl, int64_t lstride, double* z, const int* skip,
                                const Partials& dot) {
-  const bool wide = ctx->tune[GS_TUNE_F64_TC] == 4;  // 256 threads per domain
-  const int jobs = kCoarse ? mas->n_coarse_jobs : mas->n_domains[0];
-  const int sms = std::max(ctx->sm_count, 1);
-#define GS_DIGITS(S, LD, T) launch_digits<kCoarse, kDot, S, LD, T>(ctx, mas, nrhs, al, r, stride, zl, lstride, z, skip, dot)
+  const int jobs = kCoarse ? mas->n_coarse_jobs : mas->n_domains[0], sms = std::max(ctx->sm_count, 1);
+#define GS_DIGITS(S, B, C, LD) \
+  launch_digits<kCoarse, kDot, S, B, C, LD>(ctx, mas, nrhs, al, r, stride, zl, lstride, z, skip, dot)
   if (mas->N == 32) {  // 3 N = 96 or 48 (the digit storage is made only for N = 32 and 16)
-    if (!wide) return GS_DIGITS(f64tc::kSlots, 96, 128);
-    if (jobs <= sms) return GS_DIGITS(f64tc::kDigits, 96, 256);
-    if (jobs <= 2 * sms) return GS_DIGITS(f64tc::kSlotsFew, 96, 256);
-    return GS_DIGITS(f64tc::kSlots, 96, 256);
+    if (jobs <= sms) return GS_DIGITS(f64tc::kDigits, f64tc::kDigits, 1, 96);
+    if (jobs <= 2 * sms) return GS_DIGITS(f64tc::kDigits, 3, 2, 96);
+    return GS_DIGITS(3, 1, 4, 96);
   }
-  if (!wide) return GS_DIGITS(f64tc::kSlots, 48, 128);
-  return jobs <= 2 * sms ? GS_DIGITS(f64tc::kDigits, 48, 256) : GS_DIGITS(f64tc::kSlots, 48, 256);
+  return jobs <= 2 * sms ? GS_DIGITS(f64tc::kDigits, f64tc::kDigits, 2, 48) : GS_DIGITS(3, 2, 4, 48);
 #undef GS_DIGITS
 }
 
@@ -715,17 +476,6 @@ int level0_f64tc_launch(gs_ctx ctx, gs_mas mas, int nrhs, const double* r, int64
   GS_CHECK(level0_f64tc_usable(ctx, mas, nrhs), GS_ERR_UNSUPPORTED, "FP64 tensor-core apply: not available");
   if (ctx->tune[GS_TUNE_F64_TC] == 3) return f64sym_level0_launch(ctx, mas, nrhs, r, stride, zl, lstride, z, skip);
   if (mas->n_domains[0] == 0) return GS_OK;
-  if (ctx->tune[GS_TUNE_F64_TC] == 2) {  // persistent, warp-specialised: one CTA per SM
-    const size_t psmem = f64tc::psmem_bytes(3 * mas->N);
-    GS_CUDA(cudaFuncSetAttribute(f64tc::k_level0_f64tc_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)psmem));
-    const int grid = std::min<int>(mas->n_domains[0], std::max(ctx->sm_count, 1));
-    f64tc::k_level0_f64tc_persistent<<<grid, f64tc::kPThreads, psmem, ctx->stream>>>(
-        (const __nv_bfloat16*)mas->dig64[0], mas->dig64_exp[0], mas->remap0, mas->n_domains[0], mas->N, nrhs,
-        f64tc_levels(mas), r, stride, zl, lstride, z, ctx->d_flags);
-    GS_CUDA(cudaGetLastError());
-    return GS_OK;
-  }
   return dot ? launch_digits_shape<false, true>(ctx, mas, nrhs, f64tc_levels(mas), r, stride, zl, lstride, z, skip, *dot)
              : launch_digits_shape<false, false>(ctx, mas, nrhs, f64tc_levels(mas), r, stride, zl, lstride, z, skip,
                                                  Partials{});

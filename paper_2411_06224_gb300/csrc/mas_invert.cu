@@ -17,11 +17,9 @@
 // the digit pass now included), 0.28 ms for the 132 domains of a 16^3 body
 // (0.46 + 0.04 ms), where one domain's chain of steps is all there is.
 //
-// The FP64 apply's operand (7 BF16 digit matrices per inverse,
+// The FP64 apply's operand (7 digit bytes per entry of an inverse,
 // mas_apply_f64tc.cu) is cut here from the inverse in shared memory; a
 // separate pass would read the 604 MB of inverses again.
-#include <cuda_bf16.h>
-
 #include <algorithm>
 
 #include "common.cuh"
@@ -38,7 +36,7 @@ constexpr int kMaxRows = 96;  // 3 N, N <= 32
 
 struct Jobs {
   double* mat[8];           // per level: n_domains matrices of 3N x 3N, overwritten by their inverses
-  uint32_t* dig[8];         // per level: digit matrices (pairs of BF16), or null
+  uint8_t* dig[8];          // per level: digit matrices (bytes), or null
   int32_t* dexp[8];         // per level: their row exponents
   int32_t first[9];         // first CTA of each level
   int32_t n_items[8];       // real items per level (l >= 1)
@@ -311,50 +309,51 @@ __global__ void __launch_bounds__(kThreads, 4) k_invert_domains(Jobs jb, const i
   __syncthreads();
 
   // both triangles over the real part of the matrix (a warp per row), and the
-  // row's exponent a: |M_ij| < 2^(a - 1)
-  uint32_t* dig = jb.dig[l];
+  // row's exponent a: |M_ij| < 2^(a - 1), and |M_ij| 2^(56 - a) so far below 2^55
+  // that its leading balanced digit is at most 127 (the bytes hold -128 .. 127):
+  // rows whose largest magnitude has a mantissa of 0xFDFDF.. or more, 1.992 of 2,
+  // take one more
+  uint8_t* dig = jb.dig[l];
   for (int i = wid; i < n3; i += kWarps) {
     const int gi = 3 * s_lane[i / 3] + i % 3;
-    int emax = 0;
+    int top = 0;  // sign-free upper words order like the magnitudes
     for (int j = lane; j < n3; j += 32) {
       const double v = sA[j <= i ? tri(i, j) : tri(j, i)];
       M[(int64_t)gi * ld + 3 * s_lane[j / 3] + j % 3] = v;
-      emax = max(emax, biased_exp(v));
+      top = max(top, __double2hiint(v) & 0x7FFFFFFF);
     }
-    emax = __reduce_max_sync(kFull, emax);
-    if (lane == 0 && emax) s_exp[gi] = emax - 1021;
+    top = __reduce_max_sync(kFull, top);
+    if (lane == 0 && top >> 20) s_exp[gi] = (top >> 20) - 1021 + ((top & 0xFFFFF) >= 0xFDFDF);
   }
   if (!dig) return;
   __syncthreads();
   if (tid < ld) jb.dexp[l][d * ld + tid] = s_exp[tid];
-  // digit matrices in the K-major operand layout [k/8][i/8][i%8][k%8]: tile t
-  // is 128 contiguous bytes per digit, a lane two neighbouring k of one row
+  // digit matrices in the order their rows are loaded (mas_apply_f64tc.cu):
+  // [k/16][i][k%16] bytes; a warp takes 8 rows by 16 columns, 128 contiguous
+  // bytes per digit, a lane four neighbouring columns of a row
   const int G = ld / 8;
-  uint32_t* out = dig + d * kDigits * (ld * ld / 2);
-  for (int t = wid; t < G * G; t += kWarps) {
-    const int gi = 8 * (t % G) + tr, gk = 8 * (t / G) + 2 * tc;
+  uint8_t* out = dig + d * kDigits * (ld * ld);
+  for (int t = wid; t < G * (ld / 16); t += kWarps) {
+    const int gi = 8 * (t % G) + tr, gk = 16 * (t / G) + 4 * tc;
     const int ni = s_pos[gi / 3], a = s_exp[gi];
-    unsigned long long z[2];
+    unsigned long long z[4];  // the digits + 128, one byte each
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < 4; ++h) {
       const int nk = s_pos[(gk + h) / 3];
       long long x = 0;
       if (ni >= 0 && nk >= 0 && a > -100000) {
         const int i = 3 * ni + gi % 3, k = 3 * nk + (gk + h) % 3;
         x = scaled_rint(sA[k <= i ? tri(i, k) : tri(k, i)], a);
       }
-      z[h] = (unsigned long long)(x + 0x808080808080LL);  // 128 in the digits 1..6
+      z[h] = (unsigned long long)x + kBias256;
     }
-    uint32_t* o = out + t * 32 + lane;
+    uint8_t* o = out + ((t / G) * ld + gi) * 16 + 4 * tc;
 #pragma unroll
     for (int p = 0; p < kDigits; ++p) {
       uint32_t w = 0;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int dg = p == 0 ? (int)((long long)z[h] >> 48) : (int)((z[h] >> (8 * (6 - p))) & 255u) - 128;
-        w |= (uint32_t)small_int_bf16_bits(dg) << (16 * h);
-      }
-      o[p * (ld * ld / 2)] = w;
+      for (int h = 0; h < 4; ++h) w |= (uint32_t)((z[h] >> (8 * (6 - p))) & 255u) << (8 * h);
+      *(uint32_t*)(o + p * (ld * ld)) = w;
     }
   }
 }
@@ -370,7 +369,7 @@ int invert_domains_launch(gs_ctx ctx, gs_mas mas, double* fac0) {
   jb.N = mas->N;
   for (int l = 0; l < mas->L; ++l) {
     jb.mat[l] = mas->inv64[l];
-    jb.dig[l] = mas->dig64.empty() ? nullptr : (uint32_t*)mas->dig64[l];
+    jb.dig[l] = mas->dig64.empty() ? nullptr : (uint8_t*)mas->dig64[l];
     jb.dexp[l] = mas->dig64_exp.empty() ? nullptr : mas->dig64_exp[l];
     jb.n_items[l] = mas->n_items[l];
     jb.first[l + 1] = jb.first[l] + mas->n_domains[l];
