@@ -149,15 +149,18 @@ __global__ void __launch_bounds__(kT, kMin) k_pcg_spmv(Sliced A, const int32_t* 
 
 // Lanes per row by size.  The large-system shapes give each lane two
 // right-hand sides and the whole row (64^3, 8 RHS: 0.19 ms; 2 lanes sharing the
-// blocks of 8 RHS: 0.23 ms); systems whose rows do not fill the GPU share a
-// row's blocks among up to 8 lanes.
+// blocks of 8 RHS: 0.23 ms); where the rows do not fill the GPU, 2 or 4 lanes
+// share a row's blocks, and more only shorten the sums of a lane to two blocks.
+// Whole solves with the lanes of this rule / twice as many / half as many: 45^3,
+// 1 RHS (2) 2.87 / - / 3.08 ms; 40^3, 4 RHS (2) 41.8 / - / 42.7; 32^3, 1 RHS,
+// five Newton steps (2) 26.5 / 26.7 / -; 20^3, 2 RHS (4) 13.3 / 14.4 / -.
+// (Loading an entry one ahead of its use: 45^3 2.87 ms as well, 20^3 13.9.)
 template <bool kFF, int kRL, int kR>
 static int launch_spmv(gs_ctx ctx, gs_mat m, const float2* xs, const double* p, double* Ap, int nrhs,
                        const PcgScalars* s, Partials& pap) {
   const Sliced A{m->row_order, m->sl_ptr, m->sl_len, m->sl_col, m->sl_ff, m->sl_f64, m->n};
-  const int64_t fill = (int64_t)std::max(ctx->sm_count, 1) * 1024;
-  int bl = 1;
-  while (bl < 8 && bl * kRL < 32 && (int64_t)m->n * kRL * bl * 2 <= fill) bl *= 2;
+  const int64_t rows = (int64_t)m->n * kRL, sms = std::max(ctx->sm_count, 1);
+  const int bl = rows * 4 <= sms * 512 ? 4 : (rows * 2 <= sms * 2048 ? 2 : 1);
   constexpr int kMin = kFF ? 4 : 3;
   const int64_t chunks = ((int64_t)m->n * kRL * bl + kT - 1) / kT;
   pap.n = (int)std::max<int64_t>(1, std::min<int64_t>({chunks, (int64_t)kMin * std::max(ctx->sm_count, 1),
@@ -170,8 +173,7 @@ static int launch_spmv(gs_ctx ctx, gs_mat m, const float2* xs, const double* p, 
   switch (bl) {
     case 1: e = go(k_pcg_spmv<kFF, 1, kRL, kR, kMin>); break;
     case 2: e = go(k_pcg_spmv<kFF, 2, kRL, kR, kMin>); break;
-    case 4: e = go(k_pcg_spmv<kFF, 4, kRL, kR, kMin>); break;
-    default: e = go(k_pcg_spmv<kFF, 8, kRL, kR, kMin>); break;
+    default: e = go(k_pcg_spmv<kFF, 4, kRL, kR, kMin>); break;
   }
   GS_CUDA(e);
   return GS_OK;
