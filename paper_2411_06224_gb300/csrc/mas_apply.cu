@@ -38,7 +38,11 @@ struct ApplyLevels {
 // trees (FP64 adds are scarce on this part).  Groups are the domain's level-1
 // items; a level-1 item lies inside one item of every coarser level, so its
 // sums serve all levels.  Most domains are one group: then the 32 nodes'
-// values are loaded at once and summed in registers.
+// values are loaded at once and summed in registers.  Few right-hand sides leave
+// lanes over, and an addition costs the FP64 pipe the same for 3 lanes as for
+// 24: with kParts > 1, that many lanes share a value's slots (24 bodies, 188,000
+// block rows, 1 RHS: 19 -> 8 us).  FP64 preconditioners only: the
+// others round the sums to FP32, where the order of the additions would show.
 constexpr int kRestrictWarps = 4;
 // Inverse entries a thread of the dense products loads before it uses them.
 constexpr int kChunk = 16;
@@ -56,6 +60,7 @@ __device__ __forceinline__ float to_tm<float>(double v) {
 __device__ __forceinline__ double to_f64(double v) { return v; }
 __device__ __forceinline__ double to_f64(float v) { return f32_to_f64_bits(v); }
 
+template <int kParts>
 __global__ void __launch_bounds__(32 * kRestrictWarps) k_restrict(const double* __restrict__ r, int64_t stride,
                                                                   int nrhs, const int32_t* __restrict__ remap0,
                                                                   int32_t n_dom0, ApplyLevels al,
@@ -75,8 +80,10 @@ __global__ void __launch_bounds__(32 * kRestrictWarps) k_restrict(const double* 
   const int lead0 = __ffs(realm) - 1;
   const int32_t c_first = __shfl_sync(kFull, c1, lead0);
   const bool one_group = __all_sync(kFull, !real || c1 == c_first);
-  for (int k0 = 0; k0 < nrhs; k0 += 8) {
-    const int k = k0 + lane / 3, c = lane % 3;
+  constexpr int kR = 8 / kParts, kS = 32 / kParts;  // right-hand sides per pass, slots per lane
+  const int part = min(lane / (3 * kR), kParts - 1), kc = lane % (3 * kR), c = kc % 3;
+  for (int k0 = 0; k0 < nrhs; k0 += kR) {
+    const int k = k0 + kc / 3;
     const bool act = lane < 24 && k < nrhs;
     const double* rk = r + k * stride + c;
     uint32_t left = realm;
@@ -87,27 +94,41 @@ __global__ void __launch_bounds__(32 * kRestrictWarps) k_restrict(const double* 
       double sum = 0.0;
       if (one_group) {  // all real slots: loads first, then the sum in slot order
         lead = lead0, cc = c_first, g = realm;
-        double v[32];
+        double v[kS];
 #pragma unroll
-        for (int s = 0; s < 32; ++s) {
-          const int32_t ns = __shfl_sync(kFull, node, s);
+        for (int s = 0; s < kS; ++s) {
+          const int32_t ns = __shfl_sync(kFull, node, part * kS + s);
           v[s] = (act && ns >= 0) ? rk[3 * (int64_t)ns] : 0.0;
         }
 #pragma unroll
-        for (int s = 0; s < 32; ++s)
-          if ((realm >> s) & 1u) sum += v[s];
+        for (int s = 0; s < kS; ++s)
+          if (kParts > 1 || ((realm >> s) & 1u)) sum += v[s];
       } else {
         lead = __ffs(left) - 1;
         cc = __shfl_sync(kFull, c1, lead);
         g = __ballot_sync(kFull, real && c1 == cc);
-        for (uint32_t m = g; m; m &= m - 1) {
-          const int32_t ns = __shfl_sync(kFull, node, __ffs(m) - 1);
-          if (act) sum += rk[3 * (int64_t)ns];
+        const uint32_t mine = kParts == 1 ? g : (g >> (part * kS)) & ((1u << (kS & 31)) - 1u);
+        if (kParts == 1) {
+          for (uint32_t m = mine; m; m &= m - 1) {
+            const int32_t ns = __shfl_sync(kFull, node, __ffs(m) - 1);
+            if (act) sum += rk[3 * (int64_t)ns];
+          }
+        } else {  // lanes have different slots: every lane takes part in every shuffle
+#pragma unroll
+          for (int s = 0; s < kS; ++s) {
+            const int32_t ns = __shfl_sync(kFull, node, part * kS + s);
+            if (act && ((mine >> s) & 1u)) sum += rk[3 * (int64_t)ns];
+          }
         }
+      }
+#pragma unroll
+      for (int h = kParts / 2; h > 0; h /= 2) {
+        const double other = __shfl_down_sync(kFull, sum, h * 3 * kR);
+        if (part < h) sum += other;
       }
       left &= ~g;
       // a level-1 item lies inside this domain: this warp is its only writer
-      if (act) rl[k * lstride + c + 3 * (al.vec_off[1] + cc)] = sum;
+      if (act && (kParts == 1 || lane < 3 * kR)) rl[k * lstride + c + 3 * (al.vec_off[1] + cc)] = sum;
     }
   }
 }
@@ -518,10 +539,23 @@ bool mas_dot_usable(gs_ctx ctx, gs_mas mas, int nrhs) {
   return (t == 1 || t == 4) && level0_f64tc_usable(ctx, mas, nrhs);
 }
 
-// z = M^-1 r and partial sums of r . z (one per domain) from r and its level-1
-// sums (in rl, whose padding entries are zero), for the forms above.
-int mas_products_dot(gs_ctx ctx, gs_mas mas, const double* r, double* z, int nrhs, double* rl, double* zl,
-                     const int* skip, const Partials& dot) {
+// Level-1 sums of r in rl, whose padding entries are zero already.
+int mas_restrict(gs_ctx ctx, gs_mas mas, const double* r, int nrhs, double* rl, const int* skip) {
+  if (mas->L < 2) return GS_OK;
+  GS_PROF(ctx, GS_K_MAS_APPLY_COARSE);
+  const bool f64 = mas->precision == GS_PREC_FP64;
+  const auto kernel = !f64 || nrhs > 4 ? k_restrict<1> : (nrhs > 2 ? k_restrict<2> : (nrhs == 2 ? k_restrict<4> : k_restrict<8>));
+  kernel<<<ceil_div(mas->n_domains[0], kRestrictWarps), 32 * kRestrictWarps, 0, ctx->stream>>>(
+      r, 3LL * mas->n, nrhs, mas->remap0, mas->n_domains[0], apply_levels(mas, false), rl,
+      3 * std::max<int64_t>(mas->vec_items, 1), skip);
+  GS_CUDA(cudaGetLastError());
+  return GS_OK;
+}
+
+// z = M^-1 r from r and its level-1 sums (in rl, whose padding entries are zero),
+// for the forms above; dot (may be null): partial sums of r . z, one per domain.
+int mas_products(gs_ctx ctx, gs_mas mas, const double* r, double* z, int nrhs, double* rl, double* zl, const int* skip,
+                 const Partials* dot) {
   const int64_t stride = 3LL * mas->n, lstride = 3 * std::max<int64_t>(mas->vec_items, 1);
   const bool f32 = mas->precision == GS_PREC_FP32;
   if (mas->L > 1) {
@@ -541,9 +575,11 @@ int mas_products_dot(gs_ctx ctx, gs_mas mas, const double* r, double* z, int nrh
       GS_TRY(coarse_f64tc_launch(ctx, mas, nrhs, rl, zl, lstride, skip, from_kids));
     }
   }
-  if (f32) return level0_f32_launch<true>(ctx, mas, r, z, nrhs, zl, lstride, skip, dot);
+  if (f32)
+    return dot ? level0_f32_launch<true>(ctx, mas, r, z, nrhs, zl, lstride, skip, *dot)
+               : level0_f32_launch<false>(ctx, mas, r, z, nrhs, zl, lstride, skip, Partials{});
   GS_PROF(ctx, GS_K_MAS_APPLY_L0);
-  return level0_f64tc_launch(ctx, mas, nrhs, r, stride, zl, lstride, z, skip, &dot);
+  return level0_f64tc_launch(ctx, mas, nrhs, r, stride, zl, lstride, z, skip, dot);
 }
 
 template <typename Ts, typename Tm>
@@ -561,8 +597,7 @@ static int launch_apply(gs_ctx ctx, gs_mas mas, const Ts* const* d_inv, const in
   GS_CHECK(threads <= 1024, GS_ERR_UNSUPPORTED, "mas apply: too many right-hand sides (%d)", nrhs);
   if (mas->L > 1) {
     GS_CUDA(cudaMemsetAsync(rl, 0, (size_t)nrhs * lstride * sizeof(double), st));
-    { GS_PROF(ctx, GS_K_MAS_APPLY_COARSE); k_restrict<<<ceil_div(mas->n_domains[0], kRestrictWarps), 32 * kRestrictWarps, 0, st>>>(r, stride, nrhs, mas->remap0,
-                                                                              mas->n_domains[0], al, rl, lstride, skip); }
+    GS_TRY(mas_restrict(ctx, mas, r, nrhs, rl, skip));
     for (int l = 1; l + 1 < mas->L; ++l) {  // levels >= 2 from the level below, in a fixed order
       GS_PROF(ctx, GS_K_MAS_APPLY_COARSE);
       k_restrict_up<double, LevelIdxRhsMajor><<<ceil_div((int64_t)mas->n_domains[l] * 32, 128), 128, 0, st>>>(

@@ -41,8 +41,8 @@ int pcg_update_xr(gs_ctx ctx, gs_mas mas, double* x, double* r, const double* p,
 int pcg_update_p(gs_ctx ctx, gs_mat m, double* p, const double* z, float2* ps, int nrhs, PcgScalars* s,
                  const Partials& rrp, const Partials& rzp, Partials fold, double tol2, int parity);
 bool mas_dot_usable(gs_ctx ctx, gs_mas mas, int nrhs);
-int mas_products_dot(gs_ctx ctx, gs_mas mas, const double* r, double* z, int nrhs, double* rl, double* zl,
-                     const int* skip, const Partials& dot);
+int mas_products(gs_ctx ctx, gs_mas mas, const double* r, double* z, int nrhs, double* rl, double* zl, const int* skip,
+                 const Partials* dot);
 
 constexpr int kRedThreads = 256;
 constexpr int kMaxChunks = 256;     // reduction blocks per right-hand side of the kernels here
@@ -338,7 +338,7 @@ extern "C" int gs_pcg_solve(gs_ctx ctx, gs_mat mat, gs_mas mas, const double* b,
     }
     if (fused_mas) {
       rzp.n = mas->n_domains[0];
-      GS_TRY(mas_products_dot(ctx, mas, r, z, nrhs, rl, zl, &s->all_conv, rzp));
+      GS_TRY(mas_products(ctx, mas, r, z, nrhs, rl, zl, &s->all_conv, &rzp));
     } else {
       GS_TRY(mas_apply_launch_skip(ctx, mas, r, z, nrhs, rl, zl, &s->all_conv));
       GS_PROF(ctx, GS_K_PCG_VECTOR);
