@@ -472,10 +472,12 @@ int pcg_update_p(gs_ctx ctx, gs_mat m, double* p, const double* z, float2* ps, i
     rz = fold;
     rz.n = kFold;
   }
-  // about eight blocks per SM over all right-hand sides: each first adds the
-  // partial sums
+  // blocks per SM over all right-hand sides: each first adds the partial sums,
+  // so few and long ones where there is much to do (64^3, 8 RHS, 24 iterations:
+  // 2 per SM 13.5 ms, 4 13.1, 6 and 8 13.4, 24 13.8), and eight where the chain of
+  // loads of a block is all there is (40^3, 4 RHS: 8 40.8 ms, 4 41.3)
   const int gx = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(len, kT * 4),
-                                                             (8LL * std::max(ctx->sm_count, 1) + nrhs - 1) / nrhs));
+                                                             ((work > kSmallWork ? 4LL : 8LL) * std::max(ctx->sm_count, 1) + nrhs - 1) / nrhs));
   GS_CUDA(launch_chained(ctx, work, ps ? k_pcg_p<true> : k_pcg_p<false>, dim3(gx, nrhs), dim3(kT), 0, p, z, ps,
                          ps ? m->ff_k : nullptr, len, nrhs, s, rrp, rz, tol2, parity));
   return GS_OK;
