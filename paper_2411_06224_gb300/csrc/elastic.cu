@@ -97,19 +97,36 @@ namespace fem {
 // With th = (A_qq - A_pp) / 2 the rotation tangent is the smaller root of
 // t^2 + 2 (th / A_pq) t - 1 = 0, written as sgn(th) A_pq / (|th| + hypot(th, A_pq))
 // (one division, no overflow of th / A_pq); c = 1 / sqrt(1 + t^2), s = t c.
+// Small angles, |A_pq| <= 2^-20 |th|: t = A_pq / (2 th) to 2^-22, which leaves
+// 2^-22 of A_pq (kept), and c = 1 - t^2 / 2; a third of the FP64 instructions.
+__device__ __forceinline__ int exponent_field(double v) { return (__double2hiint(v) >> 20) & 0x7FF; }
+__device__ __forceinline__ float leading_bits(double v) {  // sign and leading bits, magnitude in [1, 2)
+  const int hi = __double2hiint(v);
+  return __int_as_float((hi & 0x80000000) | 0x3F800000 | ((hi & 0xFFFFF) << 3) | ((uint32_t)__double2loint(v) >> 29));
+}
 template <int p, int q>
 __device__ __forceinline__ void jacobi_rotate(double (&A)[3][3], double (&Q)[3][3]) {
   constexpr int r = 3 - p - q;
   const double apq = A[p][q];
   const double th = 0.5 * (A[q][q] - A[p][p]);
-  const double h = sqrt(th * th + apq * apq);
-  if (apq == 0.0 || h == 0.0) return;
-  const double t = (th >= 0.0 ? apq : -apq) / (fabs(th) + h);
-  const double c = rsqrt(1.0 + t * t);
+  double t, c, rest = 0.0;
+  if (fabs(apq) <= 0x1p-20 * fabs(th) && exponent_field(th) > 0) {
+    // the quotient of the leading 24 bits, exponents apart
+    const int de = exponent_field(apq) - exponent_field(th);
+    if (apq == 0.0 || de < -120) return;  // turns by less than 2^-120
+    t = (double)(__fdividef(leading_bits(apq), leading_bits(th)) * __int_as_float((126 + de) << 23));
+    c = fma(-0.5 * t, t, 1.0);
+    rest = fma(-2.0 * t, th, apq);
+  } else {
+    const double h = sqrt(th * th + apq * apq);
+    if (apq == 0.0 || h == 0.0) return;
+    t = (th >= 0.0 ? apq : -apq) / (fabs(th) + h);
+    c = rsqrt(1.0 + t * t);
+  }
   const double s = t * c;
   A[p][p] -= t * apq;
   A[q][q] += t * apq;
-  A[p][q] = A[q][p] = 0.0;
+  A[p][q] = A[q][p] = rest;
   const double arp = A[r][p], arq = A[r][q];
   A[r][p] = A[p][r] = c * arp - s * arq;
   A[r][q] = A[q][r] = s * arp + c * arq;
@@ -121,12 +138,84 @@ __device__ __forceinline__ void jacobi_rotate(double (&A)[3][3], double (&Q)[3][
   }
 }
 
-// Symmetric A = Q diag(A) Q^T on return (A diagonal, Q orthogonal).
+// The same in FP32, the rotations gathered in a quaternion h = (w, x, y, z),
+// Q = R(h): J turns about axis r by the angle of (c, s), backwards for (0, 1) and
+// (1, 2).
+template <int p, int q>
+__device__ __forceinline__ void jacobi_rotate_start(float (&a)[3][3], float (&h)[4]) {
+  constexpr int r = 3 - p - q, r1 = (r + 1) % 3, r2 = (r + 2) % 3;
+  const float apq = a[p][q], th = 0.5f * (a[q][q] - a[p][p]);
+  const float hyp = sqrtf(th * th + apq * apq);
+  if (!(hyp > 0.0f)) return;
+  const float t = __fdividef(th >= 0.0f ? apq : -apq, fabsf(th) + hyp);
+  const float c = rsqrtf(1.0f + t * t), s = t * c;
+  a[p][p] -= t * apq;
+  a[q][q] += t * apq;
+  a[p][q] = a[q][p] = 0.0f;
+  const float arp = a[r][p], arq = a[r][q];
+  a[r][p] = a[p][r] = c * arp - s * arq;
+  a[r][q] = a[q][r] = s * arp + c * arq;
+  const float ch = sqrtf(0.5f + 0.5f * c);  // |t| <= 1: c >= 0.7
+  const float sh = (r == 1 ? 0.5f : -0.5f) * __fdividef(s, ch);
+  const float w = h[0], vr = h[1 + r], v1 = h[1 + r1], v2 = h[1 + r2];
+  h[0] = w * ch - vr * sh;
+  h[1 + r] = vr * ch + w * sh;
+  h[1 + r1] = v1 * ch + v2 * sh;
+  h[1 + r2] = v2 * ch - v1 * sh;
+}
+
+// Symmetric A = Q diag(A) Q^T on return (A diagonal, Q orthogonal).  Cyclic
+// Jacobi to 1e-17 of the diagonal, begun in FP32: FP64 instructions are what
+// bounds the element kernels, and four of the five sweeps only find an angle.
+// Four FP32 sweeps of A less its mean diagonal give a rotation to about 2^-22,
+// its quaternion is normalised in FP64, and what is left of R^T A R takes one
+// or two FP64 sweeps at small angles.  k_element_hessians, 178,000 tets: 627 us
+// with all sweeps in FP64 and the 3x3 block always decomposed, 400 now.
 __device__ __forceinline__ void sym_eig3(double (&A)[3][3], double (&Q)[3][3]) {
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j) Q[i][j] = i == j ? 1.0 : 0.0;
+  const double mean = (A[0][0] + A[1][1] + A[2][2]) * (1.0 / 3.0);
+  const double d[6] = {A[0][0] - mean, A[1][1] - mean, A[2][2] - mean, A[0][1], A[0][2], A[1][2]};
+  int top = 0;  // the largest exponent field
+#pragma unroll
+  for (int i = 0; i < 6; ++i) top = max(top, (__double2hiint(d[i]) & 0x7FFFFFFF) >> 20);
+  if (top > 100 && top < 2000) {
+    float f[6], a[3][3], h[4] = {1.0f, 0.0f, 0.0f, 0.0f};
+    const double scale = __hiloint2double((2046 - top) << 20, 0);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) f[i] = (float)(d[i] * scale);
+    a[0][0] = f[0], a[1][1] = f[1], a[2][2] = f[2];
+    a[0][1] = a[1][0] = f[3], a[0][2] = a[2][0] = f[4], a[1][2] = a[2][1] = f[5];
+#pragma unroll 1
+    for (int sweep = 0; sweep < 4; ++sweep) {
+      jacobi_rotate_start<0, 1>(a, h);
+      jacobi_rotate_start<0, 2>(a, h);
+      jacobi_rotate_start<1, 2>(a, h);
+    }
+    const double w = h[0], x = h[1], y = h[2], z = h[3];
+    const double over = fma(w, w, fma(x, x, fma(y, y, fma(z, z, -1.0))));  // |h|^2 - 1, about 1e-6
+    if (fabs(over) < 1e-5) {
+      const double k = 2.0 * (1.0 - over) * fma(over, over, 1.0);  // 2 / |h|^2 to over^4
+      const double kx = k * x, ky = k * y, kz = k * z;
+      const double xx = kx * x, yy = ky * y, zz = kz * z, xy = kx * y, xz = kx * z, yz = ky * z;
+      const double wx = kx * w, wy = ky * w, wz = kz * w;
+      Q[0][0] = 1.0 - (yy + zz), Q[0][1] = xy - wz, Q[0][2] = xz + wy;
+      Q[1][0] = xy + wz, Q[1][1] = 1.0 - (xx + zz), Q[1][2] = yz - wx;
+      Q[2][0] = xz - wy, Q[2][1] = yz + wx, Q[2][2] = 1.0 - (xx + yy);
+      double M[3][3];  // A Q
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) M[i][j] = A[i][0] * Q[0][j] + A[i][1] * Q[1][j] + A[i][2] * Q[2][j];
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = i; j < 3; ++j) A[i][j] = A[j][i] = Q[0][i] * M[0][j] + Q[1][i] * M[1][j] + Q[2][i] * M[2][j];
+    }
+  }
+#pragma unroll 1
   for (int sweep = 0; sweep < 16; ++sweep) {
     const double off = A[0][1] * A[0][1] + A[0][2] * A[0][2] + A[1][2] * A[1][2];
     const double dg = A[0][0] * A[0][0] + A[1][1] * A[1][1] + A[2][2] * A[2][2];
@@ -373,14 +462,25 @@ __global__ void __launch_bounds__(128) k_element_hessians(const double* __restri
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j) As[i][j] = lam * g[i] * g[j] + (i == j ? mu : c1 * s[3 - i - j]);
-  sym_eig3(As, Es);
+  // definite already (its leading minors are positive): nothing to project
+  const double m2 = As[0][0] * As[1][1] - As[0][1] * As[0][1];
+  const double m3 = As[2][2] * m2 - As[0][0] * As[1][2] * As[1][2] +
+                    As[0][2] * (2.0 * As[0][1] * As[1][2] - As[1][1] * As[0][2]);
   double Ps[3][3];
+  if (As[0][0] > 0.0 && m2 > 0.0 && m3 > 0.0) {
 #pragma unroll
-  for (int i = 0; i < 3; ++i)
+    for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j)
-      Ps[i][j] = pos(As[0][0]) * Es[i][0] * Es[j][0] + pos(As[1][1]) * Es[i][1] * Es[j][1] +
-                 pos(As[2][2]) * Es[i][2] * Es[j][2];
+      for (int j = 0; j < 3; ++j) Ps[i][j] = As[i][j];
+  } else {
+    sym_eig3(As, Es);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        Ps[i][j] = pos(As[0][0]) * Es[i][0] * Es[j][0] + pos(As[1][1]) * Es[i][1] * Es[j][1] +
+                   pos(As[2][2]) * Es[i][2] * Es[j][2];
+  }
   // 2x2 blocks: pair (i, j) = (1, 2), (0, 2), (0, 1) for k = 0, 1, 2
   double dk[3], ok[3];
 #pragma unroll
