@@ -113,11 +113,18 @@ __global__ void __launch_bounds__(kThreads, kCtas) k_level0_f64tc(
   const int lvl = kCoarse ? job_level[blockIdx.x] : 0;
   const int32_t d = kCoarse ? job_dom[blockIdx.x] : (int32_t)blockIdx.x;
   const uint8_t* dd = dig_tab[lvl] + (int64_t)d * kDigits * LD * LD;
-  int32_t node_of[kPer];  // nodes of this thread's entries of r
+  int32_t node_of[kPer];  // nodes of this thread's entries of r; coarse: their children's lane masks
+  int32_t first_of[kPer];
 #pragma unroll
   for (int m = 0; m < kPer; ++m) {
     const int e = tid + m * kThreads;
-    node_of[m] = kCoarse ? 0 : (e / ld < nrhs && e < 8 * ld ? remap0[(int64_t)d * N + e % ld / 3] : -1);
+    const bool in = e / ld < nrhs && e < 8 * ld;
+    node_of[m] = kCoarse ? 0 : (in ? remap0[(int64_t)d * N + e % ld / 3] : -1);
+    first_of[m] = 0;
+    if (kCoarse && in && al.kids[lvl]) {
+      const int2 kid = al.kids[lvl][(int64_t)d * N + e % ld / 3];
+      first_of[m] = kid.x, node_of[m] = kid.y;
+    }
   }
   const int32_t my_node = kCoarse ? 0 : remap0[(int64_t)d * N + min(lane, N - 1)];
   if (skip && *skip) return;  // whole CTA, before any barrier or TMEM use
@@ -192,9 +199,8 @@ __global__ void __launch_bounds__(kThreads, kCtas) k_level0_f64tc(
     if (k < nrhs && k < 8) {
       if (kCoarse) {
         if (al.kids[lvl]) {
-          const int2 kid = al.kids[lvl][(int64_t)d * N + j / 3];
-          const double* rk = r + k * lstride + 3 * (al.vec_off[lvl - 1] + kid.x) + j % 3;
-          rv[m] = sum_children(rk, (uint32_t)kid.y);
+          const double* rk = r + k * lstride + 3 * (al.vec_off[lvl - 1] + first_of[m]) + j % 3;
+          rv[m] = sum_children(rk, (uint32_t)node_of[m]);
         } else {
           rv[m] = r[k * lstride + cbase + j];
         }

@@ -45,8 +45,6 @@ __global__ void __launch_bounds__(kT, kMin) k_pcg_spmv(Sliced A, const int32_t* 
                                                        const float2* __restrict__ xs, const double* __restrict__ p,
                                                        double* __restrict__ Ap, int64_t stride, int nrhs,
                                                        const PcgScalars* __restrict__ s, Partials pap) {
-  wait_for_previous_kernel();
-  if (s->all_conv) return;
   constexpr int G = kBL * kRL;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = lane % G;
   const int bl = sub % kBL, r0 = sub / kBL * kR;
@@ -60,20 +58,29 @@ __global__ void __launch_bounds__(kT, kMin) k_pcg_spmv(Sliced A, const int32_t* 
   // (rows are ordered by length within windows: the same place would always
   // meet the same lengths)
   const int64_t rounds = (chunks + gridDim.x - 1) / gridDim.x;
-  for (int64_t i = 0; i < rounds; ++i) {
+  int32_t len, row, next;
+  int64_t base;  // entry 0 of the row
+  auto open_row = [&](int64_t i) {
     const int64_t c = i * gridDim.x + (blockIdx.x + i * 37) % gridDim.x;
-    if (c >= chunks) continue;  // whole block
     const int64_t slot = c * (kT / G) + threadIdx.x / G;
-    const bool in = slot < A.n && nh > 0;
-    const int32_t len = in ? A.len[slot] : 0;
-    const int64_t base = in ? (int64_t)A.ptr[slot >> 5] * 32 + (slot & 31) : 0;  // entry 0 of the row
-    const int32_t row = in ? A.row_order[slot] : 0;
-    int32_t next = bl < len ? A.col[base + 32 * bl] : 0;
+    const bool in = c < chunks && slot < A.n && nh > 0;
+    len = in ? A.len[slot] : 0;
+    base = in ? (int64_t)A.ptr[slot >> 5] * 32 + (slot & 31) : 0;
+    row = in ? A.row_order[slot] : -1;
+    next = bl < len ? A.col[base + 32 * bl] : 0;
+  };
+  open_row(0);  // the matrix is older than the kernel before
+  wait_for_previous_kernel();
+  if (s->all_conv) return;
+  for (int64_t i = 0; i < rounds; ++i) {
+    if (i > 0) open_row(i);
+    const bool in = row >= 0;
+    const int32_t lane_slot = (int32_t)(base & 31);
     double y[kR * 3];
     if (kFF) {
       FFSum<kR * 3> acc;
       acc.clear();
-      const float2* v = A.ff + (base - (slot & 31)) * 9 + (slot & 31);
+      const float2* v = A.ff + (base - lane_slot) * 9 + lane_slot;
       for (int32_t e = bl; e < len; e += kBL) {
         const int32_t col = next;
         if (e + kBL < len) next = A.col[base + 32 * (int64_t)(e + kBL)];
@@ -95,7 +102,7 @@ __global__ void __launch_bounds__(kT, kMin) k_pcg_spmv(Sliced A, const int32_t* 
     } else {
 #pragma unroll
       for (int q = 0; q < kR * 3; ++q) y[q] = 0.0;
-      const double* v = A.f64 + (base - (slot & 31)) * 9 + (slot & 31);
+      const double* v = A.f64 + (base - lane_slot) * 9 + lane_slot;
       for (int32_t e = bl; e < len; e += kBL) {
         const int32_t col = next;
         if (e + kBL < len) next = A.col[base + 32 * (int64_t)(e + kBL)];
