@@ -52,6 +52,20 @@ __device__ __forceinline__ void write_digits256_f16(long long y, unsigned char* 
   *(uint16_t*)(col + 7 * 128) = 0;
 }
 
+// Byte p (0: the most significant of 7) of four integers as one word, z0's lowest.
+__device__ __forceinline__ void bytes_of_four(const unsigned long long (&z)[4], uint32_t (&w)[7]) {
+  const uint32_t l0 = (uint32_t)z[0], l1 = (uint32_t)z[1], l2 = (uint32_t)z[2], l3 = (uint32_t)z[3];
+  const uint32_t h0 = (uint32_t)(z[0] >> 32), h1 = (uint32_t)(z[1] >> 32), h2 = (uint32_t)(z[2] >> 32),
+                 h3 = (uint32_t)(z[3] >> 32);
+  const uint32_t a = __byte_perm(l0, l1, 0x5140), b = __byte_perm(l2, l3, 0x5140);  // bytes 0, 0', 1, 1'
+  const uint32_t c = __byte_perm(l0, l1, 0x7362), d = __byte_perm(l2, l3, 0x7362);  // bytes 2, 2', 3, 3'
+  const uint32_t e = __byte_perm(h0, h1, 0x5140), f = __byte_perm(h2, h3, 0x5140);
+  w[6] = __byte_perm(a, b, 0x5410), w[5] = __byte_perm(a, b, 0x7632);
+  w[4] = __byte_perm(c, d, 0x5410), w[3] = __byte_perm(c, d, 0x7632);
+  w[2] = __byte_perm(e, f, 0x5410), w[1] = __byte_perm(e, f, 0x7632);
+  w[0] = __byte_perm(__byte_perm(h0, h1, 0x0062), __byte_perm(h2, h3, 0x0062), 0x5410);
+}
+
 // Four digit bytes (digit + 128 each) as two F16 pairs.
 __device__ __forceinline__ void expand_digit_bytes(uint32_t w, uint32_t& d01, uint32_t& d23) {
   const uint32_t off = 0x64806480u;

@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(kThreads) k_level0_tc(const __nv_bfloat16* __r
     if (mbar_wait(&bars[0], 0)) {
       fence_after_sync();
       for (int s = 0; s < ld / 16; ++s)
-        mma_bf16(tmem, smem_desc(a0 + 2u * s * lbo_a, lbo_a, 128), smem_desc(b0 + 512u * s, 256, 128), idesc1,
+        mma_f16(tmem, smem_desc(a0 + 2u * s * lbo_a, lbo_a, 128), smem_desc(b0 + 512u * s, 256, 128), idesc1,
                  s > 0 ? 1u : 0u);
       mma_commit(&bars[1]);
     } else {
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(kThreads) k_level0_tc(const __nv_bfloat16* __r
       // K-direction step between core matrices (128 bytes) and its stride
       // offset the M-direction step (ld*16 bytes), as for K-major operands
       for (int s = 0; s < ld / 16; ++s)
-        mma_bf16(tmem + 16, smem_desc(a0 + 256u * s, 128, lbo_a), smem_desc(b0 + 512u * s, 256, 128), idesc2,
+        mma_f16(tmem + 16, smem_desc(a0 + 256u * s, 128, lbo_a), smem_desc(b0 + 512u * s, 256, 128), idesc2,
                  s > 0 ? 1u : 0u);
       mma_commit(&bars[2]);
     } else {

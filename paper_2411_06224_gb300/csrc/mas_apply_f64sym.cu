@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(kThreads) k_f64sym(const uint8_t* const* __res
       const uint64_t db0 = smem_desc(smem_u32(sB), 1024, 128);
 #pragma unroll
       for (int ks = 0; ks < ld / 16; ++ks)
-        mma_bf16(tmem + 8u * p, da + ((uint64_t)ks * 2u * lbo >> 4), db0 + ((uint64_t)ks * 2048u >> 4), idesc,
+        mma_f16(tmem + 8u * p, da + ((uint64_t)ks * 2u * lbo >> 4), db0 + ((uint64_t)ks * 2048u >> 4), idesc,
                  (p > 0 || ks > 0) ? 1u : 0u);
       mma_commit(&aempty[as]);
     }

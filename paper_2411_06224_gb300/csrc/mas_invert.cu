@@ -1,47 +1,40 @@
-// Domain inverses of the MAS preconditioner (Alg. 1 "invert unpadded parts")
-// and their digit matrices, one CTA per domain of every level.
+// Domain inverses of the MAS preconditioner (Alg. 1 "invert unpadded parts"),
+// one CTA per domain of every level.
 //
 // The real part of a domain matrix (3k x 3k, 3k <= 96) is factorised in
-// shared memory (Cholesky, FP64), the factor inverted, and W^T W = L^-T L^-1
-// written over the matrix.  Rows beyond 3k up to the next multiple of 8 hold
-// the identity, so every step works on whole 8 x 8 tiles.
+// shared memory (Cholesky, FP64) and the factor inverted, W = L^-1.  For domains
+// of 16 and 32 nodes W is written over the matrix and mas_square.cu forms W^T W =
+// M^-1 on the tensor cores; for other sizes W^T W is formed here.  Rows beyond 3k
+// up to the next multiple of 8 hold the identity, so every step works on whole 8 x
+// 8 tiles.
 //
-// What bounds it: FP64 arithmetic, 3 (3k)^3 / 6 FMA per domain at 2 per clock
-// and SM (5.9 ms for the 8,456 domains of a 64^3 body), where an instruction
-// costs its 16 cycles however few lanes take part.  So the three products run
-// on tiles whose 32 lanes all work (lane (r, c) owns entries (r, c) and
-// (r, c + 4)), with a few block barriers per 8 columns instead of three per
-// column; square roots and reciprocals, 96 one-lane chains of a library
-// division and square root before, are one chain of a few FMA per column.
-// Measured: 8.43 ms on that body (11.77 ms column by column, plus 1.62 ms for
-// the digit pass now included), 0.28 ms for the 132 domains of a 16^3 body
-// (0.46 + 0.04 ms), where one domain's chain of steps is all there is.
-//
-// The FP64 apply's operand (7 digit bytes per entry of an inverse,
-// mas_apply_f64tc.cu) is cut here from the inverse in shared memory; a
-// separate pass would read the 604 MB of inverses again.
+// What bounds it: FP64 arithmetic, (3k)^3 / 6 FMA per domain and product at 2 per
+// clock and SM (4.0 ms for the two products and the 8,456 domains of a 64^3 body),
+// where an instruction costs its 16 cycles however few lanes take part.  So the
+// products run on tiles whose 32 lanes all work (lane (r, c) owns entries (r, c)
+// and (r, c + 4)), with a few block barriers per 8 columns instead of three per
+// column; square roots and reciprocals, 96 one-lane chains of a library division
+// and square root before, are one chain of a few FMA per column.  Measured on the
+// 1,060 domains of a 32^3 body: 0.78 ms (all three products 1.10, column by column
+// and with a separate digit pass 1.72 + 0.09).
 #include <algorithm>
 
 #include "common.cuh"
 #include "fp64split.cuh"
 #include "primitives.cuh"
+#include "square.cuh"
 
 namespace gs {
+
+int square_factors_launch(gs_ctx ctx, const square::Jobs& jb, int N, const int32_t* remap0);
+
 namespace invert {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kDigits = 7;
 constexpr int kMaxRows = 96;  // 3 N, N <= 32
 
-struct Jobs {
-  double* mat[8];           // per level: n_domains matrices of 3N x 3N, overwritten by their inverses
-  uint8_t* dig[8];          // per level: digit matrices (bytes), or null
-  int32_t* dexp[8];         // per level: their row exponents
-  int32_t first[9];         // first CTA of each level
-  int32_t n_items[8];       // real items per level (l >= 1)
-  int L, N;
-};
+using square::Jobs;
 
 __device__ __forceinline__ int tri(int i, int j) { return i * (i + 1) / 2 + j; }
 
@@ -75,13 +68,13 @@ __device__ __forceinline__ void sqrt_and_inverse(double d, double& root, double&
   inv = scale_exp(y, -k);
 }
 
+// kSquare: the inverses; else the factors W, packed by rows in the matrices' place.
+template <bool kSquare>
 __global__ void __launch_bounds__(kThreads, 4) k_invert_domains(Jobs jb, const int32_t* __restrict__ remap0,
                                                                 int* __restrict__ flags, double* __restrict__ fac0) {
   extern __shared__ double sA[];  // lower triangle packed by rows: (i, j), j <= i, at i (i + 1) / 2 + j
   __shared__ double s_inv[kMaxRows];  // 1 / L_ii
-  __shared__ int s_exp[kMaxRows];     // digit exponent of every row of the full domain
   __shared__ int s_lane[32];          // compacted node -> lane of the domain
-  __shared__ int s_pos[32];           // lane -> compacted node, -1: padding
   __shared__ int s_k, s_bad;
   const int job = blockIdx.x;
   int l = 0;
@@ -96,10 +89,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_invert_domains(Jobs jb, const i
     const uint32_t rm = __ballot_sync(kFull, real);
     const int pos = __popc(rm & ((1u << tid) - 1u));
     if (real) s_lane[pos] = tid;
-    s_pos[tid] = real ? pos : -1;
     if (tid == 0) s_k = __popc(rm), s_bad = 0;
   }
-  if (tid < kMaxRows) s_exp[tid] = -100000;
   __syncthreads();
   const int n3 = 3 * s_k, nb = (n3 + 7) / 8, np = 8 * nb;
   for (int i = wid; i < np; i += kWarps) {
@@ -257,6 +248,11 @@ __global__ void __launch_bounds__(kThreads, 4) k_invert_domains(Jobs jb, const i
     }
   }
 
+  if (!kSquare) {
+    for (int i = tid; i < np * (np + 1) / 2; i += kThreads) M[i] = sA[i];
+    return;
+  }
+
   // Inverse = W^T W, lower triangle, in place.  Tile (I, J) reads rows
   // 8 I .. of W, so the row blocks 0..7 can be overwritten before the tiles of
   // the last row blocks are formed; each warp holds its tiles of one half in
@@ -308,53 +304,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_invert_domains(Jobs jb, const i
   }
   __syncthreads();
 
-  // both triangles over the real part of the matrix (a warp per row), and the
-  // row's exponent a: |M_ij| < 2^(a - 1), and |M_ij| 2^(56 - a) so far below 2^55
-  // that its leading balanced digit is at most 127 (the bytes hold -128 .. 127):
-  // rows whose largest magnitude has a mantissa of 0xFDFDF.. or more, 1.992 of 2,
-  // take one more
-  uint8_t* dig = jb.dig[l];
+  // both triangles over the real part of the matrix (a warp per row)
   for (int i = wid; i < n3; i += kWarps) {
     const int gi = 3 * s_lane[i / 3] + i % 3;
-    int top = 0;  // sign-free upper words order like the magnitudes
-    for (int j = lane; j < n3; j += 32) {
-      const double v = sA[j <= i ? tri(i, j) : tri(j, i)];
-      M[(int64_t)gi * ld + 3 * s_lane[j / 3] + j % 3] = v;
-      top = max(top, __double2hiint(v) & 0x7FFFFFFF);
-    }
-    top = __reduce_max_sync(kFull, top);
-    if (lane == 0 && top >> 20) s_exp[gi] = (top >> 20) - 1021 + ((top & 0xFFFFF) >= 0xFDFDF);
-  }
-  if (!dig) return;
-  __syncthreads();
-  if (tid < ld) jb.dexp[l][d * ld + tid] = s_exp[tid];
-  // digit matrices in the order their rows are loaded (mas_apply_f64tc.cu):
-  // [k/16][i][k%16] bytes; a warp takes 8 rows by 16 columns, 128 contiguous
-  // bytes per digit, a lane four neighbouring columns of a row
-  const int G = ld / 8;
-  uint8_t* out = dig + d * kDigits * (ld * ld);
-  for (int t = wid; t < G * (ld / 16); t += kWarps) {
-    const int gi = 8 * (t % G) + tr, gk = 16 * (t / G) + 4 * tc;
-    const int ni = s_pos[gi / 3], a = s_exp[gi];
-    unsigned long long z[4];  // the digits + 128, one byte each
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      const int nk = s_pos[(gk + h) / 3];
-      long long x = 0;
-      if (ni >= 0 && nk >= 0 && a > -100000) {
-        const int i = 3 * ni + gi % 3, k = 3 * nk + (gk + h) % 3;
-        x = scaled_rint(sA[k <= i ? tri(i, k) : tri(k, i)], a);
-      }
-      z[h] = (unsigned long long)x + kBias256;
-    }
-    uint8_t* o = out + ((t / G) * ld + gi) * 16 + 4 * tc;
-#pragma unroll
-    for (int p = 0; p < kDigits; ++p) {
-      uint32_t w = 0;
-#pragma unroll
-      for (int h = 0; h < 4; ++h) w |= (uint32_t)((z[h] >> (8 * (6 - p))) & 255u) << (8 * h);
-      *(uint32_t*)(o + p * (ld * ld)) = w;
-    }
+    for (int j = lane; j < n3; j += 32) M[(int64_t)gi * ld + 3 * s_lane[j / 3] + j % 3] = sA[j <= i ? tri(i, j) : tri(j, i)];
   }
 }
 
@@ -377,9 +330,12 @@ int invert_domains_launch(gs_ctx ctx, gs_mas mas, double* fac0) {
   const int np = (3 * mas->N + 7) / 8 * 8;
   const size_t smem = ((size_t)np * (np + 1) / 2 + 8) * sizeof(double);
   GS_PROF(ctx, GS_K_MAS_INVERT);
-  invert::k_invert_domains<<<jb.first[mas->L], invert::kThreads, smem, ctx->stream>>>(jb, mas->remap0, ctx->d_flags,
-                                                                                      fac0);
+  const bool factors = mas->N == 16 || mas->N == 32;  // the tensor cores square them
+  (factors ? invert::k_invert_domains<false> : invert::k_invert_domains<true>)<<<jb.first[mas->L], invert::kThreads,
+                                                                                smem, ctx->stream>>>(
+      jb, mas->remap0, ctx->d_flags, fac0);
   GS_CUDA(cudaGetLastError());
+  if (factors) GS_TRY(square_factors_launch(ctx, jb, mas->N, mas->remap0));
   return GS_OK;
 }
 
