@@ -113,6 +113,18 @@ __global__ void __launch_bounds__(256) k_slice_values(const int32_t* __restrict_
   }
 }
 
+// The device has no room for the copy: none is kept, and the error of that one
+// allocation does not stand.
+static int no_room(gs_ctx ctx, gs_mat m) {
+  if (cudaPeekAtLastError() != cudaErrorMemoryAllocation) return GS_ERR_CUDA;
+  cudaGetLastError();
+  const int window = m->sl_window;
+  release_sliced(ctx, m, true);
+  m->sl_window = window;
+  return GS_OK;
+}
+
+
 // The sliced copy with float-float (ff) or FP64 values, made on first use and
 // kept with the matrix; new values (gs_fem_refill) drop the values only.
 int ensure_sliced(gs_ctx ctx, gs_mat m, bool ff) {
@@ -133,17 +145,20 @@ int ensure_sliced(gs_ctx ctx, gs_mat m, bool ff) {
     GS_CUDA(cudaMemcpyAsync(ctx->h_pinned + 8, m->sl_ptr + slices, 4, cudaMemcpyDeviceToHost, st));
     GS_CUDA(cudaStreamSynchronize(st));
     m->sl_entries = 32LL * ctx->h_pinned[8];
-    GS_TRY(ctx->alloc((void**)&m->sl_col, (size_t)std::max<int64_t>(m->sl_entries, 1) * 4));
-    GS_TRY(ctx->alloc((void**)&m->sl_blk, (size_t)std::max<int64_t>(m->sl_entries, 1) * 4));
-    { GS_PROF(ctx, GS_K_OTHER); k_slice_entries<<<ceil_div(n, 256), 256, 0, st>>>(m->row_order, m->row_ptr, m->cid, m->lo_ptr, m->lo_idx, m->lo_col, n, m->sl_ptr, m->sl_col, m->sl_blk); }
     m->sl_window = m->row_order_window;
+    if (m->sl_entries > 4 * m->nnzb + (1 << 20)) return GS_OK;  // mostly padding: a row very much longer than the rest
+    const size_t words = (size_t)std::max<int64_t>(m->sl_entries, 1);
+    if (ctx->alloc((void**)&m->sl_blk, words * 4) != GS_OK || ctx->alloc((void**)&m->sl_col, words * 4) != GS_OK)
+      return no_room(ctx, m);
+    { GS_PROF(ctx, GS_K_OTHER); k_slice_entries<<<ceil_div(n, 256), 256, 0, st>>>(m->row_order, m->row_ptr, m->cid, m->lo_ptr, m->lo_idx, m->lo_col, n, m->sl_ptr, m->sl_col, m->sl_blk); }
   }
+  if (!m->sl_col) return GS_OK;
   if (ff ? m->sl_ff != nullptr : m->sl_f64 != nullptr) return GS_OK;
   if (ff) {
     GS_TRY(ensure_ff_scales(ctx, m));
-    GS_TRY(ctx->alloc((void**)&m->sl_ff, (size_t)std::max<int64_t>(m->sl_entries, 1) * 72));
+    if (ctx->alloc((void**)&m->sl_ff, (size_t)std::max<int64_t>(m->sl_entries, 1) * 72) != GS_OK) return no_room(ctx, m);
   } else {
-    GS_TRY(ctx->alloc((void**)&m->sl_f64, (size_t)std::max<int64_t>(m->sl_entries, 1) * 72));
+    if (ctx->alloc((void**)&m->sl_f64, (size_t)std::max<int64_t>(m->sl_entries, 1) * 72) != GS_OK) return no_room(ctx, m);
   }
   GS_PROF(ctx, GS_K_OTHER);
   const dim3 grid(ceil_div(n, 256), n < 65536 ? 8 : 2);
