@@ -476,7 +476,7 @@ def kernel_lines(B, ctx, dev, clk, spmv, prec, nrhs, N, V, nnzb, ndom, mp, live,
         # per diagonal block and two per off-diagonal block
         ff_inst = nrhs * 9 * 12.0 * (V + 2.0 * n_off)
         fp32_peak = sms * 128 * sm_mhz_max * 1e6 / 1e12  # T FP32 instructions/s
-        kname = "k_spmv_ff_ws" if spmv_ws else "k_spmv_ff_row"
+        kname = "k_pcg_spmv" if nrhs <= 8 else ("k_spmv_ff_ws" if spmv_ws else "k_spmv_ff_row")
         spmv_line = {"bound": "alu", "achieved": ff_inst / t_spmv / 1e12, "peak": fp32_peak,
                      "unit": "T FP32 instructions/s", "frac": ff_inst / t_spmv / 1e12 / fp32_peak,
                      "traffic": (recorded_traffic(kname, f"{traffic_key},ff_rhs{B.gs_tune_get(ctx, B.GS_TUNE_SPMV_FF_RHS)}")
@@ -490,7 +490,8 @@ def kernel_lines(B, ctx, dev, clk, spmv, prec, nrhs, N, V, nnzb, ndom, mp, live,
                                  "frac": ff_inst / t_spmv_iso / 1e12 / fp32_peak,
                                  "hbm_frac": spmv_bytes / t_spmv_iso / 1e9 / hbm}
     else:
-        kname = "k_spmv_row_ws" if spmv_ws else f"k_spmv_{spmv}"
+        kname = ("k_pcg_spmv" if nrhs <= 8 and spmv != "srbk" else
+                 "k_spmv_row_ws" if spmv_ws else f"k_spmv_{spmv}")
         spmv_line = fp64_line(spmv_flops, spmv_bytes, t_spmv,
                               recorded_traffic(kname, traffic_key) if traffic_key else None)
         spmv_line["kernel"] = kname

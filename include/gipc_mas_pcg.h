@@ -327,7 +327,10 @@ int gs_adjoint(gs_ctx ctx, gs_mat mat, gs_mas mas, const double* x, const double
 /* ---------------------------------------------------------------- tuning */
 /* Launch shapes a context uses, set by the autotuner (or by hand).  Values
  * outside the listed set return GS_ERR_INVALID.  Results do not depend on
- * the choice except through the order of floating-point sums. */
+ * the choice except through the order of floating-point sums.  The SpMV shapes
+ * steer gs_spmv, and gs_pcg_solve with more than 8 right-hand sides; with up to 8
+ * gs_pcg_solve runs its own product over a sliced copy of the matrix (made on
+ * first use, freed with the matrix), except for GS_SPMV_SRBK. */
 #define GS_TUNE_SPMV_LANES 0      /* lanes per block row of the FP64 row SpMV: 1, 2 (default), 4, 8 */
 #define GS_TUNE_SPMV32_LANES 1    /* lanes per block row of the FP32 SpMV of the mixed solve: 2 (default), 4 */
 #define GS_TUNE_APPLY_RHS 2       /* right-hand sides per thread in the level-0 MAS product: 2, 4 (default), 8 */

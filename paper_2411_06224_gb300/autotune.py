@@ -10,7 +10,8 @@ sums; a shape the problem cannot launch (too many threads per block) is
 skipped.
 
 The shapes and the kernels they steer:
-  * GS_TUNE_SPMV_LANES   lanes per block row of the row SpMV, FP64 or float-float (Sec. 5.3);
+  * GS_TUNE_SPMV_LANES   lanes per block row of the row SpMV, FP64 or float-float (Sec. 5.3;
+                         PCG with up to 8 right-hand sides has its own shapes);
   * GS_TUNE_APPLY_RHS    right-hand sides per thread in the level-0 MAS product (Eq. 6);
   * GS_TUNE_SPMV32_LANES lanes per block row of the FP32 SpMV inside the mixed solve;
   * GS_TUNE_BATCH_CHUNK  vector entries per work item of the batched PCG reductions;
