@@ -130,6 +130,14 @@ struct RowWords {
   int32_t n_long, too_long;
 };
 
+// What the host waits for, into pinned memory in one launch.
+__global__ void k_row_words(const RowWords* __restrict__ words, const int32_t* __restrict__ total,
+                            int* __restrict__ host) {
+  host[4] = words->n_long;
+  host[5] = words->too_long;
+  host[8] = *total;
+}
+
 __global__ void k_row_count(const int32_t* __restrict__ rows, const int32_t* __restrict__ cols, int64_t nb, int32_t n,
                             int32_t* __restrict__ cnt, int32_t* __restrict__ rank, int32_t* __restrict__ key_of_input,
                             int* __restrict__ flags) {
@@ -351,8 +359,7 @@ static int reduce_rows(gs_ctx ctx, gs_mat m, const int32_t* rows, const int32_t*
     k_row_sort_block<<<std::max(1, std::min(2 * ctx->sm_count, n)), T, 0, st>>>(start, list, cnt, words, long_rows);
   }
   { GS_PROF(ctx, GS_K_ASSEMBLE); GS_TRY(exclusive_scan_i32(st, cnt, m->row_ptr, (int64_t)n + 1, temp, tb)); }
-  GS_CUDA(cudaMemcpyAsync(ctx->h_pinned + 4, words, sizeof(RowWords), cudaMemcpyDeviceToHost, st));
-  GS_CUDA(cudaMemcpyAsync(ctx->h_pinned + 8, m->row_ptr + n, 4, cudaMemcpyDeviceToHost, st));
+  k_row_words<<<1, 1, 0, st>>>(words, m->row_ptr + n, ctx->h_pinned);
   int flags = 0;
   GS_TRY(ctx->take_flags(&flags));
   if (flags) return status_from_flags(flags);
