@@ -462,12 +462,18 @@ __global__ void __launch_bounds__(128) k_element_hessians(const double* __restri
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j) As[i][j] = lam * g[i] * g[j] + (i == j ? mu : c1 * s[3 - i - j]);
-  // definite already (its leading minors are positive): nothing to project
+  // definite already (its leading minors are positive): nothing to project.  Every
+  // term of a minor is a product of entries, so its rounding is below 2^-48 of t^2
+  // or t^3, t the sum of the magnitudes; minors within 2^-40 of zero are decomposed:
+  // at the uniform stretch with mu = c1 s two eigenvalues vanish, and their product
+  // says nothing about their signs.
   const double m2 = As[0][0] * As[1][1] - As[0][1] * As[0][1];
   const double m3 = As[2][2] * m2 - As[0][0] * As[1][2] * As[1][2] +
                     As[0][2] * (2.0 * As[0][1] * As[1][2] - As[1][1] * As[0][2]);
+  const double ts = As[0][0] + As[1][1] + fabs(As[2][2]) + fabs(As[0][1]) + fabs(As[0][2]) + fabs(As[1][2]);
+  const double tm = 0x1p-40 * ts * ts;
   double Ps[3][3];
-  if (As[0][0] > 0.0 && m2 > 0.0 && m3 > 0.0) {
+  if (As[0][0] > 0.0 && m2 > tm && m3 > tm * ts) {
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
