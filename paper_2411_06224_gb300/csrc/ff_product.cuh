@@ -72,7 +72,7 @@ struct FFSum {
 // acc += H x for right-hand sides 0 .. nh - 1 of the column operand xb (3 pairs
 // each); vec: xb is 16-byte aligned, two RHS at a time.
 template <int kR>
-__device__ __forceinline__ void ff_block_product(const float2 (&H)[9], const float2* __restrict__ xb, int nh, bool vec,
+__device__ __forceinline__ void ff_block_product(const float2 (&H)[9], const float2* xb, int nh, bool vec,
                                                  FFSum<kR * 3>& acc) {
 #pragma unroll
   for (int q = 0; q < kR; q += 2) {

@@ -235,11 +235,10 @@ constexpr int kF32Unroll = 4;
 
 template <int kR, bool kDot>
 __global__ void __launch_bounds__(96) k_level0_f32(const float* __restrict__ invp, int pitch, int N, int nrhs,
-                                                   const double* __restrict__ r, double* __restrict__ z,
-                                                   int64_t stride, const int32_t* __restrict__ remap0,
-                                                   const double* __restrict__ zl, int64_t lstride, ApplyLevels al,
-                                                   const int* __restrict__ skip, int* __restrict__ flags,
-                                                   Partials dot) {
+                                                   const double* r, double* __restrict__ z, int64_t stride,
+                                                   const int32_t* __restrict__ remap0, const double* zl,
+                                                   int64_t lstride, ApplyLevels al, const int* skip,
+                                                   int* __restrict__ flags, Partials dot) {
   using namespace umma;
   // with kDot the kernel before is this preconditioner's coarse product or the
   // update of r: it wrote neither the inverses nor *skip
@@ -381,8 +380,8 @@ template <int kR>
 __global__ void __launch_bounds__(256) k_coarse_f32(const float* const* __restrict__ inv,
                                                     const int32_t* __restrict__ job_level,
                                                     const int32_t* __restrict__ job_dom, int N, int nrhs,
-                                                    const double* __restrict__ rl, double* __restrict__ zl,
-                                                    int64_t lstride, ApplyLevels al, const int* __restrict__ skip) {
+                                                    const double* rl, double* __restrict__ zl, int64_t lstride,
+                                                    ApplyLevels al, const int* skip) {
   if (skip && *skip) return;
   extern __shared__ float sm[];  // [ld][ld], then [ld][kR]
   const int ld = 3 * N, tid = threadIdx.x;

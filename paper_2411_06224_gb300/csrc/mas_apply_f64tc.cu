@@ -87,9 +87,8 @@ template <bool kCoarse, bool kDot, int kSlots, int kBufs, int kCtas, int LD>
 __global__ void __launch_bounds__(kThreads, kCtas) k_level0_f64tc(
     const uint8_t* const* __restrict__ dig_tab, const int32_t* const* __restrict__ exp_tab,
     const int32_t* __restrict__ job_level, const int32_t* __restrict__ job_dom, const int32_t* __restrict__ remap0,
-    int N, int nrhs, Levels al, const double* __restrict__ r, int64_t stride,
-    const double* __restrict__ zl, int64_t lstride, double* __restrict__ z, int* __restrict__ flags,
-    const int* __restrict__ skip, Partials dot) {
+    int N, int nrhs, Levels al, const double* r, int64_t stride, const double* zl, int64_t lstride,
+    double* __restrict__ z, int* __restrict__ flags, const int* skip, Partials dot) {
   using namespace umma;
   // The digits may be copied before the kernel ahead has ended where that is the
   // restriction or the coarse product: it wrote neither them nor *skip.

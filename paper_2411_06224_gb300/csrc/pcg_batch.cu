@@ -116,9 +116,8 @@ __global__ void __launch_bounds__(kT) k_binit(const double* __restrict__ b, doub
 
 // Partial sums of u . v; kCopy also writes dst = v.
 template <bool kCopy>
-__global__ void __launch_bounds__(kT) k_bdot(const double* __restrict__ u_, const double* __restrict__ v_,
-                                             double* __restrict__ dst, const Head* h, Arrays a,
-                                             double* __restrict__ out) {
+__global__ void __launch_bounds__(kT) k_bdot(const double* u_, const double* v_, double* __restrict__ dst,
+                                             const Head* h, Arrays a, double* __restrict__ out) {
   wait_for_previous_kernel();
   if (!kCopy && h->all_conv) return;
   const Span sp = my_span(a);
@@ -163,8 +162,7 @@ __global__ void k_bfirst_running(Head* h) { h->all_conv = h->running == 0; }
 // sums of ||r||^2.  The system's first block keeps what the sums decide; the
 // others may read conv and bad before or after, the answer is the same.
 __global__ void __launch_bounds__(kT) k_bupdate_xr(double* __restrict__ x, double* __restrict__ r,
-                                                   const double* __restrict__ p, const double* __restrict__ Ap,
-                                                   Head* h, Arrays a) {
+                                                   const double* p, const double* Ap, Head* h, Arrays a) {
   wait_for_previous_kernel();
   if (h->all_conv) return;
   __shared__ double s_alpha;
@@ -216,8 +214,8 @@ __global__ void __launch_bounds__(kT) k_bupdate_xr(double* __restrict__ x, doubl
 
 // The convergence test from the partial sums of ||r||^2, beta from those of
 // r . z, and p = z + beta p.
-__global__ void __launch_bounds__(kT) k_bupdate_p(double* __restrict__ p, const double* __restrict__ z, Head* h,
-                                                  Arrays a, double tol2) {
+__global__ void __launch_bounds__(kT) k_bupdate_p(double* __restrict__ p, const double* z, Head* h, Arrays a,
+                                                  double tol2) {
   wait_for_previous_kernel();
   if (h->all_conv) return;
   __shared__ double s_beta;

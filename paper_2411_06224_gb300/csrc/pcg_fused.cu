@@ -42,9 +42,8 @@ struct Sliced {  // the sliced matrix (sliced.cu)
 // with the entry's own values.
 template <bool kFF, int kBL, int kRL, int kR, int kMin>
 __global__ void __launch_bounds__(kT, kMin) k_pcg_spmv(Sliced A, const int32_t* __restrict__ kk,
-                                                       const float2* __restrict__ xs, const double* __restrict__ p,
-                                                       double* __restrict__ Ap, int64_t stride, int nrhs,
-                                                       const PcgScalars* __restrict__ s, Partials pap) {
+                                                       const float2* xs, const double* p, double* __restrict__ Ap,
+                                                       int64_t stride, int nrhs, const PcgScalars* s, Partials pap) {
   constexpr int G = kBL * kRL;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = lane % G;
   const int bl = sub % kBL, r0 = sub / kBL * kR;
@@ -217,8 +216,8 @@ constexpr int kPitch = 99;  // doubles per right-hand side: 3 N <= 96, spread ov
 
 template <int kR>
 __global__ void __launch_bounds__(kT, 3) k_pcg_xr(double* __restrict__ x, double* __restrict__ r,
-                                                  const double* __restrict__ p, const double* __restrict__ Ap,
-                                                  int64_t stride, int nrhs, const int32_t* __restrict__ remap0,
+                                                  const double* p, const double* Ap, int64_t stride, int nrhs,
+                                                  const int32_t* __restrict__ remap0,
                                                   int32_t n_dom, int N, const int32_t* __restrict__ item1,
                                                   int64_t off1, double* __restrict__ rl, int64_t lstride,
                                                   PcgScalars* s, Partials pap, Partials rrp, int parity) {
@@ -358,7 +357,7 @@ int pcg_update_xr(gs_ctx ctx, gs_mas mas, double* x, double* r, const double* p,
 // across right-hand sides; the new p's bound gathers in the other parity's fp.
 // A converged RHS keeps p, ps and its bounds.
 template <bool kFF>
-__global__ void __launch_bounds__(kT) k_pcg_p(double* __restrict__ p, const double* __restrict__ z,
+__global__ void __launch_bounds__(kT) k_pcg_p(double* __restrict__ p, const double* z,
                                               float2* __restrict__ ps, const int32_t* __restrict__ kk, int64_t len,
                                               int nrhs, PcgScalars* s, Partials rrp, Partials rzp, double tol2,
                                               int parity) {
@@ -445,7 +444,7 @@ __global__ void __launch_bounds__(kT) k_pcg_p(double* __restrict__ p, const doub
 
 // Folds the partial sums of a reduction over very many domains to 64 per RHS.
 constexpr int kFold = 64;
-__global__ void __launch_bounds__(kT) k_fold(Partials a, Partials out, const int* __restrict__ skip) {
+__global__ void __launch_bounds__(kT) k_fold(Partials a, Partials out, const int* skip) {
   wait_for_previous_kernel();
   if (*skip) return;
   const int k = blockIdx.y, per = (a.n + kFold - 1) / kFold, g0 = blockIdx.x * per;

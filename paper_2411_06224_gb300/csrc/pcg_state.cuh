@@ -126,7 +126,11 @@ __device__ __forceinline__ bool test_convergence(PcgScalars* s, int k, double rr
 
 // Programmatic dependent launch: a kernel may be resident before the one ahead
 // of it in the stream has finished; it waits here for that kernel's results.
-// Without the launch attribute both are no-ops.
+// Without the launch attribute both are no-ops.  Such a kernel lives while the one
+// before it writes, so its pointers to the iteration's vectors and words are not
+// `const __restrict__`: that would say nobody writes them meanwhile, and let the
+// compiler load them ahead of the wait or without coherence.  Tables older than
+// the solve are.
 __device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next_kernel_launch() { asm volatile("griddepcontrol.launch_dependents;"); }
 

@@ -88,7 +88,7 @@ struct LevelIdxNodeMajor {
 
 // Sum of rk[3 b] over the set bits b of mask, ascending, 16 loads in flight:
 // a coarse item's value from its children (the sum of k_restrict_up).
-__device__ __forceinline__ double sum_children(const double* __restrict__ rk, uint32_t mask) {
+__device__ __forceinline__ double sum_children(const double* rk, uint32_t mask) {
   double sum = 0.0;
 #pragma unroll 1
   for (int b = 0; b < 32; b += 16) {
