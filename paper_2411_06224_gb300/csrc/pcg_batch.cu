@@ -217,14 +217,17 @@ __global__ void __launch_bounds__(kT) k_bupdate_xr(double* __restrict__ x, doubl
 __global__ void __launch_bounds__(kT) k_bupdate_p(double* __restrict__ p, const double* z, Head* h, Arrays a,
                                                   double tol2) {
   wait_for_previous_kernel();
-  if (h->all_conv) return;
   __shared__ double s_beta;
   __shared__ int s_stop;
   const Span sp = my_span(a);
   const int s = a.w_seg[sp.w];
   if (threadIdx.x < 32) {
-    const double rr = system_sum(a.rrp, a, s), rz = system_sum(a.rzp, a, s);
-    if (threadIdx.x == 0) {
+    // all_conv is read once for the block: this grid's recording blocks may set it
+    const bool over = __shfl_sync(kFull, threadIdx.x == 0 ? h->all_conv : 0, 0) != 0;
+    const double rr = over ? 0.0 : system_sum(a.rrp, a, s), rz = over ? 0.0 : system_sum(a.rzp, a, s);
+    if (over) {
+      if (threadIdx.x == 0) s_stop = 1;
+    } else if (threadIdx.x == 0) {
       const bool record = sp.at == kParts * a.w_start[s];
       const bool was = a.conv[s] != 0, bad = a.bad[s] != 0 || !isfinite(rr);
       const bool stop = was || bad || rr <= tol2 * a.bnorm2[s];

@@ -375,12 +375,16 @@ __global__ void __launch_bounds__(kT) k_pcg_p(double* __restrict__ p, const doub
   double rr = 0.0;
   if (threadIdx.x < 32) rr = warp_sum_partials(rrp, k);
   wait_for_previous_kernel();
-  if (s->all_conv) return;
+  // all_conv is read once for the block: this grid's recording blocks may set it
   double rz = 0.0;
-  if (threadIdx.x < 32) rz = warp_sum_partials(rzp, k);
+  bool over = false;
+  if (threadIdx.x < 32) {
+    over = __shfl_sync(kFull, threadIdx.x == 0 ? s->all_conv : 0, 0) != 0;
+    if (!over) rz = warp_sum_partials(rzp, k);
+  }
   if (threadIdx.x == 0) {
     s_ex[0] = s_ex[1] = kExpNone;
-    s_stop = test_convergence(s, k, rr, tol2, record);
+    s_stop = over || test_convergence(s, k, rr, tol2, record);
     s_beta = rz / s->rz[parity][k];
   }
   int ex = kExpNone;

@@ -55,3 +55,13 @@ def test_only_tables_are_promised_constant():
         text = source(os.path.join(CSRC, path))
         at = text.index(helper + "(")
         assert "__restrict__" not in text[at : text.index("{", at)], helper
+
+
+def test_kernels_that_set_all_conv_decide_once_per_block():
+    """A grid whose recording block may set all_conv must not let each thread test it:
+    the warps of a later block could part, and go on with shared words that nobody set."""
+    writers = {n: b for n, (_, b) in chained_kernels().items() if "test_convergence(" in b or "all_conv = 1" in b}
+    assert set(writers) == {"k_pcg_p", "k_bupdate_p"}
+    for name, body in writers.items():
+        assert not re.search(r"if\s*\([^)]*all_conv[^)]*\)\s*return", body), name
+        assert body.index("all_conv") < body.index("__syncthreads()") < body.index("if (s_stop)"), name
