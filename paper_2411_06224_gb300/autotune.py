@@ -19,9 +19,9 @@ The shapes and the kernels they steer:
   * GS_TUNE_F64_TC       FP64 apply on the tensor cores (exact digit
                          splitting) or on the FP64 cores.  The digit storage is
                          made when the preconditioner is built, so the sweep
-                         stays within the storage built: the symmetric digit
-                         bytes (3) or the FP64 cores, or the digit bytes of
-                         every entry (1, 2 and 4 alike) or the FP64 cores;
+                         chooses between the value built with (3, the symmetric
+                         digit bytes, or 1, 2 and 4, one kernel from the digit
+                         bytes of every entry) and the FP64 cores;
   * GS_TUNE_SPMV_WS      one thread group per row, or a persistent grid whose
                          warps steal the next rows;
   * GS_TUNE_SPMV_FF_RHS  right-hand sides per thread of the float-float SpMV
@@ -46,7 +46,7 @@ CANDIDATES = {
     B.GS_TUNE_SPMV32_LANES: (2, 4),
     B.GS_TUNE_BATCH_CHUNK: (1024, 2048, 4096, 8192, 16384),
     B.GS_TUNE_BF16_TC: (1, 0),
-    B.GS_TUNE_F64_TC: (1, 2, 0),
+    B.GS_TUNE_F64_TC: (4, 0),
     B.GS_TUNE_SPMV_WINDOW: (0, 256, 1024, 4096, 16384),
     B.GS_TUNE_SPMV_WS: (0, 1),
     B.GS_TUNE_SPMV_FF_RHS: (8, 4, 2, 1),
@@ -125,7 +125,7 @@ def tune(ctx, mat, mas, nrhs=1, reps=10, mixed=False, node_off=None, iters=20, s
     apply = lambda: B.gs_mas_apply(ctx, mas, x, y, nrhs=nrhs)
     if fp64:
         built = B.gs_tune_get(ctx, B.GS_TUNE_F64_TC)  # the value `mas` was built with
-        cands = (3, 0) if built == 3 else (1, 4, 2, 0) if built in (1, 2, 4) else (0,)
+        cands = (built, 0) if built else (0,)
         out[NAMES[B.GS_TUNE_F64_TC]] = sweep(ctx, B.GS_TUNE_F64_TC, B.GS_K_MAS_APPLY_L0, apply, reps, cands)
     if not fp64 or B.gs_tune_get(ctx, B.GS_TUNE_F64_TC) == 0:  # the FP64-core kernel's shape
         out[NAMES[B.GS_TUNE_APPLY_RHS]] = sweep(ctx, B.GS_TUNE_APPLY_RHS, B.GS_K_MAS_APPLY_L0, apply, reps)

@@ -166,7 +166,7 @@ int level0_f64tc_prepare(gs_ctx ctx, gs_mas mas);
 // Inverts the level matrices in place and cuts their digit matrices (mas_invert.cu)
 int invert_domains_launch(gs_ctx ctx, gs_mas mas, double* fac0);
 // skip (device, may be null): the kernels return at once while *skip is set
-// dot (GS_TUNE_F64_TC 1 or 4): also partial sums of r . z, one per domain
+// dot (GS_TUNE_F64_TC 1, 2 or 4): also partial sums of r . z, one per domain
 struct Partials;
 int level0_f64tc_launch(gs_ctx ctx, gs_mas mas, int nrhs, const double* r, int64_t stride, const double* zl,
                         int64_t lstride, double* z, const int* skip = nullptr, const Partials* dot = nullptr);

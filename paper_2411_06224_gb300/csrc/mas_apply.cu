@@ -529,13 +529,13 @@ static int level0_f32_launch(gs_ctx ctx, gs_mas mas, const double* r, double* z,
   return launch_level0_f32<8, kDot>(ctx, mas, r, z, nrhs, zl, lstride, skip, dot);
 }
 
-// Forms whose level-0 product can also reduce r . z: FP64 from digit bytes
-// (one CTA per domain), FP32 from packed inverses; at most 8 RHS.
+// Forms whose level-0 product can also reduce r . z: FP64 from digit bytes of every
+// entry (GS_TUNE_F64_TC 1, 2 and 4, one kernel), FP32 from packed inverses; at most
+// 8 RHS.
 bool mas_dot_usable(gs_ctx ctx, gs_mas mas, int nrhs) {
   if (nrhs > 8) return false;
   if (mas->precision == GS_PREC_FP32) return level0_f32_bulk_usable(mas, nrhs);
-  const int t = ctx->tune[GS_TUNE_F64_TC];
-  return (t == 1 || t == 4) && level0_f64tc_usable(ctx, mas, nrhs);
+  return ctx->tune[GS_TUNE_F64_TC] != 3 && level0_f64tc_usable(ctx, mas, nrhs);
 }
 
 // Level-1 sums of r in rl, whose padding entries are zero already.
