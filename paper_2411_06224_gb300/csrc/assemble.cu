@@ -10,9 +10,10 @@
 // counts the rows and ranks the input within its row, one scatter of 8-byte
 // (column, index) keys) followed by a sort of every row's keys in a warp's
 // registers or a block's shared memory; the runs of a sorted row are then
-// summed by one warp, nine lanes to a block (reduce_rows).  A row of more
-// than 4,096 inputs sends the matrix to the general path: keys packed as
-// (row << b) | col with b the bit width of n, which keeps the (row, col) order
+// summed by one warp, nine lanes to a block (reduce_rows).  The inputs of rows of
+// more than 4,096 are radix-sorted among themselves and summed by as many warps
+// as they need.  Matrices of mostly empty rows take the general path: keys packed
+// as (row << b) | col with b the bit width of n, which keeps the (row, col) order
 // of the paper's (row << 32) | col encoding while shortening the radix sort
 // to 2b bits, values gathered through the sorted index, run flags, scan and
 // FastSegmentReduction (reduce_sorted_keys).
@@ -124,33 +125,55 @@ __global__ void k_row_ptr(const int32_t* __restrict__ rid, int64_t U, int32_t n,
 constexpr int kRowWarp = 256;   // longest row sorted by one warp
 constexpr int kRowBlock = kRowSerial;  // longest row sorted by one block (32 KB of keys)
 
-// Words the host reads back: [0] rows longer than kRowWarp, [1] set if a row
-// is longer than kRowBlock.
+// Words of the row path: rows that a block sorts, and the rows longer than
+// kRowBlock as (their number << 32) | their inputs, which the host reads back.
 struct RowWords {
-  int32_t n_long, too_long;
+  uint64_t huge;
+  int32_t n_long;
 };
 
-// What the host waits for, into pinned memory in one launch.
+// What the host waits for, and the error word (cleared), into pinned memory in one
+// launch.
 __global__ void k_row_words(const RowWords* __restrict__ words, const int32_t* __restrict__ total,
-                            int* __restrict__ host) {
-  host[4] = words->n_long;
-  host[5] = words->too_long;
+                            int* __restrict__ flags, int* __restrict__ host) {
+  host[0] = *flags;
+  *flags = 0;
+  host[4] = (int)(words->huge >> 32);
+  host[5] = (int)(uint32_t)words->huge;
   host[8] = *total;
 }
 
+// Counts the rows' inputs and ranks each within its row, in no fixed order.  The
+// lanes of the warp's first four rows add once per row: a row of very many inputs
+// (the reduced rows of a body of thousands of nodes) is one address for all of them,
+// and 2M atomics on four addresses took 0.7 ms, 0.19 so.
 __global__ void k_row_count(const int32_t* __restrict__ rows, const int32_t* __restrict__ cols, int64_t nb, int32_t n,
                             int32_t* __restrict__ cnt, int32_t* __restrict__ rank, int32_t* __restrict__ key_of_input,
                             int* __restrict__ flags) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nb) return;
-  const int32_t r = rows[i], c = cols[i];
-  int32_t k = -1;
-  if (r < 0 || r >= n || c < 0 || c >= n)
-    atomicOr(flags, kErrIndex);
-  else if (r <= c)
-    k = atomicAdd(&cnt[r], 1);
-  rank[i] = k;
-  if (k < 0) key_of_input[i] = -1;
+  const int lane = threadIdx.x & 31;
+  const bool in = i < nb;
+  const int32_t r = in ? rows[i] : 0, c = in ? cols[i] : 0;
+  const bool inside = in && r >= 0 && r < n && c >= 0 && c < n;
+  if (in && !inside) atomicOr(flags, kErrIndex);
+  const bool counts = inside && r <= c;
+  uint32_t left = __ballot_sync(kFull, counts), group = 1u << lane;  // lanes that add with this one
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (!left) break;  // whole warp
+    const int32_t rl = __shfl_sync(kFull, r, __ffs(left) - 1);
+    const bool mine = counts && r == rl;
+    const uint32_t same = __ballot_sync(kFull, mine);
+    if (mine) group = same;
+    left &= ~same;
+  }
+  const int lead = __ffs(group) - 1;
+  int32_t first = 0;
+  if (counts && lane == lead) first = atomicAdd(&cnt[r], __popc(group));
+  first = __shfl_sync(kFull, first, lead);
+  if (!in) return;
+  rank[i] = counts ? first + __popc(group & ((1u << lane) - 1u)) : -1;
+  if (!counts) key_of_input[i] = -1;
 }
 
 // The ranks of a row's inputs are in no fixed order; the sort by (column,
@@ -212,9 +235,13 @@ __device__ __forceinline__ int32_t sort_row(uint64_t* __restrict__ row, int32_t 
   return unique;
 }
 
+// Rows of up to kRowWarp inputs; the others go to the lists of k_row_sort_block
+// (long_rows, from the front) and of the huge rows (long_rows, from the back, and
+// their first places among all inputs of huge rows).
 __global__ void __launch_bounds__(256) k_row_sort(const int32_t* __restrict__ start, int32_t n,
                                                   uint64_t* __restrict__ list, int32_t* __restrict__ unique,
-                                                  RowWords* __restrict__ words, int32_t* __restrict__ long_rows) {
+                                                  RowWords* __restrict__ words, int32_t* __restrict__ long_rows,
+                                                  int32_t* __restrict__ huge_base) {
   const int32_t r = (int32_t)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= n) return;  // whole warp
@@ -223,12 +250,17 @@ __global__ void __launch_bounds__(256) k_row_sort(const int32_t* __restrict__ st
   int32_t u = 0;
   if (len > kRowWarp) {
     if (lane == 0) {
-      if (len > kRowBlock)
-        words->too_long = 1;
-      else
+      if (len > kRowBlock) {
+        const uint64_t old =
+            atomicAdd((unsigned long long*)&words->huge, (1ull << 32) | (unsigned long long)(uint32_t)len);
+        const int32_t h = (int32_t)(old >> 32);
+        long_rows[n - 1 - h] = r;
+        huge_base[h] = (int32_t)(uint32_t)old;
+      } else {
         long_rows[atomicAdd(&words->n_long, 1)] = r;
+      }
     }
-    return;  // k_row_sort_block writes this row's count
+    return;  // k_row_sort_block or k_huge_unique writes this row's count
   }
   if (len > 128)
     u = sort_row<8>(row, len, lane);
@@ -294,7 +326,7 @@ __global__ void __launch_bounds__(256) k_row_reduce(const int32_t* __restrict__ 
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (r >= n) return;  // whole warp
   const int32_t s0 = start[r], len = start[r + 1] - s0;
-  if (len == 0) return;
+  if (len == 0 || len > kRowBlock) return;
   int32_t next = row_ptr[r];  // the next run's stored block
   uint32_t before = 0;        // column of the last entry of the previous 32
   double cv = 0.0;
@@ -330,49 +362,173 @@ __global__ void __launch_bounds__(256) k_row_reduce(const int32_t* __restrict__ 
   if (lane < 9) R[(size_t)cd * 9 + lane] = cv;
 }
 
-// Rows sorted one by one.  *done stays false when a row is too long for it
-// (nothing but scratch and m->row_ptr, m->key_of_input was touched).
+// ---------------------------------------------------------------- rows of more than kRowBlock inputs
+// Their inputs are sorted together by (row's number h, column, input) in one radix
+// sort, and summed in pieces of 256 sorted entries (64 where 256 would leave SMs
+// idle) whatever the rows are, a warp each, added to the zeroed output.  The other
+// rows are summed as ever.  Sending the whole matrix to the general path instead,
+// once the row path had met a row too long for it, paid for both: 13.4M inputs with
+// one row of 5,000 2.72 ms (0.92 so; 2.25 in the general path alone), 2M inputs on
+// four rows 1.48 (0.73; 0.78), a two-level assembly with a body of 8,192 nodes 0.99
+// (0.59; 0.85), 20,000 inputs with a row of 4,200 0.165 (0.144; 0.149).
+__global__ void k_huge_keys(const uint64_t* __restrict__ list, const int32_t* __restrict__ start,
+                            const int32_t* __restrict__ last_row, const int32_t* __restrict__ base, int32_t n_huge,
+                            int32_t m, int cb, int ib, uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= m) return;
+  int32_t lo = 0, hi = n_huge;  // base[lo] <= p < base[hi]
+  while (hi - lo > 1) {
+    const int32_t mid = (lo + hi) / 2;
+    if (base[mid] <= p)
+      lo = mid;
+    else
+      hi = mid;
+  }
+  const uint64_t e = list[(int64_t)start[*(last_row - lo)] + (p - base[lo])];
+  keys[p] = ((uint64_t)lo << (cb + ib)) | (e >> 32 << ib) | (uint32_t)e;
+  vals[p] = (uint32_t)e;
+}
+
+// head[p]: sorted entry p begins a run (head[m]: 0, the end of the scan).
+__global__ void k_huge_heads(const uint64_t* __restrict__ keys, int32_t m, int ib, int32_t* __restrict__ head) {
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p <= m) head[p] = p < m && (p == 0 || keys[p] >> ib != keys[p - 1] >> ib);
+}
+
+__global__ void k_huge_unique(const int32_t* __restrict__ last_row, const int32_t* __restrict__ base, int32_t n_huge,
+                              int32_t m, const int32_t* __restrict__ before, int32_t* __restrict__ unique) {
+  const int32_t h = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (h < n_huge) unique[*(last_row - h)] = before[h + 1 < n_huge ? base[h + 1] : m] - before[base[h]];
+}
+
+__global__ void __launch_bounds__(256) k_huge_reduce(const uint64_t* __restrict__ keys,
+                                                     const uint32_t* __restrict__ vals,
+                                                     const int32_t* __restrict__ before,
+                                                     const int32_t* __restrict__ last_row,
+                                                     const int32_t* __restrict__ base, int32_t m, int piece, int cb,
+                                                     int ib, const int32_t* __restrict__ row_ptr,
+                                                     const double* __restrict__ blocks, double* __restrict__ R,
+                                                     int32_t* __restrict__ rid, int32_t* __restrict__ cid,
+                                                     int32_t* __restrict__ key_of_input) {
+  __shared__ uint32_t s_idx[8][kPiece];
+  __shared__ int32_t s_dst[8][kPiece];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t p0 = ((int64_t)blockIdx.x * 8 + w) * piece;
+  if (p0 >= m) return;  // whole warp
+  const int len = (int)min((int64_t)piece, m - p0);
+  for (int j = lane; j < len; j += 32) {
+    const int64_t p = p0 + j;
+    const uint64_t key = keys[p];
+    const int32_t h = (int32_t)(key >> (cb + ib)), r = *(last_row - h);
+    const int32_t u = row_ptr[r] + before[p + 1] - 1 - before[base[h]];
+    const uint32_t i = vals[p];
+    if (before[p + 1] != before[p]) {
+      rid[u] = r;
+      cid[u] = (int32_t)(key >> ib & ((1ull << cb) - 1));
+    }
+    s_idx[w][j] = i;
+    s_dst[w][j] = u;
+    key_of_input[i] = u;
+  }
+  __syncwarp();
+  double cv = 0.0;
+  int32_t cd = -1;
+  sum_piece<true>(blocks, s_idx[w], s_dst[w], len, R, cv, cd, lane);
+  if (lane < 9) atomicAdd(R + (size_t)cd * 9 + lane, cv);
+}
+
+// Sorted entries of the rows of more than kRowBlock inputs.
+struct HugeRows {
+  const int32_t *last_row, *base;  // row h at last_row[-h]; its first place
+  int32_t n, m;                    // rows, inputs
+  int cb, ib;                      // bits of a column and of an input
+  uint64_t* keys;
+  uint32_t* vals;
+  int32_t* before;  // runs before a sorted entry (m + 1)
+};
+
+// Sorts the huge rows' inputs and writes their unique counts.  rank's slot takes
+// the sort's values.
+static int sort_huge_rows(gs_ctx ctx, const uint64_t* list, const int32_t* start, int64_t nb, int32_t* unique,
+                          HugeRows& g) {
+  cudaStream_t st = ctx->stream;
+  const int T = 256;
+  uint64_t* keys = nullptr;
+  uint32_t* vals = nullptr;
+  void* temp = nullptr;
+  const size_t tb = std::max(radix_sort_temp_bytes(g.m), scan_temp_bytes((int64_t)g.m + 1));
+  GS_TRY(ctx->scratch_buf(kSlotSortKeysOut, (size_t)g.m * 16, (void**)&keys));
+  GS_TRY(ctx->scratch_buf(kSlotSortValsIn, (size_t)nb * 4, (void**)&vals));
+  GS_TRY(ctx->scratch_buf(kSlotSortValsOut, (size_t)g.m * 4, (void**)&g.vals));
+  GS_TRY(ctx->scratch_buf(kSlotSortTemp, tb, &temp));
+  g.keys = keys + g.m;
+  g.before = (int32_t*)keys;  // the unsorted keys' place
+  { GS_PROF(ctx, GS_K_ASSEMBLE); k_huge_keys<<<ceil_div(g.m, T), T, 0, st>>>(list, start, g.last_row, g.base, g.n, g.m, g.cb, g.ib, keys, vals); }
+  { GS_PROF(ctx, GS_K_ASSEMBLE); GS_TRY(radix_sort_pairs(st, keys, g.keys, vals, g.vals, g.m, bits_for(g.n) + g.cb + g.ib, temp, tb)); }
+  { GS_PROF(ctx, GS_K_ASSEMBLE); k_huge_heads<<<ceil_div((int64_t)g.m + 1, T), T, 0, st>>>(g.keys, g.m, g.ib, g.before); }
+  { GS_PROF(ctx, GS_K_ASSEMBLE); GS_TRY(exclusive_scan_i32(st, g.before, g.before, (int64_t)g.m + 1, temp, tb)); }
+  { GS_PROF(ctx, GS_K_ASSEMBLE); k_huge_unique<<<ceil_div(g.n, T), T, 0, st>>>(g.last_row, g.base, g.n, g.m, g.before, unique); }
+  return GS_OK;
+}
+
+// Rows sorted one by one.  *done stays false where the huge rows' keys do not fit 64
+// bits (nothing but scratch and m->row_ptr, m->key_of_input was touched).
 static int reduce_rows(gs_ctx ctx, gs_mat m, const int32_t* rows, const int32_t* cols, const double* blocks, int64_t nb,
                        bool* done) {
   cudaStream_t st = ctx->stream;
   const int32_t n = m->n;
   const int T = 256;
-  // counts / unique counts, row starts, worklist of long rows, words
-  int32_t *cnt = nullptr, *rank = nullptr;
+  // counts / unique counts, row starts, worklists of long and huge rows, words
+  int32_t* rank = nullptr;
   uint64_t* list = nullptr;
   void* temp = nullptr;
   const size_t tb = scan_temp_bytes((int64_t)n + 1);
-  GS_TRY(ctx->scratch_buf(kSlotScan, (3 * (size_t)n + 8) * 4, (void**)&cnt));
+  RowWords* words = nullptr;  // then the counts
+  const size_t ints = 3 * (size_t)n + 2 + (size_t)(nb / kRowBlock) + 1;
+  GS_TRY(ctx->scratch_buf(kSlotScan, sizeof(RowWords) + ints * 4, (void**)&words));
   GS_TRY(ctx->scratch_buf(kSlotSortValsIn, (size_t)nb * 4, (void**)&rank));
   GS_TRY(ctx->scratch_buf(kSlotSortKeysIn, (size_t)nb * 8, (void**)&list));
   GS_TRY(ctx->scratch_buf(kSlotSortTemp, tb, &temp));
-  int32_t *start = cnt + n + 1, *long_rows = start + n + 1;
-  RowWords* words = (RowWords*)(long_rows + n);
-  GS_CUDA(cudaMemsetAsync(cnt, 0, ((size_t)n + 1) * 4, st));
-  GS_CUDA(cudaMemsetAsync(words, 0, sizeof(RowWords), st));
+  int32_t *cnt = (int32_t*)(words + 1), *start = cnt + n + 1, *long_rows = start + n + 1, *huge_base = long_rows + n;
+  GS_CUDA(cudaMemsetAsync(words, 0, sizeof(RowWords) + ((size_t)n + 1) * 4, st));
   { GS_PROF(ctx, GS_K_ASSEMBLE); k_row_count<<<ceil_div(nb, T), T, 0, st>>>(rows, cols, nb, n, cnt, rank, m->key_of_input, ctx->d_flags); }
   { GS_PROF(ctx, GS_K_ASSEMBLE); GS_TRY(exclusive_scan_i32(st, cnt, start, (int64_t)n + 1, temp, tb)); }
   { GS_PROF(ctx, GS_K_ASSEMBLE); k_row_scatter<<<ceil_div(nb, T), T, 0, st>>>(rows, cols, rank, start, nb, list); }
-  { GS_PROF(ctx, GS_K_ASSEMBLE); k_row_sort<<<ceil_div(32LL * n, T), T, 0, st>>>(start, n, list, cnt, words, long_rows); }
+  { GS_PROF(ctx, GS_K_ASSEMBLE); k_row_sort<<<ceil_div(32LL * n, T), T, 0, st>>>(start, n, list, cnt, words, long_rows, huge_base); }
   {
     GS_PROF(ctx, GS_K_ASSEMBLE);
     k_row_sort_block<<<std::max(1, std::min(2 * ctx->sm_count, n)), T, 0, st>>>(start, list, cnt, words, long_rows);
   }
-  { GS_PROF(ctx, GS_K_ASSEMBLE); GS_TRY(exclusive_scan_i32(st, cnt, m->row_ptr, (int64_t)n + 1, temp, tb)); }
-  k_row_words<<<1, 1, 0, st>>>(words, m->row_ptr + n, ctx->h_pinned);
-  int flags = 0;
-  GS_TRY(ctx->take_flags(&flags));
-  if (flags) return status_from_flags(flags);
-  const RowWords h = *(const RowWords*)(ctx->h_pinned + 4);
-  if (h.too_long) return GS_OK;
+  HugeRows huge{};
+  for (int pass = 0;; ++pass) {
+    { GS_PROF(ctx, GS_K_ASSEMBLE); GS_TRY(exclusive_scan_i32(st, cnt, m->row_ptr, (int64_t)n + 1, temp, tb)); }
+    k_row_words<<<1, 1, 0, st>>>(words, m->row_ptr + n, ctx->d_flags, ctx->h_pinned);
+    GS_CUDA(cudaGetLastError());
+    GS_TRY(ctx->sync());
+    if (ctx->h_pinned[0]) return status_from_flags(ctx->h_pinned[0]);
+    huge.n = ctx->h_pinned[4], huge.m = ctx->h_pinned[5];
+    if (pass || !huge.n) break;
+    huge.last_row = long_rows + n - 1, huge.base = huge_base;
+    huge.cb = bits_for(n), huge.ib = bits_for(nb);
+    if (bits_for(huge.n) + huge.cb + huge.ib > 64) return GS_OK;
+    GS_TRY(sort_huge_rows(ctx, list, start, nb, cnt, huge));
+    GS_TRY(ctx->scratch_buf(kSlotSortTemp, tb, &temp));  // may have grown
+  }
   const int64_t U = ctx->h_pinned[8];
   m->nnzb = U;
   GS_TRY(ctx->alloc((void**)&m->au, (size_t)U * 72));
   GS_TRY(ctx->alloc((void**)&m->rid, (size_t)U * 4));
   GS_TRY(ctx->alloc((void**)&m->cid, (size_t)U * 4));
   if (U > 0) {
+    if (huge.n) GS_CUDA(cudaMemsetAsync(m->au, 0, (size_t)U * 72, st));
     { GS_PROF(ctx, GS_K_ASSEMBLE); k_row_reduce<<<ceil_div(32LL * n, T), T, 0, st>>>(start, m->row_ptr, list, blocks, n, m->au, m->rid, m->cid,
                                                                                     m->key_of_input); }
+  }
+  if (huge.n) {
+    GS_PROF(ctx, GS_K_ASSEMBLE);
+    const int piece = huge.m <= 2 * 8 * 64 * std::max(ctx->sm_count, 1) ? 64 : kPiece;  // 2 blocks per SM
+    k_huge_reduce<<<ceil_div(huge.m, 8 * piece), T, 0, st>>>(huge.keys, huge.vals, huge.before, huge.last_row, huge.base, huge.m, piece,
+                                                             huge.cb, huge.ib, m->row_ptr, blocks, m->au, m->rid, m->cid, m->key_of_input);
   }
   *done = true;
   return GS_OK;

@@ -205,6 +205,77 @@ __global__ void __launch_bounds__(1024) k_scan_one(const int32_t* in, int32_t* o
     }
 }
 
+// Small sorts whole, one block, by the same passes: a pass is one launch of 3 to 7 us
+// for its histogram, one for its scan and one for its scatter, 19 us together; here 10 (4,200
+// pairs).  A warp takes a contiguous part of the pairs, kOnePer of them per lane,
+// loaded before any pass is over (in and out of a pass differ).
+constexpr int kOnePer = 8;
+constexpr int64_t kSortOneMax = 1024 * kOnePer;
+__global__ void __launch_bounds__(1024) k_sort_one(const uint64_t* k_in, const uint32_t* v_in, uint64_t* k_out,
+                                                   uint32_t* v_out, uint64_t* k_tmp, uint32_t* v_tmp, int n,
+                                                   int end_bit) {
+  __shared__ int32_t wcnt[32][256];  // running, then prefixed, count of each digit per warp
+  __shared__ int32_t toff[256], s_warp[32], total;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int per = (n + 1023) / 1024, wbase = warp * 32 * per, passes = (end_bit + 7) / 8;
+  const unsigned lt = (1u << lane) - 1u;
+  const uint64_t* ki = k_in;
+  const uint32_t* vi = v_in;
+  for (int p = 1; p <= passes; ++p) {
+    uint64_t* ko = (passes - p) % 2 == 0 ? k_out : k_tmp;
+    uint32_t* vo = (passes - p) % 2 == 0 ? v_out : v_tmp;
+    const int shift = 8 * (p - 1);
+    const uint32_t mask = (1u << min(8, end_bit - shift)) - 1u;
+    for (int d = tid; d < 32 * 256; d += 1024) (&wcnt[0][0])[d] = 0;
+    uint64_t k[kOnePer];
+    uint32_t v[kOnePer];
+    int dg[kOnePer], rank[kOnePer];
+#pragma unroll
+    for (int i = 0; i < kOnePer; ++i) {
+      const int e = wbase + i * 32 + lane;
+      const bool valid = i < per && e < n;
+      k[i] = valid ? ki[e] : 0;
+      v[i] = valid ? vi[e] : 0;
+      dg[i] = valid ? (int)((k[i] >> shift) & mask) : 256 + lane;  // an invalid lane matches nobody
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kOnePer; ++i) {
+      if (i >= per) break;  // whole block
+      const unsigned peers = __match_any_sync(kFull, dg[i]);
+      const bool valid = dg[i] < 256;
+      const int before = valid ? wcnt[warp][dg[i]] : 0;
+      __syncwarp();
+      rank[i] = before + __popc(peers & lt);
+      if (valid && (peers & lt) == 0) wcnt[warp][dg[i]] = before + __popc(peers);
+      __syncwarp();
+    }
+    __syncthreads();
+    int s = 0;
+    if (tid < 256) {  // exclusive prefix of the warps' counts, per digit, in warp order
+#pragma unroll 8
+      for (int w = 0; w < 32; ++w) {
+        const int c = wcnt[w][tid];
+        wcnt[w][tid] = s;
+        s += c;
+      }
+    }
+    const int first = block_exclusive_scan(s, s_warp, &total);  // every thread
+    if (tid < 256) toff[tid] = first;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kOnePer; ++i) {
+      if (i >= per || dg[i] >= 256) continue;
+      const int pos = toff[dg[i]] + wcnt[warp][dg[i]] + rank[i];
+      ko[pos] = k[i];
+      vo[pos] = v[i];
+    }
+    __syncthreads();  // the next pass reads them
+    ki = ko;
+    vi = vo;
+  }
+}
+
 }  // namespace prim
 
 static inline size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -251,6 +322,11 @@ int radix_sort_pairs(cudaStream_t st, const uint64_t* k_in, uint64_t* k_out, con
   int32_t* hist = (int32_t*)t;
   t += align256((size_t)256 * tiles * 4);
   void* stemp = t;
+  if (n <= prim::kSortOneMax) {
+    prim::k_sort_one<<<1, 1024, 0, st>>>(k_in, v_in, k_out, v_out, tk, tv, (int)n, end_bit);
+    GS_CUDA(cudaGetLastError());
+    return GS_OK;
+  }
   const int passes = (end_bit + 7) / 8;
   const uint64_t* ki = k_in;
   const uint32_t* vi = v_in;
