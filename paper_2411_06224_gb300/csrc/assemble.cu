@@ -10,7 +10,7 @@
 // counts the rows and ranks the input within its row, one scatter of 8-byte
 // (column, index) keys) followed by a sort of every row's keys in a warp's
 // registers or a block's shared memory; the runs of a sorted row are then
-// summed by one warp, nine lanes to a block (reduce_rows).  The inputs of rows of
+// summed by that warp or block, nine lanes to a 3x3 block (reduce_rows).  The inputs of rows of
 // more than 4,096 are radix-sorted among themselves and summed by as many warps
 // as they need.  Matrices of mostly empty rows take the general path: keys packed
 // as (row << b) | col with b the bit width of n, which keeps the (row, col) order
@@ -122,8 +122,8 @@ __global__ void k_row_ptr(const int32_t* __restrict__ rid, int64_t U, int32_t n,
 // twice.  Measured, gs_assemble and gs_mat_export: 2.48 -> 1.29 ms (64^3, 13.4M
 // inputs), 0.21 -> 0.13 ms (16^3, 0.18M), two-level 1.34 -> 0.80 ms (40^3 and
 // 1,000 bodies).
-constexpr int kRowWarp = 256;   // longest row sorted by one warp
-constexpr int kRowBlock = kRowSerial;  // longest row sorted by one block (32 KB of keys)
+constexpr int kRowWarp = kPiece;       // longest row sorted, and summed, by one warp
+constexpr int kRowBlock = kRowSerial;  // longest row sorted, and summed, by one block (32 KB of keys)
 
 // Words of the row path: rows that a block sorts, and the rows longer than
 // kRowBlock as (their number << 32) | their inputs, which the host reads back.
@@ -140,6 +140,7 @@ __global__ void k_row_words(const RowWords* __restrict__ words, const int32_t* _
   *flags = 0;
   host[4] = (int)(words->huge >> 32);
   host[5] = (int)(uint32_t)words->huge;
+  host[6] = words->n_long;
   host[8] = *total;
 }
 
@@ -274,7 +275,8 @@ __global__ void __launch_bounds__(256) k_row_sort(const int32_t* __restrict__ st
 }
 
 // The long rows, a block each.
-__global__ void __launch_bounds__(256) k_row_sort_block(const int32_t* __restrict__ start, uint64_t* __restrict__ list,
+constexpr int kSortBlock = 512;  // threads of it
+__global__ void __launch_bounds__(kSortBlock) k_row_sort_block(const int32_t* __restrict__ start, uint64_t* __restrict__ list,
                                                         int32_t* __restrict__ unique,
                                                         const RowWords* __restrict__ words,
                                                         const int32_t* __restrict__ long_rows) {
@@ -311,9 +313,39 @@ __global__ void __launch_bounds__(256) k_row_sort_block(const int32_t* __restric
   }
 }
 
-// The runs of every sorted row, a warp per row: in pieces of 256 entries it
-// finds the runs, writes their keys and each input's stored block, and sums
-// them (run_reduce.cuh).
+// Keys of a piece of m sorted entries from entry p0 of row r (list: the row's), whose
+// first run is the stored block `next` where it begins with a head, else next - 1:
+// each input's stored block, and the runs' keys.
+__device__ __forceinline__ void number_runs(const uint64_t* __restrict__ list, int32_t p0, int m, int32_t r,
+                                            int32_t next, uint32_t* s_idx, int32_t* s_dst, int32_t* __restrict__ rid,
+                                            int32_t* __restrict__ cid, int32_t* __restrict__ key_of_input, int lane) {
+  uint32_t before = p0 > 0 ? (uint32_t)(list[p0 - 1] >> 32) : 0;  // column of the entry ahead
+  for (int j = 0; j < m; j += 32) {
+    const int32_t p = p0 + j + lane;
+    const bool in = j + lane < m;
+    const uint64_t key = in ? list[p] : ~0ull;
+    const uint32_t c = (uint32_t)(key >> 32);
+    uint32_t prev = __shfl_up_sync(kFull, c, 1);
+    if (lane == 0) prev = before;
+    before = __shfl_sync(kFull, c, 31);
+    const bool head = in && (p == 0 || c != prev);
+    const uint32_t hm = __ballot_sync(kFull, head);
+    const int32_t u = next + __popc(hm & (0xffffffffu >> (31 - lane))) - 1;
+    if (head) {
+      rid[u] = r;
+      cid[u] = (int32_t)c;
+    }
+    if (in) {
+      s_idx[j + lane] = (uint32_t)key;
+      s_dst[j + lane] = u;
+      key_of_input[(uint32_t)key] = u;
+    }
+    next += __popc(hm);
+  }
+}
+
+// The runs of every sorted row of up to kPiece inputs, a warp per row: finds the runs,
+// writes their keys and each input's stored block, and sums them (run_reduce.cuh).
 __global__ void __launch_bounds__(256) k_row_reduce(const int32_t* __restrict__ start,
                                                     const int32_t* __restrict__ row_ptr,
                                                     const uint64_t* __restrict__ list,
@@ -326,40 +358,42 @@ __global__ void __launch_bounds__(256) k_row_reduce(const int32_t* __restrict__ 
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (r >= n) return;  // whole warp
   const int32_t s0 = start[r], len = start[r + 1] - s0;
-  if (len == 0 || len > kRowBlock) return;
-  int32_t next = row_ptr[r];  // the next run's stored block
-  uint32_t before = 0;        // column of the last entry of the previous 32
+  if (len == 0 || len > kPiece) return;
+  number_runs(list + s0, 0, len, r, row_ptr[r], s_idx[w], s_dst[w], rid, cid, key_of_input, lane);
+  __syncwarp();
   double cv = 0.0;
   int32_t cd = -1;
-  for (int32_t p0 = 0; p0 < len; p0 += kPiece) {
-    const int m = min(kPiece, len - p0);
-    for (int j = 0; j < m; j += 32) {
-      const int32_t p = p0 + j + lane;
-      const bool in = j + lane < m;
-      const uint64_t key = in ? list[s0 + p] : ~0ull;
-      const uint32_t c = (uint32_t)(key >> 32);
-      uint32_t prev = __shfl_up_sync(kFull, c, 1);
-      if (lane == 0) prev = before;
-      before = __shfl_sync(kFull, c, 31);
-      const bool head = in && (p == 0 || c != prev);
-      const uint32_t hm = __ballot_sync(kFull, head);
-      const int32_t u = next + __popc(hm & (0xffffffffu >> (31 - lane))) - 1;
-      if (head) {
-        rid[u] = r;
-        cid[u] = (int32_t)c;
-      }
-      if (in) {
-        s_idx[w][j + lane] = (uint32_t)key;
-        s_dst[w][j + lane] = u;
-        key_of_input[(uint32_t)key] = u;
-      }
-      next += __popc(hm);
-    }
-    __syncwarp();
-    sum_piece<false>(blocks, s_idx[w], s_dst[w], m, R, cv, cd, lane);
-    __syncwarp();
-  }
+  sum_piece<false>(blocks, s_idx[w], s_dst[w], len, R, cv, cd, lane);
   if (lane < 9) R[(size_t)cd * 9 + lane] = cv;
+}
+
+// The same for the rows that a block sorted, a block each.
+__global__ void __launch_bounds__(32 * kRowWarps) k_row_reduce_block(
+    const int32_t* __restrict__ start, const int32_t* __restrict__ row_ptr, const uint64_t* __restrict__ list,
+    const double* __restrict__ blocks, const int32_t* __restrict__ long_rows, double* __restrict__ R,
+    int32_t* __restrict__ rid, int32_t* __restrict__ cid, int32_t* __restrict__ key_of_input) {
+  __shared__ uint32_t s_idx[kRowWarps][kRowPiece];
+  __shared__ int32_t s_dst[kRowWarps][kRowPiece];
+  __shared__ RowEnds ends;
+  __shared__ int s_heads[kRowWarps];
+  const int32_t r = long_rows[blockIdx.x];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int32_t s0 = start[r], len = start[r + 1] - s0;
+  const int per = row_piece(len), p0 = w * per, m = max(0, min(per, len - p0));
+  const uint64_t* row = list + s0;
+  int heads = 0;
+  for (int j = lane; j < m; j += 32) {
+    const int32_t p = p0 + j;
+    heads += p == 0 || (row[p] >> 32) != (row[p - 1] >> 32);
+  }
+  heads = __reduce_add_sync(kFull, heads);
+  if (lane == 0) s_heads[w] = heads;
+  __syncthreads();
+  int32_t next = row_ptr[r];
+  for (int i = 0; i < w; ++i) next += s_heads[i];
+  if (m > 0) number_runs(row, p0, m, r, next, s_idx[w], s_dst[w], rid, cid, key_of_input, lane);  // whole warp
+  __syncwarp();
+  sum_row_block(blocks, s_idx[w], s_dst[w], m, R, &ends, w, lane);
 }
 
 // ---------------------------------------------------------------- rows of more than kRowBlock inputs
@@ -497,7 +531,7 @@ static int reduce_rows(gs_ctx ctx, gs_mat m, const int32_t* rows, const int32_t*
   { GS_PROF(ctx, GS_K_ASSEMBLE); k_row_sort<<<ceil_div(32LL * n, T), T, 0, st>>>(start, n, list, cnt, words, long_rows, huge_base); }
   {
     GS_PROF(ctx, GS_K_ASSEMBLE);
-    k_row_sort_block<<<std::max(1, std::min(2 * ctx->sm_count, n)), T, 0, st>>>(start, list, cnt, words, long_rows);
+    k_row_sort_block<<<std::max(1, std::min(2 * ctx->sm_count, n)), kSortBlock, 0, st>>>(start, list, cnt, words, long_rows);
   }
   HugeRows huge{};
   for (int pass = 0;; ++pass) {
@@ -523,6 +557,10 @@ static int reduce_rows(gs_ctx ctx, gs_mat m, const int32_t* rows, const int32_t*
     if (huge.n) GS_CUDA(cudaMemsetAsync(m->au, 0, (size_t)U * 72, st));
     { GS_PROF(ctx, GS_K_ASSEMBLE); k_row_reduce<<<ceil_div(32LL * n, T), T, 0, st>>>(start, m->row_ptr, list, blocks, n, m->au, m->rid, m->cid,
                                                                                     m->key_of_input); }
+  }
+  if (const int n_long = ctx->h_pinned[6]) {
+    GS_PROF(ctx, GS_K_ASSEMBLE);
+    k_row_reduce_block<<<n_long, 32 * kRowWarps, 0, st>>>(start, m->row_ptr, list, blocks, long_rows, m->au, m->rid, m->cid, m->key_of_input);
   }
   if (huge.n) {
     GS_PROF(ctx, GS_K_ASSEMBLE);

@@ -65,8 +65,10 @@ struct gs_fem_s {
   int64_t U_e = 0;
   uint64_t* e_keys = nullptr;  // U_e unique element keys, ascending
   int32_t* e_start = nullptr;  // V + 1: first sorted input of every row
-  int32_t* e_long = nullptr;   // count, then the rows of more than kRowSerial inputs
-  int32_t n_long_rows = 0;
+  int32_t* e_long = nullptr;   // [0], [1] counts; rows of more than kPiece inputs from the front, of more than
+                               // kRowSerial from the back
+  int32_t n_long_rows = 0, n_huge_rows = 0;
+  int64_t long_cap = 0;        // entries of e_long
   double* e_vals = nullptr;    // n_in * 9 input blocks (numeric scratch)
   double* forces = nullptr;    // T * 12 node forces of the elements
   double* energy = nullptr;    // T + nc + V energy terms
@@ -571,8 +573,8 @@ __global__ void k_mass_blocks(const double* __restrict__ mass, int32_t V, double
 
 // Numeric assembly through the stored order: sorted entry i carries input
 // sidx[i] into stored block O[i] (ascending); row r holds the entries
-// start[r] .. start[r + 1] - 1.  A warp per row sums its runs in pieces of 256
-// entries (run_reduce.cuh, as gs_assemble does).  32^3 body, 1.5M inputs:
+// start[r] .. start[r + 1] - 1.  A warp per row sums its runs, a block per row of
+// more than 256 entries (run_reduce.cuh, as gs_assemble does).  32^3 body, 1.5M inputs:
 // 0.053 ms (0.142 ms with a thread per input and a segmented warp reduction).
 __device__ __forceinline__ void load_piece(const uint32_t* __restrict__ sidx, const int32_t* __restrict__ O, int64_t i0,
                                            int m, uint32_t* s_idx, int32_t* s_dst, int lane) {
@@ -590,32 +592,49 @@ __global__ void __launch_bounds__(256) k_reduce_rows(const uint32_t* __restrict_
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (r >= n) return;  // whole warp
   const int32_t i0 = start[r], len = start[r + 1] - i0;
-  if (len == 0 || len > kRowSerial) return;
+  if (len == 0 || len > kPiece) return;
   double cv = 0.0;
   int32_t cd = -1;
-  for (int32_t p = 0; p < len; p += kPiece) {
-    const int m = min(kPiece, len - p);
-    load_piece(sidx, O, i0 + p, m, s_idx[w], s_dst[w], lane);
-    sum_piece<false>(vals, s_idx[w], s_dst[w], m, R, cv, cd, lane);
-  }
+  load_piece(sidx, O, i0, len, s_idx[w], s_dst[w], lane);
+  sum_piece<false>(vals, s_idx[w], s_dst[w], len, R, cv, cd, lane);
   if (lane < 9) R[(size_t)cd * 9 + lane] = cv;
 }
 
-// Rows of more than kRowSerial entries (a vertex of thousands of elements): a
-// block each, its warps taking pieces in turn and adding their sums to the
-// zeroed output atomically.
-__global__ void __launch_bounds__(256) k_reduce_long_rows(const uint32_t* __restrict__ sidx,
-                                                          const int32_t* __restrict__ O,
-                                                          const int32_t* __restrict__ start,
-                                                          const int32_t* __restrict__ rows,
-                                                          const double* __restrict__ vals, double* __restrict__ R) {
-  __shared__ uint32_t s_idx[8][kPiece];
-  __shared__ int32_t s_dst[8][kPiece];
+// Rows of more than kPiece entries, a block each.
+__global__ void __launch_bounds__(32 * kRowWarps) k_reduce_long_rows(const uint32_t* __restrict__ sidx,
+                                                                     const int32_t* __restrict__ O,
+                                                                     const int32_t* __restrict__ start,
+                                                                     const int32_t* __restrict__ rows,
+                                                                     const double* __restrict__ vals,
+                                                                     double* __restrict__ R) {
+  __shared__ uint32_t s_idx[kRowWarps][kRowPiece];
+  __shared__ int32_t s_dst[kRowWarps][kRowPiece];
+  __shared__ RowEnds ends;
   const int32_t r = rows[blockIdx.x];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int32_t i0 = start[r], len = start[r + 1] - i0;
-  for (int32_t p = w * kPiece; p < len; p += 8 * kPiece) {
-    const int m = min(kPiece, len - p);
+  const int per = row_piece(len), p0 = w * per, m = max(0, min(per, len - p0));
+  load_piece(sidx, O, i0 + p0, m, s_idx[w], s_dst[w], lane);
+  sum_row_block(vals, s_idx[w], s_dst[w], m, R, &ends, w, lane);
+}
+
+// Rows of more than kRowSerial entries (a vertex of thousands of elements): as many
+// blocks as fill the GPU, their warps taking pieces of 64 to 256 in turn and adding
+// their sums to the zeroed output atomically (row blockIdx.x from the list's end).
+__global__ void __launch_bounds__(256) k_reduce_huge_rows(const uint32_t* __restrict__ sidx,
+                                                          const int32_t* __restrict__ O,
+                                                          const int32_t* __restrict__ start,
+                                                          const int32_t* __restrict__ last_row,
+                                                          const double* __restrict__ vals, double* __restrict__ R) {
+  __shared__ uint32_t s_idx[8][kPiece];
+  __shared__ int32_t s_dst[8][kPiece];
+  const int32_t r = *(last_row - blockIdx.x);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int32_t i0 = start[r], len = start[r + 1] - i0;
+  const int64_t warps = gridDim.y * 8;
+  const int per = (int)max((int64_t)64, min((int64_t)kPiece, (len + warps - 1) / warps));
+  for (int64_t p = (blockIdx.y * 8 + w) * (int64_t)per; p < len; p += warps * per) {
+    const int m = (int)min((int64_t)per, len - p);
     double cv = 0.0;
     int32_t cd = -1;
     load_piece(sidx, O, i0 + p, m, s_idx[w], s_dst[w], lane);
@@ -624,8 +643,7 @@ __global__ void __launch_bounds__(256) k_reduce_long_rows(const uint32_t* __rest
   }
 }
 
-// First sorted input of every row, and the rows longer than kRowSerial
-// (long_rows[0] counts them).
+// First sorted input of every row.
 __global__ void k_row_starts(const uint64_t* __restrict__ keys, const int32_t* __restrict__ O, int64_t n, int shift,
                              int32_t n_rows, int32_t* __restrict__ start) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -635,9 +653,15 @@ __global__ void k_row_starts(const uint64_t* __restrict__ keys, const int32_t* _
   for (int32_t r = prev + 1; r <= here; ++r) start[r] = (int32_t)i;
 }
 
-__global__ void k_long_rows(const int32_t* __restrict__ start, int32_t n_rows, int32_t* __restrict__ long_rows) {
+// The rows of more than kPiece inputs, and those of more than kRowSerial (gs_fem_s::e_long).
+__global__ void k_long_rows(const int32_t* __restrict__ start, int32_t n_rows, int64_t cap,
+                            int32_t* __restrict__ long_rows) {
   const int32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < n_rows && start[r + 1] - start[r] > kRowSerial) long_rows[1 + atomicAdd(long_rows, 1)] = r;
+  const int32_t len = r < n_rows ? start[r + 1] - start[r] : 0;
+  if (len > kRowSerial)
+    long_rows[cap - 1 - atomicAdd(long_rows + 1, 1)] = r;
+  else if (len > kPiece)
+    long_rows[2 + atomicAdd(long_rows, 1)] = r;
 }
 
 __global__ void k_add_blocks(const int32_t* __restrict__ pos, const double* __restrict__ src, int64_t n,
@@ -1175,7 +1199,12 @@ int refill(gs_ctx ctx, gs_fem f, const double* x, gs_mat m) {
   }
   if (f->n_long_rows) {
     GS_PROF(ctx, GS_K_ASSEMBLE);
-    k_reduce_long_rows<<<f->n_long_rows, 256, 0, st>>>(f->e_sidx, f->O_m, f->e_start, f->e_long + 1, f->e_vals, m->au);
+    k_reduce_long_rows<<<f->n_long_rows, 32 * kRowWarps, 0, st>>>(f->e_sidx, f->O_m, f->e_start, f->e_long + 2, f->e_vals, m->au);
+  }
+  if (f->n_huge_rows) {
+    GS_PROF(ctx, GS_K_ASSEMBLE);
+    const dim3 g(f->n_huge_rows, std::min(65535, std::max(1, ceil_div(4LL * ctx->sm_count, f->n_huge_rows))));
+    k_reduce_huge_rows<<<g, 256, 0, st>>>(f->e_sidx, f->O_m, f->e_start, f->e_long + f->long_cap - 1, f->e_vals, m->au);
   }
   if (f->c_mat && f->c_mat->nnzb) {
     GS_PROF(ctx, GS_K_ASSEMBLE);
@@ -1286,12 +1315,12 @@ int gs_fem_create(gs_ctx ctx, int32_t n_vertices, int64_t n_tets, const double* 
     if ((s = ctx->alloc((void**)&f->e_keys, (size_t)f->U_e * 8))) return fail(s);
     { GS_PROF(ctx, GS_K_ASSEMBLE); k_unique_keys<<<ceil_div(n, 256), 256, 0, st>>>(skeys, f->e_O, n, f->e_keys); }
     if ((s = ctx->alloc((void**)&f->e_start, (size_t)(V + 1) * 4)) ||
-        (s = ctx->alloc((void**)&f->e_long, (size_t)(n / kRowSerial + 2) * 4)))
+        (s = ctx->alloc((void**)&f->e_long, (size_t)(f->long_cap = n / kPiece + 2) * 4)))
       return fail(s);
     { GS_PROF(ctx, GS_K_ASSEMBLE); k_row_starts<<<ceil_div(n + 1, 256), 256, 0, st>>>(f->e_keys, f->e_O, n, f->shift, V, f->e_start); }
-    if (cudaMemsetAsync(f->e_long, 0, 4, st) != cudaSuccess) return fail(GS_ERR_CUDA);
-    { GS_PROF(ctx, GS_K_ASSEMBLE); k_long_rows<<<ceil_div(V, 256), 256, 0, st>>>(f->e_start, V, f->e_long); }
-    if ((s = read_i32(ctx, f->e_long, &f->n_long_rows))) return fail(s);
+    if (cudaMemsetAsync(f->e_long, 0, 8, st) != cudaSuccess) return fail(GS_ERR_CUDA);
+    { GS_PROF(ctx, GS_K_ASSEMBLE); k_long_rows<<<ceil_div(V, 256), 256, 0, st>>>(f->e_start, V, f->long_cap, f->e_long); }
+    if ((s = read_i32(ctx, f->e_long, &f->n_long_rows)) || (s = read_i32(ctx, f->e_long + 1, &f->n_huge_rows))) return fail(s);
     if ((s = check_flags(ctx, "gs_fem_create"))) return fail(s);
   }
   if ((s = merge_pattern(ctx, f))) return fail(s);
