@@ -10,7 +10,8 @@ namespace gs {
 
 // Accumulate the term (ah + al)(xh + xl) into the pair (S, L).  The rounded
 // intrinsics keep the compiler from contracting or reordering the
-// transformations.
+// transformations.  The term's small parts are added among themselves first, so
+// that only one of the four roundings is at the size of L.
 __device__ __forceinline__ void ff_term(float ah, float al, float xh, float xl, float& S, float& L) {
   const float p = __fmul_rn(ah, xh);
   const float e = __fmaf_rn(ah, xh, -p);
@@ -18,9 +19,7 @@ __device__ __forceinline__ void ff_term(float ah, float al, float xh, float xl, 
   const float bp = __fsub_rn(s, S);
   const float err = __fadd_rn(__fsub_rn(S, __fsub_rn(s, bp)), __fsub_rn(p, bp));
   S = s;
-  L = __fadd_rn(L, __fadd_rn(err, e));
-  L = __fmaf_rn(ah, xl, L);
-  L = __fmaf_rn(al, xh, L);
+  L = __fadd_rn(L, __fmaf_rn(al, xh, __fmaf_rn(ah, xl, __fadd_rn(err, e))));
 }
 
 // (S, L) += (S2, L2): two-sum of the large parts, the rest gathered in L.
@@ -50,6 +49,16 @@ struct FFSum {
   __device__ __forceinline__ void clear() {
 #pragma unroll
     for (int q = 0; q < kV; ++q) S[q] = 0.f, L[q] = 0.f;
+  }
+  // (S, L) = two_sum(S, L): the same sum, L small again.
+  __device__ __forceinline__ void settle() {
+#pragma unroll
+    for (int q = 0; q < kV; ++q) {
+      const float s = __fadd_rn(S[q], L[q]);
+      const float bp = __fsub_rn(s, S[q]);
+      L[q] = __fadd_rn(__fsub_rn(S[q], __fsub_rn(s, bp)), __fsub_rn(L[q], bp));
+      S[q] = s;
+    }
   }
   // Sum over kLanes neighbouring lanes, in a fixed order.
   template <int kLanes>

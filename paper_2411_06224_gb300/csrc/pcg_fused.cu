@@ -37,9 +37,15 @@ struct Sliced {  // the sliced matrix (sliced.cu)
 
 // One row by kBL * kRL lanes: kRL groups take kR right-hand sides each, the kBL
 // lanes of a group share the row's entries and merge in a fixed order.  kFF:
-// float-float (spmv_ff.cu), xs the split operand; else FP64, x the operand.  An
+// float-float (spmv_ff.cu), xs the split operand; else FP64, x the operand.  A lane
+// that sums a whole row gathers twice the small parts that each of two lanes
+// would, with as much more rounding, so its pairs are settled every kSettle entries.
+// 64^3, 8 RHS, 24 iterations: error 9.4e-14, 13.13 ms (1.7e-13 and 13.12 with three
+// roundings a term at the size of L and never settled; 1.16e-13 with two lanes to a
+// row; settling every fourth entry 5.8e-14 and 13.4).  An
 // entry's column is loaded one entry ahead, so that its operand's gather leaves
 // with the entry's own values.
+constexpr int kSettle = 16;
 template <bool kFF, int kBL, int kRL, int kR, int kMin>
 __global__ void __launch_bounds__(kT, kMin) k_pcg_spmv(Sliced A, const int32_t* __restrict__ kk,
                                                        const float2* xs, const double* p, double* __restrict__ Ap,
@@ -80,13 +86,17 @@ __global__ void __launch_bounds__(kT, kMin) k_pcg_spmv(Sliced A, const int32_t* 
       FFSum<kR * 3> acc;
       acc.clear();
       const float2* v = A.ff + (base - lane_slot) * 9 + lane_slot;
-      for (int32_t e = bl; e < len; e += kBL) {
-        const int32_t col = next;
-        if (e + kBL < len) next = A.col[base + 32 * (int64_t)(e + kBL)];
-        float2 H[9];
+      for (int32_t e = bl; e < len;) {
+        const int32_t end = min(len, e + kSettle * kBL);
+        for (; e < end; e += kBL) {
+          const int32_t col = next;
+          if (e + kBL < len) next = A.col[base + 32 * (int64_t)(e + kBL)];
+          float2 H[9];
 #pragma unroll
-        for (int q = 0; q < 9; ++q) H[q] = v[(int64_t)e * 288 + 32 * q];
-        ff_block_product<kR>(H, xs + ((int64_t)col * nrhs + r0) * 3, nh, vec, acc);
+          for (int q = 0; q < 9; ++q) H[q] = v[(int64_t)e * 288 + 32 * q];
+          ff_block_product<kR>(H, xs + ((int64_t)col * nrhs + r0) * 3, nh, vec, acc);
+        }
+        acc.settle();
       }
       acc.template merge<kBL>();
       if (in && bl == 0) {

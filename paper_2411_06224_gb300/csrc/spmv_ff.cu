@@ -23,7 +23,7 @@
 //   * Each term a x = ah xh + (ah xl + al xh) + al xl: ah xh is taken exactly
 //     as p + e (p = ah * xh rounded, e = fma(ah, xh, -p)), the row sum of the
 //     p runs through Knuth's two-sum (s, err), and the small parts
-//     err + e + ah xl + al xh gather in a second float; al xl (below 2^-47 of
+//     err + e + ah xl + al xh, added up, gather in a second float; al xl (below 2^-47 of
 //     the term) is dropped.  y_r = 2^(k_r + K + F) (S + L), added in FP64.
 //
 // Error per output (u = 2^-24, m = terms of the row, 3 per stored block of
