@@ -39,7 +39,9 @@ struct Sliced {  // the sliced matrix (sliced.cu)
 // lanes of a group share the row's entries and merge in a fixed order.  kFF:
 // float-float (spmv_ff.cu), xs the split operand; else FP64, x the operand.  A lane
 // that sums a whole row gathers twice the small parts that each of two lanes
-// would, with as much more rounding, so its pairs are settled every kSettle entries.
+// would, with as much more rounding, so its pairs are settled every kSettle entries
+// (where 2 or 4 lanes share it, not: the chain is short, and the loop in pieces cost
+// 3 % at 40^3, 1 RHS).
 // 64^3, 8 RHS, 24 iterations: error 9.4e-14, 13.13 ms (1.7e-13 and 13.12 with three
 // roundings a term at the size of L and never settled; 1.16e-13 with two lanes to a
 // row; settling every fourth entry 5.8e-14 and 13.4).  An
@@ -87,7 +89,7 @@ __global__ void __launch_bounds__(kT, kMin) k_pcg_spmv(Sliced A, const int32_t* 
       acc.clear();
       const float2* v = A.ff + (base - lane_slot) * 9 + lane_slot;
       for (int32_t e = bl; e < len;) {
-        const int32_t end = min(len, e + kSettle * kBL);
+        const int32_t end = kBL == 1 ? min(len, e + kSettle) : len;
         for (; e < end; e += kBL) {
           const int32_t col = next;
           if (e + kBL < len) next = A.col[base + 32 * (int64_t)(e + kBL)];
@@ -96,7 +98,7 @@ __global__ void __launch_bounds__(kT, kMin) k_pcg_spmv(Sliced A, const int32_t* 
           for (int q = 0; q < 9; ++q) H[q] = v[(int64_t)e * 288 + 32 * q];
           ff_block_product<kR>(H, xs + ((int64_t)col * nrhs + r0) * 3, nh, vec, acc);
         }
-        acc.settle();
+        if (kBL == 1) acc.settle();
       }
       acc.template merge<kBL>();
       if (in && bl == 0) {
