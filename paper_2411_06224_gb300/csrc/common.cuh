@@ -232,6 +232,7 @@ struct gs_mat_s {
   float2* sl_ff = nullptr;    // values, float-float: [(sl_ptr[s] + e) * 9 + q][32]
   double* sl_f64 = nullptr;   // the same in FP64
   int64_t sl_entries = 0;
+  int32_t sl_longest = 0;     // entries of the longest row
   int32_t sl_window = -1;     // row_order_window it was built for
   const void* pattern_owner = nullptr;  // the elastic body whose fixed pattern this matrix uses (or null)
   uint64_t pattern_version = 0;        // and that pattern's version

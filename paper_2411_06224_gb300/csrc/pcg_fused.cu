@@ -173,12 +173,18 @@ __global__ void __launch_bounds__(kT, kMin) k_pcg_spmv(Sliced A, const int32_t* 
 // 1 RHS (2) 2.87 / - / 3.08 ms; 40^3, 4 RHS (2) 41.8 / - / 42.7; 32^3, 1 RHS,
 // five Newton steps (2) 26.5 / 26.7 / -; 20^3, 2 RHS (4) 13.3 / 14.4 / -.
 // (Loading an entry one ahead of its use: 45^3 2.87 ms as well, 20^3 13.9.)
+// A row coupled to very many nodes holds up the whole product, 0.4 to 0.9 us an entry
+// and lane, so four lanes share the rows where the longest is beyond kHubRow; below it
+// the other rows' sums cost more.  24 iterations at 64^3, 4 RHS, FP64, with one row of
+// 327 / 627 / 3,027 blocks, 1 lane and 4: 18.5 / 27.6 / 100 and 14.1 / 16.1 / 32.7 ms
+// (15.4 with one lane and a row of 227); 40^3, 1 RHS, 3,027: 2 lanes 31.2, 4 17.5.
+constexpr int32_t kHubRow = 192;
 template <bool kFF, int kRL, int kR>
 static int launch_spmv(gs_ctx ctx, gs_mat m, const float2* xs, const double* p, double* Ap, int nrhs,
                        const PcgScalars* s, Partials& pap) {
   const Sliced A{m->row_order, m->sl_ptr, m->sl_len, m->sl_col, m->sl_ff, m->sl_f64, m->n};
   const int64_t rows = (int64_t)m->n * kRL, sms = std::max(ctx->sm_count, 1);
-  const int bl = rows * 4 <= sms * 512 ? 4 : (rows * 2 <= sms * 2048 ? 2 : 1);
+  const int bl = rows * 4 <= sms * 512 || m->sl_longest > kHubRow ? 4 : (rows * 2 <= sms * 2048 ? 2 : 1);
   constexpr int kMin = kFF ? 4 : 3;
   const int64_t chunks = ((int64_t)m->n * kRL * bl + kT - 1) / kT;
   pap.n = (int)std::max<int64_t>(1, std::min<int64_t>({chunks, (int64_t)kMin * std::max(ctx->sm_count, 1),

@@ -22,11 +22,11 @@ namespace gs {
 
 int ensure_row_order(gs_ctx ctx, gs_mat m);
 
-// Length of every row of the order, and the longest of each slice (a warp per
-// slice; one slice more, of length 0, ends the scan).
+// Length of every row of the order, the longest of each slice (a warp per
+// slice; one slice more, of length 0, ends the scan) and of all (*longest: 0).
 __global__ void k_slice_len(const int32_t* __restrict__ row_order, const int32_t* __restrict__ row_ptr,
                             const int32_t* __restrict__ lo_ptr, int32_t n, int32_t n_slices,
-                            int32_t* __restrict__ len, int32_t* __restrict__ most) {
+                            int32_t* __restrict__ len, int32_t* __restrict__ most, int32_t* __restrict__ longest) {
   const int32_t t = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x), s = t >> 5;
   if (s > n_slices) return;  // whole warp
   int32_t l = 0;
@@ -36,7 +36,10 @@ __global__ void k_slice_len(const int32_t* __restrict__ row_order, const int32_t
     len[t] = l;
   }
   const int32_t m = __reduce_max_sync(kFull, l);
-  if ((t & 31) == 0) most[s] = m;
+  if ((t & 31) == 0) {
+    most[s] = m;
+    if (m > *(volatile int32_t*)longest) atomicMax(longest, m);
+  }
 }
 
 // Column of every entry, and its stored block (complemented: transposed).  A
@@ -136,15 +139,19 @@ int ensure_sliced(gs_ctx ctx, gs_mat m, bool ff) {
     int32_t* most = nullptr;
     void* temp = nullptr;
     const size_t tb = scan_temp_bytes(slices + 1);
-    GS_TRY(ctx->scratch_buf(kSlotScan, ((size_t)slices + 1) * 4, (void**)&most));
+    GS_TRY(ctx->scratch_buf(kSlotScan, ((size_t)slices + 2) * 4, (void**)&most));
+    int32_t* longest = most + slices + 1;
+    GS_CUDA(cudaMemsetAsync(longest, 0, 4, st));
     GS_TRY(ctx->scratch_buf(kSlotSortTemp, tb, &temp));
     GS_TRY(ctx->alloc((void**)&m->sl_ptr, ((size_t)slices + 1) * 4));
     GS_TRY(ctx->alloc((void**)&m->sl_len, (size_t)std::max(n, 1) * 4));
-    { GS_PROF(ctx, GS_K_OTHER); k_slice_len<<<ceil_div(32LL * (slices + 1), 256), 256, 0, st>>>(m->row_order, m->row_ptr, m->lo_ptr, n, slices, m->sl_len, most); }
+    { GS_PROF(ctx, GS_K_OTHER); k_slice_len<<<ceil_div(32LL * (slices + 1), 256), 256, 0, st>>>(m->row_order, m->row_ptr, m->lo_ptr, n, slices, m->sl_len, most, longest); }
     { GS_PROF(ctx, GS_K_OTHER); GS_TRY(exclusive_scan_i32(st, most, m->sl_ptr, slices + 1, temp, tb)); }
     GS_CUDA(cudaMemcpyAsync(ctx->h_pinned + 8, m->sl_ptr + slices, 4, cudaMemcpyDeviceToHost, st));
+    GS_CUDA(cudaMemcpyAsync(ctx->h_pinned + 9, longest, 4, cudaMemcpyDeviceToHost, st));
     GS_CUDA(cudaStreamSynchronize(st));
     m->sl_entries = 32LL * ctx->h_pinned[8];
+    m->sl_longest = ctx->h_pinned[9];
     m->sl_window = m->row_order_window;
     if (m->sl_entries > 4 * m->nnzb + (1 << 20)) return GS_OK;  // mostly padding: a row very much longer than the rest
     const size_t words = (size_t)std::max<int64_t>(m->sl_entries, 1);
