@@ -172,6 +172,9 @@ __global__ void __launch_bounds__(kT, kMin) k_pcg_spmv(Sliced A, const int32_t* 
 // Whole solves with the lanes of this rule / twice as many / half as many: 45^3,
 // 1 RHS (2) 2.87 / - / 3.08 ms; 40^3, 4 RHS (2) 41.8 / - / 42.7; 32^3, 1 RHS,
 // five Newton steps (2) 26.5 / 26.7 / -; 20^3, 2 RHS (4) 13.3 / 14.4 / -.
+// With five or seven right-hand sides in a lane the blocks are two to an SM and 1 lane
+// leaves the last round empty for longer: 50^3, 5 RHS 9.1 ms with 1, 8.0 with 2; 64^3
+// 12.6 and 13.6.
 // (Loading an entry one ahead of its use: 45^3 2.87 ms as well, 20^3 13.9.)
 // A row coupled to very many nodes holds up the whole product, 0.4 to 0.9 us an entry
 // and lane, so four lanes share the rows where the longest is beyond kHubRow; below it
@@ -184,8 +187,8 @@ static int launch_spmv(gs_ctx ctx, gs_mat m, const float2* xs, const double* p, 
                        const PcgScalars* s, Partials& pap) {
   const Sliced A{m->row_order, m->sl_ptr, m->sl_len, m->sl_col, m->sl_ff, m->sl_f64, m->n};
   const int64_t rows = (int64_t)m->n * kRL, sms = std::max(ctx->sm_count, 1);
-  const int bl = rows * 4 <= sms * 512 || m->sl_longest > kHubRow ? 4 : (rows * 2 <= sms * 2048 ? 2 : 1);
-  constexpr int kMin = kFF ? 4 : 3;
+  const int bl = rows * 4 <= sms * 512 || m->sl_longest > kHubRow ? 4 : (rows * 2 <= sms * (kR > 3 ? 3072 : 2048) ? 2 : 1);
+  constexpr int kMin = kR > 3 ? 2 : (kFF && kR < 3 ? 4 : 3);
   const int64_t chunks = ((int64_t)m->n * kRL * bl + kT - 1) / kT;
   pap.n = (int)std::max<int64_t>(1, std::min<int64_t>({chunks, (int64_t)kMin * std::max(ctx->sm_count, 1),
                                                        (int64_t)kMaxRedBlocks}));
@@ -208,6 +211,25 @@ static int launch_spmv_rhs(gs_ctx ctx, gs_mat m, const float2* xs, const double*
                            const PcgScalars* s, Partials& pap) {
   if (nrhs == 1) return launch_spmv<kFF, 1, 1>(ctx, m, xs, p, Ap, nrhs, s, pap);
   if (nrhs == 2) return launch_spmv<kFF, 2, 1>(ctx, m, xs, p, Ap, nrhs, s, pap);
+  // Odd counts and 6 leave places of 2 x 2 or 4 x 2 empty, and an instruction costs the
+  // same for a lane without a right-hand side: other shares, but not on systems so
+  // small that lanes are what is missing (12^3, 5 RHS: 1.1 ms with 4 lanes of 2, 1.2
+  // with 2 of 3), nor where 7 in one lane leave too few (32^3: 3.9 and 4.2).  24
+  // iterations at 64^3, FP32 preconditioner, with the shares of 4 and 8 / these / the
+  // former product: row 3 RHS 10.7 / 10.0 / 10.4 ms, 5 17.5 / 12.6 / 13.6, 6 17.8 / 15.1 /
+  // 15.2, 7 18.2 / 16.0 / 17.0; float-float 3 RHS 7.6 / 7.1 / 9.0, 5 10.9 / 9.3 / 10.5, 6
+  // 10.7 / 9.9 / 11.0.
+  if (m->n >= 4096) {
+    if (kFF) {
+      if (nrhs == 3) return launch_spmv<true, 1, 3>(ctx, m, xs, p, Ap, nrhs, s, pap);
+      if (nrhs == 5 || nrhs == 6) return launch_spmv<true, 2, 3>(ctx, m, xs, p, Ap, nrhs, s, pap);
+    } else {
+      if (nrhs == 3) return launch_spmv<false, 1, 3>(ctx, m, xs, p, Ap, nrhs, s, pap);
+      if (nrhs == 5) return launch_spmv<false, 1, 5>(ctx, m, xs, p, Ap, nrhs, s, pap);
+      if (nrhs == 6) return launch_spmv<false, 2, 3>(ctx, m, xs, p, Ap, nrhs, s, pap);
+      if (nrhs == 7 && m->n > 512LL * ctx->sm_count) return launch_spmv<false, 1, 7>(ctx, m, xs, p, Ap, nrhs, s, pap);
+    }
+  }
   if (nrhs <= 4) return launch_spmv<kFF, 2, 2>(ctx, m, xs, p, Ap, nrhs, s, pap);
   return launch_spmv<kFF, 4, 2>(ctx, m, xs, p, Ap, nrhs, s, pap);
 }
