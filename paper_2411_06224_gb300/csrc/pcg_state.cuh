@@ -136,10 +136,13 @@ __device__ __forceinline__ void let_next_kernel_launch() { asm volatile("griddep
 
 // Up to this many block rows x right-hand sides an iteration is bound by its
 // launches and latencies, beyond it by bytes and arithmetic.  Kernels of the
-// first kind are chained (below) and fused further (pcg.cu).  Whole solves so,
-// against neither: 16^3, 4 RHS 5.7 / 9.4 ms; 40^3, 4 RHS 42 / 54; 45^3, 1 RHS
-// 3.7 / 4.8; 64^3, 8 RHS 16.1 / 14.5.
-constexpr int64_t kSmallWork = 1 << 19;
+// first kind are chained (below) and fused further (pcg.cu).  24 iterations, float-
+// float product, with / without, by rows x RHS, FP64 preconditioner: 182,000 (45^3 x
+// 2) 3.25 / 4.21 ms; 375,000 (50^3 x 3) 5.19 / 5.59; 547,000 (45^3 x 6) 5.52 / 6.07;
+// 702,000 (56^3 x 4) 6.98 / 7.27; 750,000 (50^3 x 6) 7.21 / 7.63; 786,000 (64^3 x 3)
+// 9.35 / 9.13; 1.05M (64^3 x 4) 9.55 / 9.26; 2.1M (64^3 x 8) 14.4 / 12.9.  FP32: 702,000
+// 5.60 / 6.18; 1.05M 7.63 / 7.71; 1.4M (56^3 x 8) 9.59 / 9.22.
+constexpr int64_t kSmallWork = 750 << 10;
 
 // Launch `kernel` on the context's stream so that, for small work, its blocks
 // may become resident while the kernel before it drains (the kernel calls
