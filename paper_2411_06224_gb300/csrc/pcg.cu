@@ -262,11 +262,6 @@ extern "C" int gs_pcg_solve(gs_ctx ctx, gs_mat mat, gs_mas mas, const double* b,
   GS_TRY(ctx->scratch_buf(kSlotPcgVectors, (ff ? 5 : 4) * vbytes, (void**)&vec));
   double *r = vec, *z = r + nrhs * len, *p = z + nrhs * len, *Ap = p + nrhs * len;
   float2* ps = (float2*)(Ap + nrhs * len);  // float-float operand (same size as a vector)
-  bool fused_spmv = nrhs <= 8 && variant != GS_SPMV_SRBK;
-  if (fused_spmv) {  // the sliced copy, built once per matrix; without one the product is a pass of its own
-    GS_TRY(ensure_sliced(ctx, mat, ff));
-    fused_spmv = ff ? mat->sl_ff != nullptr : mat->sl_f64 != nullptr;
-  }
   // beyond kSmallWork the separate passes are faster: x, r streamed (55 us at
   // 64^3, 8 RHS), restricted (22), r . z streamed (22)
   const bool fused_mas = mas_dot_usable(ctx, mas, nrhs) && (int64_t)mat->n * nrhs <= kSmallWork;
@@ -287,6 +282,13 @@ extern "C" int gs_pcg_solve(gs_ctx ctx, gs_mat mat, gs_mas mas, const double* b,
   double *rl, *zl;
   GS_TRY(mas_level_vectors(ctx, mas, nrhs, &rl, &zl));
   GS_CUDA(cudaMemsetAsync(s, 0, sizeof(PcgScalars), st));
+  // the sliced copy, built once per matrix, last of all: it is optional (without one the
+  // product is a pass of its own) and must not take the room of what is not
+  bool fused_spmv = nrhs <= 8 && variant != GS_SPMV_SRBK;
+  if (fused_spmv) {
+    GS_TRY(ensure_sliced(ctx, mat, ff));
+    fused_spmv = ff ? mat->sl_ff != nullptr : mat->sl_f64 != nullptr;
+  }
   if (!fused_spmv) {
     if (variant != GS_SPMV_SRBK) GS_TRY(ensure_row_order(ctx, mat));
     if (ff) GS_TRY(ensure_ff(ctx, mat));

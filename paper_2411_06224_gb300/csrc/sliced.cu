@@ -116,17 +116,15 @@ __global__ void __launch_bounds__(256) k_slice_values(const int32_t* __restrict_
   }
 }
 
-// The device has no room for the copy: none is kept, and the error of that one
-// allocation does not stand.
+// The device has no room for the copy: none is kept (nor tried again for this row
+// order), and the error of that one allocation does not stand.
 static int no_room(gs_ctx ctx, gs_mat m) {
   if (cudaPeekAtLastError() != cudaErrorMemoryAllocation) return GS_ERR_CUDA;
   cudaGetLastError();
-  const int window = m->sl_window;
   release_sliced(ctx, m, true);
-  m->sl_window = window;
+  m->sl_window = m->row_order_window;
   return GS_OK;
 }
-
 
 // The sliced copy with float-float (ff) or FP64 values, made on first use and
 // kept with the matrix; new values (gs_fem_refill) drop the values only.
@@ -139,12 +137,13 @@ int ensure_sliced(gs_ctx ctx, gs_mat m, bool ff) {
     int32_t* most = nullptr;
     void* temp = nullptr;
     const size_t tb = scan_temp_bytes(slices + 1);
-    GS_TRY(ctx->scratch_buf(kSlotScan, ((size_t)slices + 2) * 4, (void**)&most));
+    if (ctx->scratch_buf(kSlotScan, ((size_t)slices + 2) * 4, (void**)&most) != GS_OK ||
+        ctx->scratch_buf(kSlotSortTemp, tb, &temp) != GS_OK ||
+        ctx->alloc((void**)&m->sl_ptr, ((size_t)slices + 1) * 4) != GS_OK ||
+        ctx->alloc((void**)&m->sl_len, (size_t)std::max(n, 1) * 4) != GS_OK)
+      return no_room(ctx, m);
     int32_t* longest = most + slices + 1;
     GS_CUDA(cudaMemsetAsync(longest, 0, 4, st));
-    GS_TRY(ctx->scratch_buf(kSlotSortTemp, tb, &temp));
-    GS_TRY(ctx->alloc((void**)&m->sl_ptr, ((size_t)slices + 1) * 4));
-    GS_TRY(ctx->alloc((void**)&m->sl_len, (size_t)std::max(n, 1) * 4));
     { GS_PROF(ctx, GS_K_OTHER); k_slice_len<<<ceil_div(32LL * (slices + 1), 256), 256, 0, st>>>(m->row_order, m->row_ptr, m->lo_ptr, n, slices, m->sl_len, most, longest); }
     { GS_PROF(ctx, GS_K_OTHER); GS_TRY(exclusive_scan_i32(st, most, m->sl_ptr, slices + 1, temp, tb)); }
     GS_CUDA(cudaMemcpyAsync(ctx->h_pinned + 8, m->sl_ptr + slices, 4, cudaMemcpyDeviceToHost, st));
