@@ -40,6 +40,27 @@ TOL = 1e-6
 METRIC = "Newton solves/s to 1e-6 rel. residual (FP64 vs mixed MAS-PCG); SpMV HBM GB/s"
 
 
+# what brief() leaves out beside lists and long texts
+DETAILS = {"phase_ms", "phase_ms_one_step", "phase_ms_one_solve", "launches_one_step", "kernels", "roofline", "host",
+           "clocks"}
+
+
+def brief(form):
+    """A form's record without its tables, lists and long texts, numbers to five digits."""
+    out = {}
+    for k, v in form.items():
+        if isinstance(v, dict) and k not in DETAILS:
+            v = brief(v)
+            if v:
+                out[k] = v
+        elif isinstance(v, bool) or (isinstance(v, str) and (len(v) <= 60 or k == "error")):
+            out[k] = v
+        elif hasattr(v, "item") or isinstance(v, (int, float)):
+            v = v.item() if hasattr(v, "item") else v
+            out[k] = float(f"{v:.5g}") if isinstance(v, float) else v
+    return out
+
+
 def _json_scalar(o):
     """numpy scalars in the output line as plain numbers."""
     if hasattr(o, "item"):
@@ -1689,7 +1710,10 @@ def main():
             line["cpu_baseline"] = {"value": None, "error": str(e)[:300]}
     B.gs_destroy(ctx)
     if rank == 0:
-        print(json.dumps(line, default=_json_scalar))
+        # the forms' whole records (16 KB) go to stderr: a line that long is cut by what reads it
+        print("forms: " + json.dumps(line["forms"], default=_json_scalar), file=sys.stderr, flush=True)
+        line["forms"] = brief(line["forms"])
+        print(json.dumps(line, default=_json_scalar), flush=True)
     if world > 1:
         dist.destroy_process_group()
 
