@@ -65,9 +65,9 @@ struct gs_fem_s {
   int64_t U_e = 0;
   uint64_t* e_keys = nullptr;  // U_e unique element keys, ascending
   int32_t* e_start = nullptr;  // V + 1: first sorted input of every row
-  int32_t* e_long = nullptr;   // [0], [1] counts; rows of more than kPiece inputs from the front, of more than
-                               // kRowSerial from the back
-  int32_t n_long_rows = 0, n_huge_rows = 0;
+  int32_t* e_long = nullptr;   // [0..2] counts (long, huge, longer); rows of more than kPiece inputs from the front,
+                               // of more than kRowSerial (huge) from the back
+  int32_t n_long_rows = 0, n_longer_rows = 0, n_huge_rows = 0;  // longer: of more than kRowMid
   int64_t long_cap = 0;        // entries of e_long
   double* e_vals = nullptr;    // n_in * 9 input blocks (numeric scratch)
   double* forces = nullptr;    // T * 12 node forces of the elements
@@ -600,22 +600,24 @@ __global__ void __launch_bounds__(256) k_reduce_rows(const uint32_t* __restrict_
   if (lane < 9) R[(size_t)cd * 9 + lane] = cv;
 }
 
-// Rows of more than kPiece entries, a block each.
-__global__ void __launch_bounds__(32 * kRowWarps) k_reduce_long_rows(const uint32_t* __restrict__ sidx,
-                                                                     const int32_t* __restrict__ O,
-                                                                     const int32_t* __restrict__ start,
-                                                                     const int32_t* __restrict__ rows,
-                                                                     const double* __restrict__ vals,
-                                                                     double* __restrict__ R) {
-  __shared__ uint32_t s_idx[kRowWarps][kRowPiece];
-  __shared__ int32_t s_dst[kRowWarps][kRowPiece];
-  __shared__ RowEnds ends;
+// Rows of more than kPiece entries, a block each; those of the other kWarps return.
+template <int kWarps>
+__global__ void __launch_bounds__(32 * kWarps) k_reduce_long_rows(const uint32_t* __restrict__ sidx,
+                                                                  const int32_t* __restrict__ O,
+                                                                  const int32_t* __restrict__ start,
+                                                                  const int32_t* __restrict__ rows,
+                                                                  const double* __restrict__ vals,
+                                                                  double* __restrict__ R) {
+  __shared__ uint32_t s_idx[kWarps][kRowPiece];
+  __shared__ int32_t s_dst[kWarps][kRowPiece];
+  __shared__ RowEnds<kWarps> ends;
   const int32_t r = rows[blockIdx.x];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int32_t i0 = start[r], len = start[r + 1] - i0;
-  const int per = row_piece(len), p0 = w * per, m = max(0, min(per, len - p0));
+  if (!row_is_mine<kWarps>(len)) return;  // whole block
+  const int per = row_piece<kWarps>(len), p0 = w * per, m = max(0, min(per, len - p0));
   load_piece(sidx, O, i0 + p0, m, s_idx[w], s_dst[w], lane);
-  sum_row_block(vals, s_idx[w], s_dst[w], m, R, &ends, w, lane);
+  sum_row_block<kWarps>(vals, s_idx[w], s_dst[w], m, R, &ends, w, lane);
 }
 
 // Rows of more than kRowSerial entries (a vertex of thousands of elements): as many
@@ -660,8 +662,10 @@ __global__ void k_long_rows(const int32_t* __restrict__ start, int32_t n_rows, i
   const int32_t len = r < n_rows ? start[r + 1] - start[r] : 0;
   if (len > kRowSerial)
     long_rows[cap - 1 - atomicAdd(long_rows + 1, 1)] = r;
-  else if (len > kPiece)
-    long_rows[2 + atomicAdd(long_rows, 1)] = r;
+  else if (len > kPiece) {
+    long_rows[3 + atomicAdd(long_rows, 1)] = r;
+    if (len > kRowMid) atomicAdd(long_rows + 2, 1);
+  }
 }
 
 __global__ void k_add_blocks(const int32_t* __restrict__ pos, const double* __restrict__ src, int64_t n,
@@ -1197,9 +1201,13 @@ int refill(gs_ctx ctx, gs_fem f, const double* x, gs_mat m) {
     GS_PROF(ctx, GS_K_ASSEMBLE);
     if (f->n_in) k_reduce_rows<<<ceil_div(32LL * f->V, 256), 256, 0, st>>>(f->e_sidx, f->O_m, f->e_start, f->V, f->e_vals, m->au);
   }
-  if (f->n_long_rows) {
+  if (f->n_long_rows > f->n_longer_rows) {
     GS_PROF(ctx, GS_K_ASSEMBLE);
-    k_reduce_long_rows<<<f->n_long_rows, 32 * kRowWarps, 0, st>>>(f->e_sidx, f->O_m, f->e_start, f->e_long + 2, f->e_vals, m->au);
+    k_reduce_long_rows<kMidWarps><<<f->n_long_rows, 32 * kMidWarps, 0, st>>>(f->e_sidx, f->O_m, f->e_start, f->e_long + 3, f->e_vals, m->au);
+  }
+  if (f->n_longer_rows) {
+    GS_PROF(ctx, GS_K_ASSEMBLE);
+    k_reduce_long_rows<kRowWarps><<<f->n_long_rows, 32 * kRowWarps, 0, st>>>(f->e_sidx, f->O_m, f->e_start, f->e_long + 3, f->e_vals, m->au);
   }
   if (f->n_huge_rows) {
     GS_PROF(ctx, GS_K_ASSEMBLE);
@@ -1315,12 +1323,14 @@ int gs_fem_create(gs_ctx ctx, int32_t n_vertices, int64_t n_tets, const double* 
     if ((s = ctx->alloc((void**)&f->e_keys, (size_t)f->U_e * 8))) return fail(s);
     { GS_PROF(ctx, GS_K_ASSEMBLE); k_unique_keys<<<ceil_div(n, 256), 256, 0, st>>>(skeys, f->e_O, n, f->e_keys); }
     if ((s = ctx->alloc((void**)&f->e_start, (size_t)(V + 1) * 4)) ||
-        (s = ctx->alloc((void**)&f->e_long, (size_t)(f->long_cap = n / kPiece + 2) * 4)))
+        (s = ctx->alloc((void**)&f->e_long, (size_t)(f->long_cap = n / kPiece + 3) * 4)))
       return fail(s);
     { GS_PROF(ctx, GS_K_ASSEMBLE); k_row_starts<<<ceil_div(n + 1, 256), 256, 0, st>>>(f->e_keys, f->e_O, n, f->shift, V, f->e_start); }
-    if (cudaMemsetAsync(f->e_long, 0, 8, st) != cudaSuccess) return fail(GS_ERR_CUDA);
+    if (cudaMemsetAsync(f->e_long, 0, 12, st) != cudaSuccess) return fail(GS_ERR_CUDA);
     { GS_PROF(ctx, GS_K_ASSEMBLE); k_long_rows<<<ceil_div(V, 256), 256, 0, st>>>(f->e_start, V, f->long_cap, f->e_long); }
-    if ((s = read_i32(ctx, f->e_long, &f->n_long_rows)) || (s = read_i32(ctx, f->e_long + 1, &f->n_huge_rows))) return fail(s);
+    if ((s = read_i32(ctx, f->e_long, &f->n_long_rows)) || (s = read_i32(ctx, f->e_long + 1, &f->n_huge_rows)) ||
+        (s = read_i32(ctx, f->e_long + 2, &f->n_longer_rows)))
+      return fail(s);
     if ((s = check_flags(ctx, "gs_fem_create"))) return fail(s);
   }
   if ((s = merge_pattern(ctx, f))) return fail(s);

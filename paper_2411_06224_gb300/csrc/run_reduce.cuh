@@ -12,10 +12,11 @@
 // addition for the whole warp.  A group per run left the warp waiting for the
 // longest run (the diagonal's) at three times the additions.
 // A warp alone needs 12 us for 256 entries, one batch of loads after the other, so a
-// longer row is shared by the 32 warps of a block: 20,000 inputs with a row of 4,000
-// assembled in 369 us by one warp, 137 so; numeric assembly of a fan of 1,000 tets (a
-// row of 4,000 inputs) 287 and 103; the 40^3 body with 1,000 affine cubes, whose rows
-// of bodies are 257 to 500 inputs long, 633 and 584.
+// longer row is shared by the 8 or 32 warps of a block: 20,000 inputs with a row of 4,000
+// assembled in 369 us by one warp, 119 so; numeric assembly of a fan of 1,000 tets (a
+// row of 4,000 inputs) 287 and 102; the 40^3 body with 1,000 affine cubes, whose rows
+// of bodies are 257 to 500 inputs long, 633 and 587; 1M inputs on 3,000 rows 355 and 194
+// (325 with 32 warps to every row).
 #pragma once
 
 #include "primitives.cuh"
@@ -23,9 +24,9 @@
 namespace gs {
 
 constexpr int kPiece = 256;      // entries that a warp sums at a time, and the longest row of a warp alone
-constexpr int kRowWarps = 32;    // warps that share a longer row
-constexpr int kRowPiece = 128;   // entries of it that one of them sums
-constexpr int kRowSerial = kRowWarps * kRowPiece;  // longest row of a block, summed in a fixed order
+constexpr int kRowPiece = 128;   // entries of a longer row that one of a block's warps sums
+constexpr int kMidWarps = 8, kRowMid = kMidWarps * kRowPiece;      // rows of a block of 8 warps
+constexpr int kRowWarps = 32, kRowSerial = kRowWarps * kRowPiece;  // longest row of a block, summed in a fixed order
 
 template <bool kAtomic>
 __device__ __forceinline__ void put_sum(double* dst, double v) {
@@ -107,21 +108,30 @@ __device__ __forceinline__ void sum_piece(const double* __restrict__ blocks, con
   sum_piece<kAtomic>(blocks, s_idx, s_dst, m, R, cv, cd, -1, none, lane);
 }
 
-// A row shared by the kRowWarps warps of a block, warp w its piece w of row_piece(len)
-// entries (fewer, or none, at the row's end).
-__device__ __forceinline__ int row_piece(int len) { return (len + kRowWarps - 1) / kRowWarps; }
+// A row shared by the kWarps warps of a block (8 for up to kRowMid entries, else 32),
+// warp w its piece w of row_piece(len) entries (fewer, or none, at the row's end).
+template <int kWarps>
+__device__ __forceinline__ bool row_is_mine(int len) {
+  return kWarps == kMidWarps ? len <= kRowMid : len > kRowMid;
+}
+template <int kWarps>
+__device__ __forceinline__ int row_piece(int len) {
+  return (len + kWarps - 1) / kWarps;
+}
 
 // The first and last runs of the block's pieces, which may go on in the next piece.
+template <int kWarps>
 struct RowEnds {
-  double first[kRowWarps][9], last[kRowWarps][9];
-  int32_t fd[kRowWarps], ld[kRowWarps];
+  double first[kWarps][9], last[kWarps][9];
+  int32_t fd[kWarps], ld[kWarps];
 };
 
 // Whole block: sums of the row's runs from each warp's piece of m entries; the pieces'
 // ends are joined in order by the first warp.
+template <int kWarps>
 __device__ __forceinline__ void sum_row_block(const double* __restrict__ blocks, const uint32_t* s_idx,
-                                              const int32_t* s_dst, int m, double* __restrict__ R, RowEnds* e, int w,
-                                              int lane) {
+                                              const int32_t* s_dst, int m, double* __restrict__ R, RowEnds<kWarps>* e,
+                                              int w, int lane) {
   if (m > 0) {  // whole warp
     const int32_t open = s_dst[0];
     double cv = 0.0, ov = 0.0;
@@ -136,7 +146,7 @@ __device__ __forceinline__ void sum_row_block(const double* __restrict__ blocks,
   if (w > 0 || lane >= 9) return;
   double cv = 0.0;
   int32_t cd = -1;
-  for (int i = 0; i < kRowWarps && e->fd[i] >= 0; ++i) {
+  for (int i = 0; i < kWarps && e->fd[i] >= 0; ++i) {
     const int32_t f = e->fd[i], l = e->ld[i];
     if (cd >= 0 && cd != f) R[(size_t)cd * 9 + lane] = cv;
     cv = (cd == f ? cv : 0.0) + e->first[i][lane];
