@@ -171,7 +171,7 @@ __device__ __forceinline__ void jacobi_rotate_start(float (&a)[3][3], float (&h)
 // bounds the element kernels, and four of the five sweeps only find an angle.
 // Four FP32 sweeps of A less its mean diagonal give a rotation to about 2^-22,
 // its quaternion is normalised in FP64, and what is left of R^T A R takes one
-// or two FP64 sweeps at small angles.  k_element_hessians, 178,000 tets: 627 us
+// or two FP64 sweeps at small angles.  k_element_hessians, 148,955 tets: 627 us
 // with all sweeps in FP64 and the 3x3 block always decomposed, 400 now.
 __device__ __forceinline__ void sym_eig3(double (&A)[3][3], double (&Q)[3][3]) {
 #pragma unroll

@@ -21,8 +21,10 @@
 //   * z_ik = 2^(a_i + b_k - 72) sum_{s=2..9} G_s 256^(9-s), combined in
 //     64-bit integers (two halves) and rounded once to a double in integer
 //     arithmetic, so the epilogue spends one FP64 add (the coarse levels).
-// Dropped terms (p + q > 9) and the roundings of X, Y are below 2^-54 of the
-// row and column maxima, the level of FP64's own rounding.
+// The roundings of X and Y move z_ik by at most 2^(a_i - 57) sum_j |r_jk| + 2^(b_k - 57)
+// sum_j |M_ij|, half a unit of each operand against the other, and the dropped terms
+// (p + q > 9) by 2^(a_i + b_k - 57): within the bound of the sum in FP64, 96 2^-53 of
+// the row's and column's largest, and 96 2^-57 of 2^(a_i + b_k) altogether.
 //
 // One CTA of 256 threads per domain.  The digit bytes come into a shared-memory
 // ring by bulk asynchronous copies; two threads per row read them, expand them

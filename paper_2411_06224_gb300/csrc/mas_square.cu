@@ -9,8 +9,10 @@
 //   G_s = sum_{p + q = s} (X^p)^T X^q,  s = 2 .. 9,
 // products of digits <= 2^14, 96 terms, <= 7 pairs: exact in FP32.  M^-1_ij =
 // 2^(c_i + c_j - 72) sum_s G_s 256^(9-s), combined in 64-bit integers and rounded
-// once.  Dropped terms and the roundings of X are below 2^-54 of 2^(c_i + c_j),
-// and 2^(2 c_i) <= 4 M^-1_ii 4: below FP64's own rounding of the sum, 96 2^-53.
+// once.  The roundings of X, 96 of half a unit on either operand against magnitudes
+// up to 2^55, come to 96 2^-57 of 2^(c_i + c_j) at most, the dropped terms to 2^-57;
+// 2^(2 c_i) <= 16 max W_ki^2 <= 16 M^-1_ii, so the bound is 96 2^-53 sqrt(M^-1_ii
+// M^-1_jj), that of the sum in FP64 (2^-57 16 beyond it).
 //
 // The groups 2 .. 6 fill the tensor memory (5 x 96 of 512 columns); 2 .. 5 are read
 // as the result's high part while 6 is formed, then 7 .. 9 take their place.  W is

@@ -15,7 +15,7 @@
 // the same fixed order, so all see the same bits.  What a kernel reads that is
 // older than the kernel just before it is loaded before that one has ended.
 // Per iteration, before and now: 16^3, 4 RHS 110 / 42 us; 40^3, 4 RHS, FP32
-// preconditioner 205 / 122; 45^3, 1 RHS 197 / 152; 64^3, 8 RHS 655 / 603.
+// preconditioner 205 / 119; 45^3, 1 RHS 197 / 121; 64^3, 8 RHS 655 / 547.
 #include <algorithm>
 
 #include "common.cuh"
