@@ -500,7 +500,8 @@ def kernel_lines(B, ctx, dev, clk, spmv, prec, nrhs, N, V, nnzb, ndom, mp, live,
         kname = "k_pcg_spmv" if nrhs <= 8 else ("k_spmv_ff_ws" if spmv_ws else "k_spmv_ff_row")
         spmv_line = {"bound": "alu", "achieved": ff_inst / t_spmv / 1e12, "peak": fp32_peak,
                      "unit": "T FP32 instructions/s", "frac": ff_inst / t_spmv / 1e12 / fp32_peak,
-                     "traffic": (recorded_traffic(kname, f"{traffic_key},ff_rhs{B.gs_tune_get(ctx, B.GS_TUNE_SPMV_FF_RHS)}")
+                     "traffic": (recorded_traffic(kname, traffic_key if kname == "k_pcg_spmv" else
+                                                  f"{traffic_key},ff_rhs{B.gs_tune_get(ctx, B.GS_TUNE_SPMV_FF_RHS)}")
                                  if traffic_key else None),
                      "hbm_gbs": spmv_bytes / t_spmv / 1e9, "hbm_frac": spmv_bytes / t_spmv / 1e9 / hbm,
                      "fp64_equivalent_tflops": spmv_flops / t_spmv / 1e12,
