@@ -1003,7 +1003,7 @@ def newton_form(args, B, dev, clk):
                            "ms_refill_element_kernels": kms[B.GS_K_ELEMENT] / reps,
                            "ms_refill_reduction": kms[B.GS_K_ASSEMBLE] / reps,
                            "resort": "gs_fem_triplets (same element kernel, triplets copied out) + gs_assemble "
-                                     "(key encode, radix sort, run flags, scan, segmented reduction)"}
+                                     "(inputs counted and scattered by row, rows sorted, row reduction)"}
         # the Newton loop
         def newton_run():
             x = x0.clone()
