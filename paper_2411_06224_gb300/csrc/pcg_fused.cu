@@ -48,19 +48,26 @@ struct Sliced {  // the sliced matrix (sliced.cu)
 // entry's column is loaded one entry ahead, so that its operand's gather leaves
 // with the entry's own values.
 constexpr int kSettle = 16;
-template <bool kFF, int kBL, int kRL, int kR, int kMin>
-__global__ void __launch_bounds__(kT, kMin) k_pcg_spmv(Sliced A, const int32_t* __restrict__ kk,
-                                                       const float2* xs, const double* p, double* __restrict__ Ap,
-                                                       int64_t stride, int nrhs, const PcgScalars* s, Partials pap) {
+template <bool kFF, int kBL, int kRL, int kR, int kThreads, int kMin>
+__global__ void __launch_bounds__(kThreads, kMin) k_pcg_spmv(Sliced A, const int32_t* __restrict__ kk,
+                                                             const float2* xs, const double* p,
+                                                             double* __restrict__ Ap, int64_t stride, int nrhs,
+                                                             const PcgScalars* s, Partials pap) {
   constexpr int G = kBL * kRL;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = lane % G;
   const int bl = sub % kBL, r0 = sub / kBL * kR;
   const int nh = min(kR, nrhs - r0);  // may be <= 0
+  // an FP64 row's sums end up in two of its lanes, half of the right-hand sides each:
+  // half the additions and products of p . Ap (53^3, 7 RHS: 12.55 -> 12.2 ms)
+  constexpr bool kHalves = !kFF && kBL > 1;
+  constexpr int kH = kHalves ? (kR + 1) / 2 : kR;
+  const bool up = kHalves && (bl & 1), holds = bl < (kHalves ? 2 : 1);
+  const int q0 = up ? kH : 0;
   const bool vec = kR % 2 == 0 && (nrhs & 1) == 0;
-  double dot[kR];
+  double dot[kH];
 #pragma unroll
-  for (int q = 0; q < kR; ++q) dot[q] = 0.0;
-  const int64_t chunks = ((int64_t)A.n * G + kT - 1) / kT;
+  for (int q = 0; q < kH; ++q) dot[q] = 0.0;
+  const int64_t chunks = ((int64_t)A.n * G + kThreads - 1) / kThreads;
   // blocks take one chunk of every gridDim.x, another place of it each time
   // (rows are ordered by length within windows: the same place would always
   // meet the same lengths)
@@ -69,7 +76,7 @@ __global__ void __launch_bounds__(kT, kMin) k_pcg_spmv(Sliced A, const int32_t* 
   int64_t base;  // entry 0 of the row
   auto open_row = [&](int64_t i) {
     const int64_t c = i * gridDim.x + (blockIdx.x + i * 37) % gridDim.x;
-    const int64_t slot = c * (kT / G) + threadIdx.x / G;
+    const int64_t slot = c * (kThreads / G) + threadIdx.x / G;
     const bool in = c < chunks && slot < A.n && nh > 0;
     len = in ? A.len[slot] : 0;
     base = in ? (int64_t)A.ptr[slot >> 5] * 32 + (slot & 31) : 0;
@@ -131,15 +138,22 @@ __global__ void __launch_bounds__(kT, kMin) k_pcg_spmv(Sliced A, const int32_t* 
           }
       }
 #pragma unroll
-      for (int o = kBL / 2; o > 0; o >>= 1)
+      for (int o = kBL / 2; o > 1; o >>= 1)
 #pragma unroll
         for (int q = 0; q < kR * 3; ++q) y[q] += __shfl_xor_sync(kFull, y[q], o, kBL);
-    }
-    if (in && bl == 0) {
+      if (kHalves)
 #pragma unroll
-      for (int q = 0; q < kR; ++q)
-        if (q < nh) {
-          const int64_t o = (r0 + q) * stride + 3 * (int64_t)row;
+        for (int q = 0; q < kH * 3; ++q) {
+          const double hi = q + 3 * kH < 3 * kR ? y[q + 3 * kH] : 0.0;
+          const double other = __shfl_xor_sync(kFull, up ? y[q] : hi, 1, kBL);
+          y[q] = (up ? hi : y[q]) + other;
+        }
+    }
+    if (in && holds) {
+#pragma unroll
+      for (int q = 0; q < kH; ++q)
+        if (q0 + q < nh) {
+          const int64_t o = (r0 + q0 + q) * stride + 3 * (int64_t)row;
 #pragma unroll
           for (int j = 0; j < 3; ++j) {
             Ap[o + j] = y[3 * q + j];
@@ -149,18 +163,18 @@ __global__ void __launch_bounds__(kT, kMin) k_pcg_spmv(Sliced A, const int32_t* 
     }
   }
   let_next_kernel_launch();
-  __shared__ double red[kWarps][8];
+  __shared__ double red[kThreads / 32][8];
 #pragma unroll
-  for (int q = 0; q < kR; ++q) {
+  for (int q = 0; q < kH; ++q) {
 #pragma unroll
     for (int o = G; o < 32; o <<= 1) dot[q] += __shfl_xor_sync(kFull, dot[q], o);
-    if (lane < G && bl == 0) red[w][r0 + q] = dot[q];
+    if (lane < G && holds && q0 + q < kR) red[w][r0 + q0 + q] = dot[q];
   }
   __syncthreads();
   if ((int)threadIdx.x < nrhs) {
     double v = 0.0;
 #pragma unroll
-    for (int i = 0; i < kWarps; ++i) v += red[i][threadIdx.x];
+    for (int i = 0; i < kThreads / 32; ++i) v += red[i][threadIdx.x];
     pap.sum[threadIdx.x * pap.pitch + blockIdx.x] = v;
   }
 }
@@ -181,6 +195,12 @@ __global__ void __launch_bounds__(kT, kMin) k_pcg_spmv(Sliced A, const int32_t* 
 // the other rows' sums cost more.  24 iterations at 64^3, 4 RHS, FP64, with one row of
 // 327 / 627 / 3,027 blocks, 1 lane and 4: 18.5 / 27.6 / 100 and 14.1 / 16.1 / 32.7 ms
 // (15.4 with one lane and a row of 227); 40^3, 1 RHS, 3,027: 2 lanes 31.2, 4 17.5.
+// The FP64 product of 3, 5 and 7 right-hand sides in a lane goes out in blocks of 128
+// threads, twice as many, where a block has few chunks: the last round is then better
+// shared.  FP64 row product, FP32 preconditioner, 256 / 128 threads: 6 RHS (2 x 3) 50^3
+// 9.2 / 8.7 ms, 60^3 14.0 / 13.3, 64^3 15.0 / 15.1, 76^3 22.8 / 23.9; 7 RHS, 2 lanes,
+// 44^3 7.6 / 7.1, 53^3 12.2 / 11.7, 56^3 12.7 / 12.7, 60^3 14.8 / 15.1; 1 lane 64^3
+// 16.1 / 17.9.
 constexpr int32_t kHubRow = 192;
 template <bool kFF, int kRL, int kR>
 static int launch_spmv(gs_ctx ctx, gs_mat m, const float2* xs, const double* p, double* Ap, int nrhs,
@@ -189,18 +209,29 @@ static int launch_spmv(gs_ctx ctx, gs_mat m, const float2* xs, const double* p, 
   const int64_t rows = (int64_t)m->n * kRL, sms = std::max(ctx->sm_count, 1);
   const int bl = rows * 4 <= sms * 512 || m->sl_longest > kHubRow ? 4 : (rows * 2 <= sms * (kR > 3 ? 3072 : 2048) ? 2 : 1);
   constexpr int kMin = kR > 3 ? 2 : (kFF && kR < 3 ? 4 : 3);
-  const int64_t chunks = ((int64_t)m->n * kRL * bl + kT - 1) / kT;
-  pap.n = (int)std::max<int64_t>(1, std::min<int64_t>({chunks, (int64_t)kMin * std::max(ctx->sm_count, 1),
-                                                       (int64_t)kMaxRedBlocks}));
-  auto go = [&](auto kernel) {
-    return launch_chained(ctx, (int64_t)m->n * nrhs, kernel, dim3(pap.n), dim3(kT), 0, A, m->ff_k, xs, p, Ap,
+  auto go = [&](auto kernel, int threads, int per_sm) {
+    const int64_t chunks = (rows * bl + threads - 1) / threads;
+    pap.n = (int)std::max<int64_t>(1, std::min<int64_t>({chunks, per_sm * sms, (int64_t)kMaxRedBlocks}));
+    return launch_chained(ctx, (int64_t)m->n * nrhs, kernel, dim3(pap.n), dim3(threads), 0, A, m->ff_k, xs, p, Ap,
                           3LL * m->n, nrhs, s, pap);
   };
   cudaError_t e = cudaSuccess;
+  if constexpr (!kFF && kR >= 3) {
+    const bool few = rows * bl <= sms * (kR > 3 ? 2048 : 3072);  // lanes in all
+    if (few && bl == 2) {
+      GS_CUDA(go(k_pcg_spmv<kFF, 2, kRL, kR, kT / 2, 2 * kMin>, kT / 2, 2 * kMin));
+      return GS_OK;
+    }
+    if constexpr (kR == 3)
+      if (few && bl == 1) {
+        GS_CUDA(go(k_pcg_spmv<kFF, 1, kRL, kR, kT / 2, 2 * kMin>, kT / 2, 2 * kMin));
+        return GS_OK;
+      }
+  }
   switch (bl) {
-    case 1: e = go(k_pcg_spmv<kFF, 1, kRL, kR, kMin>); break;
-    case 2: e = go(k_pcg_spmv<kFF, 2, kRL, kR, kMin>); break;
-    default: e = go(k_pcg_spmv<kFF, 4, kRL, kR, kMin>); break;
+    case 1: e = go(k_pcg_spmv<kFF, 1, kRL, kR, kT, kMin>, kT, kMin); break;
+    case 2: e = go(k_pcg_spmv<kFF, 2, kRL, kR, kT, kMin>, kT, kMin); break;
+    default: e = go(k_pcg_spmv<kFF, 4, kRL, kR, kT, kMin>, kT, kMin); break;
   }
   GS_CUDA(e);
   return GS_OK;
@@ -214,11 +245,12 @@ static int launch_spmv_rhs(gs_ctx ctx, gs_mat m, const float2* xs, const double*
   // Odd counts and 6 leave places of 2 x 2 or 4 x 2 empty, and an instruction costs the
   // same for a lane without a right-hand side: other shares, but not on systems so
   // small that lanes are what is missing (12^3, 5 RHS: 1.1 ms with 4 lanes of 2, 1.2
-  // with 2 of 3), nor where 7 in one lane leave too few (32^3: 3.9 and 4.2).  24
-  // iterations at 64^3, FP32 preconditioner, with the shares of 4 and 8 / these / the
-  // former product: row 3 RHS 10.7 / 10.0 / 10.4 ms, 5 17.5 / 12.6 / 13.6, 6 17.8 / 15.1 /
-  // 15.2, 7 18.2 / 16.0 / 17.0; float-float 3 RHS 7.6 / 7.1 / 9.0, 5 10.9 / 9.3 / 10.5, 6
-  // 10.7 / 9.9 / 11.0.
+  // with 2 of 3), nor where 7 in one lane leave too few (32^3: 3.4 and 3.7 ms; 34^3 4.3
+  // and 3.9).  24 iterations at 64^3, FP32 preconditioner, with the shares of 4 and 8 /
+  // these / the former product: row 3 RHS 10.7 / 9.8 / 10.5 ms, 5 17.5 / 12.6 / 13.6, 6
+  // 17.8 / 15.0 / 15.2, 7 18.2 / 16.0 / 17.0; float-float 3 RHS 7.6 / 7.1 / 9.0, 5 10.9 /
+  // 9.3 / 10.5, 6 10.7 / 9.9 / 11.0.  Row product, 53^3: 5 RHS 8.9 (former 9.6), 6 10.6
+  // (10.7), 7 11.7 (11.7).
   if (m->n >= 4096) {
     if (kFF) {
       if (nrhs == 3) return launch_spmv<true, 1, 3>(ctx, m, xs, p, Ap, nrhs, s, pap);
@@ -227,7 +259,7 @@ static int launch_spmv_rhs(gs_ctx ctx, gs_mat m, const float2* xs, const double*
       if (nrhs == 3) return launch_spmv<false, 1, 3>(ctx, m, xs, p, Ap, nrhs, s, pap);
       if (nrhs == 5) return launch_spmv<false, 1, 5>(ctx, m, xs, p, Ap, nrhs, s, pap);
       if (nrhs == 6) return launch_spmv<false, 2, 3>(ctx, m, xs, p, Ap, nrhs, s, pap);
-      if (nrhs == 7 && m->n > 512LL * ctx->sm_count) return launch_spmv<false, 1, 7>(ctx, m, xs, p, Ap, nrhs, s, pap);
+      if (nrhs == 7 && m->n > 256LL * ctx->sm_count) return launch_spmv<false, 1, 7>(ctx, m, xs, p, Ap, nrhs, s, pap);
     }
   }
   if (nrhs <= 4) return launch_spmv<kFF, 2, 2>(ctx, m, xs, p, Ap, nrhs, s, pap);
